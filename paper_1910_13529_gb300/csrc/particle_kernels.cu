@@ -688,10 +688,10 @@ __device__ __forceinline__ void push_deposit_2d_chunks(const GridP& g, const Spe
         const int fzl = any ? ((box[1] + 1 - fz0 + 3) & ~3) : 0, fxl = any ? box[3] - box[2] + 1 : 0;
         const int fvol = fzl * fxl;
         const bool ftile = any && 6 * fvol <= F_CAP && fxl <= g.nx + 2 * K;
-        // current box: every deposition window lies within one node below and two above the
-        // gather stencils (the move is under one cell per axis)
+        // current box: every deposition window starts at most one node below the gather stencils and
+        // its K + 1 nodes end at most one node above them (the move is under one cell per axis)
         const int jz0 = any ? ((box[0] - 1) & ~3) : 0, jx0 = box[2] - 1;
-        const int jzl = any ? ((box[1] + 3 - jz0 + 3) & ~3) : 0, jxl = any ? box[3] - box[2] + 4 : 0;
+        const int jzl = any ? ((box[1] + 2 - jz0 + 3) & ~3) : 0, jxl = any ? box[3] - box[2] + 3 : 0;
         const int jvol = jzl * jxl;
         const bool jtile = any && 3 * jvol <= J_CAP && jxl <= g.nx + 2 * KW;
         float2* P1 = reinterpret_cast<float2*>(sF);
@@ -935,8 +935,10 @@ __device__ __forceinline__ void push_deposit_2d_chunks(const GridP& g, const Spe
 // constant divisors.  A chunk of 256 particles sorted in 4 x 4 x 4-cell tiles spans at most three
 // tiles of a uniform 2-per-cell plasma (chunk and tile boundaries do not line up); three tiles
 // along z, whatever their alignment to the 4-cell groups after window shifts, need at most 18 x 7 x 7
-// field nodes and 21 x 10 x 10 current nodes.  A chunk whose boxes do not fit (a tile row ends
-// inside it, sparse regions, particles injected since the last sort) takes the general path.  The current box is cleared once when the
+// field nodes and 20 x 9 x 9 current nodes: both boxes leave room for one cell of drift along x and y
+// between sorts (in the developed wake of the 512 x 256 x 256 run 17% of the chunks use it).  A chunk
+// whose boxes do not fit (a tile row ends inside it, sparse regions, particles injected since the last
+// sort) goes on a list.  The current box is cleared once when the
 // CTA starts and then by the flush that empties it, so a chunk does not clear it again.
 // Field rows hold up to 20 z nodes, current rows up to 24: with row pitches of 20 and 24 words the
 // cells of a sorted warp (4 along z, 4 along x) fall on distinct shared-memory banks (a pitch of
@@ -1112,15 +1114,16 @@ __device__ __forceinline__ void push_deposit_3d_chunks(const GridP& g, const Spe
         const int fz0 = bc[0] & ~3, fx0 = bc[2], fy0 = bc[4];
         const int fzl = bc[1] + 1 - fz0, fxl = bc[3] - bc[2] + 1, fyl = bc[5] - bc[4] + 1;
         const bool ftile = any && fzl <= FZ3 && fxl <= FX3 && fyl <= FY3;
-        // every deposition window lies within one node below and two above the gather stencils
+        // every deposition window lies within one node below and one above the gather stencils: it
+        // starts at the lower of two supports at most one node apart and holds K + 1 nodes
         const int jz0 = (bc[0] - 1) & ~3, jx0 = bc[2] - 1, jy0 = bc[4] - 1;
-        const int jzl = bc[1] + 3 - jz0, jxl = bc[3] - bc[2] + 4, jyl = bc[5] - bc[4] + 4;
+        const int jzl = bc[1] + 2 - jz0, jxl = bc[3] - bc[2] + 3, jyl = bc[5] - bc[4] + 3;
         const bool jtile = any && jzl <= JZ3 && jxl <= JX3 && jyl <= JY3;
         if (DEFER && any && !(ftile && jtile)) {
             // boxes the general path holds in shared memory (its own rounding of the z extents) go to
             // the general kernel's list, the rest (the plasma injected since the last sort: one
             // long row of cells) to the per-particle kernel's list
-            const int gfz = (bc[1] + 1 - fz0 + 3) & ~3, gjz = (bc[1] + 3 - jz0 + 3) & ~3;
+            const int gfz = (bc[1] + 1 - fz0 + 3) & ~3, gjz = (bc[1] + 2 - jz0 + 3) & ~3;
             const bool general = 6 * gfz * fxl * fyl <= F_CAP3 && fxl <= g.nx + 2 * K && fyl <= g.ny + 2 * K &&
                                  3 * gjz * jxl * jyl <= J_CAP3 && jxl <= g.nx + 2 * KW && jyl <= g.ny + 2 * KW;
             int* list = general ? defer : defer2;
@@ -1384,38 +1387,6 @@ __global__ void __launch_bounds__(FUSED_T, 3) push_deposit_3d_kernel(GridP g, Sp
                                         defer, defer2);
 }
 
-// The chunks of defer2 (see push_deposit_3d_chunks): per particle, gather from global memory, push,
-// move and deposit with global atomics (contributions that are exactly zero are not added); a
-// light kernel at full occupancy.  The last CTA to finish clears the list (defer2[1] counts CTAs).
-template <int SHAPE>
-__global__ void __launch_bounds__(FUSED_T, 2) push_deposit_3d_particles_kernel(GridP g, SpeciesP sp,
-                                                                            const float* __restrict__ E,
-                                                                            const float* __restrict__ B,
-                                                                            float* __restrict__ J, int shift,
-                                                                            int* __restrict__ defer2) {
-    const int nd = *(volatile int*)defer2;
-    const long long n = *sp.count;
-    for (int k = blockIdx.x; k < nd; k += gridDim.x) {
-        const long long p = (long long)defer2[2 + k] * FUSED_T + threadIdx.x;
-        if (p >= n) continue;
-        Pos p0, p1;
-        float v3;
-        if (advance_one<3, SHAPE, MODE_FUSED>(g, sp, E, B, shift, p, sp.cap, p0, p1, v3)) {
-            GlobalAcc acc{&g, J};
-            deposit<3, SHAPE>(g, sp.qv, v3, p0, p1, acc);
-        }
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        __threadfence();
-        if (atomicAdd(defer2 + 1, 1) == (int)gridDim.x - 1) {
-            defer2[0] = 0;
-            defer2[1] = 0;
-            __threadfence();
-        }
-    }
-}
-
 constexpr int SMEM_3D_GEN = F_CAP3 + J_CAP3 + 2 * PF3 * FUSED_T;
 
 // .x = sum Wza Wxa Wya Fa, .y = sum Wzb Wxb Wyb Fb over K^3 nodes of [y][x][z] boxes (row fzl,
@@ -1444,13 +1415,14 @@ __device__ __forceinline__ float2 tile_interp3_pair(const float* __restrict__ Fa
     return acc;
 }
 
-// The general path for the chunks push_deposit_3d_kernel leaves (list[0 .. nlist)): boxes of any
-// shape up to F_CAP3 / J_CAP3 words, runtime strides; larger boxes use global memory.
+// The general path for the chunks push_deposit_3d_kernel leaves (list[k0], list[k0 + kst], .. below
+// nlist): boxes of any shape up to F_CAP3 / J_CAP3 words (the main kernel lists no larger ones
+// here), runtime strides.
 template <int SHAPE>
 __device__ __forceinline__ void push_deposit_3d_general(const GridP& g, const SpeciesP& sp,
                                                         const float* __restrict__ E, const float* __restrict__ B,
                                                         float* __restrict__ J, int shift, const int* __restrict__ list,
-                                                        int nlist, float* sF, float* sJ, int* box) {
+                                                        int nlist, int k0, int kst, float* sF, float* sJ, int* box) {
     constexpr int K = Shape<SHAPE>::K;
     constexpr int KW = K + 1;
     const long long n = *sp.count;
@@ -1474,7 +1446,6 @@ __device__ __forceinline__ void push_deposit_3d_general(const GridP& g, const Sp
         cp_async_commit();
     };
     int buf = 0;
-    const int k0 = blockIdx.x, kst = gridDim.x;
     auto chunk_base = [&](int k) { return k < nlist ? (long long)list[k] * FUSED_T : n; };
     prefetch(chunk_base(k0), 0);
     // box[0..6] and box[7..13] serve alternate chunks (see push_deposit_2d_chunks): no barrier at
@@ -1545,8 +1516,8 @@ __device__ __forceinline__ void push_deposit_3d_general(const GridP& g, const Sp
         const int fvol = fzl * fxl * fyl;
         const bool ftile = any && 6 * fvol <= F_CAP3 && fxl <= g.nx + 2 * K && fyl <= g.ny + 2 * K;
         const int jz0 = any ? ((bc[0] - 1) & ~3) : 0, jx0 = bc[2] - 1, jy0 = bc[4] - 1;
-        const int jzl = any ? ((bc[1] + 3 - jz0 + 3) & ~3) : 0;
-        const int jxl = any ? bc[3] - bc[2] + 4 : 0, jyl = any ? bc[5] - bc[4] + 4 : 0;
+        const int jzl = any ? ((bc[1] + 2 - jz0 + 3) & ~3) : 0;
+        const int jxl = any ? bc[3] - bc[2] + 3 : 0, jyl = any ? bc[5] - bc[4] + 3 : 0;
         const int jvol = jzl * jxl * jyl;
         const bool jtile = any && 3 * jvol <= J_CAP3 && jxl <= g.nx + 2 * KW && jyl <= g.ny + 2 * KW;
         // groups (c, y, x, z4) of the [c][y][x][z] box, copied asynchronously (all of a thread's
@@ -1606,7 +1577,7 @@ __device__ __forceinline__ void push_deposit_3d_general(const GridP& g, const Sp
         // ---- gather (E1 z+, E2 x+, E3 y+, B1 x+ y+, B2 z+ y+, B3 z+ x+) ----
         float eb[6];
         if (ok) {
-            if (ftile) {
+            {
                 const float* F = sF;
                 const float2 q1 = tile_interp3_pair<K>(F, bzh - fz0, bxn - fx0, byn - fy0, Wzh, Wxn, Wyn,
                                                        F + 4 * fvol, bzh - fz0, bxn - fx0, byh - fy0, Wzh, Wxn,
@@ -1623,8 +1594,6 @@ __device__ __forceinline__ void push_deposit_3d_general(const GridP& g, const Sp
                 eb[3] = q2.y;
                 eb[2] = q3.x;
                 eb[5] = q3.y;
-            } else {
-                gather<3, SHAPE>(g, E, B, p0, eb);
             }
         }
         // ---- push and move ----
@@ -1703,14 +1672,6 @@ __device__ __forceinline__ void push_deposit_3d_general(const GridP& g, const Sp
                 Py[k] = S0y[k] + 0.5f * DSy[k];
                 Qy[k] = 0.5f * S0y[k] + (1.f / 3.f) * DSy[k];
             }
-            // window origins are >= -2 and below 2^20 - 4 on every axis: an exact 64-bit key
-            const unsigned long long key =
-                ok ? (((unsigned long long)(bz + 4) << 40) | ((unsigned long long)(bx + 4) << 20) |
-                      (unsigned long long)(by + 4))
-                   : (0xFFFFF00000000000ull | (unsigned)threadIdx.x);
-            // direct atomics when at most 4 lanes share a window (144 deposits per particle make
-            // conflicts costlier than in 2D), else sums over runs of lanes first
-            const int gmax = __reduce_max_sync(0xffffffffu, __popc(__match_any_sync(0xffffffffu, key)));
             int* s0 = iJ + ((by - jy0) * jxl + (bx - jx0)) * jzl + (bz - jz0);
             const float MAGIC = 12582912.f;           // 1.5 2^23
             auto terms = [&](auto&& put) {
@@ -1729,18 +1690,7 @@ __device__ __forceinline__ void push_deposit_3d_general(const GridP& g, const Sp
                         }
                     }
             };
-            if (gmax <= 4) {
-                if (ok) terms([&](int o, float biased) { atomicAdd(s0 + o, __float_as_int(biased) - 0x4B400000); });
-            } else {
-                const SegReduce seg = make_segments(key);
-                terms([&](int o, float biased) {
-                    const int v = seg.sum(__float_as_int(biased) - 0x4B400000);
-                    if (seg.head && ok && v != 0) atomicAdd(s0 + o, v);
-                });
-            }
-        } else if (any && !jtile && ok) {
-            GlobalAcc acc{&g, J};
-            deposit<3, SHAPE>(g, sp.qv, 0.f, p0, p1, acc);
+            if (ok) terms([&](int o, float biased) { atomicAdd(s0 + o, __float_as_int(biased) - 0x4B400000); });
         }
         __syncthreads();
         if (jtile && mbits != 0) {
@@ -1770,25 +1720,59 @@ __device__ __forceinline__ void push_deposit_3d_general(const GridP& g, const Sp
     cp_async_wait_all_p();                         // the last (empty) prefetch group
 }
 
-// The chunks push_deposit_3d_kernel deferred (defer[0] of them, chunk indices from defer[2]), on the
-// general path.  The last CTA to finish clears the list (defer[1] counts finished CTAs).
+// Everything push_deposit_3d_kernel left, of all species, in one launch: defer[s][2 ..] holds the
+// chunks for the general path (count in defer[s][0]), defer2[s][2 ..] those whose boxes are beyond it
+// (a chunk of particles that crossed the periodic seam since the last sort).  The latter go per
+// particle (gather from global memory, global atomics, exact zeros not added) in units of one warp,
+// dealt to the CTAs in turn: a warp's scattered atomics pass through its SM one lane at a time, so a
+// chunk's eight warps on eight SMs finish in an eighth of the time of one CTA.  One launch for all
+// species: the few chunks of one species run beside those of the others.
+// The last CTA to finish clears the lists (defer[0][1] counts finished CTAs).
 template <int SHAPE>
-__global__ void __launch_bounds__(FUSED_T, 2) push_deposit_3d_deferred_kernel(GridP g, SpeciesP sp,
+__global__ void __launch_bounds__(FUSED_T, 2) push_deposit_3d_leftover_kernel(GridP g, LeftoverP lp,
                                                                               const float* __restrict__ E,
                                                                               const float* __restrict__ B,
-                                                                              float* __restrict__ J, int shift,
-                                                                              int* __restrict__ defer) {
+                                                                              float* __restrict__ J, int shift) {
     extern __shared__ float4 smem4[];
     float* smem = reinterpret_cast<float*>(smem4);
     __shared__ int box[14];
-    const int nd = *(volatile int*)defer;
-    push_deposit_3d_general<SHAPE>(g, sp, E, B, J, shift, defer + 2, nd, smem, smem + F_CAP3, box);
+    const int grid = (int)gridDim.x;
+    int first = 0;                                   // chunks of the species before this one, modulo the grid
+#pragma unroll 1
+    for (int s = 0; s < lp.n; ++s) {
+        const int nd = *(volatile int*)lp.defer[s];
+        const int k0 = (int)blockIdx.x >= first ? (int)blockIdx.x - first : (int)blockIdx.x - first + grid;
+        if (k0 < nd)
+            push_deposit_3d_general<SHAPE>(g, lp.sp[s], E, B, J, shift, lp.defer[s] + 2, nd, k0, grid, smem,
+                                           smem + F_CAP3, box);
+        first = (first + nd) % grid;
+        __syncthreads();
+    }
+    const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    int item = wid * grid + ((int)blockIdx.x >= first ? (int)blockIdx.x - first : (int)blockIdx.x - first + grid);
+#pragma unroll 1
+    for (int s = 0; s < lp.n; ++s) {
+        const SpeciesP& sp = lp.sp[s];
+        const int nw = *(volatile int*)lp.defer2[s] * (FUSED_T / 32);
+        const long long n = *sp.count;
+        for (; item < nw; item += grid * (FUSED_T / 32)) {
+            const long long p =
+                (long long)lp.defer2[s][2 + item / (FUSED_T / 32)] * FUSED_T + (item % (FUSED_T / 32)) * 32 + lane;
+            Pos p0, p1;
+            float v3;
+            if (p < n && advance_one<3, SHAPE, MODE_FUSED>(g, sp, E, B, shift, p, sp.cap, p0, p1, v3)) {
+                GlobalAcc acc{&g, J};
+                deposit<3, SHAPE>(g, sp.qv, v3, p0, p1, acc);
+            }
+        }
+        item -= nw;
+    }
     __syncthreads();
     if (threadIdx.x == 0) {
         __threadfence();
-        if (atomicAdd(defer + 1, 1) == (int)gridDim.x - 1) {
-            defer[0] = 0;
-            defer[1] = 0;
+        if (atomicAdd(lp.defer[0] + 1, 1) == grid - 1) {
+            for (int s = 0; s < lp.n; ++s) lp.defer[s][0] = lp.defer2[s][0] = 0;
+            lp.defer[0][1] = 0;
             __threadfence();
         }
     }
@@ -2195,26 +2179,42 @@ cudaError_t launch_push(const GridP& g0, const SpeciesP& sp, const float* E, con
                 if (e != cudaSuccess) return e;
                 configured = true;
             }
-            // two lists of deferred chunks, each 2 + ceil(cap / FUSED_T) ints
-            int* defer2 = defer + 2 + (sp.cap + FUSED_T - 1) / FUSED_T;
-            k<<<pblocks(extent), FUSED_T, smem, s>>>(g, sp, E, B, J, shift, defer, defer2);
-            // the deferred chunks: a fixed grid (their count is on the device)
-            auto kd = push_deposit_3d_deferred_kernel<SH>;
-            const size_t smem_d = SMEM_3D_GEN * sizeof(float);
-            static bool configured_d = false;
-            if (!configured_d) {
-                cudaError_t e = cudaFuncSetAttribute(kd, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_d);
-                if (e != cudaSuccess) return e;
-                configured_d = true;
-            }
-            const long long nchunk = (extent + FUSED_T - 1) / FUSED_T;
-            const unsigned nb = (unsigned)(nchunk < 152 * 2 ? (nchunk < 1 ? 1 : nchunk) : 152 * 2);
-            kd<<<nb, FUSED_T, smem_d, s>>>(g, sp, E, B, J, shift, defer);
-            const unsigned nb2 = (unsigned)(nchunk < 152 * 4 ? (nchunk < 1 ? 1 : nchunk) : 152 * 4);
-            push_deposit_3d_particles_kernel<SH><<<nb2, FUSED_T, 0, s>>>(g, sp, E, B, J, shift, defer2);
+            k<<<pblocks(extent), FUSED_T, smem, s>>>(g, sp, E, B, J, shift, defer, defer + defer_len(sp.cap));
         } else {
             push_kernel<ND, SH><<<pblocks(extent), 256, 0, s>>>(g, sp, E, B, shift);
         }
+        return cudaGetLastError();
+    });
+}
+
+cudaError_t launch_push_leftover(const GridP& g0, const SpeciesP* sp, int* const* defer, const long long* extent, int n,
+                                 const float* E, const float* B, float* J, int shift, cudaStream_t s) {
+    const GridP g = prep(g0);
+    LeftoverP lp;
+    lp.n = 0;
+    long long nchunk = 0;
+    for (int i = 0; i < n; ++i) {
+        if (extent[i] <= 0) continue;
+        lp.sp[lp.n] = sp[i];
+        lp.defer[lp.n] = defer[i];
+        lp.defer2[lp.n] = defer[i] + defer_len(sp[i].cap);
+        nchunk += (extent[i] + FUSED_T - 1) / FUSED_T;
+        ++lp.n;
+    }
+    if (lp.n == 0) return cudaSuccess;
+    return dispatch(3, g.shape, [&](auto nd, auto sh) {
+        (void)nd;
+        auto k = push_deposit_3d_leftover_kernel<decltype(sh)::value>;
+        const size_t smem = SMEM_3D_GEN * sizeof(float);
+        static bool configured = false;
+        if (!configured) {
+            cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            if (e != cudaSuccess) return e;
+            configured = true;
+        }
+        // the lists' lengths are on the device: a full grid, or one CTA per warp of a small extent
+        const long long want = nchunk * (FUSED_T / 32);
+        k<<<(unsigned)(want < 152 * 2 ? want : 152 * 2), FUSED_T, smem, s>>>(g, lp, E, B, J, shift);
         return cudaGetLastError();
     });
 }

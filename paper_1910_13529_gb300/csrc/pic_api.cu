@@ -620,19 +620,31 @@ pic_status pic_step(pic_t* h, int nsteps, void* stream) {
             Scope sc(h, PIC_T_DEPOSIT, 1, s);
             CK(h, cudaMemsetAsync(h->J, 0, sizeof(float) * 3 * N, s), "zero J");
         }
+        SpeciesP sps[PIC_MAX_SPECIES];
+        int* defers[PIC_MAX_SPECIES];
+        long long extents[PIC_MAX_SPECIES];
+        int nsp = 0;
         for (int i = 0; i < PIC_MAX_SPECIES; ++i) {
             if (!h->sp[i].bound) continue;
             SpeciesSlot& q = h->sp[i];
             if (h->cfg.ndim == 3 && !q.defer) {
-                const long long len = 2 + (q.cap + 255) / 256;       // two lists of this length
+                const long long len = defer_len(q.cap);              // two lists of this length
                 if ((st = dalloc(h, &q.defer, 2 * len, "deferred chunk lists"))) return st;
                 CK(h, cudaMemsetAsync(q.defer, 0, sizeof(int32_t) * 2, s), "clear deferred chunk list");
                 CK(h, cudaMemsetAsync(q.defer + len, 0, sizeof(int32_t) * 2, s), "clear deferred chunk list");
             }
             SpeciesP sp = species_params(h, i);
-            Scope sc(h, PIC_T_PARTICLES, h->cfg.ndim == 3 ? 3 : 1, s);
+            sps[nsp] = sp;
+            defers[nsp] = q.defer;
+            extents[nsp++] = q.extent;
+            Scope sc(h, PIC_T_PARTICLES, 1, s);
             CK(h, launch_push(h->g, sp, Ec, Bc, h->J, h->pending_shift, 0, q.extent, q.defer, s),
                "fused push/deposit kernel");
+        }
+        if (h->cfg.ndim == 3 && nsp > 0) {
+            Scope sc(h, PIC_T_PARTICLES, 1, s);
+            CK(h, launch_push_leftover(h->g, sps, defers, extents, nsp, Ec, Bc, h->J, h->pending_shift, s),
+               "deferred chunks kernel");
         }
         h->pending_shift = 0;
         if ((st = smooth_current(h, s))) return st;

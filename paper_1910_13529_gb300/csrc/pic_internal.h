@@ -77,6 +77,14 @@ struct SpeciesP {
     float* prev_off;
 };
 
+// The species of a step whose deferred chunks one launch finishes (3D fused mode).
+struct LeftoverP {
+    int n;
+    SpeciesP sp[PIC_MAX_SPECIES];
+    int* defer[PIC_MAX_SPECIES];     // chunks for the general path (count in [0], chunks from [2])
+    int* defer2[PIC_MAX_SPECIES];    // chunks beyond it
+};
+
 // One instance of a batched run: its grid, its (single) species, its two field buffers.
 struct PartInst {
     GridP g;
@@ -126,11 +134,14 @@ cudaError_t launch_correct_j1_batch(const CorrInst* inst, int ninst, int max_row
 cudaError_t launch_push_batch(const PartInst* inst, int ninst, int ndim, int shape, long long max_extent, int parity,
                               cudaStream_t s);
 cudaError_t launch_zero_j_batch(const PartInst* inst, int ninst, long long max_ncell, cudaStream_t s);
-// defer (3D fused mode): library scratch of two lists of 2 + ceil(cap / 256) ints each, their
-// first two ints zero on first use: the chunks whose shared-memory boxes do not fit, processed by
-// the general and the per-particle kernels, which clear the lists.
+// defer (3D fused mode): library scratch of two lists of defer_len(cap) ints each, their first two
+// ints zero on first use: the chunks whose shared-memory boxes do not fit.  launch_push_leftover,
+// after launch_push of every species, processes the lists of all of them and clears them.
+constexpr long long defer_len(long long cap) { return 2 + (cap + 255) / 256; }
 cudaError_t launch_push(const GridP& g, const SpeciesP& sp, const float* E, const float* B,
                         float* J, int shift, int mode, long long extent, int* defer, cudaStream_t s);
+cudaError_t launch_push_leftover(const GridP& g, const SpeciesP* sp, int* const* defer, const long long* extent, int n,
+                                 const float* E, const float* B, float* J, int shift, cudaStream_t s);
 cudaError_t launch_deposit_unfused(const GridP& g, const SpeciesP& sp, float* J, long long extent,
                                    cudaStream_t s);
 // Appends the new column's cold plasma (3D: at the count rounded up to 256, patch-ordered);
