@@ -8,6 +8,8 @@
 // offset and placed into the deposition window by an integer shift, which makes the "new"
 // shape of one step bit-identical to the "old" shape of the next: charge is conserved to FP32
 // round-off per step with no drift from re-rounded positions.
+#include <cuda.h>
+#include <cudaTypedefs.h>
 #include <cuda_runtime.h>
 
 #include <climits>
@@ -949,6 +951,12 @@ constexpr int JZ3 = 24, JZP3 = 24, JX3 = 10, JY3 = 10;   // current box per comp
 constexpr int JV3 = JZP3 * JX3 * JY3;
 constexpr int PF3 = 7;                           // prefetched words per particle (cell, 3 offsets, 3 momenta)
 constexpr int SMEM_3D = 6 * FV3 + 3 * JV3 + 2 * PF3 * FUSED_T;
+// Words about a chunk that its warps agree on: the lower ends of its gather box along z, x, y, the
+// upper ends negated (so that all six are minima), the largest current contribution (float bits) and
+// whether any particle moves.  Three sets in turn: one chunk's is read while the next one's is
+// gathered and the one after that is reset.  One more word says that a copy did not arrive.
+enum { BW_LO = 0, BW_HI = 3, BW_MAX = 6, BW_MOVING = 7, BW_N = 8, BW_ABORT = 3 * BW_N, BW_SHARED = BW_ABORT + 1 };
+__device__ __forceinline__ int box_word_init(int k) { return k < BW_MAX ? INT_MAX : 0; }
 static_assert((3 * JV3) % 4 == 0 && FZP3 % 4 == 0 && JZP3 % 4 == 0, "16-byte groups");
 
 // i / d for the box extents d = 1..32 as (i m_d) >> 16 with m_d = ceil(2^16 / d): the product
@@ -1014,15 +1022,61 @@ __device__ __noinline__ void deposit3_global(const GridP g, float qv, const Pos 
     deposit<3, SHAPE>(g, qv, 0.f, p0, p1, acc);
 }
 
+// a compile-time false condition
+struct Never {
+    __device__ constexpr operator bool() const { return false; }
+};
+
+// Waits for phase `parity` of an mbarrier that a TMA copy completes; gives up after about a second
+// (false).
+__device__ __forceinline__ bool mbar_wait(unsigned bar, unsigned parity) {
+    for (int k = 0; k < (1 << 20); ++k) {
+        unsigned done;
+        asm volatile("{\n.reg .pred q;\nmbarrier.try_wait.parity.shared::cta.b64 q, [%1], %2, 0x3e8;\n"
+                     "selp.u32 %0, 1, 0, q;\n}\n"
+                     : "=r"(done)
+                     : "r"(bar), "r"(parity)
+                     : "memory");
+        if (done) return true;
+    }
+    return false;
+}
+
+// One TMA copy of the FZP3 x FX3 x FY3 x 3 field box at (z, x, y) into dst; cells outside the grid
+// read as zero.
+__device__ __forceinline__ void tma_box(float* dst, const CUtensorMap* map, int z, int x, int y, unsigned bar) {
+    asm volatile("cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], "
+                 "[%1, {%2, %3, %4, %5}], [%6];\n" ::"r"((unsigned)__cvta_generic_to_shared(dst)),
+                 "l"(map), "r"(z), "r"(x), "r"(y), "r"(0), "r"(bar)
+                 : "memory");
+}
+
+// The fused step on chunks of FUSED_T particles.  Software pipeline, two barriers per chunk:
+//   top      this chunk's gather box was agreed on during the previous chunk and, when it lies inside
+//            the periodic x and y range, its fields were copied by TMA (one elected thread, two
+//            copies; z cells outside the grid arrive as zeros) behind the previous chunk's deposits.
+//            Boxes across the seam are staged here by every thread (cp.async), and grids that TMA
+//            cannot address (rows not 16-byte aligned) by every thread where the copy is asked for;
+//   then     the next chunk's particle words, copied one chunk ahead, give that chunk's gather box;
+//            gather, push, store, deposition weights of this chunk;
+//   barrier  the next chunk's fields are requested (all gathers are done), deposits of this chunk;
+//   barrier  the current box goes to J and is cleared.
+// The staging loop with its index arithmetic took about 230 of 1780 instructions per 32 particles,
+// and the four barriers of a chunk that first agreed on its box, then staged, a sixth of the time
+// (512 x 256 x 256 wake, both species of a step: 5.97 ms before, 5.30 ms now; issue slots 63% and
+// shared-memory wavefronts 68% busy).
 // DEFER: a chunk whose boxes do not fit is appended to defer[2..] (count in defer[0]) for the
-// general kernel, or to defer2[2..] for the per-particle kernel when even the general path's boxes
+// general path, or to defer2[2..] for the per-particle path when even the general path's boxes
 // would not hold it; without DEFER it takes the out-of-line global-memory path here.
-template <int SHAPE, bool DEFER>
+// TMA: mapE, mapB are tensor maps of E and B; without, the threads stage every chunk.
+template <int SHAPE, bool DEFER, bool TMA>
 __device__ __forceinline__ void push_deposit_3d_chunks(const GridP& g, const SpeciesP& sp,
                                                        const float* __restrict__ E, const float* __restrict__ B,
                                                        float* __restrict__ J, int shift, long long chunk0,
                                                        long long stride, float* sF, float* sJ, int* box,
-                                                       int* __restrict__ defer, int* __restrict__ defer2) {
+                                                       int* __restrict__ defer, int* __restrict__ defer2,
+                                                       const CUtensorMap* mapE, const CUtensorMap* mapB,
+                                                       unsigned long long* mbar, int* status) {
     constexpr int K = Shape<SHAPE>::K;
     constexpr int KW = K + 1;
     const long long n = *sp.count;
@@ -1032,6 +1086,7 @@ __device__ __forceinline__ void push_deposit_3d_chunks(const GridP& g, const Spe
     const bool jvec = (g.nz & 3) == 0 && aligned16(J);
     int* const iJ = reinterpret_cast<int*>(sJ);
     float* const pfb = sJ + 3 * JV3;                  // [2][PF3][FUSED_T]
+    const unsigned bar = (unsigned)__cvta_generic_to_shared(mbar);
     auto prefetch = [&](long long b, int buf) {
         const long long q = b + threadIdx.x;
         if (q < n) {
@@ -1046,30 +1101,159 @@ __device__ __forceinline__ void push_deposit_3d_chunks(const GridP& g, const Spe
         }
         cp_async_commit();
     };
-    int buf = 0;
+    // the gather box of the chunk at b from its particle words (a shape's half-cell support starts at
+    // the node below the cell and its nodal one there or, for K = 3 or the linear upper half, a node up)
+    auto agree = [&](long long b, int buf, int* bw) {
+        const float* w = pfb + buf * PF3 * FUSED_T + threadIdx.x;
+        int v[6] = {INT_MAX, INT_MAX, INT_MAX, INT_MAX, INT_MAX, INT_MAX};
+        bool moving = false;
+        if (b + threadIdx.x < n) {
+            const int cell = __float_as_int(w[0]);
+            if (cell >= 0) {
+                int c[3];
+                decode(g, cell, c[0], c[1], c[2]);
+                c[0] -= 1 + shift;
+                if (c[0] >= 0 && c[0] < g.nz) {
+                    moving = w[4 * FUSED_T] != 0.f || w[5 * FUSED_T] != 0.f || w[6 * FUSED_T] != 0.f;
+#pragma unroll
+                    for (int a = 0; a < 3; ++a) {
+                        // quadratic: nodes [cell - 1, cell + 1] and, upper half, [cell, cell + 2];
+                        // linear: [cell, cell + 1] and, lower half, [cell - 1, cell]
+                        const bool up = w[(1 + a) * FUSED_T] >= 0.5f;
+                        v[BW_LO + a] = K == 3 || !up ? c[a] - 1 : c[a];
+                        v[BW_HI + a] = -(K == 3 && up ? c[a] + 2 : c[a] + 1);
+                    }
+                }
+            }
+        }
+        int mine = 0;
+#pragma unroll
+        for (int a = 0; a < 6; ++a) {
+            const int m = __reduce_min_sync(0xffffffffu, v[a]);
+            if ((threadIdx.x & 31) == a) mine = m;
+        }
+        if ((threadIdx.x & 31) < 6 && mine != INT_MAX) atomicMin(bw + (threadIdx.x & 31), mine);
+        if (__any_sync(0xffffffffu, moving) && (threadIdx.x & 31) == 0) bw[BW_MOVING] = 1;
+    };
+    struct Ext {
+        int fz0, fx0, fy0, fzl, fxl, fyl;
+        bool any, ftile, tma;
+    };
+    auto extents = [&](const int* bw) {
+        Ext e;
+        e.any = bw[BW_LO] != INT_MAX;
+        e.fz0 = bw[BW_LO] & ~3, e.fx0 = bw[BW_LO + 1], e.fy0 = bw[BW_LO + 2];
+        e.fzl = 1 - bw[BW_HI] - e.fz0, e.fxl = 1 - bw[BW_HI + 1] - e.fx0, e.fyl = 1 - bw[BW_HI + 2] - e.fy0;
+        e.ftile = e.any && e.fzl <= FZ3 && e.fxl <= FX3 && e.fyl <= FY3;
+        e.tma = TMA && e.ftile && e.fx0 >= 0 && e.fy0 >= 0 && e.fx0 + e.fxl <= g.nx && e.fy0 + e.fyl <= g.ny;
+        return e;
+    };
+    // groups (c, y, x, z4) of the [c][y][x][z] box, only those inside the used extents; z groups start
+    // at multiples of 4, so with nz % 4 == 0 a group lies wholly inside or wholly outside 0 <= z < nz
+    auto staged = [&](const Ext& e, auto&& f) {
+        const int ngz = (e.fzl + 3) >> 2;
+        const unsigned mgz = kInv16.m[ngz], mfx = kInv16.m[e.fxl], mfy = kInv16.m[e.fyl];
+#pragma unroll 2
+        for (int i = threadIdx.x; i < 6 * e.fyl * e.fxl * ngz; i += FUSED_T) {
+            const int r = qdiv(i, mgz), zg = i - r * ngz;
+            const int r2 = qdiv(r, mfx), x = r - r2 * e.fxl;
+            const int c = qdiv(r2, mfy), y = r2 - c * e.fyl;
+            f(c, x, y, zg);
+        }
+    };
+    static_assert(6 * FY3 * FX3 * (FZ3 / 4) < 2048 && FX3 <= 32 && FY3 <= 32 && FZ3 / 4 <= 32, "qdiv range");
+    auto stage = [&](const Ext& e) {
+        staged(e, [&](int c, int x, int y, int zg) {
+            const long long row = ((long long)wrapi(e.fy0 + y, g.ny) * g.nx + wrapi(e.fx0 + x, g.nx)) * g.nz;
+            const float* f = (c < 3 ? E + c * N : B + (c - 3) * N) + row;
+            float* d = sF + c * FV3 + (y * FX3 + x) * FZP3 + 4 * zg;
+            const int gz = e.fz0 + 4 * zg;
+            if (fvec) {
+                const bool in = gz >= 0 && gz < g.nz;
+                cp_async16z(d, f + (in ? gz : 0), in);
+            } else {
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const bool in = (unsigned)(gz + j) < (unsigned)g.nz;
+                    cp_async4z(d + j, f + (in ? gz + j : 0), in);
+                }
+            }
+        });
+        cp_async_commit();
+    };
+    // the fields of the next chunk (its box is agreed on, every gather from the box is done): one
+    // thread asks for the TMA copies; without tensor maps every thread issues its share of the groups
+    auto request = [&](const int* bw) {
+        if (TMA && threadIdx.x != 0) return;
+        const Ext e = extents(bw);
+        if (!TMA && e.ftile) stage(e);
+        if (!e.tma) return;
+        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(bar),
+                     "r"((unsigned)(6 * FV3 * sizeof(float)))
+                     : "memory");
+        tma_box(sF, mapE, e.fz0, e.fx0, e.fy0, bar);
+        tma_box(sF + 3 * FV3, mapB, e.fz0, e.fx0, e.fy0, bar);
+    };
     prefetch(chunk0 * FUSED_T, 0);
-    // box[0..6] and box[7..13] serve alternate chunks: no barrier at the top of the loop or after
-    // the flush.  The current box starts cleared.
-    if (threadIdx.x < 14) {
-        const int q = threadIdx.x % 7;
-        box[threadIdx.x] = q == 6 ? 0 : (q & 1) ? INT_MIN : INT_MAX;
+    prefetch((chunk0 + stride) * FUSED_T, 1);
+    if (threadIdx.x < BW_SHARED) box[threadIdx.x] = threadIdx.x < BW_ABORT ? box_word_init(threadIdx.x % BW_N) : 0;
+    if (TMA && threadIdx.x == 0) {
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(bar) : "memory");
+        asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     }
     for (int i = threadIdx.x; i < (3 * JV3) / 4; i += FUSED_T)
         reinterpret_cast<int4*>(iJ)[i] = make_int4(0, 0, 0, 0);
     __syncthreads();
-    int cur = 0;
-    for (long long base = chunk0 * FUSED_T; base < n; base += stride * FUSED_T, buf ^= 1, cur ^= 7) {
-        int* const bc = box + cur;
-        if (threadIdx.x < 7) box[(cur ^ 7) + threadIdx.x] = threadIdx.x == 6 ? 0 : (threadIdx.x & 1) ? INT_MIN : INT_MAX;
-        prefetch(base + stride * FUSED_T, buf ^ 1);
-        cp_async_wait_prev();                      // this thread's words of this chunk
-        const long long p = base + threadIdx.x;
-        const float* mine = pfb + buf * PF3 * FUSED_T + threadIdx.x;
+    cp_async_wait_prev();
+    agree(chunk0 * FUSED_T, 0, box);
+    __syncthreads();
+    request(box);
+    int buf = 0, cur = 0;
+    unsigned parity = 0;
+    for (long long base = chunk0 * FUSED_T; base < n; base += stride * FUSED_T, buf ^= 1) {
+        int* const bc = box + cur * BW_N;
+        const int nxt = cur == 2 ? 0 : cur + 1;
+        cp_async_wait_all_p();                     // the next chunk's particle words
+        agree(base + stride * FUSED_T, buf ^ 1, box + nxt * BW_N);
+        const Ext e = extents(bc);
+        const bool any = e.any, ftile = e.ftile;
+        const int fz0 = e.fz0, fx0 = e.fx0, fy0 = e.fy0;
+        // every deposition window lies within one node below and one above the gather stencils: it
+        // starts at the lower of two supports at most one node apart and holds K + 1 nodes
+        const int jz0 = (bc[BW_LO] - 1) & ~3, jx0 = fx0 - 1, jy0 = fy0 - 1;
+        const int jzl = 2 - bc[BW_HI] - jz0, jxl = e.fxl + 2, jyl = e.fyl + 2;
+        const bool jtile = any && jzl <= JZ3 && jxl <= JX3 && jyl <= JY3;
+        const bool listed = DEFER && any && !(ftile && jtile);
+        if (listed && threadIdx.x == 0) {
+            // boxes the general path holds in shared memory (its own rounding of the z extents) go to
+            // its list, the rest to the per-particle one
+            const int gfz = (e.fzl + 3) & ~3, gjz = (jzl + 3) & ~3;
+            const bool general = 6 * gfz * e.fxl * e.fyl <= F_CAP3 && e.fxl <= g.nx + 2 * K && e.fyl <= g.ny + 2 * K &&
+                                 3 * gjz * jxl * jyl <= J_CAP3 && jxl <= g.nx + 2 * KW && jyl <= g.ny + 2 * KW;
+            int* list = general ? defer : defer2;
+            list[2 + atomicAdd(list, 1)] = (int)(base / FUSED_T);
+        }
+        if (e.tma) {
+            if (!mbar_wait(bar, parity)) {         // the copy did not arrive: report, give it more time, stop
+                atomicOr(status, STATUS_TIMEOUT);
+                mbar_wait(bar, parity);
+                box[BW_ABORT] = 1;
+            }
+            parity ^= 1;
+        } else if (ftile) {
+            if (TMA) stage(e);                     // a box across the periodic seam: not asked for ahead
+            cp_async_wait_all_p();
+            // these writes come before a later TMA copy into the same box
+            if (TMA) asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+            __syncthreads();
+        }
         // ---- load and decode ----
+        const long long p = base + threadIdx.x;
         bool ok = false;
         Pos p0;
         float u[3] = {0.f, 0.f, 0.f};
-        if (p < n) {
+        if (p < n && !listed) {
+            const float* mine = pfb + buf * PF3 * FUSED_T + threadIdx.x;
             int cell = __float_as_int(mine[0]);
             if (cell >= 0) {
                 int izg;
@@ -1088,108 +1272,34 @@ __device__ __forceinline__ void push_deposit_3d_chunks(const GridP& g, const Spe
                 }
             }
         }
-        // ---- gather weights and the chunk's boxes ----
-        float Wzn[K], Wzh[K], Wxn[K], Wxh[K], Wyn[K], Wyh[K];
-        int bzn = 0, bzh = 0, bxn = 0, bxh = 0, byn = 0, byh = 0;
-        if (ok) {
-            bzn = p0.iz + Shape<SHAPE>::w(p0.oz, Wzn);
-            bzh = half_weights<SHAPE>(p0.iz, p0.oz, Wzh);
-            bxn = p0.ix + Shape<SHAPE>::w(p0.ox, Wxn);
-            bxh = half_weights<SHAPE>(p0.ix, p0.ox, Wxh);
-            byn = p0.iy + Shape<SHAPE>::w(p0.oy, Wyn);
-            byh = half_weights<SHAPE>(p0.iy, p0.oy, Wyh);
-        }
-        box_reduce(bc, ok ? min(bzn, bzh) : INT_MAX, ok ? max(bzn, bzh) + K - 1 : INT_MIN,
-                   ok ? min(bxn, bxh) : INT_MAX, ok ? max(bxn, bxh) + K - 1 : INT_MIN);
-        {
-            const int c = __reduce_min_sync(0xffffffffu, ok ? min(byn, byh) : INT_MAX);
-            const int d = __reduce_max_sync(0xffffffffu, ok ? max(byn, byh) + K - 1 : INT_MIN);
-            if ((threadIdx.x & 31) == 0 && c != INT_MAX) {
-                atomicMin(bc + 4, c);
-                atomicMax(bc + 5, d);
-            }
-        }
-        __syncthreads();
-        const bool any = bc[0] != INT_MAX;
-        const int fz0 = bc[0] & ~3, fx0 = bc[2], fy0 = bc[4];
-        const int fzl = bc[1] + 1 - fz0, fxl = bc[3] - bc[2] + 1, fyl = bc[5] - bc[4] + 1;
-        const bool ftile = any && fzl <= FZ3 && fxl <= FX3 && fyl <= FY3;
-        // every deposition window lies within one node below and one above the gather stencils: it
-        // starts at the lower of two supports at most one node apart and holds K + 1 nodes
-        const int jz0 = (bc[0] - 1) & ~3, jx0 = bc[2] - 1, jy0 = bc[4] - 1;
-        const int jzl = bc[1] + 2 - jz0, jxl = bc[3] - bc[2] + 3, jyl = bc[5] - bc[4] + 3;
-        const bool jtile = any && jzl <= JZ3 && jxl <= JX3 && jyl <= JY3;
-        if (DEFER && any && !(ftile && jtile)) {
-            // boxes the general path holds in shared memory (its own rounding of the z extents) go to
-            // the general kernel's list, the rest (the plasma injected since the last sort: one
-            // long row of cells) to the per-particle kernel's list
-            const int gfz = (bc[1] + 1 - fz0 + 3) & ~3, gjz = (bc[1] + 2 - jz0 + 3) & ~3;
-            const bool general = 6 * gfz * fxl * fyl <= F_CAP3 && fxl <= g.nx + 2 * K && fyl <= g.ny + 2 * K &&
-                                 3 * gjz * jxl * jyl <= J_CAP3 && jxl <= g.nx + 2 * KW && jyl <= g.ny + 2 * KW;
-            int* list = general ? defer : defer2;
-            if (threadIdx.x == 0) list[2 + atomicAdd(list, 1)] = (int)(base / FUSED_T);
-            __syncthreads();                       // everyone has read this chunk's box words
-            continue;
-        }
-        // groups (c, y, x, z4) of the [c][y][x][z] box, only those inside the used extents, copied
-        // asynchronously (all of a thread's groups in flight at once); z groups start at multiples of
-        // 4, so with nz % 4 == 0 a group lies wholly inside or wholly outside 0 <= z < nz
-        const int ngz = ftile ? (fzl + 3) >> 2 : 0;
-        const unsigned mgz = ftile ? kInv16.m[ngz] : 0u, mfx = ftile ? kInv16.m[fxl] : 0u,
-                       mfy = ftile ? kInv16.m[fyl] : 0u;
-        const int nstage = 6 * fyl * fxl * ngz;
-        auto staged = [&](auto&& f) {
-#pragma unroll 2
-            for (int i = threadIdx.x; i < nstage; i += FUSED_T) {
-                const int r = qdiv(i, mgz), zg = i - r * ngz;
-                const int r2 = qdiv(r, mfx), x = r - r2 * fxl;
-                const int c = qdiv(r2, mfy), y = r2 - c * fyl;
-                f(c, x, y, zg);
-            }
-        };
-        static_assert(6 * FY3 * FX3 * (FZ3 / 4) < 2048 && FX3 <= 32 && FY3 <= 32 && FZ3 / 4 <= 32, "qdiv range");
-        if (ftile) {
-            staged([&](int c, int x, int y, int zg) {
-                const long long row = ((long long)wrapi(fy0 + y, g.ny) * g.nx + wrapi(fx0 + x, g.nx)) * g.nz;
-                const float* f = (c < 3 ? E + c * N : B + (c - 3) * N) + row;
-                float* d = sF + c * FV3 + (y * FX3 + x) * FZP3 + 4 * zg;
-                const int gz = fz0 + 4 * zg;
-                if (fvec) {
-                    const bool in = gz >= 0 && gz < g.nz;
-                    cp_async16z(d, f + (in ? gz : 0), in);
-                } else {
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        const bool in = (unsigned)(gz + j) < (unsigned)g.nz;
-                        cp_async4z(d + j, f + (in ? gz + j : 0), in);
-                    }
-                }
-            });
-        }
-        cp_async_commit();
-        cp_async_wait_all_p();                     // the box (and the next chunk's particle words)
         // a particle at rest in zero fields stays at rest and carries no current: a chunk with no
         // moving particle reads its staged groups back to see whether they are all zero
-        const bool moving = ok && (u[0] != 0.f || u[1] != 0.f || u[2] != 0.f);
-        bool live = __syncthreads_or(moving);
-        if (!live && ftile) {
+        if (ftile && !bc[BW_MOVING]) {
             unsigned fbits = 0u;
-            staged([&](int c, int x, int y, int zg) {
+            staged(e, [&](int c, int x, int y, int zg) {
                 const float4 v = *reinterpret_cast<const float4*>(sF + c * FV3 + (y * FX3 + x) * FZP3 + 4 * zg);
                 fbits |= __float_as_uint(v.x) | __float_as_uint(v.y) | __float_as_uint(v.z) | __float_as_uint(v.w);
             });
-            live = __syncthreads_or(fbits != 0u);
-        }
-        if (!live && ftile) {
-            // a quiet chunk (every particle at rest, every field of its footprint zero): nothing
-            // moves and no current flows; only a pending window shift is applied to the cells,
-            // and the rest of the chunk runs with every particle switched off
-            if (shift && ok) sp.cell[p] = encode(g, p0.iz, p0.ix, p0.iy);
-            ok = false;
+            if (!__syncthreads_or(fbits != 0u)) {
+                // a quiet chunk (every particle at rest, every field of its footprint zero): nothing
+                // moves and no current flows; only a pending window shift is applied to the cells,
+                // and the rest of the chunk runs with every particle switched off
+                if (shift && ok) sp.cell[p] = encode(g, p0.iz, p0.ix, p0.iy);
+                ok = false;
+            }
         }
         // ---- gather (E1 z+, E2 x+, E3 y+, B1 x+ y+, B2 z+ y+, B3 z+ x+) ----
+        float Wzn[K], Wxn[K], Wyn[K];
+        int bzn = 0, bxn = 0, byn = 0;
         float eb[6];
         if (ok) {
+            float Wzh[K], Wxh[K], Wyh[K];
+            bzn = p0.iz + Shape<SHAPE>::w(p0.oz, Wzn);
+            bxn = p0.ix + Shape<SHAPE>::w(p0.ox, Wxn);
+            byn = p0.iy + Shape<SHAPE>::w(p0.oy, Wyn);
+            const int bzh = half_weights<SHAPE>(p0.iz, p0.oz, Wzh);
+            const int bxh = half_weights<SHAPE>(p0.ix, p0.ox, Wxh);
+            const int byh = half_weights<SHAPE>(p0.iy, p0.oy, Wyh);
             if (ftile) {
                 auto at = [&](int comp, int z, int x, int y) {
                     return sF + comp * FV3 + ((y - fy0) * FX3 + (x - fx0)) * FZP3 + (z - fz0);
@@ -1237,6 +1347,7 @@ __device__ __forceinline__ void push_deposit_3d_chunks(const GridP& g, const Spe
                 sp.u[2 * cap + p] = u[2];
             }
         }
+        prefetch(base + 2 * stride * FUSED_T, buf);      // this chunk's words are done with
         // ---- deposition ----
         float S0z[KW], DSz[KW], S0x[KW], DSx[KW], S0y[KW], DSy[KW];
         int bz = 0, bx = 0, by = 0;
@@ -1267,10 +1378,13 @@ __device__ __forceinline__ void push_deposit_3d_chunks(const GridP& g, const Spe
         // fixed-point scale of the chunk (see push_deposit_2d_chunks): s = 2^(22-e), max mb < 2^e
         if (jtile) {
             const unsigned wm = __reduce_max_sync(0xffffffffu, ok ? __float_as_uint(mb) : 0u);
-            if ((threadIdx.x & 31) == 0 && wm) atomicMax(reinterpret_cast<unsigned*>(bc + 6), wm);
+            if ((threadIdx.x & 31) == 0 && wm) atomicMax(reinterpret_cast<unsigned*>(bc + BW_MAX), wm);
         }
         __syncthreads();
-        const int mbits = bc[6];
+        if (TMA && box[BW_ABORT]) break;
+        request(box + nxt * BW_N);
+        if (threadIdx.x < BW_N) box[(3 - cur - nxt) * BW_N + threadIdx.x] = box_word_init(threadIdx.x);
+        const int mbits = bc[BW_MAX];
         const int sexp = min(275 - (mbits >> 23), 253);
         const float fs = __int_as_float(sexp << 23), inv_s = __int_as_float((254 - sexp) << 23);
         if (jtile && mbits != 0) {
@@ -1295,50 +1409,57 @@ __device__ __forceinline__ void push_deposit_3d_chunks(const GridP& g, const Spe
             const bool uz = __any_sync(0xffffffffu, S0z[KW - 1] != 0.f || DSz[KW - 1] != 0.f);
             const bool ux = __any_sync(0xffffffffu, S0x[KW - 1] != 0.f || DSx[KW - 1] != 0.f);
             const bool uy = __any_sync(0xffffffffu, S0y[KW - 1] != 0.f || DSy[KW - 1] != 0.f);
-            // one component at a time: fewer values live at once
-            auto terms = [&](auto&& put) {
+            // one component at a time: fewer values live at once; (hz, hx, hy): whether the last node
+            // of the window along an axis takes part
+            auto terms = [&](auto&& put, auto hz, auto hx, auto hy) {
 #pragma unroll
                 for (int c = 0; c < KW; ++c) {
-                    if (c == KW - 1 && !uy) continue;
+                    if (c == KW - 1 && !hy) continue;
                     const float py = P_(S0y[c], DSy[c]), qy = Q_(S0y[c], DSy[c]);
 #pragma unroll
                     for (int b = 0; b < KW; ++b) {
-                        if (b == KW - 1 && !ux) continue;
+                        if (b == KW - 1 && !hx) continue;
                         const float t = fmaf(S0x[b], py, DSx[b] * qy);
 #pragma unroll
                         for (int a = 0; a < KW - 1; ++a) {
-                            if (a == KW - 2 && !uz) continue;
+                            if (a == KW - 2 && !hz) continue;
                             put((c * JX3 + b) * JZP3 + a, fmaf(cz[a], t, MAGIC));
                         }
                     }
 #pragma unroll
                     for (int a = 0; a < KW; ++a) {
-                        if (a == KW - 1 && !uz) continue;
+                        if (a == KW - 1 && !hz) continue;
                         const float t = fmaf(S0z[a], py, DSz[a] * qy);
 #pragma unroll
                         for (int b = 0; b < KW - 1; ++b) {
-                            if (b == KW - 2 && !ux) continue;
+                            if (b == KW - 2 && !hx) continue;
                             put(JV3 + (c * JX3 + b) * JZP3 + a, fmaf(cx[b], t, MAGIC));
                         }
                     }
                 }
 #pragma unroll
                 for (int b = 0; b < KW; ++b) {
-                    if (b == KW - 1 && !ux) continue;
+                    if (b == KW - 1 && !hx) continue;
                     const float px = P_(S0x[b], DSx[b]), qx = Q_(S0x[b], DSx[b]);
 #pragma unroll
                     for (int a = 0; a < KW; ++a) {
-                        if (a == KW - 1 && !uz) continue;
+                        if (a == KW - 1 && !hz) continue;
                         const float t = fmaf(S0z[a], px, DSz[a] * qx);
 #pragma unroll
                         for (int c = 0; c < KW - 1; ++c) {
-                            if (c == KW - 2 && !uy) continue;
+                            if (c == KW - 2 && !hy) continue;
                             put(2 * JV3 + (c * JX3 + b) * JZP3 + a, fmaf(cy[c], t, MAGIC));
                         }
                     }
                 }
             };
-            if (ok) terms([&](int o, float biased) { atomicAdd(s0 + o, __float_as_int(biased) - 0x4B400000); });
+            if (ok) {
+                auto put = [&](int o, float biased) { atomicAdd(s0 + o, __float_as_int(biased) - 0x4B400000); };
+                if (!(uz || ux || uy))
+                    terms(put, Never(), Never(), Never());
+                else
+                    terms(put, uz, ux, uy);
+            }
         } else if (!DEFER && any && !jtile && ok) {
             deposit3_global<SHAPE>(g, sp.qv, p0, p1, J);
         }
@@ -1371,20 +1492,24 @@ __device__ __forceinline__ void push_deposit_3d_chunks(const GridP& g, const Spe
                 }
             }
         }
+        cur = nxt;
     }
-    cp_async_wait_all_p();                         // the last (empty) prefetch group
+    cp_async_wait_all_p();                         // the last (empty) prefetch groups
 }
 
-template <int SHAPE>
+template <int SHAPE, bool TMA>
 __global__ void __launch_bounds__(FUSED_T, 3) push_deposit_3d_kernel(GridP g, SpeciesP sp, const float* __restrict__ E,
                                                                      const float* __restrict__ B, float* __restrict__ J,
                                                                      int shift, int* __restrict__ defer,
-                                                                     int* __restrict__ defer2) {
-    extern __shared__ float4 smem4[];
+                                                                     int* __restrict__ defer2,
+                                                                     const __grid_constant__ CUtensorMap mapE,
+                                                                     const __grid_constant__ CUtensorMap mapB, int* status) {
+    extern __shared__ __align__(128) float4 smem4[];
     float* smem = reinterpret_cast<float*>(smem4);
-    __shared__ int box[14];
-    push_deposit_3d_chunks<SHAPE, true>(g, sp, E, B, J, shift, blockIdx.x, gridDim.x, smem, smem + 6 * FV3, box,
-                                        defer, defer2);
+    __shared__ int box[BW_SHARED];
+    __shared__ __align__(8) unsigned long long mbar;
+    push_deposit_3d_chunks<SHAPE, true, TMA>(g, sp, E, B, J, shift, blockIdx.x, gridDim.x, smem, smem + 6 * FV3, box,
+                                             defer, defer2, &mapE, &mapB, &mbar, status);
 }
 
 constexpr int SMEM_3D_GEN = F_CAP3 + J_CAP3 + 2 * PF3 * FUSED_T;
@@ -1782,11 +1907,11 @@ template <int SHAPE>
 __global__ void __launch_bounds__(FUSED_T, 2) push_deposit_3d_batch_kernel(const PartInst* __restrict__ inst, int parity) {
     extern __shared__ float4 smem4[];
     float* smem = reinterpret_cast<float*>(smem4);
-    __shared__ int box[14];
+    __shared__ int box[BW_SHARED];
     const PartInst& q = inst[blockIdx.y];
     const GridP g = prep_device(q.g);
-    push_deposit_3d_chunks<SHAPE, false>(g, q.sp, q.E[parity], q.B[parity], q.J, 0, blockIdx.x, gridDim.x, smem,
-                                         smem + 6 * FV3, box, nullptr, nullptr);
+    push_deposit_3d_chunks<SHAPE, false, false>(g, q.sp, q.E[parity], q.B[parity], q.J, 0, blockIdx.x, gridDim.x, smem,
+                                                smem + 6 * FV3, box, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr);
 }
 
 template <int SHAPE>
@@ -2152,10 +2277,36 @@ inline unsigned pblocks(long long extent) {
     return (unsigned)(b < 1 ? 1 : (b > 152 * 16 ? 152 * 16 : b));
 }
 
+// The driver's tensor-map encoder (null when the driver has none).
+PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
+    static const PFN_cuTensorMapEncodeTiled_v12000 fn = [] {
+        void* p = nullptr;
+        cudaDriverEntryPointQueryResult r;
+        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &r) != cudaSuccess ||
+            r != cudaDriverEntryPointSuccess)
+            p = nullptr;
+        return reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(p);
+    }();
+    return fn;
+}
+
+// Map of a field's three components [c][y][x][z] with the field box of push_deposit_3d_chunks; false
+// when TMA cannot address the array (rows or base not 16-byte aligned).
+bool field_box_map(CUtensorMap* map, const float* F, const GridP& g) {
+    const auto fn = tensor_map_encoder();
+    if (!fn || g.nz % 4 != 0 || ((uintptr_t)F & 15) != 0) return false;
+    const cuuint64_t dims[4] = {(cuuint64_t)g.nz, (cuuint64_t)g.nx, (cuuint64_t)g.ny, 3};
+    const cuuint64_t strides[3] = {4ull * g.nz, 4ull * g.nz * g.nx, 4ull * g.ncell};
+    const cuuint32_t boxd[4] = {FZP3, FX3, FY3, 3}, es[4] = {1, 1, 1, 1};
+    return fn(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, const_cast<float*>(F), dims, strides, boxd, es,
+              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 }  // namespace
 
 cudaError_t launch_push(const GridP& g0, const SpeciesP& sp, const float* E, const float* B, float* J,
-                        int shift, int mode, long long extent, int* defer, cudaStream_t s) {
+                        int shift, int mode, long long extent, int* defer, int* status, cudaStream_t s) {
     const GridP g = prep(g0);
     if (extent <= 0) return cudaSuccess;
     return dispatch(g.ndim, g.shape, [&](auto nd, auto sh) {
@@ -2171,15 +2322,18 @@ cudaError_t launch_push(const GridP& g0, const SpeciesP& sp, const float* E, con
             }
             k<<<pblocks(extent), FUSED_T, smem, s>>>(g, sp, E, B, J, shift);
         } else if (mode == MODE_FUSED) {
-            auto k = push_deposit_3d_kernel<SH>;
             const size_t smem = SMEM_3D * sizeof(float);
-            static bool configured = false;
-            if (!configured) {
+            CUtensorMap mapE{}, mapB{};
+            const bool tma = field_box_map(&mapE, E, g) && field_box_map(&mapB, B, g);
+            auto k = tma ? push_deposit_3d_kernel<SH, true> : push_deposit_3d_kernel<SH, false>;
+            static bool configured[2] = {false, false};
+            if (!configured[tma]) {
                 cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
                 if (e != cudaSuccess) return e;
-                configured = true;
+                configured[tma] = true;
             }
-            k<<<pblocks(extent), FUSED_T, smem, s>>>(g, sp, E, B, J, shift, defer, defer + defer_len(sp.cap));
+            k<<<pblocks(extent), FUSED_T, smem, s>>>(g, sp, E, B, J, shift, defer, defer + defer_len(sp.cap), mapE, mapB,
+                                                     status);
         } else {
             push_kernel<ND, SH><<<pblocks(extent), 256, 0, s>>>(g, sp, E, B, shift);
         }

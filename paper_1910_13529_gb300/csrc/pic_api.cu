@@ -561,7 +561,8 @@ pic_status pic_gather_push(pic_t* h, void* stream) {
         }
         SpeciesP sp = species_params(h, i);
         Scope sc(h, PIC_T_PARTICLES, 1, s);
-        CK(h, launch_push(h->g, sp, h->E, h->B, nullptr, h->pending_shift, 1, q.extent, nullptr, s), "push kernel");
+        CK(h, launch_push(h->g, sp, h->E, h->B, nullptr, h->pending_shift, 1, q.extent, nullptr, h->status, s),
+           "push kernel");
     }
     h->pending_shift = 0;
     h->state = 1;
@@ -638,7 +639,7 @@ pic_status pic_step(pic_t* h, int nsteps, void* stream) {
             defers[nsp] = q.defer;
             extents[nsp++] = q.extent;
             Scope sc(h, PIC_T_PARTICLES, 1, s);
-            CK(h, launch_push(h->g, sp, Ec, Bc, h->J, h->pending_shift, 0, q.extent, q.defer, s),
+            CK(h, launch_push(h->g, sp, Ec, Bc, h->J, h->pending_shift, 0, q.extent, q.defer, h->status, s),
                "fused push/deposit kernel");
         }
         if (h->cfg.ndim == 3 && nsp > 0) {
@@ -762,6 +763,7 @@ pic_status pic_diag(pic_t* h, double* out, void* stream) {
     out[PIC_DIAG_SHIFTS] = (double)h->shifts;
     out[PIC_DIAG_STATUS] = (double)status;
     out[PIC_DIAG_INTERIOR] = acc[5];
+    if (status & STATUS_TIMEOUT) return fail(h, PIC_ERR_TIMEOUT, "a field copy of the particle kernel did not arrive");
     if (status & STATUS_CAPACITY) return fail(h, PIC_ERR_CAPACITY, "particle capacity exceeded during injection");
     return PIC_OK;
 }
@@ -804,6 +806,7 @@ pic_status pic_sync(pic_t* h, void* stream) {
     CK(h, cudaStreamSynchronize((cudaStream_t)stream), "synchronise");
     int status = 0;
     CK(h, cudaMemcpy(&status, h->status, sizeof(int), cudaMemcpyDeviceToHost), "read status");
+    if (status & STATUS_TIMEOUT) return fail(h, PIC_ERR_TIMEOUT, "a field copy of the particle kernel did not arrive");
     if (status & STATUS_CAPACITY) return fail(h, PIC_ERR_CAPACITY, "particle capacity exceeded during injection");
     return PIC_OK;
 }
