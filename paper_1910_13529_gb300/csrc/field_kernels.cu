@@ -16,6 +16,7 @@
 #include <climits>
 
 #include <cstdint>
+#include <vector>
 
 #include "pic_internal.h"
 
@@ -781,268 +782,347 @@ __device__ __forceinline__ void march_bnew_store(const FieldP& p, const float* e
 }
 
 // ---- 2D x-marching rows -------------------------------------------------------------------
-// A CTA owns z in [z0, z0 + TZ) and walks x over [xa, xa + xc): every row of B^{n+1/2} and
-// E^{n+1} is computed once (no x halo), register-blocked along z as above.  The rows a step
-// needs next are copied by cp.async one step ahead into a ring of 4 E, 3 B and 2 J rows:
-// for output row k the step computes B^{n+1/2}(k+1) from E^n(k+1), E^n(k+2); E^{n+1}(k+1) from
-// B^{n+1/2}(k+1), B^{n+1/2}(k), J(k+1); B^{n+1}(k) from E^{n+1}(k), E^{n+1}(k+1), B^{n+1/2}(k),
-// while E^n(k+3), B^n(k+2), J(k+2) land.
-template <int MAXM, int TZ>
-struct March2T {
+// A CTA owns a z segment and walks x over [xa, xb).  A lane owns eight consecutive z cells of the
+// segment in every stage and keeps them in registers from row to row, so everything that is
+// pointwise in z (the x differences, B1, E1, the rows x and x - 1 of each stage) costs no shared
+// memory; only the two components that are differentiated along z go through it, interleaved as
+// pairs (E2, E3) or (B2, B3): both have the same stencil, so one 64-bit operand carries both and a
+// packed FP32 subtraction and a packed FMA do a tap of the two.  Per row r = x + 1:
+//   B^{n+1/2}(r)   from the pair window of E^n(r) and E^n(r), E^n(r + 1) at the lane's cells;
+//   E^{n+1}(r)     from the pair window of B^{n+1/2}(r), B^{n+1/2}(r), B^{n+1/2}(r - 1) and J(r);
+//   B^{n+1}(r - 1) from the part of it that the pair window of E^{n+1}(r - 1) gave a row earlier and
+//                  the x differences of E^{n+1}(r) and E^{n+1}(r - 1).
+// E^n(r + 2), B^n(r + 1) and J(r + 1) arrive by cp.async behind the stages.  A segment of NT lanes
+// produces the NT - 6 D lanes in its middle, D = the lanes a window reaches on either side: each stage
+// loses D lanes at both ends.
+// A lane's eight pairs take five 16-byte groups (one is padding): the lanes of a quarter warp then read
+// a window from eight different groups modulo 8, without bank conflicts.
+// What bounds it: HBM for Yee and M <= 4, the FP32 pipe (a packed operation counts twice there) and
+// the latency of two warps per scheduler for M = 16.  The form before it staged every component with
+// its halo and read two windows of 2 M + 4 floats for four cells (69% of the shared-memory rate, issue
+// 71%).  Before and now, us per advance, best segment length: 8192 x 2048 Yee 188 and 163 (91% of the
+// copy bandwidth), M = 16 240 and 213 (69%); 4099 x 1030 M = 16 145 and 91 (rows not 16-byte aligned);
+// 4096 x 1024 M = 16 84 and 64.  64 threads win everywhere: fewer barrier partners outweigh the
+// 6 D lanes of a segment that produce nothing.  Below about 1e6 cells the blocked tiles are faster
+// (one row at a time is a serial chain).
+constexpr int ROW_Z = 8;                                       // cells of a lane
+constexpr int ROW_G = 5;                                       // 16-byte groups of a lane's pairs
+
+template <int MAXM, int NT, bool VEC>
+struct RowT {
     static constexpr int MP = (MAXM + 3) & ~3;
-    static constexpr int H2 = MP, H1 = 2 * MP, H0 = 3 * MP;
-    static constexpr int WE = TZ + 2 * H0, WB = TZ + 2 * H1, WJ = TZ + 2 * H2;
-    static constexpr int SE = 3 * WE, SB = 3 * WB, SJ = 3 * WJ;           // one row, 3 components
-    static constexpr size_t smem_bytes = sizeof(float) * (4 * SE + 3 * SB + 2 * SJ);
-    static_assert(TZ % 4 == 0, "the z tile holds whole groups of four cells");
+    static constexpr int D = (MP + ROW_Z - 1) / ROW_Z;         // lanes a window reaches on one side
+    static constexpr int R = ROW_Z * NT;                       // cells of the segment
+    static constexpr int OUT = ROW_Z * (NT - 6 * D);           // cells it produces
+    static constexpr int PB = (NT + 2 * D) * ROW_G * 4;        // floats of a pair buffer
+    // E, B, J rows, three pair buffers and, for rows that are not 16-byte aligned, the output rows
+    static constexpr size_t smem_bytes = sizeof(float) * (9 * R + 3 * PB + (VEC ? 0 : 6 * R));
+    static_assert(NT > 6 * D, "a segment has lanes left to produce");
 };
 
-// B^{n+1/2} in place over the B^n row b from the E^n rows e (x) and e1 (x + 1).
-template <int MAXM, int TZ>
-__device__ __forceinline__ void march2_bhalf(const FieldP& p, float* b, const float* e, const float* e1, int z0) {
-    using T = March2T<MAXM, TZ>;
-    constexpr int MP = T::MP, WE = T::WE, WB = T::WB, NG = WB / 4;
-    const GridP& g = p.g;
-    const float hz = 0.5f * g.dt / g.dz, hx = 0.5f * g.dt / g.dx;
-    for (int gi = threadIdx.x; gi < NG; gi += blockDim.x) {
-        const int z = 4 * gi - T::H1, gz = z0 + z;
-        if (gz + 3 < 0 || gz >= g.nz) continue;                     // B^n = B^{n+1/2} = 0 there
-        const int eo = z + T::H0;
-        float d2[4], d3[4], E2[4], E3[4], E1[4], E1x[4], E3x[4];
-        window_dz<MAXM, MP, true>(p.st, e + WE + eo - MP, d2, E2);
-        window_dz<MAXM, MP, true>(p.st, e + 2 * WE + eo - MP, d3, E3);
-        lds4(E1, e + eo);
-        lds4(E1x, e1 + eo);
-        lds4(E3x, e1 + 2 * WE + eo);
-        const int bo = 4 * gi;
-        float b0[4], b1[4], b2[4];
-        lds4(b0, b + bo);
-        lds4(b1, b + WB + bo);
-        lds4(b2, b + 2 * WB + bo);
+__device__ __forceinline__ void lds8(float (&a)[8], const float* s) {
+    float t[4];
+    lds4(t, s);
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const bool in = gz + j >= 0 && gz + j < g.nz;
-            b0[j] = in ? b0[j] - hx * (E3x[j] - E3[j]) : 0.f;
-            b1[j] = in ? b1[j] + hz * d3[j] : 0.f;
-            b2[j] = in ? b2[j] - (hz * d2[j] - hx * (E1x[j] - E1[j])) : 0.f;
-        }
-        sts4(b + bo, b0);
-        sts4(b + WB + bo, b1);
-        sts4(b + 2 * WB + bo, b2);
-    }
+    for (int j = 0; j < 4; ++j) a[j] = t[j];
+    lds4(t, s + 4);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) a[4 + j] = t[j];
 }
 
-// E^{n+1} in place over the E^n row e from the B^{n+1/2} rows b (x), bm (x - 1) and the J row j.
-template <int MAXM, int TZ>
-__device__ __forceinline__ void march2_enew(const FieldP& p, float* e, const float* b, const float* bm, const float* j,
-                                            int z0) {
-    using T = March2T<MAXM, TZ>;
-    constexpr int MP = T::MP, WE = T::WE, WB = T::WB, WJ = T::WJ, NG = WJ / 4;
-    const GridP& g = p.g;
-    const float dt = g.dt, fz = dt / g.dz, fx = dt / g.dx;
-    for (int gi = threadIdx.x; gi < NG; gi += blockDim.x) {
-        const int z = 4 * gi - T::H2, gz = z0 + z;
-        if (gz + 3 < 0 || gz >= g.nz) continue;                     // E^n = E^{n+1} = 0 there
-        const int eo = z + T::H0, bo = z + T::H1;
-        float d2[4], d3[4], B2[4], B3[4], B1[4], B1x[4], B3x[4];
-        window_dz<MAXM, MP, false>(p.st, b + WB + bo - MP, d2, B2);
-        window_dz<MAXM, MP, false>(p.st, b + 2 * WB + bo - MP, d3, B3);
-        lds4(B1, b + bo);
-        lds4(B1x, bm + bo);
-        lds4(B3x, bm + 2 * WB + bo);
-        const int jo = 4 * gi;
-        float e0[4], e1[4], e2[4], j0[4], j1[4], j2[4];
-        lds4(e0, e + eo);
-        lds4(e1, e + WE + eo);
-        lds4(e2, e + 2 * WE + eo);
-        lds4(j0, j + jo);
-        lds4(j1, j + WJ + jo);
-        lds4(j2, j + 2 * WJ + jo);
+// pairs (a[j], b[j]) of a lane
+__device__ __forceinline__ void put_pairs(float* own, const float (&a)[8], const float (&b)[8]) {
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const bool in = gz + q >= 0 && gz + q < g.nz;
-            e0[q] = in ? e0[q] + fx * (B3[q] - B3x[q]) - dt * j0[q] : 0.f;
-            e1[q] = in ? e1[q] - fz * d3[q] - dt * j1[q] : 0.f;
-            e2[q] = in ? e2[q] + (fz * d2[q] - fx * (B1[q] - B1x[q])) - dt * j2[q] : 0.f;
-        }
-        sts4(e + eo, e0);
-        sts4(e + WE + eo, e1);
-        sts4(e + 2 * WE + eo, e2);
-    }
+    for (int q = 0; q < 4; ++q)
+        *reinterpret_cast<float4*>(own + 4 * q) = make_float4(a[2 * q], b[2 * q], a[2 * q + 1], b[2 * q + 1]);
 }
 
-// B^{n+1} of row gx from the E^{n+1} rows e (x), e1 (x + 1) and the B^{n+1/2} row b; stores
-// E^{n+1}(x), B^{n+1}(x) (one cell towards -z if the window moves).
-template <int MAXM, int TZ>
-__device__ __forceinline__ void march2_bnew_store(const FieldP& p, const float* e, const float* e1, const float* b,
-                                                  int z0, int gx, bool vec) {
-    using T = March2T<MAXM, TZ>;
-    constexpr int MP = T::MP, WE = T::WE, WB = T::WB, NG = TZ / 4;
-    const GridP& g = p.g;
-    const long long N = g.ncell;
-    const float hz = 0.5f * g.dt / g.dz, hx = 0.5f * g.dt / g.dx;
-    const long long row = (long long)gx * g.nz;
-    for (int gi = threadIdx.x; gi < NG; gi += blockDim.x) {
-        const int z = 4 * gi, gz = z0 + z;
-        if (gz >= g.nz) continue;
-        const int eo = z + T::H0, bo = z + T::H1;
-        float d2[4], d3[4], E2[4], E3[4], E1[4], E1x[4], E3x[4];
-        window_dz<MAXM, MP, true>(p.st, e + WE + eo - MP, d2, E2);
-        window_dz<MAXM, MP, true>(p.st, e + 2 * WE + eo - MP, d3, E3);
-        lds4(E1, e + eo);
-        lds4(E1x, e1 + eo);
-        lds4(E3x, e1 + 2 * WE + eo);
-        float b0[4], b1[4], b2[4];
-        lds4(b0, b + bo);
-        lds4(b1, b + WB + bo);
-        lds4(b2, b + 2 * WB + bo);
+// d[j] = the axial difference (see window_dz) of both components of a pair at the lane's cells
+template <int MAXM, int MP, bool PLUS>
+__device__ __forceinline__ void window_pairs(const StencilP& st, const float* own, float2 (&d)[8]) {
+    constexpr int NW = 2 * MP + ROW_Z;
+    float2 w[NW];
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            b0[q] -= hx * (E3x[q] - E3[q]);
-            b1[q] += hz * d3[q];
-            b2[q] -= hz * d2[q] - hx * (E1x[q] - E1[q]);
-        }
-        if (vec && !p.shift) {
-            const long long o = row + gz;
-            *reinterpret_cast<float4*>(p.Eout + o) = make_float4(E1[0], E1[1], E1[2], E1[3]);
-            *reinterpret_cast<float4*>(p.Eout + N + o) = make_float4(E2[0], E2[1], E2[2], E2[3]);
-            *reinterpret_cast<float4*>(p.Eout + 2 * N + o) = make_float4(E3[0], E3[1], E3[2], E3[3]);
-            *reinterpret_cast<float4*>(p.Bout + o) = make_float4(b0[0], b0[1], b0[2], b0[3]);
-            *reinterpret_cast<float4*>(p.Bout + N + o) = make_float4(b1[0], b1[1], b1[2], b1[3]);
-            *reinterpret_cast<float4*>(p.Bout + 2 * N + o) = make_float4(b2[0], b2[1], b2[2], b2[3]);
-            continue;
-        }
+    for (int k = 0; k < NW; k += 2) {
+        const int rel = k - MP + 64 * ROW_Z, lane = rel / ROW_Z - 64, cell = rel % ROW_Z;
+        const float4 v = *reinterpret_cast<const float4*>(own + lane * (4 * ROW_G) + 2 * cell);
+        w[k] = make_float2(v.x, v.y);
+        w[k + 1] = make_float2(v.z, v.w);
+    }
+    const float2 minus = make_float2(-1.f, -1.f);
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const int gzq = gz + q;
-            if (gzq >= g.nz) break;
-            const int oz = gzq - p.shift;
-            if (oz >= 0) {
-                const long long o = row + oz;
-                p.Eout[o] = E1[q];
-                p.Eout[N + o] = E2[q];
-                p.Eout[2 * N + o] = E3[q];
-                p.Bout[o] = b0[q];
-                p.Bout[N + o] = b1[q];
-                p.Bout[2 * N + o] = b2[q];
-            }
-            if (p.shift && gzq == g.nz - 1) {
-                const long long o = row + gzq;
-                p.Eout[o] = 0.f;
-                p.Eout[N + o] = 0.f;
-                p.Eout[2 * N + o] = 0.f;
-                p.Bout[o] = 0.f;
-                p.Bout[N + o] = 0.f;
-                p.Bout[2 * N + o] = 0.f;
-            }
+    for (int j = 0; j < ROW_Z; ++j) d[j] = make_float2(0.f, 0.f);
+#pragma unroll
+    for (int l = 1; l <= MAXM; ++l) {
+#pragma unroll
+        for (int j = 0; j < ROW_Z; ++j) {
+            const float2 hi = PLUS ? w[MP + j + l] : w[MP + j + l - 1];
+            const float2 lo = PLUS ? w[MP + j - l + 1] : w[MP + j - l];
+            d[j] = __ffma2_rn(PLUS ? st.C2[l - 1] : st.Cm2[l - 1], __ffma2_rn(lo, minus, hi), d[j]);
         }
     }
 }
 
 __device__ __forceinline__ void cp_async_commit_group() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_prev_group() { asm volatile("cp.async.wait_group 1;\n" ::: "memory"); }
+__device__ __forceinline__ void cp_async_wait_groups() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
 
-// One z segment [z0, z0 + TZ) of rows xa .. xb - 1 (the body of the x-marching kernels).
-template <int MAXM, int TZ>
-__device__ __forceinline__ void march2_segment(const FieldP& p, int z0, int xa, int xb, float* sm) {
-    using T = March2T<MAXM, TZ>;
+// Row x of a field's three components over the segment's cells from zr0 on; zero outside the grid.
+template <int NT, bool VEC>
+__device__ __forceinline__ void stage_row(float* dst, const float* __restrict__ f0, const float* __restrict__ f1,
+                                          const float* __restrict__ f2, int zr0, int x, const GridP& g) {
+    constexpr int R = ROW_Z * NT;
+    const long long row = (long long)wrapi(x, g.nx) * g.nz;
+    const float* f[3] = {f0 + row, f1 + row, f2 + row};
+    if (VEC) {
+#pragma unroll
+        for (int k = 0; k < R / 4; k += NT) {
+            const int i = 4 * (k + threadIdx.x), gz = zr0 + i;
+            const bool in = gz >= 0 && gz < g.nz;
+#pragma unroll
+            for (int c = 0; c < 3; ++c) cp_async16(dst + c * R + i, f[c] + (in ? gz : 0), in);
+        }
+    } else {
+#pragma unroll
+        for (int k = 0; k < R; k += NT) {
+            const int i = k + threadIdx.x, gz = zr0 + i;
+            const bool in = gz >= 0 && gz < g.nz;
+#pragma unroll
+            for (int c = 0; c < 3; ++c) cp_async4z(dst + c * R + i, f[c] + (in ? gz : 0), in);
+        }
+    }
+}
+
+// Stores a lane's cells gz .. gz + 7 of three components at `row` (16-byte aligned rows), one cell
+// towards -z when the window moves: an output group then takes its last cell from the next lane, by
+// shuffle; where the next lane is in another warp or segment (`last`) that lane stores it itself
+// (`first`).  Every lane of a warp calls; the front column is zeroed.
+__device__ __forceinline__ void store_row(float* f, long long N, long long row, int gz, const GridP& g, bool owned, int shift,
+                                          bool first, bool last, const float (&a)[8], const float (&b)[8],
+                                          const float (&c)[8]) {
+    const float(*v[3])[8] = {&a, &b, &c};
+    if (!shift) {
+        if (!owned || gz >= g.nz) return;
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+            float* o = f + q * N + row + gz;
+            *reinterpret_cast<float4*>(o) = make_float4((*v[q])[0], (*v[q])[1], (*v[q])[2], (*v[q])[3]);
+            if (gz + 4 < g.nz)
+                *reinterpret_cast<float4*>(o + 4) = make_float4((*v[q])[4], (*v[q])[5], (*v[q])[6], (*v[q])[7]);
+        }
+        return;
+    }
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+        const float nx = __shfl_down_sync(0xffffffffu, (*v[q])[0], 1);
+        if (!owned || gz >= g.nz) continue;
+        float* o = f + q * N + row + gz;
+        const bool half = gz + 4 >= g.nz, front = gz + 8 >= g.nz;
+        *reinterpret_cast<float4*>(o) =
+            make_float4((*v[q])[1], (*v[q])[2], (*v[q])[3], half ? 0.f : (*v[q])[4]);
+        if (!half) {
+            if (front || !last) {
+                *reinterpret_cast<float4*>(o + 4) =
+                    make_float4((*v[q])[5], (*v[q])[6], (*v[q])[7], front ? 0.f : nx);
+            } else {
+                o[4] = (*v[q])[5];
+                o[5] = (*v[q])[6];
+                o[6] = (*v[q])[7];
+            }
+        }
+        if (first && gz > 0) o[-1] = (*v[q])[0];
+    }
+}
+
+// Rows xa .. xb - 1 of the segment producing the cells [z0, z0 + tz) (tz a multiple of ROW_Z, at most
+// RowT::OUT).
+template <int MAXM, int NT, bool VEC>
+__device__ __forceinline__ void march_rows(const FieldP& p, int z0, int tz, int xa, int xb, float* sm) {
+    using T = RowT<MAXM, NT, VEC>;
+    constexpr int MP = T::MP, R = T::R;
     const GridP& g = p.g;
     const long long N = g.ncell;
-    const bool vec = p.vec4 != 0;
-    auto Eslot = [&](int i) { return sm + i * T::SE; };
-    auto Bslot = [&](int i) { return sm + 4 * T::SE + i * T::SB; };
-    auto Jslot = [&](int i) { return sm + 4 * T::SE + 3 * T::SB + i * T::SJ; };
-    auto stageE = [&](int i, int x) {
-        stage_plane(Eslot(i), T::WE, p.Ein, p.Ein + N, p.Ein + 2 * N, 1, T::WE, z0 - T::H0, wrapi(x, g.nx), 0, 0, g,
-                    vec);
-    };
-    auto stageB = [&](int i, int x) {
-        stage_plane(Bslot(i), T::WB, p.Bin, p.Bin + N, p.Bin + 2 * N, 1, T::WB, z0 - T::H1, wrapi(x, g.nx), 0, 0, g,
-                    vec);
-    };
-    auto stageJ = [&](int i, int x) {
-        stage_plane(Jslot(i), T::WJ, p.J1, p.J2, p.J3, 1, T::WJ, z0 - T::H2, wrapi(x, g.nx), 0, 0, g, vec);
-    };
-    auto landed_all = [&]() {
-        cp_async_wait_all();
-        __syncthreads();
-    };
-    // prologue: B^{n+1/2}(xa-1), B^{n+1/2}(xa), E^{n+1}(xa), and the first prefetch
-    stageE(0, xa - 1);
-    stageE(1, xa);
-    stageB(0, xa - 1);
-    landed_all();
-    march2_bhalf<MAXM, TZ>(p, Bslot(0), Eslot(0), Eslot(1), z0);
-    stageE(2, xa + 1);
-    stageB(1, xa);
-    stageJ(0, xa);
-    landed_all();
-    march2_bhalf<MAXM, TZ>(p, Bslot(1), Eslot(1), Eslot(2), z0);
-    __syncthreads();
-    march2_enew<MAXM, TZ>(p, Eslot(1), Bslot(1), Bslot(0), Jslot(0), z0);
-    __syncthreads();
-    // E: ec = E^{n+1}(k), en = E^n(k+1), ef = E^n(k+2) (in flight), eg = free
-    // B: bc = B^{n+1/2}(k), bf = B^n(k+1) (in flight), bg = free;  J: jf = J(k+1) (in flight), jg = free
-    int ec = 1, en = 2, ef = 3, eg = 0, bc = 1, bf = 2, bg = 0, jf = 1, jg = 0;
-    stageE(ef, xa + 2);
-    stageB(bf, xa + 1);
-    stageJ(jf, xa + 1);
-    cp_async_commit_group();
-    for (int k = xa; k < xb; ++k) {
-        // the next step's rows, while this step computes
-        stageE(eg, k + 3);
-        stageB(bg, k + 2);
-        stageJ(jg, k + 2);
-        {
-            cp_async_commit_group();
-            cp_async_wait_prev_group();             // this step's rows (committed one step earlier)
+    const int t = threadIdx.x;
+    const float dt = g.dt, hz = 0.5f * dt / g.dz, fz = dt / g.dz, hx = 0.5f * dt / g.dx, fx = dt / g.dx;
+    float *sE = sm, *sB = sm + 3 * R, *sJ = sm + 6 * R;
+    float *own1 = sm + 9 * R + (t + T::D) * (4 * ROW_G), *own2 = own1 + T::PB, *own3 = own2 + T::PB;
+    float* sO = sm + 9 * R + 3 * T::PB;                        // !VEC: output rows E, B
+    const int zr0 = z0 - 3 * T::D * ROW_Z, gz = zr0 + ROW_Z * t;
+    const bool inside = gz >= 0 && gz + ROW_Z <= g.nz;
+    const bool owned = gz >= z0 && gz < z0 + tz;
+    const bool first = owned && ((t & 31) == 0 || gz == z0);
+    const bool last = owned && ((t & 31) == 31 || gz + ROW_Z >= z0 + tz);
+    auto mask = [&](float (&a)[8]) {
+        if (!inside) {
+#pragma unroll
+            for (int j = 0; j < 8; ++j) a[j] = (gz + j >= 0 && gz + j < g.nz) ? a[j] : 0.f;
         }
+    };
+    auto read3 = [&](const float* s, float (&a)[8], float (&b)[8], float (&c)[8]) {
+        lds8(a, s + ROW_Z * t);
+        lds8(b, s + R + ROW_Z * t);
+        lds8(c, s + 2 * R + ROW_Z * t);
+    };
+    // !VEC: own cells to an output row; after a barrier the CTA stores it with consecutive lanes on
+    // consecutive cells
+    auto keep3 = [&](float* o, const float (&a)[8], const float (&b)[8], const float (&c)[8]) {
+        const float(*v[3])[8] = {&a, &b, &c};
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+            float* d = o + q * R + ROW_Z * t;
+            *reinterpret_cast<float4*>(d) = make_float4((*v[q])[0], (*v[q])[1], (*v[q])[2], (*v[q])[3]);
+            *reinterpret_cast<float4*>(d + 4) = make_float4((*v[q])[4], (*v[q])[5], (*v[q])[6], (*v[q])[7]);
+        }
+    };
+    auto flush3 = [&](const float* o, float* f, int x) {
+        const long long row = (long long)x * g.nz;
+        for (int i = z0 - zr0 + t; i < z0 - zr0 + tz; i += NT) {
+            const int z = zr0 + i;
+            if (z >= g.nz) break;
+            const bool front = p.shift && z == g.nz - 1;
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                float* d = f + c * N + row + z;
+                if (z >= p.shift) d[-p.shift] = o[c * R + i];
+                if (front) d[0] = 0.f;
+            }
+        }
+    };
+    float En1[8], En2[8], En3[8];                              // E^n of the row ahead
+    stage_row<NT, VEC>(sE, p.Ein, p.Ein + N, p.Ein + 2 * N, zr0, xa - 1, g);
+    cp_async_commit_group();
+    cp_async_wait_groups();
+    __syncthreads();
+    read3(sE, En1, En2, En3);
+    put_pairs(own1, En2, En3);
+    __syncthreads();
+    stage_row<NT, VEC>(sE, p.Ein, p.Ein + N, p.Ein + 2 * N, zr0, xa, g);
+    stage_row<NT, VEC>(sB, p.Bin, p.Bin + N, p.Bin + 2 * N, zr0, xa - 1, g);
+    cp_async_commit_group();
+    stage_row<NT, VEC>(sJ, p.J1, p.J2, p.J3, zr0, xa, g);
+    cp_async_commit_group();
+    float Bm1[8], Bm3[8];                                      // B^{n+1/2} of the row behind
+    float Bp1[8], Bp2[8], Bp3[8];                              // B^{n+1} of it without the x differences
+    float Em1[8], Em3[8];                                      // E^{n+1} of it
+#pragma unroll 1
+    for (int r = xa - 1; r <= xb; ++r) {
+        float E1[8], E2[8], E3[8], b1[8], b2[8], b3[8];
+        float2 d[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) E1[j] = En1[j], E2[j] = En2[j], E3[j] = En3[j];
+        cp_async_wait_prev_group();                            // E^n(r + 1), B^n(r)
         __syncthreads();
-        march2_bhalf<MAXM, TZ>(p, Bslot(bf), Eslot(en), Eslot(ef), z0);
+        read3(sE, En1, En2, En3);
+        read3(sB, b1, b2, b3);
+        window_pairs<MAXM, MP, true>(p.st, own1, d);
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            b1[j] -= hx * (En3[j] - E3[j]);
+            b2[j] += hz * d[j].y;
+            b3[j] -= hz * d[j].x - hx * (En1[j] - E1[j]);
+        }
+        mask(b1);
+        mask(b2);
+        mask(b3);
+        put_pairs(own2, b2, b3);
+        cp_async_wait_groups();                                // J(r)
         __syncthreads();
-        march2_enew<MAXM, TZ>(p, Eslot(en), Bslot(bf), Bslot(bc), Jslot(jf), z0);
+        stage_row<NT, VEC>(sE, p.Ein, p.Ein + N, p.Ein + 2 * N, zr0, r + 2, g);
+        stage_row<NT, VEC>(sB, p.Bin, p.Bin + N, p.Bin + 2 * N, zr0, r + 1, g);
+        cp_async_commit_group();
+        put_pairs(own1, En2, En3);
+        if (r >= xa) {
+            float j1[8], j2[8], j3[8];
+            window_pairs<MAXM, MP, false>(p.st, own2, d);
+            read3(sJ, j1, j2, j3);
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                E1[j] = E1[j] + fx * (b3[j] - Bm3[j]) - dt * j1[j];
+                E2[j] = E2[j] - fz * d[j].y - dt * j2[j];
+                E3[j] = E3[j] + (fz * d[j].x - fx * (b1[j] - Bm1[j])) - dt * j3[j];
+            }
+            mask(E1);
+            mask(E2);
+            mask(E3);
+            put_pairs(own3, E2, E3);
+            if (r < xb) {
+                if (VEC) store_row(p.Eout, N, (long long)r * g.nz, gz, g, owned, p.shift, first, last, E1, E2, E3);
+                else keep3(sO, E1, E2, E3);
+            }
+            if (r > xa) {
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    Bp1[j] -= hx * (E3[j] - Em3[j]);
+                    Bp3[j] += hx * (E1[j] - Em1[j]);
+                }
+                if (VEC) store_row(p.Bout, N, (long long)(r - 1) * g.nz, gz, g, owned, p.shift, first, last, Bp1, Bp2, Bp3);
+                else keep3(sO + 3 * R, Bp1, Bp2, Bp3);
+            }
+#pragma unroll
+            for (int j = 0; j < 8; ++j) Em1[j] = E1[j], Em3[j] = E3[j];
+        }
+#pragma unroll
+        for (int j = 0; j < 8; ++j) Bm1[j] = b1[j], Bm3[j] = b3[j];
         __syncthreads();
-        march2_bnew_store<MAXM, TZ>(p, Eslot(ec), Eslot(en), Bslot(bc), z0, k, vec);
-        __syncthreads();
-        int t = ec;
-        ec = en;
-        en = ef;
-        ef = eg;
-        eg = t;
-        t = bc;
-        bc = bf;
-        bf = bg;
-        bg = t;
-        t = jf;
-        jf = jg;
-        jg = t;
+        stage_row<NT, VEC>(sJ, p.J1, p.J2, p.J3, zr0, r + 1, g);
+        cp_async_commit_group();
+        if (r >= xa) {
+            if (!VEC) {
+                if (r < xb) flush3(sO, p.Eout, r);
+                if (r > xa) flush3(sO + 3 * R, p.Bout, r - 1);
+            }
+            if (r < xb) {
+                window_pairs<MAXM, MP, true>(p.st, own3, d);
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    Bp1[j] = b1[j];
+                    Bp2[j] = b2[j] + hz * d[j].y;
+                    Bp3[j] = b3[j] - hz * d[j].x;
+                }
+            }
+        }
     }
-    cp_async_wait_all();                   // no copy may outlive the CTA's shared memory
+    cp_async_wait_groups();                                    // no copy may outlive the CTA's shared memory
 }
 
-template <int MAXM, int TZ, int NT>
-__global__ void __launch_bounds__(NT) field_advance_march2_kernel(FieldP p, int xc) {
+// cells per segment, a multiple of ROW_Z, for nseg segments of a row of nz cells
+__host__ __device__ inline int row_segment(int nz, int nseg) {
+    const int c = (nz + nseg - 1) / nseg;
+    return (c + ROW_Z - 1) / ROW_Z * ROW_Z;
+}
+
+template <int MAXM, int NT, bool VEC>
+__global__ void __launch_bounds__(NT) field_advance_rows_kernel(FieldP p, int tz, int xc) {
     extern __shared__ float4 smem4[];
-    const int z0 = blockIdx.x * TZ;
     const int xa = blockIdx.y * xc, xb = min(xa + xc, p.g.nx);
-    march2_segment<MAXM, TZ>(p, z0, xa, xb, reinterpret_cast<float*>(smem4));
+    march_rows<MAXM, NT, VEC>(p, blockIdx.x * tz, tz, xa, xb, reinterpret_cast<float*>(smem4));
 }
 
-// Many independent 2D grids: a persistent grid walks a work list of (instance, z segment, first
+// An instance's parameters to shared memory, by all threads.
+__device__ __forceinline__ void load_params(FieldP* dst, const FieldP* __restrict__ src) {
+    static_assert(sizeof(FieldP) % 8 == 0, "copied in 8-byte words");
+    for (int i = threadIdx.x; i < (int)(sizeof(FieldP) / 8); i += blockDim.x)
+        reinterpret_cast<unsigned long long*>(dst)[i] = __ldg(reinterpret_cast<const unsigned long long*>(src) + i);
+}
+
+// Many independent 2D grids: a persistent grid walks a work list of (instance, z0 | cells << 16, first
 // row, last row + 1) items; inst[2 i + parity] holds instance i's parameters for this step's
-// buffer direction.  Every item is the x-marching segment of field_advance_march2_kernel.
-template <int MAXM, int TZ, int NT>
-__global__ void __launch_bounds__(NT) field_advance_march2_batch_kernel(const FieldP* __restrict__ inst,
-                                                                        const int4* __restrict__ work, int nwork,
-                                                                        int parity) {
+// buffer direction.
+template <int MAXM, int NT>
+__global__ void __launch_bounds__(NT) field_advance_rows_batch_kernel(const FieldP* __restrict__ inst,
+                                                                      const int4* __restrict__ work, int nwork,
+                                                                      int parity) {
     extern __shared__ float4 smem4[];
     __shared__ FieldP sp;
+    float* sm = reinterpret_cast<float*>(smem4);
     for (int w = blockIdx.x; w < nwork; w += gridDim.x) {
         const int4 it = work[w];
         __syncthreads();                        // the previous item is done with sp
-        if (threadIdx.x == 0) sp = inst[2 * it.x + parity];
+        load_params(&sp, inst + 2 * it.x + parity);
         __syncthreads();
-        march2_segment<MAXM, TZ>(sp, it.y, it.z, it.w, reinterpret_cast<float*>(smem4));
+        const int z0 = it.y & 0xffff, tz = (unsigned)it.y >> 16;
+        if (sp.vec4) march_rows<MAXM, NT, true>(sp, z0, tz, it.z, it.w, sm);
+        else march_rows<MAXM, NT, false>(sp, z0, tz, it.z, it.w, sm);
     }
 }
 
@@ -1202,57 +1282,29 @@ __global__ void __launch_bounds__(256) field_advance_kernel(FieldP p) {
     advance_tile<NDIM, MAXM, TZ, TX, TY>(p, blockIdx.x, blockIdx.y, blockIdx.z, smem);
 }
 
-// Many independent grids in one launch: block b takes tile b of the concatenated tile list;
-// tile_start[i] is the first tile of instance i (tile_start[ninst] = total).  inst[2 i + parity]
-// holds instance i's parameters for this step's buffer direction.
+// Many independent grids in one launch: block b takes tile work[b] = (instance, tz, tx, ty);
+// inst[2 i + parity] holds instance i's parameters for this step's buffer direction.
 template <int NDIM, int MAXM, int TZ, int TX, int TY>
 __global__ void __launch_bounds__(256) field_advance_batch_kernel(const FieldP* __restrict__ inst,
-                                                                  const int* __restrict__ tile_start, int ninst,
-                                                                  int parity) {
+                                                                  const int4* __restrict__ work, int parity) {
     extern __shared__ float smem[];
     __shared__ FieldP sp;
-    __shared__ int sidx, slocal;
-    if (threadIdx.x == 0) {
-        const int t = blockIdx.x;
-        int lo = 0, hi = ninst - 1;          // last instance whose first tile is <= t
-        while (lo < hi) {
-            int mid = (lo + hi + 1) >> 1;
-            if (tile_start[mid] <= t) lo = mid; else hi = mid - 1;
-        }
-        sidx = lo;
-        slocal = t - tile_start[lo];
-        sp = inst[2 * lo + parity];
-    }
+    const int4 it = __ldg(work + blockIdx.x);
+    load_params(&sp, inst + 2 * it.x + parity);
     __syncthreads();
-    const int ntz = (sp.g.nz + TZ - 1) / TZ, ntx = (sp.g.nx + TX - 1) / TX;
-    const int l = slocal;
-    const int tz = l % ntz, tx = (l / ntz) % ntx, ty = NDIM == 3 ? l / (ntz * ntx) : 0;
-    advance_tile<NDIM, MAXM, TZ, TX, TY>(sp, tz, tx, ty, smem);
+    advance_tile<NDIM, MAXM, TZ, TX, TY>(sp, it.y, it.z, it.w, smem);
 }
 
 // The same tile list with the register-blocked tile (advance_tile_rb).
 template <int NDIM, int MAXM, int TZ, int TX, int TY>
 __global__ void __launch_bounds__(256, 2) field_advance_rb_batch_kernel(const FieldP* __restrict__ inst,
-                                                                        const int* __restrict__ tile_start, int ninst,
-                                                                        int parity) {
+                                                                        const int4* __restrict__ work, int parity) {
     extern __shared__ float4 smem4[];
     __shared__ FieldP sp;
-    __shared__ int slocal;
-    if (threadIdx.x == 0) {
-        const int t = blockIdx.x;
-        int lo = 0, hi = ninst - 1;          // last instance whose first tile is <= t
-        while (lo < hi) {
-            int mid = (lo + hi + 1) >> 1;
-            if (tile_start[mid] <= t) lo = mid; else hi = mid - 1;
-        }
-        slocal = t - tile_start[lo];
-        sp = inst[2 * lo + parity];
-    }
+    const int4 it = __ldg(work + blockIdx.x);
+    load_params(&sp, inst + 2 * it.x + parity);
     __syncthreads();
-    const int ntz = (sp.g.nz + TZ - 1) / TZ, ntx = (sp.g.nx + TX - 1) / TX;
-    const int l = slocal;
-    const int tz = l % ntz, tx = (l / ntz) % ntx, ty = NDIM == 3 ? l / (ntz * ntx) : 0;
-    advance_tile_rb<NDIM, MAXM, TZ, TX, TY>(sp, tz, tx, ty, reinterpret_cast<float*>(smem4));
+    advance_tile_rb<NDIM, MAXM, TZ, TX, TY>(sp, it.y, it.z, it.w, reinterpret_cast<float*>(smem4));
 }
 
 template <int NDIM, int MAXM, int TZ, int TX, int TY>
@@ -1329,28 +1381,42 @@ cudaError_t launch_fa_march(const FieldP& p, cudaStream_t s) {
     return cudaGetLastError();
 }
 
-template <int MAXM, int TZ, int NT>
-cudaError_t launch_fa_march2(const FieldP& p, cudaStream_t s) {
-    using T = March2T<MAXM, TZ>;
-    auto k = field_advance_march2_kernel<MAXM, TZ, NT>;
-    static bool configured = false;
-    if (!configured) {
-        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)T::smem_bytes);
-        if (e != cudaSuccess) return e;
-        configured = true;
-    }
-    // x chunks: one wave of CTAs over the SMs, each chunk at least 16 rows (the prologue of a
-    // chunk recomputes two rows)
+// CTAs of k that one SM holds (k already has its shared-memory limit), once per kernel
+template <typename K>
+int resident_ctas(K k, int nt, size_t smem) {
+    int n = 0;
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, nt, smem) == cudaSuccess && n > 0 ? n : 1;
+}
+
+inline int sm_count() {
     int dev = 0, nsm = 152;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    const int cols = (p.g.nz + TZ - 1) / TZ;
-    int per_sm = (int)((227 * 1024) / (T::smem_bytes + 1024));
-    per_sm = per_sm < 1 ? 1 : (per_sm > 2048 / NT ? 2048 / NT : per_sm);
-    const int xc = march_chunk(p.g.nx, cols, nsm * per_sm, 16);
-    dim3 grid(cols, (p.g.nx + xc - 1) / xc, 1);
-    k<<<grid, NT, T::smem_bytes, s>>>(p, xc);
+    return nsm;
+}
+
+template <int MAXM, int NT, bool VEC>
+cudaError_t launch_fa_rows_v(const FieldP& p, cudaStream_t s) {
+    using T = RowT<MAXM, NT, VEC>;
+    auto k = field_advance_rows_kernel<MAXM, NT, VEC>;
+    static int per_sm = 0;
+    if (!per_sm) {
+        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)T::smem_bytes);
+        if (e != cudaSuccess) return e;
+        per_sm = resident_ctas(k, NT, T::smem_bytes);
+    }
+    // equal segments along z; x chunks for one wave of CTAs, each of at least 8 rows (a chunk's first
+    // two rows of B^{n+1/2} and one of E^{n+1} are computed by its neighbours as well)
+    const int nseg = (p.g.nz + T::OUT - 1) / T::OUT, tz = row_segment(p.g.nz, nseg);
+    const int cols = (p.g.nz + tz - 1) / tz;
+    const int xc = march_chunk(p.g.nx, cols, sm_count() * per_sm, 8);
+    k<<<dim3(cols, (p.g.nx + xc - 1) / xc, 1), NT, T::smem_bytes, s>>>(p, tz, xc);
     return cudaGetLastError();
+}
+
+template <int MAXM, int NT>
+cudaError_t launch_fa_rows(const FieldP& p, cudaStream_t s) {
+    return p.vec4 ? launch_fa_rows_v<MAXM, NT, true>(p, s) : launch_fa_rows_v<MAXM, NT, false>(p, s);
 }
 
 template <int MAXM, int TZ, int TX, int NT>
@@ -1377,7 +1443,7 @@ cudaError_t launch_fa_march_ring(const FieldP& p, cudaStream_t s) {
 }
 
 template <int NDIM, int MAXM, int TZ, int TX, int TY>
-cudaError_t launch_fa_batch(const FieldP* inst, const int* tile_start, int ninst, int total, int parity,
+cudaError_t launch_fa_batch(const FieldP* inst, const int4* work, int total, int parity,
                             cudaStream_t s) {
     using T = Tile<NDIM, MAXM, TZ, TX, TY>;
     auto k = field_advance_batch_kernel<NDIM, MAXM, TZ, TX, TY>;
@@ -1387,14 +1453,14 @@ cudaError_t launch_fa_batch(const FieldP* inst, const int* tile_start, int ninst
         if (e != cudaSuccess) return e;
         configured = true;
     }
-    k<<<(unsigned)total, 256, T::smem_bytes, s>>>(inst, tile_start, ninst, parity);
+    k<<<(unsigned)total, 256, T::smem_bytes, s>>>(inst, work, parity);
     return cudaGetLastError();
 }
 
 }  // namespace
 
 template <int NDIM, int MAXM, int TZ, int TX, int TY>
-cudaError_t launch_fa_rb_batch(const FieldP* inst, const int* tile_start, int ninst, int total, int parity,
+cudaError_t launch_fa_rb_batch(const FieldP* inst, const int4* work, int total, int parity,
                                cudaStream_t s) {
     using T = TileRB<NDIM, MAXM, TZ, TX, TY>;
     auto k = field_advance_rb_batch_kernel<NDIM, MAXM, TZ, TX, TY>;
@@ -1404,84 +1470,129 @@ cudaError_t launch_fa_rb_batch(const FieldP* inst, const int* tile_start, int ni
         if (e != cudaSuccess) return e;
         configured = true;
     }
-    k<<<(unsigned)total, 256, T::smem_bytes, s>>>(inst, tile_start, ninst, parity);
+    k<<<(unsigned)total, 256, T::smem_bytes, s>>>(inst, work, parity);
     return cudaGetLastError();
 }
 
-template <int MAXM, int TZ, int NT>
-cudaError_t launch_fa_march2_batch(const FieldP* inst, const int4* work, int nwork, int parity, cudaStream_t s) {
-    using T = March2T<MAXM, TZ>;
-    auto k = field_advance_march2_batch_kernel<MAXM, TZ, NT>;
-    static bool configured = false;
-    if (!configured) {
-        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)T::smem_bytes);
-        if (e != cudaSuccess) return e;
-        configured = true;
+// CTAs of the batched x-march that run at once (its shared memory holds either kind of instance)
+template <int MAXM>
+int rows_batch_slots_m() {
+    using T = RowT<MAXM, ROWS_BATCH_NT, false>;
+    static int per_sm = 0;
+    if (!per_sm) {
+        auto k = field_advance_rows_batch_kernel<MAXM, ROWS_BATCH_NT>;
+        if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)T::smem_bytes) != cudaSuccess)
+            return 1;
+        per_sm = resident_ctas(k, ROWS_BATCH_NT, T::smem_bytes);
     }
-    int dev = 0, nsm = 152;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    int per_sm = (int)((227 * 1024) / (T::smem_bytes + 1024));
-    per_sm = per_sm < 1 ? 1 : (per_sm > 2048 / NT ? 2048 / NT : per_sm);
-    const int grid = nwork < nsm * per_sm ? nwork : nsm * per_sm;
-    if (grid <= 0) return cudaSuccess;
-    k<<<grid, NT, T::smem_bytes, s>>>(inst, work, nwork, parity);
+    return sm_count() * per_sm;
+}
+
+int rows_batch_slots(int maxm) {
+    return maxm <= 1 ? rows_batch_slots_m<1>() : maxm <= 4 ? rows_batch_slots_m<4>()
+         : maxm <= 8 ? rows_batch_slots_m<8>() : rows_batch_slots_m<16>();
+}
+
+template <int MAXM>
+cudaError_t launch_fa_rows_batch(const FieldP* inst, const int4* work, int nwork, int parity, cudaStream_t s) {
+    using T = RowT<MAXM, ROWS_BATCH_NT, false>;
+    const int slots = rows_batch_slots_m<MAXM>();
+    field_advance_rows_batch_kernel<MAXM, ROWS_BATCH_NT>
+        <<<nwork < slots ? nwork : slots, ROWS_BATCH_NT, T::smem_bytes, s>>>(inst, work, nwork, parity);
     return cudaGetLastError();
 }
 
-// Tiles of one grid in the batched field advance (same tile shapes as launch_field_advance_batch).
-// Batched 2D x-march: z segments of MARCH2_BATCH_TZ cells (64 threads), rows in chunks.
-cudaError_t launch_field_advance_march2_batch(const FieldP* inst, const int4* work, int nwork, int maxm, int parity,
-                                              cudaStream_t s) {
+// Batched 2D x-march: items of one z segment and a chunk of rows.
+cudaError_t launch_field_advance_rows_batch(const FieldP* inst, const int4* work, int nwork, int maxm, int parity,
+                                            cudaStream_t s) {
     if (nwork <= 0) return cudaSuccess;
-    if (maxm <= 1) return launch_fa_march2_batch<1, MARCH2_BATCH_TZ, 64>(inst, work, nwork, parity, s);
-    if (maxm <= 4) return launch_fa_march2_batch<4, MARCH2_BATCH_TZ, 64>(inst, work, nwork, parity, s);
-    if (maxm <= 8) return launch_fa_march2_batch<8, MARCH2_BATCH_TZ, 64>(inst, work, nwork, parity, s);
-    return launch_fa_march2_batch<16, MARCH2_BATCH_TZ, 64>(inst, work, nwork, parity, s);
+    if (maxm <= 1) return launch_fa_rows_batch<1>(inst, work, nwork, parity, s);
+    if (maxm <= 4) return launch_fa_rows_batch<4>(inst, work, nwork, parity, s);
+    if (maxm <= 8) return launch_fa_rows_batch<8>(inst, work, nwork, parity, s);
+    return launch_fa_rows_batch<16>(inst, work, nwork, parity, s);
 }
 
-int field_tiles(int ndim, int maxm, int nz, int nx, int ny) {
-    (void)maxm;
-    if (ndim == 2) return ((nz + 127) / 128) * ((nx + 7) / 8);
-    return ((nz + 63) / 64) * ((nx + 3) / 4) * ((ny + 3) / 4);
+int rows_batch_segment(int maxm, int nz) {
+    const int out = maxm <= 4 ? RowT<4, ROWS_BATCH_NT, false>::OUT
+                  : maxm <= 8 ? RowT<8, ROWS_BATCH_NT, false>::OUT : RowT<16, ROWS_BATCH_NT, false>::OUT;
+    return row_segment(nz, (nz + out - 1) / out);
 }
 
-cudaError_t launch_field_advance_rb_batch(const FieldP* inst, const int* tile_start, int ninst, int total_tiles,
+// Work items of the x-march over grids nz[i] x nx[i]: rows in equal chunks of at most `most`.
+// The CTAs of one wave share the items, so of the chunk lengths from 8 to 128 rows the one with the
+// fewest waves times rows a CTA walks (its chunk and the prologue's 2.5) is taken: on 128 instances of
+// 128..1024 x 64..256 cells a fixed chunk of 32 rows leaves the third of its waves 30% full.
+std::vector<int4> rows_batch_work(int maxm, const std::vector<int>& nz, const std::vector<int>& nx) {
+    const int slots = rows_batch_slots(maxm);
+    auto chunk = [](int n, int most) { return (n + (n + most - 1) / most - 1) / ((n + most - 1) / most); };
+    int best = 32;
+    double best_cost = 1e300;
+    for (int most = 8; most <= 128; ++most) {
+        long long items = 0;
+        for (size_t i = 0; i < nz.size(); ++i) {
+            const int tz = rows_batch_segment(maxm, nz[i]), c = chunk(nx[i], most);
+            items += (long long)((nz[i] + tz - 1) / tz) * ((nx[i] + c - 1) / c);
+        }
+        const double cost = (double)((items + slots - 1) / slots) * (most + 2.5);
+        if (cost < best_cost) {
+            best_cost = cost;
+            best = most;
+        }
+    }
+    std::vector<int4> work;
+    for (size_t i = 0; i < nz.size(); ++i) {
+        const int tz = rows_batch_segment(maxm, nz[i]), c = chunk(nx[i], best);
+        for (int z0 = 0; z0 < nz[i]; z0 += tz)
+            for (int xa = 0; xa < nx[i]; xa += c)
+                work.push_back(make_int4((int)i, z0 | tz << 16, xa, xa + c < nx[i] ? xa + c : nx[i]));
+    }
+    return work;
+}
+
+// Appends one grid's tiles to the list of the batched field advance (tile shapes of
+// launch_field_advance_batch and launch_field_advance_rb_batch).
+void batch_tiles(std::vector<int4>& work, int inst, int ndim, int nz, int nx, int ny) {
+    const int tz = ndim == 2 ? 128 : 64, tx = ndim == 2 ? 8 : 4, ty = ndim == 2 ? 1 : 4;
+    for (int k = 0; k < (ny + ty - 1) / ty; ++k)
+        for (int j = 0; j < (nx + tx - 1) / tx; ++j)
+            for (int i = 0; i < (nz + tz - 1) / tz; ++i) work.push_back(make_int4(inst, i, j, k));
+}
+
+cudaError_t launch_field_advance_rb_batch(const FieldP* inst, const int4* work, int total_tiles,
                                           int ndim, int maxm, int parity, cudaStream_t s) {
-    if (ninst <= 0 || total_tiles <= 0) return cudaSuccess;
+    if (total_tiles <= 0) return cudaSuccess;
     if (ndim == 2) {
-        if (maxm <= 1) return launch_fa_rb_batch<2, 1, 128, 8, 1>(inst, tile_start, ninst, total_tiles, parity, s);
-        if (maxm <= 4) return launch_fa_rb_batch<2, 4, 128, 8, 1>(inst, tile_start, ninst, total_tiles, parity, s);
-        if (maxm <= 8) return launch_fa_rb_batch<2, 8, 128, 8, 1>(inst, tile_start, ninst, total_tiles, parity, s);
-        return launch_fa_rb_batch<2, 16, 128, 8, 1>(inst, tile_start, ninst, total_tiles, parity, s);
+        if (maxm <= 1) return launch_fa_rb_batch<2, 1, 128, 8, 1>(inst, work, total_tiles, parity, s);
+        if (maxm <= 4) return launch_fa_rb_batch<2, 4, 128, 8, 1>(inst, work, total_tiles, parity, s);
+        if (maxm <= 8) return launch_fa_rb_batch<2, 8, 128, 8, 1>(inst, work, total_tiles, parity, s);
+        return launch_fa_rb_batch<2, 16, 128, 8, 1>(inst, work, total_tiles, parity, s);
     }
-    if (maxm <= 1) return launch_fa_rb_batch<3, 1, 64, 4, 4>(inst, tile_start, ninst, total_tiles, parity, s);
-    if (maxm <= 4) return launch_fa_rb_batch<3, 4, 64, 4, 4>(inst, tile_start, ninst, total_tiles, parity, s);
-    if (maxm <= 8) return launch_fa_rb_batch<3, 8, 64, 4, 4>(inst, tile_start, ninst, total_tiles, parity, s);
-    return launch_fa_rb_batch<3, 16, 64, 4, 4>(inst, tile_start, ninst, total_tiles, parity, s);
+    if (maxm <= 1) return launch_fa_rb_batch<3, 1, 64, 4, 4>(inst, work, total_tiles, parity, s);
+    if (maxm <= 4) return launch_fa_rb_batch<3, 4, 64, 4, 4>(inst, work, total_tiles, parity, s);
+    if (maxm <= 8) return launch_fa_rb_batch<3, 8, 64, 4, 4>(inst, work, total_tiles, parity, s);
+    return launch_fa_rb_batch<3, 16, 64, 4, 4>(inst, work, total_tiles, parity, s);
 }
 
-cudaError_t launch_field_advance_batch(const FieldP* inst, const int* tile_start, int ninst, int total_tiles,
+cudaError_t launch_field_advance_batch(const FieldP* inst, const int4* work, int total_tiles,
                                        int ndim, int maxm, int parity, cudaStream_t s) {
-    if (ninst <= 0 || total_tiles <= 0) return cudaSuccess;
+    if (total_tiles <= 0) return cudaSuccess;
     if (ndim == 2) {
-        if (maxm <= 1) return launch_fa_batch<2, 1, 128, 8, 1>(inst, tile_start, ninst, total_tiles, parity, s);
-        if (maxm <= 4) return launch_fa_batch<2, 4, 128, 8, 1>(inst, tile_start, ninst, total_tiles, parity, s);
-        if (maxm <= 8) return launch_fa_batch<2, 8, 128, 8, 1>(inst, tile_start, ninst, total_tiles, parity, s);
-        return launch_fa_batch<2, 16, 128, 8, 1>(inst, tile_start, ninst, total_tiles, parity, s);
+        if (maxm <= 1) return launch_fa_batch<2, 1, 128, 8, 1>(inst, work, total_tiles, parity, s);
+        if (maxm <= 4) return launch_fa_batch<2, 4, 128, 8, 1>(inst, work, total_tiles, parity, s);
+        if (maxm <= 8) return launch_fa_batch<2, 8, 128, 8, 1>(inst, work, total_tiles, parity, s);
+        return launch_fa_batch<2, 16, 128, 8, 1>(inst, work, total_tiles, parity, s);
     }
-    if (maxm <= 1) return launch_fa_batch<3, 1, 64, 4, 4>(inst, tile_start, ninst, total_tiles, parity, s);
-    if (maxm <= 4) return launch_fa_batch<3, 4, 64, 4, 4>(inst, tile_start, ninst, total_tiles, parity, s);
-    if (maxm <= 8) return launch_fa_batch<3, 8, 64, 4, 4>(inst, tile_start, ninst, total_tiles, parity, s);
-    return launch_fa_batch<3, 16, 64, 4, 4>(inst, tile_start, ninst, total_tiles, parity, s);
+    if (maxm <= 1) return launch_fa_batch<3, 1, 64, 4, 4>(inst, work, total_tiles, parity, s);
+    if (maxm <= 4) return launch_fa_batch<3, 4, 64, 4, 4>(inst, work, total_tiles, parity, s);
+    if (maxm <= 8) return launch_fa_batch<3, 8, 64, 4, 4>(inst, work, total_tiles, parity, s);
+    return launch_fa_batch<3, 16, 64, 4, 4>(inst, work, total_tiles, parity, s);
 }
 
 // Tile variants the autotuner chooses from.  2D: (TZ, TX); 3D: (TZ, TX, TY); rb = register-
 // blocked tile (four z cells per thread).
 //   2D: 0 = 128 x 8, 1 = 256 x 4, 2 = 64 x 16, 3 = 256 x 8,
 //       4 = rb 128 x 8, 5 = rb 256 x 4, 6 = rb 128 x 4, 7 = rb 256 x 8,
-//       8 = x-march z 448 (128 threads), 9 = x-march z 384 (128 threads),
-//       10 = x-march z 960 (256 threads), 11 = x-march z 192 (64 threads)
+//       8 .. 11 = x-march, eight z cells per thread, segments of 128, 96, 256 and 64 threads
 //   3D: 0 = 64 x 4 x 4, 1 = 128 x 4 x 2, 2 = 32 x 8 x 4,
 //       3 = rb 64 x 4 x 4, 4 = rb 128 x 4 x 2, 5 = rb 32 x 8 x 4,
 //       6 = y-march 128 x 4 (256 threads), 7 = y-march 128 x 4 (128 threads),
@@ -1508,10 +1619,10 @@ cudaError_t launch_fa_variant(const FieldP& p, int v, cudaStream_t s) {
             case 5: return launch_fa_rb<2, MAXM, 256, 4, 1>(p, s);
             case 6: return launch_fa_rb<2, MAXM, 128, 4, 1>(p, s);
             case 7: return launch_fa_rb<2, MAXM, 256, 8, 1>(p, s);
-            case 8: return launch_fa_march2<MAXM, 448, 128>(p, s);
-            case 9: return launch_fa_march2<MAXM, 384, 128>(p, s);
-            case 10: return launch_fa_march2<MAXM, 960, 256>(p, s);
-            case 11: return launch_fa_march2<MAXM, 192, 64>(p, s);
+            case 8: return launch_fa_rows<MAXM, 128>(p, s);
+            case 9: return launch_fa_rows<MAXM, 96>(p, s);
+            case 10: return launch_fa_rows<MAXM, 256>(p, s);
+            case 11: return launch_fa_rows<MAXM, 64>(p, s);
             default: return launch_fa<2, MAXM, 128, 8, 1>(p, s);
         }
     }

@@ -482,6 +482,8 @@ pic_status pic_destroy(pic_t* h) {
         cudaEventDestroy(h->ev_a[i]);
         cudaEventDestroy(h->ev_b[i]);
     }
+        h->st.C2[l] = make_float2(h->st.C[l], h->st.C[l]);
+        h->st.Cm2[l] = make_float2(h->st.Cm[l], h->st.Cm[l]);
     for (auto& q : h->sp) {
         dfree(q.prev_cell);
         dfree(q.prev_off);
@@ -958,8 +960,8 @@ struct pic_batch_t {
     struct FieldGroup {
         std::vector<int> members;
         FieldP* d_inst = nullptr;
-        int* d_tiles = nullptr;
-        int4* d_work = nullptr;      // 2D: x-marching work items (instance, z0, first row, end row)
+        int4* d_tiles = nullptr;     // tiles (instance, tz, tx, ty)
+        int4* d_work = nullptr;      // 2D: x-marching work items (instance, z0 | cells << 16, first row, end row)
         int total = 0, maxm = 1, nwork = 0;
         int variant = 1;             // 0: one cell per thread, 1: register-blocked, 2: x-marching (2D)
         double ms[3] = {0, 0, 0};    // batch autotune: time of one launch per variant (0: not timed)
@@ -1043,8 +1045,8 @@ pic_status batch_build(pic_batch_t* b) {
     for (int c = 0; c < 4; ++c) {
         auto& f = b->fg[c];
         std::vector<FieldP> inst;
-        std::vector<int> tiles(1, 0);
-        std::vector<int4> work;
+        std::vector<int4> tiles;
+        std::vector<int> nzs, nxs;
         for (int j = 0; j < (int)f.members.size(); ++j) {
             pic_t* h = b->h[f.members[j]];
             const bool aligned = ((uintptr_t)h->E | (uintptr_t)h->B | (uintptr_t)h->J | (uintptr_t)h->E2 |
@@ -1064,13 +1066,13 @@ pic_status batch_build(pic_batch_t* b) {
                 p.vec4 = (h->g.nz % 4 == 0 && aligned) ? 1 : 0;
                 inst.push_back(p);
             }
-            tiles.push_back(tiles.back() + field_tiles(b->ndim, maxm_of[c], h->g.nz, h->g.nx, h->g.ny));
-            if (b->ndim == 2)
-                for (int z0 = 0; z0 < h->g.nz; z0 += MARCH2_BATCH_TZ)
-                    for (int xa = 0; xa < h->g.nx; xa += MARCH2_BATCH_XC)
-                        work.push_back(make_int4(j, z0, xa, std::min(xa + MARCH2_BATCH_XC, h->g.nx)));
+            batch_tiles(tiles, j, b->ndim, h->g.nz, h->g.nx, h->g.ny);
+            nzs.push_back(h->g.nz);
+            nxs.push_back(h->g.nx);
         }
-        f.total = tiles.back();
+        std::vector<int4> work;
+        if (b->ndim == 2) work = rows_batch_work(maxm_of[c], nzs, nxs);
+        f.total = (int)tiles.size();
         f.maxm = maxm_of[c];
         f.nwork = (int)work.size();
         if (upload(&f.d_inst, inst) != cudaSuccess || upload(&f.d_tiles, tiles) != cudaSuccess ||
@@ -1108,11 +1110,10 @@ pic_status batch_build(pic_batch_t* b) {
 
 cudaError_t batch_field_launch(pic_batch_t* b, const pic_batch_t::FieldGroup& f, int variant, int parity,
                                cudaStream_t s) {
-    const int n = (int)f.members.size();
     if (variant == 2 && b->ndim == 2)
-        return launch_field_advance_march2_batch(f.d_inst, f.d_work, f.nwork, f.maxm, parity, s);
-    if (variant == 1) return launch_field_advance_rb_batch(f.d_inst, f.d_tiles, n, f.total, b->ndim, f.maxm, parity, s);
-    return launch_field_advance_batch(f.d_inst, f.d_tiles, n, f.total, b->ndim, f.maxm, parity, s);
+        return launch_field_advance_rows_batch(f.d_inst, f.d_work, f.nwork, f.maxm, parity, s);
+    if (variant == 1) return launch_field_advance_rb_batch(f.d_inst, f.d_tiles, f.total, b->ndim, f.maxm, parity, s);
+    return launch_field_advance_batch(f.d_inst, f.d_tiles, f.total, b->ndim, f.maxm, parity, s);
 }
 
 // Batch autotune: per stencil class, time one field-advance launch (parity 0: reads E, B, J,

@@ -2,6 +2,7 @@
 #pragma once
 
 #include <cstdint>
+#include <vector>
 #include <cuda_runtime.h>
 
 #include "../../include/pic.h"
@@ -43,6 +44,7 @@ struct StencilP {
     int M;
     float C[PIC_MAX_M];
     float Cm[PIC_MAX_M];
+    float2 C2[PIC_MAX_M], Cm2[PIC_MAX_M];   // each coefficient twice: operands of packed arithmetic
 };
 
 // Field-advance launch parameters.
@@ -118,18 +120,18 @@ int field_variants(int ndim);
 int default_field_variant(int ndim, int M);
 
 // batched: instance tables live in device memory
-cudaError_t launch_field_advance_batch(const FieldP* inst, const int* tile_start, int ninst, int total_tiles,
-                                       int ndim, int maxm, int parity, cudaStream_t s);
-int field_tiles(int ndim, int maxm, int nz, int nx, int ny);
-// Batched 2D field advance with the x-marching segments: work[w] = (instance, z0, first row,
-// last row + 1); z segments of MARCH2_BATCH_TZ cells.
-constexpr int MARCH2_BATCH_TZ = 192;
-constexpr int MARCH2_BATCH_XC = 32;
+cudaError_t launch_field_advance_batch(const FieldP* inst, const int4* work, int total_tiles, int ndim, int maxm,
+                                       int parity, cudaStream_t s);
+void batch_tiles(std::vector<int4>& work, int inst, int ndim, int nz, int nx, int ny);
+// Batched 2D field advance with the x-marching segments: work[w] = (instance, z0 | cells << 16, first
+// row, last row + 1).
+constexpr int ROWS_BATCH_NT = 64;
+std::vector<int4> rows_batch_work(int maxm, const std::vector<int>& nz, const std::vector<int>& nx);
 // The same tile list as launch_field_advance_batch with register-blocked tiles.
-cudaError_t launch_field_advance_rb_batch(const FieldP* inst, const int* tile_start, int ninst, int total_tiles,
-                                          int ndim, int maxm, int parity, cudaStream_t s);
-cudaError_t launch_field_advance_march2_batch(const FieldP* inst, const int4* work, int nwork, int maxm, int parity,
-                                              cudaStream_t s);
+cudaError_t launch_field_advance_rb_batch(const FieldP* inst, const int4* work, int total_tiles, int ndim, int maxm,
+                                          int parity, cudaStream_t s);
+cudaError_t launch_field_advance_rows_batch(const FieldP* inst, const int4* work, int nwork, int maxm, int parity,
+                                            cudaStream_t s);
 cudaError_t launch_correct_j1_batch(const CorrInst* inst, int ninst, int max_rows, int max_nz, cudaStream_t s);
 cudaError_t launch_push_batch(const PartInst* inst, int ninst, int ndim, int shape, long long max_extent, int parity,
                               cudaStream_t s);
