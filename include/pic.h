@@ -310,9 +310,18 @@ pic_status pic_timing_read(pic_t* h, double* ms, int64_t* launches, void* stream
  *           it in J (the filter precedes the correction and does not depend on C);
  *   aE, aB: device, updated in place; grad: device double[M], accumulated (not cleared).
  * The transposed operators use d-x = (d+x)^T (the pair of Appendix C), so the adjoint step is
- * the leapfrog with the roles of d+ and d- exchanged.  Library scratch: 7 nz nx ny floats.  */
+ * the leapfrog with the roles of d+ and d- exchanged.  Library scratch: 3 nz nx ny floats.  */
 pic_status pic_adjoint_step(pic_t* h, const float* E, const float* B, const float* J, float* aE, float* aB,
                             double* grad, void* stream);
+/* The two passes of a backward run over recorded steps (device arrays of contiguous steps):
+ *   pic_step_record: nsteps steps as pic_step makes them, but from E[0], B[0] (3 nz nx ny floats per
+ *     step) into E[1], B[1], .., E[nsteps], B[nsteps], the current of step k into J[k]; the bound
+ *     fields and the bound J are not touched.  Finite-difference solvers, no moving window.
+ *   pic_adjoint_run: nsteps x pic_adjoint_step over such a record, from its last step to its first;
+ *     E holds nsteps + 1 entries, so a step's new E need not be rebuilt.                        */
+pic_status pic_step_record(pic_t* h, int nsteps, float* E, float* B, float* J, void* stream);
+pic_status pic_adjoint_run(pic_t* h, int nsteps, const float* E, const float* B, const float* J, float* aE, float* aB,
+                           double* grad, void* stream);
 
 /* ---- tile autotuner ----------------------------------------------------------------------
  * pic_autotune times each field-advance tile variant on the handle's bound fields (results go
@@ -322,7 +331,7 @@ pic_status pic_adjoint_step(pic_t* h, const float* E, const float* B, const floa
  * PIC_MAX_TILE_VARIANTS entries) and the number of variants.  2D (z x x): 0 = 128x8,
  * 1 = 256x4, 2 = 64x16, 3 = 256x8 with one cell per thread and stage, 4 = 128x8, 5 = 256x4,
  * 6 = 128x4, 7 = 256x8 register-blocked (four z cells per thread, 128-bit shared loads),
- * 8..11 register-blocked z segments of 448, 384, 960, 192 cells that march along x with the
+ * 8..11 z segments of 128, 96, 256, 64 threads with eight cells each that march along x with the
  * next rows prefetched;
  * 3D (z x x x y): 0 = 64x4x4, 1 = 128x4x2, 2 = 32x8x4, 3..5 the same shapes register-
  * blocked, 6..9 register-blocked columns that march along y (z x x = 128x4 with 256 or 128

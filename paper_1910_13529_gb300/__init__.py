@@ -31,7 +31,7 @@ EXPORTS = ["pic_create", "pic_destroy", "pic_last_error", "pic_fit_coefficients"
            "pic_get_count", "pic_get_state", "pic_sync", "pic_timing", "pic_timing_read", "pic_gauss_static",
            "pic_batch_create", "pic_batch_instance", "pic_batch_step", "pic_batch_destroy", "pic_batch_get_tuning",
            "pic_autotune", "pic_get_tuning", "pic_set_tuning", "pic_adjoint_step",
-           "pic_set_state", "pic_get_next_id"]
+           "pic_step_record", "pic_adjoint_run", "pic_set_state", "pic_get_next_id"]
 TIMING_KEYS = ["particles", "deposit", "correction", "fields", "sort", "window", "diag", "filter"]
 
 
@@ -101,6 +101,8 @@ def _load():
         "pic_get_tuning": ([vp, ip, dp, ip], ctypes.c_int),
         "pic_set_tuning": ([vp, ctypes.c_int], ctypes.c_int),
         "pic_adjoint_step": ([vp, vp, vp, vp, vp, vp, vp, vp], ctypes.c_int),
+        "pic_step_record": ([vp, ctypes.c_int, vp, vp, vp, vp], ctypes.c_int),
+        "pic_adjoint_run": ([vp, ctypes.c_int, vp, vp, vp, vp, vp, vp, vp], ctypes.c_int),
         "pic_batch_get_tuning": ([vp, ip, dp], ctypes.c_int),
         "pic_set_state": ([vp, ctypes.c_int64, ctypes.c_int64, ctypes.c_int, ctypes.c_int64], ctypes.c_int),
         "pic_get_next_id": ([vp, i64p], ctypes.c_int),
@@ -306,6 +308,14 @@ def pic_set_tuning(h, variant):
 
 def pic_adjoint_step(h, E_ptr, B_ptr, J_ptr, aE_ptr, aB_ptr, grad_ptr, stream):
     _check(lib.pic_adjoint_step(h, E_ptr, B_ptr, J_ptr, aE_ptr, aB_ptr, grad_ptr, stream), h)
+
+
+def pic_step_record(h, nsteps, E_ptr, B_ptr, J_ptr, stream):
+    _check(lib.pic_step_record(h, int(nsteps), E_ptr, B_ptr, J_ptr, stream), h)
+
+
+def pic_adjoint_run(h, nsteps, E_ptr, B_ptr, J_ptr, aE_ptr, aB_ptr, grad_ptr, stream):
+    _check(lib.pic_adjoint_run(h, int(nsteps), E_ptr, B_ptr, J_ptr, aE_ptr, aB_ptr, grad_ptr, stream), h)
 
 
 def pic_set_state(h, step, shifts, pending_shift, next_id):

@@ -67,7 +67,7 @@ struct pic_t {
     std::vector<int> ev_cat;
     size_t ev_used = 0;
     long long launches[PIC_TIMING_N] = {0};
-    float* adj_scratch = nullptr; // adjoint: B', E', W (7 N floats)
+    float* adj_scratch = nullptr; // adjoint: E' of the step (3 N floats)
     double* static_rho = nullptr; // device address of g_static_rho on this handle's device
     int fa_variant = 0;           // field-advance tile variant (pic_autotune)
     KSpaceState* ks = nullptr;    // k-space solvers: transforms, buffers and symbol tables
@@ -294,6 +294,62 @@ pic_status do_sort(pic_t* h, cudaStream_t s) {
     return PIC_OK;
 }
 
+pic_status adjoint_supported(pic_t* h, const char* who) {
+    if (h->split) return fail(h, PIC_ERR_ARG, "%s needs one coefficient set (no coef_b)", who);
+    if (h->ks) return fail(h, PIC_ERR_ARG, "%s: finite-difference solvers only", who);
+    return PIC_OK;
+}
+
+// The three stages of one adjoint step; Ep: the step's E^{n+1} (components 2 and 3 are read).
+pic_status adjoint_stages(pic_t* h, const float* E, const float* B, const float* J, const float* Ep, float* aE, float* aB,
+                          double* grad, cudaStream_t s) {
+    CK(h, launch_adjoint_ampere(h->g, h->st, Ep, aB, aE, grad, s), "adjoint: third stage");
+    CK(h, launch_adjoint_faraday(h->g, h->st, E, B, J, aE, aB, h->hf, h->hlen, grad, s), "adjoint: second stage");
+    CK(h, launch_adjoint_ampere(h->g, h->st, E, aB, aE, grad, s), "adjoint: first stage");
+    return PIC_OK;
+}
+
+// One step n: particles and currents of every species into J, then the fields from (Ein, Bin) into
+// (Eout, Bout).
+pic_status one_step(pic_t* h, const float* Ein, const float* Bin, float* Eout, float* Bout, cudaStream_t s) {
+    pic_status st;
+    if (h->cfg.sort_every > 0 && h->step % h->cfg.sort_every == 0)
+        if ((st = do_sort(h, s))) return st;
+    {
+        Scope sc(h, PIC_T_DEPOSIT, 1, s);
+        CK(h, cudaMemsetAsync(h->J, 0, sizeof(float) * 3 * h->g.ncell, s), "zero J");
+    }
+    SpeciesP sps[PIC_MAX_SPECIES];
+    int* defers[PIC_MAX_SPECIES];
+    long long extents[PIC_MAX_SPECIES];
+    int nsp = 0;
+    for (int i = 0; i < PIC_MAX_SPECIES; ++i) {
+        if (!h->sp[i].bound) continue;
+        SpeciesSlot& q = h->sp[i];
+        if (h->cfg.ndim == 3 && !q.defer) {
+            const long long len = defer_len(q.cap);              // two lists of this length
+            if ((st = dalloc(h, &q.defer, 2 * len, "deferred chunk lists"))) return st;
+            CK(h, cudaMemsetAsync(q.defer, 0, sizeof(int32_t) * 2, s), "clear deferred chunk list");
+            CK(h, cudaMemsetAsync(q.defer + len, 0, sizeof(int32_t) * 2, s), "clear deferred chunk list");
+        }
+        SpeciesP sp = species_params(h, i);
+        sps[nsp] = sp;
+        defers[nsp] = q.defer;
+        extents[nsp++] = q.extent;
+        Scope sc(h, PIC_T_PARTICLES, 1, s);
+        CK(h, launch_push(h->g, sp, Ein, Bin, h->J, h->pending_shift, 0, q.extent, q.defer, h->status, s),
+           "fused push/deposit kernel");
+    }
+    if (h->cfg.ndim == 3 && nsp > 0) {
+        Scope sc(h, PIC_T_PARTICLES, 1, s);
+        CK(h, launch_push_leftover(h->g, sps, defers, extents, nsp, Ein, Bin, h->J, h->pending_shift, s),
+           "deferred chunks kernel");
+    }
+    h->pending_shift = 0;
+    if ((st = smooth_current(h, s))) return st;
+    return advance_fields(h, Ein, Bin, Eout, Bout, s);
+}
+
 }  // namespace
 
 extern "C" {
@@ -426,6 +482,8 @@ pic_status pic_create(const pic_config* cfg, pic_t** out) {
         h->C64b[l] = l < M ? CB[l] : 0.0;
         h->st.C[l] = (float)h->C64[l];
         h->st.Cm[l] = (float)h->C64b[l];
+        h->st.C2[l] = make_float2(h->st.C[l], h->st.C[l]);
+        h->st.Cm2[l] = make_float2(h->st.Cm[l], h->st.Cm[l]);
         yee_b = yee_b && h->C64b[l] == (l == 0 ? 1.0 : 0.0);
     }
     // Sec. 3 correction: P = [k]_B1 / [k]_Yee, from the B-side coefficients
@@ -482,8 +540,6 @@ pic_status pic_destroy(pic_t* h) {
         cudaEventDestroy(h->ev_a[i]);
         cudaEventDestroy(h->ev_b[i]);
     }
-        h->st.C2[l] = make_float2(h->st.C[l], h->st.C[l]);
-        h->st.Cm2[l] = make_float2(h->st.Cm[l], h->st.Cm[l]);
     for (auto& q : h->sp) {
         dfree(q.prev_cell);
         dfree(q.prev_off);
@@ -617,41 +673,7 @@ pic_status pic_step(pic_t* h, int nsteps, void* stream) {
     const long long N = h->g.ncell;
     float *Ec = h->E, *Bc = h->B, *En = h->E2, *Bn = h->B2;
     for (int it = 0; it < nsteps; ++it) {
-        if (h->cfg.sort_every > 0 && h->step % h->cfg.sort_every == 0)
-            if ((st = do_sort(h, s))) return st;
-        {
-            Scope sc(h, PIC_T_DEPOSIT, 1, s);
-            CK(h, cudaMemsetAsync(h->J, 0, sizeof(float) * 3 * N, s), "zero J");
-        }
-        SpeciesP sps[PIC_MAX_SPECIES];
-        int* defers[PIC_MAX_SPECIES];
-        long long extents[PIC_MAX_SPECIES];
-        int nsp = 0;
-        for (int i = 0; i < PIC_MAX_SPECIES; ++i) {
-            if (!h->sp[i].bound) continue;
-            SpeciesSlot& q = h->sp[i];
-            if (h->cfg.ndim == 3 && !q.defer) {
-                const long long len = defer_len(q.cap);              // two lists of this length
-                if ((st = dalloc(h, &q.defer, 2 * len, "deferred chunk lists"))) return st;
-                CK(h, cudaMemsetAsync(q.defer, 0, sizeof(int32_t) * 2, s), "clear deferred chunk list");
-                CK(h, cudaMemsetAsync(q.defer + len, 0, sizeof(int32_t) * 2, s), "clear deferred chunk list");
-            }
-            SpeciesP sp = species_params(h, i);
-            sps[nsp] = sp;
-            defers[nsp] = q.defer;
-            extents[nsp++] = q.extent;
-            Scope sc(h, PIC_T_PARTICLES, 1, s);
-            CK(h, launch_push(h->g, sp, Ec, Bc, h->J, h->pending_shift, 0, q.extent, q.defer, h->status, s),
-               "fused push/deposit kernel");
-        }
-        if (h->cfg.ndim == 3 && nsp > 0) {
-            Scope sc(h, PIC_T_PARTICLES, 1, s);
-            CK(h, launch_push_leftover(h->g, sps, defers, extents, nsp, Ec, Bc, h->J, h->pending_shift, s),
-               "deferred chunks kernel");
-        }
-        h->pending_shift = 0;
-        if ((st = smooth_current(h, s))) return st;
-        if ((st = advance_fields(h, Ec, Bc, En, Bn, s))) return st;
+        if ((st = one_step(h, Ec, Bc, En, Bn, s))) return st;
         float* t = Ec;
         Ec = En;
         En = t;
@@ -666,6 +688,24 @@ pic_status pic_step(pic_t* h, int nsteps, void* stream) {
     }
     h->state = 0;
     return PIC_OK;
+}
+
+pic_status pic_step_record(pic_t* h, int nsteps, float* E, float* B, float* J, void* stream) {
+    if (!h) return PIC_ERR_ARG;
+    if (nsteps < 0 || !E || !B || !J) return fail(h, PIC_ERR_ARG, "pic_step_record: nsteps < 0 or a null array");
+    if (h->cfg.moving_window || h->ks)
+        return fail(h, PIC_ERR_ARG, "pic_step_record: finite-difference solvers without a moving window");
+    if (h->state == 1) return fail(h, PIC_ERR_STATE, "pic_step_record after pic_gather_push without pic_deposit");
+    const long long n3 = 3 * h->g.ncell;
+    float* const bound = h->J;
+    pic_status st = PIC_OK;
+    for (int k = 0; !st && k < nsteps; ++k) {
+        h->J = J + k * n3;
+        st = one_step(h, E + k * n3, B + k * n3, E + (k + 1) * n3, B + (k + 1) * n3, (cudaStream_t)stream);
+    }
+    h->J = bound;
+    if (!st) h->state = 0;
+    return st;
 }
 
 pic_status pic_filter_current(pic_t* h, void* stream) {
@@ -842,34 +882,23 @@ pic_status pic_timing_read(pic_t* h, double* ms, int64_t* launches, void* stream
 pic_status pic_adjoint_step(pic_t* h, const float* E, const float* B, const float* J, float* aE, float* aB,
                             double* grad, void* stream) {
     if (!h || !E || !B || !J || !aE || !aB || !grad) return PIC_ERR_ARG;
-    if (h->split) return fail(h, PIC_ERR_ARG, "pic_adjoint_step needs one coefficient set (no coef_b)");
-    if (h->ks) return fail(h, PIC_ERR_ARG, "pic_adjoint_step: finite-difference solvers only");
-    const long long N = h->g.ncell;
-    if (!h->adj_scratch) {
-        pic_status st = dalloc(h, &h->adj_scratch, 7 * N, "adjoint scratch");
-        if (st) return st;
-    }
     cudaStream_t s = (cudaStream_t)stream;
-    float* Bh = h->adj_scratch;        // B' = B - h T E
-    float* Ep = Bh + 3 * N;            // E' = E + dt (S B' - J)
-    float* W = Ep + 3 * N;             // P^{-1} aE1
-    const float dt = h->g.dt, hh = 0.5f * dt;
-    const int M = h->st.M;
-    const GridP& g = h->g;
-    CK(h, launch_curl_plus_update(g, h->st, B, E, -hh, Bh, s), "adjoint: B half step");
-    CK(h, launch_curl_minus_update(g, h->st, E, Bh, J, dt, -dt, Ep, s), "adjoint: E step");
-    CK(h, launch_grad_plus(g, M, aB, Ep, -(double)hh, grad, s), "adjoint: gradient (third stage)");
-    CK(h, launch_curl_minus_update(g, h->st, aE, aB, nullptr, -hh, 0.f, aE, s), "adjoint: third stage");
-    CK(h, launch_grad_minus(g, M, aE, Bh, (double)dt, grad, s), "adjoint: gradient (second stage)");
-    if (h->hlen > 0) {
-        CK(h, cudaMemcpyAsync(W, aE, sizeof(float) * N, cudaMemcpyDeviceToDevice, s), "adjoint: copy aE1");
-        CK(h, launch_correct_j1(g, h->hf, h->hlen, W, s), "adjoint: P^-1 aE1");
-        CK(h, launch_grad_corr(g, M, W, J, (double)dt, grad, s), "adjoint: gradient (correction)");
-    }
-    CK(h, launch_curl_plus_update(g, h->st, aB, aE, dt, aB, s), "adjoint: second stage");
-    CK(h, launch_grad_plus(g, M, aB, E, -(double)hh, grad, s), "adjoint: gradient (first stage)");
-    CK(h, launch_curl_minus_update(g, h->st, aE, aB, nullptr, -hh, 0.f, aE, s), "adjoint: first stage");
-    return PIC_OK;
+    pic_status st = adjoint_supported(h, "pic_adjoint_step");
+    if (st) return st;
+    if (!h->adj_scratch && (st = dalloc(h, &h->adj_scratch, 3 * h->g.ncell, "adjoint scratch"))) return st;
+    CK(h, launch_adjoint_enew(h->g, h->st, E, B, J, h->adj_scratch, s), "adjoint: E step");
+    return adjoint_stages(h, E, B, J, h->adj_scratch, aE, aB, grad, s);
+}
+
+pic_status pic_adjoint_run(pic_t* h, int nsteps, const float* E, const float* B, const float* J, float* aE, float* aB,
+                           double* grad, void* stream) {
+    if (!h || nsteps < 0 || !E || !B || !J || !aE || !aB || !grad) return PIC_ERR_ARG;
+    cudaStream_t s = (cudaStream_t)stream;
+    pic_status st = adjoint_supported(h, "pic_adjoint_run");
+    const long long n3 = 3 * h->g.ncell;
+    for (int k = nsteps - 1; !st && k >= 0; --k)
+        st = adjoint_stages(h, E + k * n3, B + k * n3, J + k * n3, E + (k + 1) * n3, aE, aB, grad, s);
+    return st;
 }
 
 // Tile autotuner: time every field-advance tile variant on this handle's bound fields (the

@@ -174,16 +174,17 @@ cudaError_t launch_filter_rho(const GridP& g, double* rho, cudaStream_t s);
 cudaError_t launch_filter_current_batch(const FiltInst* inst, int ninst, long long max_rows3, cudaStream_t s);
 
 // ---- adjoint (adjoint_kernels.cu) ----
-cudaError_t launch_curl_plus_update(const GridP& g, const StencilP& st, const float* X, const float* Y, float a,
-                                    float* out, cudaStream_t s);
-cudaError_t launch_curl_minus_update(const GridP& g, const StencilP& st, const float* X, const float* Y, const float* J,
-                                     float a, float b, float* out, cudaStream_t s);
-cudaError_t launch_grad_plus(const GridP& g, int M, const float* L, const float* F, double a, double* grad,
-                             cudaStream_t s);
-cudaError_t launch_grad_minus(const GridP& g, int M, const float* L, const float* F, double a, double* grad,
-                              cudaStream_t s);
-cudaError_t launch_grad_corr(const GridP& g, int M, const float* W, const float* J1c, double a, double* grad,
-                             cudaStream_t s);
+struct TapsP {
+    float h[2 * PIC_MAX_HLEN + 1];       // centred: h[m] at PIC_MAX_HLEN + m
+};
+// E^{n+1} of a step from its E, B, J: components 2 and 3 of out
+cudaError_t launch_adjoint_enew(const GridP& g, const StencilP& st, const float* E, const float* B, const float* J,
+                                float* out, cudaStream_t s);
+// first and third stage (F: the step's E^{n+1} and E^n) and second stage of the adjoint step
+cudaError_t launch_adjoint_ampere(const GridP& g, const StencilP& st, const float* F, const float* aB, float* aE,
+                                  double* grad, cudaStream_t s);
+cudaError_t launch_adjoint_faraday(const GridP& g, const StencilP& st, const float* E, const float* B, const float* J1,
+                                   const float* aE, float* aB, const float* taps, int hlen, double* grad, cudaStream_t s);
 
 // ---- host math (host_math.cpp) ----
 int fit_coefficients(double kappa, int M, double wk, double n, double* C);

@@ -240,7 +240,7 @@ class StencilLoss:
     The particles are held rigid (their momenta never change) by giving them an effectively
     infinite mass; the loss is (1/2) sum (E^2 + B^2) dV over the cells with z index below
     (beam z index - behind).  The forward pass keeps a checkpoint (fields and particles) every
-    `every` steps; the backward pass replays each segment from its checkpoint, keeping the fields
+    `every` steps; the backward pass replays each segment from its checkpoint, recording the fields
     and currents of every step of the segment, and runs the adjoint steps in reverse."""
 
     RIGID_MASS = 1e30
@@ -282,7 +282,7 @@ class StencilLoss:
         return L
 
     def loss_and_grad(self, C):
-        from . import pic_adjoint_step
+        from . import pic_adjoint_run, pic_step_record
         sim = self._sim(C)
         ckpt = []
         # forward in runs of `every` steps (an even run ends in the bound field arrays: no copy back)
@@ -298,21 +298,20 @@ class StencilLoss:
         aB[..., :zc] = sim.B[..., :zc] * dV
         grad = torch.zeros(len(C), dtype=torch.float64, device=self.device)
         stream = sim.stream
+        # the record of one segment: fields at the start of every step and at its end, currents
+        n = min(self.every, self.nsteps)
+        E = torch.empty((n + 1, *sim.E.shape), dtype=torch.float32, device=self.device)
+        B, J = torch.empty_like(E), torch.empty_like(E[:n])
         for n0, E0, B0, parts in reversed(ckpt):
             n1 = min(n0 + self.every, self.nsteps)
-            sim.E.copy_(E0)
-            sim.B.copy_(B0)
+            E[0].copy_(E0)
+            B[0].copy_(B0)
             for s, arrs in parts.items():
                 for k, v in arrs.items():
                     sim.species[s][k].copy_(v)
-            saved = []
-            for _ in range(n0, n1):
-                En, Bn = sim.E.clone(), sim.B.clone()
-                sim.step(1)
-                saved.append((En, Bn, sim.J.clone()))
-            for En, Bn, Jn in reversed(saved):
-                pic_adjoint_step(sim.h, En.data_ptr(), Bn.data_ptr(), Jn.data_ptr(), aE.data_ptr(), aB.data_ptr(),
-                                 grad.data_ptr(), stream)
+            pic_step_record(sim.h, n1 - n0, E.data_ptr(), B.data_ptr(), J.data_ptr(), stream)
+            pic_adjoint_run(sim.h, n1 - n0, E.data_ptr(), B.data_ptr(), J.data_ptr(), aE.data_ptr(), aB.data_ptr(),
+                            grad.data_ptr(), stream)
         torch.cuda.synchronize(self.device)
         g = grad.cpu().numpy()
         sim.close()

@@ -60,3 +60,95 @@ def test_3d_chunks_of_every_path(shape, nz):
         dx, du = particle_errors(sim, osim, s, 3)
         assert dx < TOL and du < TOL
     sim.close()
+
+
+@pytest.mark.parametrize("M", [1, 5, 16])
+@pytest.mark.parametrize("nz,nx", [(1504, 12), (1503, 9), (420, 40)])
+def test_2d_marching_rows(nz, nx, M):
+    """x-marching field advance (variants 8..11) with the window shift: several z segments, whole and
+    ragged last segments, rows with and without 16-byte alignment, several chunks along x."""
+    from oracle import core as oc
+    from paper_1910_13529_gb300 import pic_set_tuning
+    C = fit.fit_coefficients(2.5, M=M) if M > 1 else np.array([1.0])
+    d = (0.5, 0.45)
+    grid = dict(ndim=2, nz=nz, nx=nx, ny=1, dz=d[0], dx=d[1], dy=1.0, dt=0.9 * fit.cfl_dt(d[0], d[1:], C),
+                solver="custom" if M > 1 else "yee", shape=1, moving_window=True)
+    rng = np.random.default_rng(nz + M)
+    start = [rng.normal(size=(3, 1, nx, nz)).astype(np.float32) for _ in range(3)]
+    osim = oracle_sim(grid, [], coef=C)
+    for oa, v in zip((osim.E, osim.B, osim.J), start):
+        oa[:] = v
+    shifted = []
+    for _ in range(3):
+        oc.field_advance(osim.g, osim.E, osim.B, osim.J)
+        osim.n += 1
+        shifted.append(oc.window_due(osim.n, osim.g.dt, osim.g.dz, osim.shifts))
+        if shifted[-1]:
+            osim.shift()
+    assert any(shifted) and not all(shifted)
+    for variant in (8, 9, 10, 11):
+        sim = gpu_sim(grid, [], coef=C)
+        pic_set_tuning(sim.h, variant)
+        for a, v in zip((sim.E, sim.B, sim.J), start):
+            a.copy_(torch.from_numpy(v))
+        for _ in range(3):
+            sim.field_advance()
+        assert field_error(sim, osim) < TOL, variant
+        sim.close()
+
+
+@pytest.mark.parametrize("ndim,nz,nx,ny,M", [(2, 37, 9, 1, 4), (2, 530, 5, 1, 16), (2, 512, 4, 1, 8), (3, 45, 6, 5, 3),
+                                             (3, 64, 5, 4, 16), (2, 50, 6, 1, 1)])
+def test_adjoint_run(ndim, nz, nx, ny, M):
+    """pic_step_record and pic_adjoint_run over two steps without particles, against FP64 central
+    differences of the oracle: gradient to 1e-4 of its largest entry (the framework's bound), and the
+    same result from pic_adjoint_step called step by step."""
+    import paper_1910_13529_gb300 as P
+    from oracle import core as oc
+    C = fit.fit_coefficients(2.5, M=M) if M > 1 else np.array([1.0])
+    d = (0.5, 0.45, 0.4)[:ndim]
+    grid = dict(ndim=ndim, nz=nz, nx=nx, ny=ny, dz=d[0], dx=d[1], dy=d[2] if ndim == 3 else 1.0,
+                dt=0.8 * fit.cfl_dt(d[0], d[1:], C), solver="custom", shape=1)
+    rng = np.random.default_rng(100 * M + nz)
+    shp = (3, ny, nx, nz)
+    E0, B0, lE, lB = (rng.normal(size=shp).astype(np.float32) for _ in range(4))
+
+    def loss(Cx):
+        osim = oracle_sim(grid, [], coef=Cx)
+        osim.E[:], osim.B[:] = E0, B0
+        for _ in range(2):
+            oc.field_advance(osim.g, osim.E, osim.B, osim.J)
+        return np.sum(lE * osim.E) + np.sum(lB * osim.B)
+
+    ref = np.zeros(M)
+    for l in range(M):
+        h = np.zeros(M)
+        h[l] = 1e-5
+        ref[l] = (loss(C + h) - loss(C - h)) / 2e-5
+    sim = gpu_sim(grid, [], coef=C)
+    dev = lambda a: torch.from_numpy(a).cuda()                                       # noqa: E731
+    E = torch.empty((3, *shp), device="cuda")
+    B, J = torch.empty_like(E), torch.empty((2, *shp), device="cuda")
+    E[0], B[0] = dev(E0), dev(B0)
+    P.pic_step_record(sim.h, 2, E.data_ptr(), B.data_ptr(), J.data_ptr(), sim.stream)
+    grads = []
+    for one_by_one in (False, True):
+        aE, aB = dev(lE), dev(lB)
+        grad = torch.zeros(M, dtype=torch.float64, device="cuda")
+        if one_by_one:
+            for k in (1, 0):
+                P.pic_adjoint_step(sim.h, E[k].data_ptr(), B[k].data_ptr(), J[k].data_ptr(), aE.data_ptr(), aB.data_ptr(),
+                                   grad.data_ptr(), sim.stream)
+        else:
+            P.pic_adjoint_run(sim.h, 2, E.data_ptr(), B.data_ptr(), J.data_ptr(), aE.data_ptr(), aB.data_ptr(),
+                              grad.data_ptr(), sim.stream)
+        torch.cuda.synchronize()
+        grads.append(grad.cpu().numpy())
+    scale = np.abs(ref).max()
+    for g in grads:
+        assert np.abs(g - ref).max() < 1e-4 * scale
+    # <l, A x> = <A^T l, x>
+    rhs = float((aE.double() * E[0].double()).sum() + (aB.double() * B[0].double()).sum())
+    lhs = float((dev(lE).double() * E[2].double()).sum() + (dev(lB).double() * B[2].double()).sum())
+    assert abs(lhs - rhs) < 1e-5 * np.linalg.norm(lE) * np.linalg.norm(E0)
+    sim.close()
