@@ -1600,11 +1600,23 @@ cudaError_t launch_field_advance_batch(const FieldP* inst, const int4* work, int
 //       10 = y-march with prefetch ring 128 x 8 (512 threads), 11 = ring 64 x 4 (128 threads)
 int field_variants(int ndim) { return ndim == 2 ? 12 : 12; }
 
-// Variant used before (or without) pic_autotune: the register-blocked tile for the customised
-// stencils, the scalar tile for Yee.
-int default_field_variant(int ndim, int M) {
-    if (M <= 1) return 0;
-    return ndim == 2 ? 4 : 10;
+// Variant used before (or without) pic_autotune.  The lines lie where the measured times of the variants
+// cross (us per advance on 16 to 33.6e6 cells; a before the rule, b with it):
+//   3D: the y-march, up to M = 8 128 x 4 (Yee 512 x 256 x 256: a 1527, b 597; 251 x 120 x 117: a 182, b 119;
+//   M = 8: a 718, b 670), for M = 16 the prefetch ring 128 x 8 (862, next best 1066).
+//   2D from 2e6 cells: the x-march with 64 threads (4096 x 1024 Yee: a 76, b 48; M = 16: a 86, b 64; 4099 x
+//   1030 M = 16: a 145, b 91), but not Yee on rows that are not 16-byte aligned (74 against 72).
+//   2D below: rows not 16-byte aligned want the one-cell tiles up to M = 4 (1501 x 700 Yee: 64 x 16 16.8,
+//   128 x 8 18.8, register-blocked 30; M = 4: 22.9 and 31) and the register-blocked ones above; aligned
+//   rows the register-blocked 128 x 8, on fewer than 1.3e5 cells 128 x 4 (256 x 128 Yee: a 8.7, b 5), and
+//   Yee from 5e5 cells 64 x 16 (2048 x 512: a 18.8, b 16.8; register-blocked 18.8).
+int default_field_variant(const GridP& g, int M) {
+    if (g.ndim == 3) return M <= 8 ? 6 : 10;
+    const bool aligned = g.nz % 4 == 0, yee = M <= 1;
+    if (g.ncell >= 2000000 && (aligned || !yee)) return 11;
+    if (!aligned) return yee ? 2 : M <= 4 ? 0 : 4;
+    if (g.ncell < 130000) return 6;
+    return yee && g.ncell >= 500000 ? 2 : 4;
 }
 
 namespace {

@@ -475,7 +475,7 @@ pic_status pic_create(const pic_config* cfg, pic_t** out) {
     g.dt = (float)c.dt;
     g.shape = c.shape;
     h->st.M = M;
-    h->fa_variant = default_field_variant(c.ndim, M);
+    h->fa_variant = default_field_variant(g, M);
     bool yee_b = true;     // B-side d- is the two-point Yee difference: no correction
     for (int l = 0; l < PIC_MAX_M; ++l) {
         h->C64[l] = l < M ? C[l] : 0.0;

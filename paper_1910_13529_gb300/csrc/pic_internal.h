@@ -117,7 +117,7 @@ enum : int { STATUS_CAPACITY = 1, STATUS_TIMEOUT = 2 };
 // ---- launchers (return cudaGetLastError of the launch) ----
 cudaError_t launch_field_advance(const FieldP& p, cudaStream_t s, int variant = 0);
 int field_variants(int ndim);
-int default_field_variant(int ndim, int M);
+int default_field_variant(const GridP& g, int M);
 
 // batched: instance tables live in device memory
 cudaError_t launch_field_advance_batch(const FieldP* inst, const int4* work, int total_tiles, int ndim, int maxm,
