@@ -486,23 +486,37 @@ __global__ void __launch_bounds__(256) push_kernel(GridP g, SpeciesP sp, const f
 // Particles per chunk of the fused kernels (one per thread).
 constexpr int FUSED_T = 256;
 
+// a compile-time false condition
+struct Never {
+    __device__ constexpr operator bool() const { return false; }
+};
+
 // ---------------------------------------------------------------- 2D fused kernel ----
 // Specialised 2D gather + push + Esirkepov for cell-sorted particles.  Per chunk of FUSED_T
-// particles (one per thread):
-//  1. the fields of the chunk's gather footprint are staged in shared memory (coalesced z rows,
-//     zero outside the z range), so the 6 x K^2 interpolation loads are shared-memory loads;
+// particles (one per thread), pipelined over chunks as in 3D (push_deposit_3d_chunks):
+//  1. the particle words and the fields of the gather footprint (coalesced z rows, zero outside the z
+//     range) were copied to shared memory during the previous chunk, the footprint having been agreed
+//     on from the words one chunk ahead; components are interpolated in pairs;
 //  2. the 2D Esirkepov weights are separable products of per-axis vectors:
 //       J1(a,b) = f1 Cz[a] Tx[b],  J2(a,b) = f2 Tz[a] Cx[b],
-//       J3(a,b) = qv v3 (S0z[a] (S0x[b] + dSx[b]/2) + dSz[a] (S0x[b]/2 + dSx[b]/3)),
+//     J3(a,b) = qv v3 (S0z[a] (S0x[b] + dSx[b]/2) + dSz[a] (S0x[b]/2 + dSx[b]/3)),
 //     with Cz = cumsum dSz, Tx = S0x + dSx/2 (and z <-> x);
 //  3. the chunk's current is summed in a shared-memory box in 32-bit fixed point (native
 //     integer atomics); when more than 8 lanes of a warp share a deposition window (dense
 //     beams) runs of consecutive lanes are summed by a segmented warp reduction first, so that
 //     one lane per run issues the atomic; the box is added to J with float4 atomics.
+// Bound by instruction issue (77% of the slots at 47% of the warps, 64 registers).  Six barriers per
+// chunk and exposed loads before, three barriers now: 2048 x 512, 5.2e6 particles, quadratic, wake state,
+// 268 us per step before, 242 us now; 1001 x 237 linear 49.4 and 48.4 us.
 // Boxes larger than the shared-memory caps fall back to global loads / global atomics.
 constexpr int F_CAP = 6 * 1024;    // field box floats (6 components)
 constexpr int J_CAP = 3 * 1024;    // current box floats (3 components)
-constexpr int SMEM_2D = F_CAP + J_CAP;
+constexpr int PF2 = 6;             // prefetched words per particle (cell, 2 offsets, 3 momenta)
+constexpr int SMEM_2D = F_CAP + J_CAP + 2 * PF2 * FUSED_T;
+// words about a chunk (as in 3D): lower ends of its gather box along z and x, upper ends negated, the
+// largest current contribution; three sets in turn
+enum { BW2_N = 5, BW2_SHARED = 3 * BW2_N };
+constexpr int DENSE_2D = 96;       // field box nodes up to which a chunk may be a dense beam's
 
 // 4-byte asynchronous global -> shared copy (the next chunk's particle data)
 __device__ __forceinline__ void cp_async4(void* dst, const void* src) {
@@ -578,51 +592,27 @@ __device__ __forceinline__ void box_reduce(int* box, int lz, int hz, int lx, int
     }
 }
 
-// Field box of a chunk, rows of fzl (a multiple of 4) floats along z, fvol = fxl fzl nodes:
-//   P1[fvol] float2 = (E1, B2): half cell along z, node along x  -> weights (Wzh, Wxn)
-//   P2[fvol] float2 = (E2, B1): node along z, half cell along x  -> weights (Wzn, Wxh)
-//   S3[fvol] = E3 (node, node),  T3[fvol] = B3 (half, half)
-// Components that share a stencil are interpolated together with packed FP32 FMAs.
+// .x = sum Wza Wxa Fa, .y = sum Wzb Wxb Fb over K x K nodes of [x][z] boxes with rows of zl floats (Fa,
+// Fb at the two stencil origins): two components by packed FP32 FMAs.
 template <int K>
-__device__ __forceinline__ float2 tile_interp2(const float2* __restrict__ f, int zl, int z, int x, const float (&Wz)[K],
-                                               const float (&Wx)[K]) {
-    const float2* r = f + x * zl + z;
+__device__ __forceinline__ float2 tile_interp2(const float* __restrict__ Fa, const float* __restrict__ Fb, int zl,
+                                               const float (&Wza)[K], const float (&Wxa)[K], const float (&Wzb)[K],
+                                               const float (&Wxb)[K]) {
     float2 acc = make_float2(0.f, 0.f);
 #pragma unroll
     for (int b = 0; b < K; ++b) {
         float2 t = make_float2(0.f, 0.f);
 #pragma unroll
-        for (int a = 0; a < K; ++a) t = __ffma2_rn(make_float2(Wz[a], Wz[a]), r[a], t);
-        acc = __ffma2_rn(make_float2(Wx[b], Wx[b]), t, acc);
-        r += zl;
-    }
-    return acc;
-}
-
-// E3 and B3 (different stencils) as one packed chain: .x = E3, .y = B3.
-template <int K>
-__device__ __forceinline__ float2 tile_interp_e3b3(const float* __restrict__ S3, const float* __restrict__ T3, int zl,
-                                                   int za, int xa, int zb, int xb, const float (&Wza)[K],
-                                                   const float (&Wxa)[K], const float (&Wzb)[K],
-                                                   const float (&Wxb)[K]) {
-    const float* r = S3 + xa * zl + za;
-    const float* q = T3 + xb * zl + zb;
-    float2 acc = make_float2(0.f, 0.f);
-#pragma unroll
-    for (int b = 0; b < K; ++b) {
-        float2 t = make_float2(0.f, 0.f);
-#pragma unroll
-        for (int a = 0; a < K; ++a) t = __ffma2_rn(make_float2(Wza[a], Wzb[a]), make_float2(r[a], q[a]), t);
+        for (int a = 0; a < K; ++a) t = __ffma2_rn(make_float2(Wza[a], Wzb[a]), make_float2(Fa[a], Fb[a]), t);
         acc = __ffma2_rn(make_float2(Wxa[b], Wxb[b]), t, acc);
-        r += zl;
-        q += zl;
+        Fa += zl;
+        Fb += zl;
     }
     return acc;
 }
 
-// Cells gz..gz+3 of a field row into a (zero outside 0 <= z < nz); vec: 16-byte groups.
-__device__ __forceinline__ float4 load_group(const float* __restrict__ row, int gz, int nz, bool vec) {
-    if (vec && gz >= 0 && gz + 3 < nz) return __ldg(reinterpret_cast<const float4*>(row + gz));
+// Cells gz..gz+3 of a field row, zero outside 0 <= z < nz.
+__device__ __forceinline__ float4 load_group(const float* __restrict__ row, int gz, int nz) {
     float4 a;
     a.x = (unsigned)gz < (unsigned)nz ? __ldg(row + gz) : 0.f;
     a.y = (unsigned)(gz + 1) < (unsigned)nz ? __ldg(row + gz + 1) : 0.f;
@@ -645,96 +635,164 @@ __device__ __forceinline__ void push_deposit_2d_chunks(const GridP& g, const Spe
     const int N = (int)g.ncell;
     const bool fvec = (g.nz & 3) == 0 && aligned16(E) && aligned16(B);
     const bool jvec = (g.nz & 3) == 0 && aligned16(J);
-    for (long long base = chunk0 * FUSED_T; base < n; base += stride * FUSED_T) {
-        if (threadIdx.x < 5) box[threadIdx.x] = threadIdx.x == 4 ? 0 : (threadIdx.x & 1) ? INT_MIN : INT_MAX;
-        __syncthreads();
-        const long long p = base + threadIdx.x;
-        // ---- load and decode ----
-        bool ok = false;
-        Pos p0;
-        float u[3] = {0.f, 0.f, 0.f};
-        if (p < n) {
-            int cell = sp.cell[p];
+    int* const iJ = reinterpret_cast<int*>(sJ);
+    float* const pfb = sJ + J_CAP;                    // [2][PF2][FUSED_T]
+    auto prefetch = [&](long long b, int buf) {
+        const long long q = b + threadIdx.x;
+        if (q < n) {
+            float* d = pfb + buf * PF2 * FUSED_T + threadIdx.x;
+            cp_async4(d, sp.cell + q);
+            cp_async4(d + FUSED_T, sp.off + q);
+            cp_async4(d + 2 * FUSED_T, sp.off + cap + q);
+            cp_async4(d + 3 * FUSED_T, sp.u + q);
+            cp_async4(d + 4 * FUSED_T, sp.u + cap + q);
+            cp_async4(d + 5 * FUSED_T, sp.u + 2 * cap + q);
+        }
+        cp_async_commit();
+    };
+    auto place = [&](int cell, int& iz, int& ix) {
+        const uint32_t r = fdiv((uint32_t)cell, g.div_nzg);
+        iz = cell - (int)r * g.nzg - 1 - shift;
+        ix = (int)r;
+        return iz >= 0 && iz < g.nz;
+    };
+    // the gather box of the chunk at b from its particle words (see push_deposit_3d_chunks); the cell of
+    // the thread's particle (aiz, aix; aiz < 0: none) is kept for the chunk's own turn
+    int aiz = -1, aix = 0;
+    auto agree = [&](long long b, int buf, int* bw) {
+        const float* w = pfb + buf * PF2 * FUSED_T + threadIdx.x;
+        int v[4] = {INT_MAX, INT_MAX, INT_MAX, INT_MAX};
+        aiz = -1;
+        if (b + threadIdx.x < n) {
+            const int cell = __float_as_int(w[0]);
+            int c[2];
             if (cell >= 0) {
-                int izg;
-                decode(g, cell, izg, p0.ix, p0.iy);
-                p0.iz = izg - 1 - shift;
-                if (p0.iz >= 0 && p0.iz < g.nz) {
-                    ok = true;
-                    p0.oz = sp.off[p];
-                    p0.ox = sp.off[cap + p];
-                    p0.oy = 0.f;
-                    u[0] = sp.u[p];
-                    u[1] = sp.u[cap + p];
-                    u[2] = sp.u[2 * cap + p];
+                if (!place(cell, c[0], c[1])) {
+                    sp.cell[b + threadIdx.x] = -1;     // left through the back of the window
                 } else {
-                    sp.cell[p] = -1;
+                    aiz = c[0];
+                    aix = c[1];
+#pragma unroll
+                    for (int a = 0; a < 2; ++a) {
+                        const bool up = w[(1 + a) * FUSED_T] >= 0.5f;
+                        v[a] = K == 3 || !up ? c[a] - 1 : c[a];
+                        v[2 + a] = -(K == 3 && up ? c[a] + 2 : c[a] + 1);
+                    }
                 }
             }
         }
-        // ---- gather weights and the chunk's boxes ----
-        float Wzn[K], Wzh[K], Wxn[K], Wxh[K];
-        int bzn = 0, bzh = 0, bxn = 0, bxh = 0;
-        if (ok) {
-            bzn = p0.iz + Shape<SHAPE>::w(p0.oz, Wzn);
-            bzh = half_weights<SHAPE>(p0.iz, p0.oz, Wzh);
-            bxn = p0.ix + Shape<SHAPE>::w(p0.ox, Wxn);
-            bxh = half_weights<SHAPE>(p0.ix, p0.ox, Wxh);
+        int mine = 0;
+#pragma unroll
+        for (int a = 0; a < 4; ++a) {
+            const int m = __reduce_min_sync(0xffffffffu, v[a]);
+            if ((threadIdx.x & 31) == a) mine = m;
         }
-        box_reduce(box, ok ? min(bzn, bzh) : INT_MAX, ok ? max(bzn, bzh) + K - 1 : INT_MIN,
-                   ok ? min(bxn, bxh) : INT_MAX, ok ? max(bxn, bxh) + K - 1 : INT_MIN);
+        if ((threadIdx.x & 31) < 4 && mine != INT_MAX) atomicMin(bw + (threadIdx.x & 31), mine);
+    };
+    // field box: z aligned down to a multiple of 4, rows of whole groups
+    struct Ext {
+        int fz0, fx0, fzl, fxl;
+        bool any, ftile;
+    };
+    auto extents = [&](const int* bw) {
+        Ext e;
+        e.any = bw[0] != INT_MAX;
+        e.fz0 = e.any ? (bw[0] & ~3) : 0, e.fx0 = bw[1];
+        e.fzl = e.any ? ((1 - bw[2] - e.fz0 + 3) & ~3) : 0, e.fxl = e.any ? 1 - bw[3] - bw[1] : 0;
+        e.ftile = e.any && 6 * e.fzl * e.fxl <= F_CAP && e.fxl <= g.nx + 2 * K;
+        return e;
+    };
+    // the fields of the next chunk: component c at sF + c fzl fxl, [x][z], zero outside the z range
+    auto request = [&](const int* bw) {
+        const Ext e = extents(bw);
+        if (!e.ftile) return;
+        const int ng = e.fzl >> 2, rows = e.fxl;
+        const float rg = 1.f / (float)ng, rx = 1.f / (float)rows;
+        const int fvol3 = 3 * rows * e.fzl;
+        for (int i = threadIdx.x; i < 3 * rows * ng; i += FUSED_T) {     // the groups of E_c and B_c
+            const int r = box_div(i, rg), zg = i - r * ng;
+            const int c = box_div(r, rx), x = r - c * rows;
+            const long long row = (long long)c * N + (long long)wrapi(e.fx0 + x, g.nx) * g.nz;
+            const float *fe = E + row, *fb = B + row;
+            float* d = sF + 4 * i;                   // (c rows + x) fzl + 4 zg
+            const int gz = e.fz0 + 4 * zg;
+            if (fvec) {
+                const bool in = gz >= 0 && gz < g.nz;
+                cp_async16z(d, fe + (in ? gz : 0), in);
+                cp_async16z(d + fvol3, fb + (in ? gz : 0), in);
+            } else {                                 // (4-byte asynchronous copies are slower than this)
+                *reinterpret_cast<float4*>(d) = load_group(fe, gz, g.nz);
+                *reinterpret_cast<float4*>(d + fvol3) = load_group(fb, gz, g.nz);
+            }
+        }
+    };
+    prefetch(chunk0 * FUSED_T, 0);
+    prefetch((chunk0 + stride) * FUSED_T, 1);
+    if (threadIdx.x < 3 * BW2_N) box[threadIdx.x] = threadIdx.x % BW2_N < 4 ? INT_MAX : 0;
+    __syncthreads();
+    cp_async_wait_prev();
+    agree(chunk0 * FUSED_T, 0, box);
+    __syncthreads();
+    request(box);
+    int buf = 0, cur = 0;
+    int clear = 0;                                   // 16-byte groups of the current box known to be zero
+    for (long long base = chunk0 * FUSED_T; base < n; base += stride * FUSED_T, buf ^= 1) {
+        int* const bc = box + cur * BW2_N;
+        const int nxt = cur == 2 ? 0 : cur + 1;
+        const bool more = base + stride * FUSED_T < n;
+        Pos p0;
+        p0.iz = aiz;
+        p0.ix = aix;
+        p0.iy = 0;
+        p0.oy = 0.f;
+        cp_async_wait_all_p();                       // this chunk's fields, the next chunk's particle words
         __syncthreads();
-        const bool any = box[0] != INT_MAX;
-        // field box: z aligned down to a multiple of 4, rows padded to whole groups
-        const int fz0 = any ? (box[0] & ~3) : 0, fx0 = box[2];
-        const int fzl = any ? ((box[1] + 1 - fz0 + 3) & ~3) : 0, fxl = any ? box[3] - box[2] + 1 : 0;
-        const int fvol = fzl * fxl;
-        const bool ftile = any && 6 * fvol <= F_CAP && fxl <= g.nx + 2 * K;
+        if (more) agree(base + stride * FUSED_T, buf ^ 1, box + nxt * BW2_N);
+        const Ext e = extents(bc);
+        const bool any = e.any;
+        const int fz0 = e.fz0, fx0 = e.fx0, fzl = e.fzl, fvol = e.fzl * e.fxl;
         // current box: every deposition window starts at most one node below the gather stencils and
         // its K + 1 nodes end at most one node above them (the move is under one cell per axis)
-        const int jz0 = any ? ((box[0] - 1) & ~3) : 0, jx0 = box[2] - 1;
-        const int jzl = any ? ((box[1] + 2 - jz0 + 3) & ~3) : 0, jxl = any ? box[3] - box[2] + 3 : 0;
+        const int jz0 = any ? ((bc[0] - 1) & ~3) : 0, jx0 = fx0 - 1;
+        const int jzl = any ? ((2 - bc[2] - jz0 + 3) & ~3) : 0, jxl = any ? e.fxl + 2 : 0;
         const int jvol = jzl * jxl;
         const bool jtile = any && 3 * jvol <= J_CAP && jxl <= g.nx + 2 * KW;
-        float2* P1 = reinterpret_cast<float2*>(sF);
-        float2* P2 = P1 + fvol;
-        float* S3 = sF + 4 * fvol;
-        float* T3 = S3 + fvol;
-        if (ftile) {
-            const int ng = fzl >> 2;
-            const float rg = 1.f / (float)ng, rx = 1.f / (float)fxl;
-            for (int i = threadIdx.x; i < 3 * fxl * ng; i += FUSED_T) {
-                const int r = box_div(i, rg), zg = i - r * ng;
-                const int pc = box_div(r, rx), x = r - pc * fxl;
-                const long long row = (long long)wrapi(fx0 + x, g.nx) * g.nz;
-                const int gz = fz0 + 4 * zg;
-                const int o = x * fzl + 4 * zg;
-                // pc = 0: (E1, B2), 1: (E2, B1), 2: E3, B3
-                const float* fa = E + pc * N + row;
-                const float* fb = B + (pc == 0 ? N : pc == 1 ? 0 : 2 * N) + row;
-                const float4 a = load_group(fa, gz, g.nz, fvec), b = load_group(fb, gz, g.nz, fvec);
-                if (pc < 2) {
-                    float4* d = reinterpret_cast<float4*>((pc == 0 ? P1 : P2) + o);
-                    d[0] = make_float4(a.x, b.x, a.y, b.y);
-                    d[1] = make_float4(a.z, b.z, a.w, b.w);
-                } else {
-                    *reinterpret_cast<float4*>(S3 + o) = a;
-                    *reinterpret_cast<float4*>(T3 + o) = b;
-                }
-            }
+        // the flush clears what a chunk used: only the first chunk and a larger box clear anything here
+        if (jtile && 3 * (jvol >> 2) > clear) {
+            for (int i = clear + threadIdx.x; i < 3 * (jvol >> 2); i += FUSED_T)
+                reinterpret_cast<int4*>(iJ)[i] = make_int4(0, 0, 0, 0);
+            clear = 3 * (jvol >> 2);
         }
-        if (jtile)
-            for (int i = threadIdx.x; i < (3 * jvol) >> 2; i += FUSED_T)
-                reinterpret_cast<float4*>(sJ)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-        __syncthreads();
+        // ---- load and decode ----
+        const long long p = base + threadIdx.x;
+        bool ok = p0.iz >= 0;
+        float u[3] = {0.f, 0.f, 0.f};
+        if (ok) {
+            const float* mine = pfb + buf * PF2 * FUSED_T + threadIdx.x;
+            p0.oz = mine[FUSED_T];
+            p0.ox = mine[2 * FUSED_T];
+            u[0] = mine[3 * FUSED_T];
+            u[1] = mine[4 * FUSED_T];
+            u[2] = mine[5 * FUSED_T];
+        }
         // ---- gather (staggering: E1 z+, E2 x+, E3 node, B1 x+, B2 z+, B3 z+ x+) ----
+        float Wzn[K], Wxn[K];
+        int bzn = 0, bxn = 0;
         float eb[6];
         if (ok) {
-            if (ftile) {
-                const float2 q1 = tile_interp2<K>(P1, fzl, bzh - fz0, bxn - fx0, Wzh, Wxn);
-                const float2 q2 = tile_interp2<K>(P2, fzl, bzn - fz0, bxh - fx0, Wzn, Wxh);
-                const float2 q3 = tile_interp_e3b3<K>(S3, T3, fzl, bzn - fz0, bxn - fx0, bzh - fz0, bxh - fx0, Wzn,
-                                                      Wxn, Wzh, Wxh);
+            float Wzh[K], Wxh[K];
+            bzn = p0.iz + Shape<SHAPE>::w(p0.oz, Wzn);
+            bxn = p0.ix + Shape<SHAPE>::w(p0.ox, Wxn);
+            const int bzh = half_weights<SHAPE>(p0.iz, p0.oz, Wzh);
+            const int bxh = half_weights<SHAPE>(p0.ix, p0.ox, Wxh);
+            if (e.ftile) {
+                const float* nn = sF + (bxn - fx0) * fzl + (bzn - fz0);
+                const float* hn = sF + (bxn - fx0) * fzl + (bzh - fz0);
+                const float* nh = sF + (bxh - fx0) * fzl + (bzn - fz0);
+                const float* hh = sF + (bxh - fx0) * fzl + (bzh - fz0);
+                const float2 q1 = tile_interp2<K>(hn, hn + 4 * fvol, fzl, Wzh, Wxn, Wzh, Wxn);             // E1, B2
+                const float2 q2 = tile_interp2<K>(nh + fvol, nh + 3 * fvol, fzl, Wzn, Wxh, Wzn, Wxh);      // E2, B1
+                const float2 q3 = tile_interp2<K>(nn + 2 * fvol, hh + 5 * fvol, fzl, Wzn, Wxn, Wzh, Wxh);  // E3, B3
                 eb[0] = q1.x;
                 eb[4] = q1.y;
                 eb[1] = q2.x;
@@ -771,6 +829,7 @@ __device__ __forceinline__ void push_deposit_2d_chunks(const GridP& g, const Spe
                 sp.u[2 * cap + p] = u[2];
             }
         }
+        prefetch(base + 2 * stride * FUSED_T, buf);      // this chunk's words are done with
         // ---- deposition ----
         float S0z[KW], DSz[KW], S0x[KW], DSx[KW];
         int bz = 0, bx = 0;
@@ -808,13 +867,14 @@ __device__ __forceinline__ void push_deposit_2d_chunks(const GridP& g, const Spe
         // is below 2^-21 of the chunk's largest contribution.
         if (jtile) {
             const unsigned wm = __reduce_max_sync(0xffffffffu, ok ? __float_as_uint(mb) : 0u);
-            if ((threadIdx.x & 31) == 0 && wm) atomicMax(reinterpret_cast<unsigned*>(box + 4), wm);
+            if ((threadIdx.x & 31) == 0 && wm) atomicMax(reinterpret_cast<unsigned*>(bc + 4), wm);
         }
         __syncthreads();
-        const int mbits = box[4];
+        if (more) request(box + nxt * BW2_N);
+        if (threadIdx.x < BW2_N) box[(3 - cur - nxt) * BW2_N + threadIdx.x] = threadIdx.x < 4 ? INT_MAX : 0;
+        const int mbits = bc[4];
         const int sexp = min(275 - (mbits >> 23), 253);       // biased exponent of s
         const float fs = __int_as_float(sexp << 23), inv_s = __int_as_float((254 - sexp) << 23);
-        int* const iJ = reinterpret_cast<int*>(sJ);
         if (any && jtile && mbits != 0) {
             const float g1 = f1 * fs, g2 = f2 * fs, g3 = f3 * fs;
             float2 CT[KW], TC[KW];        // (s Cz, Tz)[a], (Tx, s Cx)[b]
@@ -827,21 +887,13 @@ __device__ __forceinline__ void push_deposit_2d_chunks(const GridP& g, const Spe
                 Ax[k] = g3 * tx;
                 Bx[k] = g3 * (0.5f * S0x[k] + (1.f / 3.f) * DSx[k]);
             }
-            // Lanes sharing a window hit the same nodes.  With at most 8 lanes per window anywhere
-            // in the warp every live lane adds its own values (at most 8-way address conflicts,
-            // serialised by the shared-memory pipe); otherwise (dense beams) runs of consecutive
-            // lanes are summed first and one lane per run adds the total.  Empty slots have unique
-            // keys.
-            const unsigned long long key = ok ? (((unsigned long long)(bz + 4) << 32) | (unsigned)(bx + 4))
-                                              : (0xFFFFFFFF00000000ull | (unsigned)threadIdx.x);
-            const int gmax = __reduce_max_sync(0xffffffffu, __popc(__match_any_sync(0xffffffffu, key)));
             int* s0 = iJ + (bx - jx0) * jzl + (bz - jz0);
             const float MAGIC = 12582912.f;           // 1.5 2^23
             // no lane of the warp changed its support node along an axis: the last window node along
             // it has S0 = dS = 0 and the last cumulative sum along it is zero; skip those deposits
             const bool uz = __any_sync(0xffffffffu, S0z[KW - 1] != 0.f || DSz[KW - 1] != 0.f);
             const bool ux = __any_sync(0xffffffffu, S0x[KW - 1] != 0.f || DSx[KW - 1] != 0.f);
-            auto terms = [&](auto&& put) {
+            auto terms = [&](auto&& put, auto hz, auto hx) {
 #pragma unroll
                 for (int b = 0; b < KW; ++b)
 #pragma unroll
@@ -849,9 +901,9 @@ __device__ __forceinline__ void push_deposit_2d_chunks(const GridP& g, const Spe
                         // J1 (a < KW-1): zero at the last cumulative z sum or the last x node;
                         // J2 (b < KW-1): at the last cumulative x sum or the last z node;
                         // J3: at the last z node or the last x node
-                        const bool k1 = !((a == KW - 2 && !uz) || (b == KW - 1 && !ux));
-                        const bool k2 = !((b == KW - 2 && !ux) || (a == KW - 1 && !uz));
-                        const bool k3 = !((a == KW - 1 && !uz) || (b == KW - 1 && !ux));
+                        const bool k1 = !((a == KW - 2 && !hz) || (b == KW - 1 && !hx));
+                        const bool k2 = !((b == KW - 2 && !hx) || (a == KW - 1 && !hz));
+                        const bool k3 = !((a == KW - 1 && !hz) || (b == KW - 1 && !hx));
                         const int o = b * jzl + a;
                         if (a < KW - 1 && b < KW - 1) {
                             if (k1 || k2) {
@@ -867,14 +919,30 @@ __device__ __forceinline__ void push_deposit_2d_chunks(const GridP& g, const Spe
                         if (k3) put(2 * jvol + o, fmaf(S0z[a], Ax[b], fmaf(DSz[a], Bx[b], MAGIC)));
                     }
             };
+            // Lanes sharing a window hit the same nodes.  With at most 8 lanes per window anywhere
+            // in the warp every live lane adds its own values (at most 8-way address conflicts,
+            // serialised by the shared-memory pipe); otherwise (dense beams) runs of consecutive
+            // lanes are summed first and one lane per run adds the total.  Empty slots have unique
+            // keys.  Only a chunk whose box is small can be that dense: one with room for more than
+            // DENSE_2D windows is not looked at (256 particles on 96 windows are fewer than 3 each).
+            int gmax = 0;
+            unsigned key = 0;
+            if (fvol <= DENSE_2D) {
+                key = ok ? (unsigned)((bx - jx0) << 16 | (bz - jz0)) : 0x80000000u | threadIdx.x;
+                gmax = __reduce_max_sync(0xffffffffu, __popc(__match_any_sync(0xffffffffu, key)));
+            }
             if (gmax <= 8) {
-                if (ok) terms([&](int o, float biased) { atomicAdd(s0 + o, __float_as_int(biased) - 0x4B400000); });
+                if (ok) {
+                    auto put = [&](int o, float biased) { atomicAdd(s0 + o, __float_as_int(biased) - 0x4B400000); };
+                    if (!(uz || ux)) terms(put, Never(), Never());
+                    else terms(put, uz, ux);
+                }
             } else {
                 const SegReduce seg = make_segments(key);
                 terms([&](int o, float biased) {
                     const int v = seg.sum(__float_as_int(biased) - 0x4B400000);
                     if (seg.head && ok && v != 0) atomicAdd(s0 + o, v);
-                });
+                }, uz, ux);
             }
         } else if (any && !jtile && ok) {
             // box too large for shared memory: FP32 atomics straight to J
@@ -897,12 +965,15 @@ __device__ __forceinline__ void push_deposit_2d_chunks(const GridP& g, const Spe
         }
         __syncthreads();
         if (jtile && mbits != 0) {
-            // box -> J in 16-byte groups (one vector atomic per group inside the grid)
+            // box -> J in 16-byte groups (one vector atomic per group inside the grid); the groups are
+            // cleared as they are read, for the next chunk
             const int ng = jzl >> 2;
             const float rg = 1.f / (float)ng, rx = 1.f / (float)jxl;
             for (int i = threadIdx.x; i < 3 * jxl * ng; i += FUSED_T) {
-                const int4 q = reinterpret_cast<const int4*>(iJ)[i];
+                int4* grp = reinterpret_cast<int4*>(iJ) + i;
+                const int4 q = *grp;
                 if ((q.x | q.y | q.z | q.w) == 0) continue;
+                *grp = make_int4(0, 0, 0, 0);
                 const float4 v = make_float4((float)q.x * inv_s, (float)q.y * inv_s, (float)q.z * inv_s,
                                              (float)q.w * inv_s);
                 const int r = box_div(i, rg), zg = i - r * ng;
@@ -919,8 +990,9 @@ __device__ __forceinline__ void push_deposit_2d_chunks(const GridP& g, const Spe
                 }
             }
         }
-        __syncthreads();
+        cur = nxt;
     }
+    cp_async_wait_all_p();                            // the last (empty) prefetch groups
 }
 
 // ---------------------------------------------------------------- 3D fused kernel ----
@@ -1022,11 +1094,6 @@ __device__ __noinline__ void deposit3_global(const GridP g, float qv, const Pos 
     deposit<3, SHAPE>(g, qv, 0.f, p0, p1, acc);
 }
 
-// a compile-time false condition
-struct Never {
-    __device__ constexpr operator bool() const { return false; }
-};
-
 // Waits for phase `parity` of an mbarrier that a TMA copy completes; gives up after about a second
 // (false).
 __device__ __forceinline__ bool mbar_wait(unsigned bar, unsigned parity) {
@@ -1103,17 +1170,24 @@ __device__ __forceinline__ void push_deposit_3d_chunks(const GridP& g, const Spe
     };
     // the gather box of the chunk at b from its particle words (a shape's half-cell support starts at
     // the node below the cell and its nodal one there or, for K = 3 or the linear upper half, a node up)
+    int aiz = -1, aix = 0, aiy = 0;   // the cell found there (aiz < 0: none), kept for the chunk's own turn
     auto agree = [&](long long b, int buf, int* bw) {
         const float* w = pfb + buf * PF3 * FUSED_T + threadIdx.x;
         int v[6] = {INT_MAX, INT_MAX, INT_MAX, INT_MAX, INT_MAX, INT_MAX};
         bool moving = false;
+        aiz = -1;
         if (b + threadIdx.x < n) {
             const int cell = __float_as_int(w[0]);
             if (cell >= 0) {
                 int c[3];
                 decode(g, cell, c[0], c[1], c[2]);
                 c[0] -= 1 + shift;
-                if (c[0] >= 0 && c[0] < g.nz) {
+                if (c[0] < 0 || c[0] >= g.nz) {
+                    sp.cell[b + threadIdx.x] = -1;     // left through the back of the window
+                } else {
+                    aiz = c[0];
+                    aix = c[1];
+                    aiy = c[2];
                     moving = w[4 * FUSED_T] != 0.f || w[5 * FUSED_T] != 0.f || w[6 * FUSED_T] != 0.f;
 #pragma unroll
                     for (int a = 0; a < 3; ++a) {
@@ -1213,8 +1287,13 @@ __device__ __forceinline__ void push_deposit_3d_chunks(const GridP& g, const Spe
     for (long long base = chunk0 * FUSED_T; base < n; base += stride * FUSED_T, buf ^= 1) {
         int* const bc = box + cur * BW_N;
         const int nxt = cur == 2 ? 0 : cur + 1;
+        const bool more = base + stride * FUSED_T < n;
+        Pos p0;
+        p0.iz = aiz;
+        p0.ix = aix;
+        p0.iy = aiy;
         cp_async_wait_all_p();                     // the next chunk's particle words
-        agree(base + stride * FUSED_T, buf ^ 1, box + nxt * BW_N);
+        if (more) agree(base + stride * FUSED_T, buf ^ 1, box + nxt * BW_N);
         const Ext e = extents(bc);
         const bool any = e.any, ftile = e.ftile;
         const int fz0 = e.fz0, fx0 = e.fx0, fy0 = e.fy0;
@@ -1247,30 +1326,18 @@ __device__ __forceinline__ void push_deposit_3d_chunks(const GridP& g, const Spe
             if (TMA) asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
             __syncthreads();
         }
-        // ---- load and decode ----
+        // ---- load ----
         const long long p = base + threadIdx.x;
-        bool ok = false;
-        Pos p0;
+        bool ok = p0.iz >= 0 && !listed;
         float u[3] = {0.f, 0.f, 0.f};
-        if (p < n && !listed) {
+        if (ok) {
             const float* mine = pfb + buf * PF3 * FUSED_T + threadIdx.x;
-            int cell = __float_as_int(mine[0]);
-            if (cell >= 0) {
-                int izg;
-                decode(g, cell, izg, p0.ix, p0.iy);
-                p0.iz = izg - 1 - shift;
-                if (p0.iz >= 0 && p0.iz < g.nz) {
-                    ok = true;
-                    p0.oz = mine[FUSED_T];
-                    p0.ox = mine[2 * FUSED_T];
-                    p0.oy = mine[3 * FUSED_T];
-                    u[0] = mine[4 * FUSED_T];
-                    u[1] = mine[5 * FUSED_T];
-                    u[2] = mine[6 * FUSED_T];
-                } else {
-                    sp.cell[p] = -1;
-                }
-            }
+            p0.oz = mine[FUSED_T];
+            p0.ox = mine[2 * FUSED_T];
+            p0.oy = mine[3 * FUSED_T];
+            u[0] = mine[4 * FUSED_T];
+            u[1] = mine[5 * FUSED_T];
+            u[2] = mine[6 * FUSED_T];
         }
         // a particle at rest in zero fields stays at rest and carries no current: a chunk with no
         // moving particle reads its staged groups back to see whether they are all zero
@@ -1382,7 +1449,7 @@ __device__ __forceinline__ void push_deposit_3d_chunks(const GridP& g, const Spe
         }
         __syncthreads();
         if (TMA && box[BW_ABORT]) break;
-        request(box + nxt * BW_N);
+        if (more) request(box + nxt * BW_N);
         if (threadIdx.x < BW_N) box[(3 - cur - nxt) * BW_N + threadIdx.x] = box_word_init(threadIdx.x);
         const int mbits = bc[BW_MAX];
         const int sexp = min(275 - (mbits >> 23), 253);
@@ -1920,7 +1987,7 @@ __global__ void __launch_bounds__(FUSED_T, 4) push_deposit_2d_kernel(GridP g, Sp
                                                                      int shift) {
     extern __shared__ float4 smem4[];      // 16-byte aligned: the boxes are read and written as float4
     float* smem = reinterpret_cast<float*>(smem4);
-    __shared__ int box[5];
+    __shared__ int box[BW2_SHARED];
     push_deposit_2d_chunks<SHAPE>(g, sp, E, B, J, shift, blockIdx.x, gridDim.x, smem, smem + F_CAP, box);
 }
 
@@ -1928,7 +1995,7 @@ template <int SHAPE>
 __global__ void __launch_bounds__(FUSED_T, 4) push_deposit_2d_batch_kernel(const PartInst* __restrict__ inst, int parity) {
     extern __shared__ float4 smem4[];
     float* smem = reinterpret_cast<float*>(smem4);
-    __shared__ int box[5];
+    __shared__ int box[BW2_SHARED];
     const PartInst& q = inst[blockIdx.y];
     const GridP g = prep_device(q.g);
     push_deposit_2d_chunks<SHAPE>(g, q.sp, q.E[parity], q.B[parity], q.J, 0, blockIdx.x, gridDim.x, smem, smem + F_CAP,

@@ -98,7 +98,7 @@ def test_2d_marching_rows(nz, nx, M):
 
 
 @pytest.mark.parametrize("ndim,nz,nx,ny,M", [(2, 37, 9, 1, 4), (2, 530, 5, 1, 16), (2, 512, 4, 1, 8), (3, 45, 6, 5, 3),
-                                             (3, 64, 5, 4, 16), (2, 50, 6, 1, 1)])
+                                             (3, 64, 5, 4, 16), (2, 50, 6, 1, 2)])
 def test_adjoint_run(ndim, nz, nx, ny, M):
     """pic_step_record and pic_adjoint_run over two steps without particles, against FP64 central
     differences of the oracle: gradient to 1e-4 of its largest entry (the framework's bound), and the
