@@ -17,8 +17,8 @@
 // memory.  A CTA owns ADJ_SEG cells of one z row, four per thread; rows that are differentiated along z
 // are staged with their halo, everything else is read at the cell.
 //
-// The gradient sums of FP32 fields are kept to about 48 bits in pairs of FP32 numbers (exact
-// differences, products and sums: Knuth's TwoSum, FMA TwoProd) and added up in FP64 from the warp
+// The gradient sums of FP32 fields are kept to about 48 bits in pairs of FP32 numbers (pair_math.h: exact
+// differences, products and sums) and added up in FP64 from the warp
 // totals on.  FP64 arithmetic per cell was what the step waited for: this chip does 64 FP32 operations
 // for one in FP64, so that 1024 x 256 cells with M = 4 took 34 us per gradient kernel, 127 us of the
 // 163 us of an adjoint step (now 26 us).  The pairs cost 17 FP32 operations per tap and component and the step is
@@ -27,6 +27,7 @@
 
 #include <type_traits>
 
+#include "pair_math.h"
 #include "pic_internal.h"
 
 namespace pic {
@@ -38,29 +39,6 @@ constexpr int HL = PIC_MAX_HLEN;
 
 __device__ __forceinline__ int wrapm(int a, int n) { return a < 0 ? a + n : (a >= n ? a - n : a); }
 
-// sums of two FP32 numbers with their rounding errors
-__device__ __forceinline__ void add2(float a, float b, float& s, float& e) {
-    s = a + b;
-    const float bb = s - a;
-    e = (a - (s - bb)) + (b - bb);
-}
-
-// Sum of products kept as an unevaluated pair h + l.
-struct PairSum {
-    float h = 0.f, l = 0.f;
-    __device__ __forceinline__ void add(float h2, float l2) {
-        float s, e;
-        add2(h, h2, s, e);
-        h = s;
-        l += e + l2;
-    }
-    // += x (dh + dl)
-    __device__ __forceinline__ void fma(float x, float dh, float dl) {
-        const float p = x * dh;
-        add(p, fmaf(x, dl, fmaf(x, dh, -p)));
-    }
-};
-
 // grad[l] += scale * the block's sum of acc[l], l < M
 template <int MAXM>
 __device__ __forceinline__ void flush_grad(PairSum (&acc)[MAXM], int M, double scale, double* grad) {
@@ -69,12 +47,8 @@ __device__ __forceinline__ void flush_grad(PairSum (&acc)[MAXM], int M, double s
 #pragma unroll
     for (int l = 0; l < MAXM; ++l) {
         if (l >= M) break;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            const float h2 = __shfl_xor_sync(0xffffffffu, acc[l].h, o), l2 = __shfl_xor_sync(0xffffffffu, acc[l].l, o);
-            acc[l].add(h2, l2);
-        }
-        if (lane == 0) part[l][w] = (double)acc[l].h + (double)acc[l].l;
+        acc[l].warp_sum();
+        if (lane == 0) part[l][w] = acc[l].value();
     }
     __syncthreads();
     if (threadIdx.x < M) {

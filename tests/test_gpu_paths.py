@@ -152,3 +152,51 @@ def test_adjoint_run(ndim, nz, nx, ny, M):
     lhs = float((dev(lE).double() * E[2].double()).sum() + (dev(lB).double() * B[2].double()).sum())
     assert abs(lhs - rhs) < 1e-5 * np.linalg.norm(lE) * np.linalg.norm(E0)
     sim.close()
+
+
+@pytest.mark.parametrize("ndim,shape", [(2, 1), (2, 2), (3, 1), (3, 2)])
+@pytest.mark.parametrize("spread", ["cells", "patch", "grid"])
+def test_rho_and_diagnostics(ndim, shape, spread):
+    """FP64 charge density, Gauss residual and energies against the oracle: particles of a chunk in a few
+    cells (shared nodes), in a patch across the periodic seam, and all over the grid (per-particle path).
+    A contribution is rounded to 2^-45 of a particle's charge density and a divergence to 2^-46 of the
+    sum of its terms: 1e-12 of the largest value leaves a factor of ten over the sums of 256."""
+    from oracle import core as oc
+    nz, nx, ny = (517, 30, 1) if ndim == 2 else (70, 24, 20)
+    d = (0.5, 0.4, 0.45)[:ndim]
+    C = fit.fit_coefficients(2.5, M=8)
+    grid = dict(ndim=ndim, nz=nz, nx=nx, ny=ny, dz=d[0], dx=d[1], dy=d[2] if ndim == 3 else 1.0,
+                dt=0.8 * fit.cfl_dt(d[0], d[1:], C), solver="custom", shape=shape, rho_bg=0.5)
+    sp = wl.random_particles(ndim, nz, nx, ny, 700, seed=9, u_scale=0.3, u_drift=(5.0, 0, 0), margin=0)
+    if spread != "grid":
+        ext = 2 if spread == "cells" else 9
+        rng = np.random.default_rng(3)
+        sp["iz"] = nz - ext + rng.integers(0, ext, 700)
+        sp["ix"] = (nx - ext // 2 + rng.integers(0, ext, 700)) % nx
+        if ndim == 3:
+            sp["iy"] = (ny - ext // 2 + rng.integers(0, ext, 700)) % ny
+    sim, osim = gpu_sim(grid, [sp], coef=C), oracle_sim(grid, [sp], coef=C)
+    rng = np.random.default_rng(1)
+    for a, oa in ((sim.E, osim.E), (sim.B, osim.B)):
+        v = rng.normal(size=oa.shape).astype(np.float32)
+        a.copy_(torch.from_numpy(v))
+        oa[:] = v
+    s = osim.species[0]
+    ref = oc.rho(osim.g, s.xi, s.Q)
+    got = sim.rho().cpu().numpy()
+    assert np.abs(got - ref).max() < 1e-12 * np.abs(ref).max()
+    G = sim.gauss().cpu().numpy()
+    g32 = oc.Grid(ndim, nz, nx, ny, *(float(np.float32(grid[k])) for k in ("dz", "dx", "dy", "dt")),
+                  C=C.astype(np.float32).astype(np.float64), shape=shape)     # the GPU's FP32 constants
+    Gref = oc.gauss(g32, osim.E, ref) - 0.5
+    assert np.abs(G - Gref).max() < 1e-12 * np.abs(Gref).max()
+    m = 8 + 24 + 2
+    D = sim.diag()
+    assert D["gauss_max"] == pytest.approx(np.abs(Gref[..., m:nz - m]).max(), rel=1e-11)
+    assert D["gauss_rms"] == pytest.approx(np.sqrt(np.mean(Gref[..., m:nz - m] ** 2)), rel=1e-11)
+    V = np.prod(d)
+    assert D["field_energy"] == pytest.approx(0.5 * V * (np.sum(osim.E ** 2) + np.sum(osim.B ** 2)), rel=1e-12)
+    u2 = np.sum(s.u ** 2, axis=1)
+    assert D["kinetic"] == pytest.approx(sp["w"] * np.sum(u2 / (1 + np.sqrt(1 + u2))), rel=1e-12)
+    assert D["count"] == 700
+    sim.close()
