@@ -185,7 +185,9 @@ pic_status need_fields(pic_t* h) {
 
 // Field advance from (Ein, Bin) into (Eout, Bout), with the window shift and injection that
 // complete step n.  J1 has already been corrected in place for the customised stencil.
-pic_status advance_fields(pic_t* h, const float* Ein, const float* Bin, float* Eout, float* Bout,
+// first, last: this is the first, the last step of its call (between the two the
+// k-space solvers keep the transforms of the fields).
+pic_status advance_fields(pic_t* h, const float* Ein, const float* Bin, float* Eout, float* Bout, bool first, bool last,
                           cudaStream_t s) {
     const long long N = h->g.ncell;
     const long long n_done = h->step + 1;
@@ -204,7 +206,7 @@ pic_status advance_fields(pic_t* h, const float* Ein, const float* Bin, float* E
     if (h->ks) {
         Scope sc(h, PIC_T_FIELDS, 1, s);
         char kerr[256] = {0};
-        if (kspace_advance(h->ks, Ein, Bin, h->J, Eout, Bout, s, kerr, sizeof kerr))
+        if (kspace_advance(h->ks, Ein, Bin, h->J, Eout, Bout, !first, !last, s, kerr, sizeof kerr))
             return fail(h, PIC_ERR_CUDA, "%s", kerr);
     } else {
         Scope sc(h, PIC_T_FIELDS, 1, s);
@@ -311,7 +313,8 @@ pic_status adjoint_stages(pic_t* h, const float* E, const float* B, const float*
 
 // One step n: particles and currents of every species into J, then the fields from (Ein, Bin) into
 // (Eout, Bout).
-pic_status one_step(pic_t* h, const float* Ein, const float* Bin, float* Eout, float* Bout, cudaStream_t s) {
+pic_status one_step(pic_t* h, const float* Ein, const float* Bin, float* Eout, float* Bout, bool first, bool last,
+                    cudaStream_t s) {
     pic_status st;
     if (h->cfg.sort_every > 0 && h->step % h->cfg.sort_every == 0)
         if ((st = do_sort(h, s))) return st;
@@ -347,7 +350,7 @@ pic_status one_step(pic_t* h, const float* Ein, const float* Bin, float* Eout, f
     }
     h->pending_shift = 0;
     if ((st = smooth_current(h, s))) return st;
-    return advance_fields(h, Ein, Bin, Eout, Bout, s);
+    return advance_fields(h, Ein, Bin, Eout, Bout, first, last, s);
 }
 
 }  // namespace
@@ -655,7 +658,7 @@ pic_status pic_field_advance(pic_t* h, void* stream) {
     if (st) return st;
     cudaStream_t s = (cudaStream_t)stream;
     const long long N = h->g.ncell;
-    if ((st = advance_fields(h, h->E, h->B, h->E2, h->B2, s))) return st;
+    if ((st = advance_fields(h, h->E, h->B, h->E2, h->B2, true, true, s))) return st;
     Scope sc(h, PIC_T_FIELDS, 2, s);
     CK(h, cudaMemcpyAsync(h->E, h->E2, sizeof(float) * 3 * N, cudaMemcpyDeviceToDevice, s), "copy E");
     CK(h, cudaMemcpyAsync(h->B, h->B2, sizeof(float) * 3 * N, cudaMemcpyDeviceToDevice, s), "copy B");
@@ -673,7 +676,7 @@ pic_status pic_step(pic_t* h, int nsteps, void* stream) {
     const long long N = h->g.ncell;
     float *Ec = h->E, *Bc = h->B, *En = h->E2, *Bn = h->B2;
     for (int it = 0; it < nsteps; ++it) {
-        if ((st = one_step(h, Ec, Bc, En, Bn, s))) return st;
+        if ((st = one_step(h, Ec, Bc, En, Bn, it == 0, it + 1 == nsteps, s))) return st;
         float* t = Ec;
         Ec = En;
         En = t;
@@ -701,7 +704,7 @@ pic_status pic_step_record(pic_t* h, int nsteps, float* E, float* B, float* J, v
     pic_status st = PIC_OK;
     for (int k = 0; !st && k < nsteps; ++k) {
         h->J = J + k * n3;
-        st = one_step(h, E + k * n3, B + k * n3, E + (k + 1) * n3, B + (k + 1) * n3, (cudaStream_t)stream);
+        st = one_step(h, E + k * n3, B + k * n3, E + (k + 1) * n3, B + (k + 1) * n3, true, true, (cudaStream_t)stream);
     }
     h->J = bound;
     if (!st) h->state = 0;
