@@ -21,10 +21,8 @@
 //     truncated row.
 // HBM traffic: one read and one write of the row (8 bytes per FP32 cell).
 //
-// Correction, one CTA per z row: the whole row sits in shared memory, so no other CTA reads the
-// values it overwrites.  Each thread produces four consecutive outputs from the
-// (2 PIC_MAX_HLEN + 4)-float window below them, read as aligned 128-bit shared loads (taps beyond
-// hlen are zero).
+// Correction, whole z rows per CTA: a row sits in shared memory, so no other CTA reads the values it
+// overwrites; two rows at a time (correct_pair), single ones after the filter (taps beyond hlen are zero).
 #include <cuda_runtime.h>
 
 #include "pic_internal.h"
@@ -195,6 +193,108 @@ __device__ __forceinline__ void correct_row(float* row, int nz, const float* __r
     correct_from(s, row, nz, h);
 }
 
+// Two rows at a time.  The rows lie in shared memory interleaved as pairs, so one packed FMA does a tap of
+// both, and a lane produces eight consecutive cells of both from the 56 pairs around them, each read
+// once: 28 128-bit loads and 392 packed FMAs for 16 outputs, where one row and four cells per thread
+// took 13 loads and 196 FMAs for four.  The sums run over the taps in the same order as
+// correct_from's: the results are the same bits.  A lane's eight pairs take five 16-byte groups (one
+// padding): the lanes of a quarter warp read different groups modulo 8.
+// Measured: 512 x 256 x 256 128 us before, 86 us now (39 us at the copy bandwidth, 44 us of FP32 pipe);
+// 128 instances of 128..1024 x 64..256 cells 132 and 69 us.
+constexpr int CP_NT = 128, CP_G = 20;           // threads; floats of a lane's pairs with padding
+constexpr int CP_HALO = kHL / 8;                // lanes of zeros at either end
+static_assert(kHL % 8 == 0, "the halo is whole lanes");
+constexpr int CP_MAX_NZ = 16384;                // longer rows do not fit in pairs
+
+__host__ __device__ constexpr int pair_floats(int nz) { return ((nz + 7) / 8 + 2 * CP_HALO) * CP_G; }
+
+// rows r0 and r0 + nz (two: both exist) of nz cells, in place; threads tid of nt, buffer s of
+// pair_floats(nz), taps h2 (each twice) in shared memory.  Every thread of the CTA calls (barriers inside);
+// live: this group has rows.
+__device__ __forceinline__ void correct_pair(float* r0, int nz, bool live, bool two, bool vec4, const float2* h2, float* s,
+                                             int tid, int nt) {
+    float* r1 = two ? r0 + nz : r0;
+    const int lanes = (nz + 7) / 8;
+    if (live) {
+        for (int k = tid; k < 2 * CP_HALO * 4; k += nt) {             // 16-byte groups of the halo lanes
+            const int l = k >> 2;
+            const int lane = l < CP_HALO ? l : lanes + l;
+            *reinterpret_cast<float4*>(s + lane * CP_G + 4 * (k & 3)) = make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+        if (vec4) {
+            for (int q = tid; q < 2 * lanes; q += nt) {
+                float4 a = make_float4(0.f, 0.f, 0.f, 0.f), b = a;
+                if (4 * q < nz) {
+                    a = *reinterpret_cast<const float4*>(r0 + 4 * q);
+                    b = *reinterpret_cast<const float4*>(r1 + 4 * q);
+                }
+                float* d = s + (CP_HALO + (q >> 1)) * CP_G + 8 * (q & 1);
+                *reinterpret_cast<float4*>(d) = make_float4(a.x, b.x, a.y, b.y);
+                *reinterpret_cast<float4*>(d + 4) = make_float4(a.z, b.z, a.w, b.w);
+            }
+        } else {
+            for (int z = tid; z < 8 * lanes; z += nt)
+                *reinterpret_cast<float2*>(s + (CP_HALO + (z >> 3)) * CP_G + 2 * (z & 7)) =
+                    z < nz ? make_float2(r0[z], r1[z]) : make_float2(0.f, 0.f);
+        }
+    }
+    __syncthreads();
+    if (!live) return;
+    for (int l = tid; l < lanes; l += nt) {
+        float2 acc[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) acc[j] = make_float2(0.f, 0.f);
+        const float* own = s + (CP_HALO + l) * CP_G;
+        // out[j] = sum_m h[m] x[j - m]: x from the highest cell down, so that every sum starts at m = -kHL
+#pragma unroll
+        for (int r = kHL + 6; r >= -kHL; r -= 2) {
+            const int at = r + 64 * 8;
+            const float4 v = *reinterpret_cast<const float4*>(own + (at / 8 - 64) * CP_G + 2 * (at % 8));
+            const float2 x[2] = {make_float2(v.z, v.w), make_float2(v.x, v.y)};       // cells r + 1, r
+#pragma unroll
+            for (int q = 0; q < 2; ++q)
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    const int m = j - (r + 1 - q);
+                    if (m >= -kHL && m <= kHL) acc[j] = __ffma2_rn(h2[kHL + m], x[q], acc[j]);
+                }
+        }
+        const int z = 8 * l;
+        if (vec4) {
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                if (z + 4 * q >= nz) break;
+                const float2* c = acc + 4 * q;
+                *reinterpret_cast<float4*>(r0 + z + 4 * q) = make_float4(c[0].x, c[1].x, c[2].x, c[3].x);
+                if (two) *reinterpret_cast<float4*>(r1 + z + 4 * q) = make_float4(c[0].y, c[1].y, c[2].y, c[3].y);
+            }
+        } else {
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                if (z + j >= nz) break;
+                r0[z + j] = acc[j].x;
+                if (two) r1[z + j] = acc[j].y;
+            }
+        }
+    }
+}
+
+__device__ __forceinline__ void load_taps(float2* h2, const float* __restrict__ h) {
+    for (int k = threadIdx.x; k <= 2 * kHL; k += blockDim.x) h2[k] = make_float2(h[k], h[k]);
+}
+
+// CP_NT / tpr pairs of rows per CTA, tpr threads each (a multiple of 32)
+__global__ void __launch_bounds__(CP_NT) correct_j1_pairs_kernel(const __grid_constant__ CorrP p, long long rows, int tpr,
+                                                                 int vec4) {
+    extern __shared__ float4 s4[];
+    __shared__ float2 h2[2 * kHL + 1];
+    load_taps(h2, p.h);
+    const int grp = threadIdx.x / tpr, nz = p.g.nz;
+    const long long r = 2 * ((long long)blockIdx.x * (CP_NT / tpr) + grp);
+    correct_pair(p.J1 + (r < rows ? r : 0) * nz, nz, r < rows, r + 1 < rows, vec4 != 0, h2,
+                 reinterpret_cast<float*>(s4) + grp * pair_floats(nz), threadIdx.x - grp * tpr, tpr);
+}
+
 // Several rows per CTA: rows_per_cta groups of tpr threads (tpr a multiple of 32, 4 tpr >= nz for
 // one pass); vec4: rows 16-byte aligned (nz % 4 == 0), staged with 16-byte loads.
 __global__ void __launch_bounds__(256) correct_j1_rows_kernel(CorrP p, long long rows, int tpr, int vec4) {
@@ -241,12 +341,23 @@ __global__ void __launch_bounds__(128) filter_z_batch_kernel(const FiltInst* __r
     filter_row<float, 128>(row, row, q.g.nz, q.vec4 != 0, buf);
 }
 
-// Batched in-place correction: blockIdx.y = instance, blockIdx.x = z row of that instance.
-__global__ void __launch_bounds__(256) correct_j1_batch_kernel(const CorrInst* __restrict__ inst) {
+// Batched in-place correction: blockIdx.y = instance, blockIdx.x = pair of z rows of that instance.
+__global__ void __launch_bounds__(CP_NT) correct_j1_batch_kernel(const CorrInst* __restrict__ inst) {
     extern __shared__ float4 s4[];
+    __shared__ float2 h2[2 * kHL + 1];
     const CorrInst& q = inst[blockIdx.y];
-    if ((long long)blockIdx.x >= (long long)q.g.nx * q.g.ny) return;
-    correct_row(q.J1 + (long long)blockIdx.x * q.g.nz, q.g.nz, q.h, reinterpret_cast<float*>(s4));
+    const long long rows = (long long)q.g.nx * q.g.ny, r = 2LL * blockIdx.x;
+    if (r >= rows) return;
+    float* row = q.J1 + r * q.g.nz;
+    if (q.g.nz > CP_MAX_NZ) {
+        correct_row(row, q.g.nz, q.h, reinterpret_cast<float*>(s4));
+        __syncthreads();
+        if (r + 1 < rows) correct_row(row + q.g.nz, q.g.nz, q.h, reinterpret_cast<float*>(s4));
+        return;
+    }
+    load_taps(h2, q.h);
+    correct_pair(row, q.g.nz, true, r + 1 < rows, q.g.nz % 4 == 0 && ((uintptr_t)q.J1 & 15) == 0, h2,
+                 reinterpret_cast<float*>(s4), threadIdx.x, CP_NT);
 }
 
 // Filter and correction in one launch over the 3 nx ny rows of J (p.J1 = J): a J1 row is filtered
@@ -331,6 +442,20 @@ cudaError_t launch_filter_current_batch(const FiltInst* inst, int ninst, long lo
 cudaError_t launch_correct_j1(const GridP& g, const float* taps, int hlen, float* J1, cudaStream_t s) {
     CorrP p = corr_params(g, taps, hlen, J1);
     const long long rows = (long long)g.nx * g.ny;
+    const int vec4 = (g.nz % 4 == 0 && ((uintptr_t)J1 & 15) == 0) ? 1 : 0;
+    // Pairs of rows where they are short and many: a pair's buffer is 2.5 times a row's and there are half
+    // as many CTAs.  One row at a time and pairs: 512 cells x 65536 rows 128 and 86 us; 8192 x 2048 41 and 46,
+    // 2048 x 512 5.7 and 6.1 (256 CTAs on 152 SMs).
+    if (g.nz <= 1024 && rows >= 4096) {
+        // threads per pair: a lane each, in whole warps; short rows share a CTA
+        int tpr = ((g.nz + 7) / 8 + 31) / 32 * 32;
+        tpr = tpr > CP_NT / 2 ? CP_NT : tpr;
+        const int per = CP_NT / tpr;
+        const size_t smem = sizeof(float) * pair_floats(g.nz) * per;
+        static_assert(sizeof(float) * pair_floats(1024) < 48 * 1024, "default shared memory");
+        correct_j1_pairs_kernel<<<(unsigned)((rows + 2 * per - 1) / (2 * per)), per * tpr, smem, s>>>(p, rows, tpr, vec4);
+        return cudaGetLastError();
+    }
     // threads per row: enough for one pass of four outputs each, in whole warps, at most 256
     int tpr = (((g.nz + 3) / 4) + 31) / 32 * 32;
     tpr = tpr > 256 ? 256 : tpr;
@@ -343,7 +468,6 @@ cudaError_t launch_correct_j1(const GridP& g, const float* taps, int hlen, float
         if (e != cudaSuccess) return e;
         opted = smem;
     }
-    const int vec4 = (g.nz % 4 == 0 && ((uintptr_t)J1 & 15) == 0) ? 1 : 0;
     correct_j1_rows_kernel<<<(unsigned)((rows + rpc - 1) / rpc), rpc * tpr, smem, s>>>(p, rows, tpr, vec4);
     return cudaGetLastError();
 }
@@ -361,13 +485,15 @@ cudaError_t launch_filter_correct(const GridP& g, const float* taps, int hlen, f
 
 cudaError_t launch_correct_j1_batch(const CorrInst* inst, int ninst, int max_rows, int max_nz, cudaStream_t s) {
     if (ninst <= 0) return cudaSuccess;
-    const size_t smem = sizeof(float) * corr_floats(max_nz);
+    const int paired = max_nz < CP_MAX_NZ ? max_nz : CP_MAX_NZ;
+    size_t smem = sizeof(float) * pair_floats(paired);
+    if (max_nz > CP_MAX_NZ && sizeof(float) * corr_floats(max_nz) > smem) smem = sizeof(float) * corr_floats(max_nz);
     if (smem > 48 * 1024) {
         cudaError_t e = cudaFuncSetAttribute(correct_j1_batch_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              (int)smem);
         if (e != cudaSuccess) return e;
     }
-    correct_j1_batch_kernel<<<dim3((unsigned)max_rows, (unsigned)ninst), 256, smem, s>>>(inst);
+    correct_j1_batch_kernel<<<dim3((unsigned)((max_rows + 1) / 2), (unsigned)ninst), CP_NT, smem, s>>>(inst);
     return cudaGetLastError();
 }
 
