@@ -141,6 +141,7 @@ __device__ __forceinline__ RowAt row_at(const GridP& g, int r) {
 template <int MP>
 __global__ void __launch_bounds__(ADJ_NT) adjoint_ampere_kernel(GridP g, StencilP st, const float* __restrict__ F,
                                                                 const float* __restrict__ aB, float* aE, double* grad) {
+    chain_enter();
     constexpr int W = ADJ_SEG + 2 * MP;
     __shared__ __align__(16) float sB[2][W], sF[2][W];
     const long long N = g.ncell;
@@ -235,6 +236,7 @@ __global__ void __launch_bounds__(ADJ_NT) adjoint_faraday_kernel(GridP g, Stenci
                                                                  const float* __restrict__ B, const float* __restrict__ J1,
                                                                  const float* __restrict__ aE, float* aB, TapsP taps,
                                                                  int correct, double* grad) {
+    chain_enter();
     constexpr int W = ADJ_SEG + 2 * MP, W1 = ADJ_SEG + 2 * HL;
     __shared__ __align__(16) float sE[2][ADJ_SEG + 4 * MP], sH[2][W], sA[2][W], sA1[W1], sJ[W];
     const long long N = g.ncell;
@@ -319,6 +321,7 @@ template <int MP>
 __global__ void __launch_bounds__(ADJ_NT) adjoint_enew_kernel(GridP g, StencilP st, const float* __restrict__ E,
                                                               const float* __restrict__ B, const float* __restrict__ J,
                                                               float* __restrict__ out) {
+    chain_enter();
     constexpr int W = ADJ_SEG + 2 * MP;
     __shared__ __align__(16) float sE[2][ADJ_SEG + 4 * MP], sH[2][W];
     const long long N = g.ncell;
@@ -353,10 +356,9 @@ inline dim3 adj_grid(const GridP& g) {
 
 template <typename F>
 cudaError_t by_width(int M, F&& f) {
-    if (M <= 4) f(std::integral_constant<int, 4>());
-    else if (M <= 8) f(std::integral_constant<int, 8>());
-    else f(std::integral_constant<int, 16>());
-    return cudaGetLastError();
+    if (M <= 4) return f(std::integral_constant<int, 4>());
+    if (M <= 8) return f(std::integral_constant<int, 8>());
+    return f(std::integral_constant<int, 16>());
 }
 
 }  // namespace
@@ -364,14 +366,14 @@ cudaError_t by_width(int M, F&& f) {
 cudaError_t launch_adjoint_enew(const GridP& g, const StencilP& st, const float* E, const float* B, const float* J,
                                 float* out, cudaStream_t s) {
     return by_width(st.M, [&](auto m) {
-        adjoint_enew_kernel<decltype(m)::value><<<adj_grid(g), ADJ_NT, 0, s>>>(g, st, E, B, J, out);
+        return launch_chained(adjoint_enew_kernel<decltype(m)::value>, adj_grid(g), ADJ_NT, 0, s, g, st, E, B, J, out);
     });
 }
 
 cudaError_t launch_adjoint_ampere(const GridP& g, const StencilP& st, const float* F, const float* aB, float* aE,
                                   double* grad, cudaStream_t s) {
     return by_width(st.M, [&](auto m) {
-        adjoint_ampere_kernel<decltype(m)::value><<<adj_grid(g), ADJ_NT, 0, s>>>(g, st, F, aB, aE, grad);
+        return launch_chained(adjoint_ampere_kernel<decltype(m)::value>, adj_grid(g), ADJ_NT, 0, s, g, st, F, aB, aE, grad);
     });
 }
 
@@ -380,8 +382,8 @@ cudaError_t launch_adjoint_faraday(const GridP& g, const StencilP& st, const flo
     TapsP t;
     for (int m = -HL; m <= HL; ++m) t.h[HL + m] = m >= -hlen && m <= hlen ? taps[m + hlen] : 0.f;
     return by_width(st.M, [&](auto m) {
-        adjoint_faraday_kernel<decltype(m)::value>
-            <<<adj_grid(g), ADJ_NT, 0, s>>>(g, st, E, B, J1, aE, aB, t, hlen > 0 ? 1 : 0, grad);
+        return launch_chained(adjoint_faraday_kernel<decltype(m)::value>, adj_grid(g), ADJ_NT, 0, s, g, st, E, B, J1, aE, aB,
+                              t, hlen > 0 ? 1 : 0, grad);
     });
 }
 

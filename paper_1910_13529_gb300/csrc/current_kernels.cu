@@ -286,6 +286,7 @@ __device__ __forceinline__ void load_taps(float2* h2, const float* __restrict__ 
 // CP_NT / tpr pairs of rows per CTA, tpr threads each (a multiple of 32)
 __global__ void __launch_bounds__(CP_NT) correct_j1_pairs_kernel(const __grid_constant__ CorrP p, long long rows, int tpr,
                                                                  int vec4) {
+    chain_enter();
     extern __shared__ float4 s4[];
     __shared__ float2 h2[2 * kHL + 1];
     load_taps(h2, p.h);
@@ -298,6 +299,7 @@ __global__ void __launch_bounds__(CP_NT) correct_j1_pairs_kernel(const __grid_co
 // Several rows per CTA: rows_per_cta groups of tpr threads (tpr a multiple of 32, 4 tpr >= nz for
 // one pass); vec4: rows 16-byte aligned (nz % 4 == 0), staged with 16-byte loads.
 __global__ void __launch_bounds__(256) correct_j1_rows_kernel(CorrP p, long long rows, int tpr, int vec4) {
+    chain_enter();
     extern __shared__ float4 s4[];
     const int nz = p.g.nz, cf = corr_floats(nz);
     const int grp = threadIdx.x / tpr, tid = threadIdx.x - grp * tpr;
@@ -327,6 +329,7 @@ __global__ void __launch_bounds__(256) correct_j1_rows_kernel(CorrP p, long long
 
 template <typename T, int NT>
 __global__ void __launch_bounds__(NT) filter_z_kernel(T* f, int nz, int vec4) {
+    chain_enter();
     __shared__ __align__(16) T buf[8 * NT + 16];
     T* row = f + (long long)blockIdx.x * nz;
     filter_row<T, NT>(row, row, nz, vec4 != 0, buf);
@@ -365,6 +368,7 @@ __global__ void __launch_bounds__(CP_NT) correct_j1_batch_kernel(const CorrInst*
 // once and written once); J2 and J3 rows are filtered in place.
 template <int NT>
 __global__ void __launch_bounds__(NT) filter_correct_kernel(CorrP p, int vec4) {
+    chain_enter();
     extern __shared__ float4 s4[];
     __shared__ __align__(16) float buf[8 * NT + 16];
     const int nz = p.g.nz;
@@ -386,13 +390,13 @@ inline int filter_threads(int nz) { return nz <= 256 ? 32 : nz <= 512 ? 64 : nz 
 template <typename T>
 cudaError_t launch_rows(T* f, int nz, long long rows, int vec4, cudaStream_t s) {
     if (rows <= 0) return cudaSuccess;
+    const bool chain = rows * nz <= 3 * CHAIN_CELLS;   // three components
     switch (filter_threads(nz)) {
-        case 32: filter_z_kernel<T, 32><<<(unsigned)rows, 32, 0, s>>>(f, nz, vec4); break;
-        case 64: filter_z_kernel<T, 64><<<(unsigned)rows, 64, 0, s>>>(f, nz, vec4); break;
-        case 128: filter_z_kernel<T, 128><<<(unsigned)rows, 128, 0, s>>>(f, nz, vec4); break;
-        default: filter_z_kernel<T, 256><<<(unsigned)rows, 256, 0, s>>>(f, nz, vec4); break;
+        case 32: return launch_chained_if(chain, filter_z_kernel<T, 32>, (unsigned)rows, 32, 0, s, f, nz, vec4);
+        case 64: return launch_chained_if(chain, filter_z_kernel<T, 64>, (unsigned)rows, 64, 0, s, f, nz, vec4);
+        case 128: return launch_chained_if(chain, filter_z_kernel<T, 128>, (unsigned)rows, 128, 0, s, f, nz, vec4);
+        default: return launch_chained_if(chain, filter_z_kernel<T, 256>, (unsigned)rows, 256, 0, s, f, nz, vec4);
     }
-    return cudaGetLastError();
 }
 
 template <int NT>
@@ -404,8 +408,7 @@ cudaError_t launch_fc(const CorrP& p, int vec4, cudaStream_t s) {
                                              (int)smem);
         if (e != cudaSuccess) return e;
     }
-    filter_correct_kernel<NT><<<(unsigned)(3LL * p.g.nx * p.g.ny), NT, smem, s>>>(p, vec4);
-    return cudaGetLastError();
+    return launch_chained_if(few_cells(p.g), filter_correct_kernel<NT>, (unsigned)(3LL * p.g.nx * p.g.ny), NT, smem, s, p, vec4);
 }
 
 CorrP corr_params(const GridP& g, const float* taps, int hlen, float* J1) {
@@ -453,8 +456,8 @@ cudaError_t launch_correct_j1(const GridP& g, const float* taps, int hlen, float
         const int per = CP_NT / tpr;
         const size_t smem = sizeof(float) * pair_floats(g.nz) * per;
         static_assert(sizeof(float) * pair_floats(1024) < 48 * 1024, "default shared memory");
-        correct_j1_pairs_kernel<<<(unsigned)((rows + 2 * per - 1) / (2 * per)), per * tpr, smem, s>>>(p, rows, tpr, vec4);
-        return cudaGetLastError();
+        return launch_chained_if(few_cells(p.g), correct_j1_pairs_kernel, (unsigned)((rows + 2 * per - 1) / (2 * per)), per * tpr, smem, s, p,
+                              rows, tpr, vec4);
     }
     // threads per row: enough for one pass of four outputs each, in whole warps, at most 256
     int tpr = (((g.nz + 3) / 4) + 31) / 32 * 32;
@@ -468,8 +471,7 @@ cudaError_t launch_correct_j1(const GridP& g, const float* taps, int hlen, float
         if (e != cudaSuccess) return e;
         opted = smem;
     }
-    correct_j1_rows_kernel<<<(unsigned)((rows + rpc - 1) / rpc), rpc * tpr, smem, s>>>(p, rows, tpr, vec4);
-    return cudaGetLastError();
+    return launch_chained_if(few_cells(p.g), correct_j1_rows_kernel, (unsigned)((rows + rpc - 1) / rpc), rpc * tpr, smem, s, p, rows, tpr, vec4);
 }
 
 cudaError_t launch_filter_correct(const GridP& g, const float* taps, int hlen, float* J, cudaStream_t s) {

@@ -532,6 +532,7 @@ __device__ __forceinline__ void advance_tile_rb(const FieldP& p, int tz, int tx,
 
 template <int NDIM, int MAXM, int TZ, int TX, int TY>
 __global__ void __launch_bounds__(256, 2) field_advance_rb_kernel(FieldP p) {
+    chain_enter();
     extern __shared__ float4 smem4[];
     advance_tile_rb<NDIM, MAXM, TZ, TX, TY>(p, blockIdx.x, blockIdx.y, blockIdx.z, reinterpret_cast<float*>(smem4));
 }
@@ -1093,6 +1094,7 @@ __host__ __device__ inline int row_segment(int nz, int nseg) {
 
 template <int MAXM, int NT, bool VEC>
 __global__ void __launch_bounds__(NT) field_advance_rows_kernel(FieldP p, int tz, int xc) {
+    chain_enter();
     extern __shared__ float4 smem4[];
     const int xa = blockIdx.y * xc, xb = min(xa + xc, p.g.nx);
     march_rows<MAXM, NT, VEC>(p, blockIdx.x * tz, tz, xa, xb, reinterpret_cast<float*>(smem4));
@@ -1136,6 +1138,7 @@ struct MarchRingT {
 
 template <int MAXM, int TZ, int TX, int NT>
 __global__ void __launch_bounds__(NT) field_advance_march_ring_kernel(FieldP p, int yc) {
+    chain_enter();
     using T = MarchT<MAXM, TZ, TX>;
     extern __shared__ float4 smem4[];
     float* sm = reinterpret_cast<float*>(smem4);
@@ -1212,6 +1215,7 @@ __global__ void __launch_bounds__(NT) field_advance_march_ring_kernel(FieldP p, 
 
 template <int MAXM, int TZ, int TX, int NT>
 __global__ void __launch_bounds__(NT) field_advance_march_kernel(FieldP p, int yc) {
+    chain_enter();
     using T = MarchT<MAXM, TZ, TX>;
     extern __shared__ float4 smem4[];
     float* sm = reinterpret_cast<float*>(smem4);
@@ -1278,6 +1282,7 @@ __global__ void __launch_bounds__(NT) field_advance_march_kernel(FieldP p, int y
 
 template <int NDIM, int MAXM, int TZ, int TX, int TY>
 __global__ void __launch_bounds__(256) field_advance_kernel(FieldP p) {
+    chain_enter();
     extern __shared__ float smem[];
     advance_tile<NDIM, MAXM, TZ, TX, TY>(p, blockIdx.x, blockIdx.y, blockIdx.z, smem);
 }
@@ -1319,8 +1324,7 @@ cudaError_t launch_fa(const FieldP& p, cudaStream_t s) {
         configured = true;
     }
     dim3 grid((p.g.nz + TZ - 1) / TZ, (p.g.nx + TX - 1) / TX, NDIM == 3 ? (p.g.ny + TY - 1) / TY : 1);
-    k<<<grid, 256, T::smem_bytes, s>>>(p);
-    return cudaGetLastError();
+    return launch_chained_if(few_cells(p.g), k, grid, 256, T::smem_bytes, s, p);
 }
 
 template <int NDIM, int MAXM, int TZ, int TX, int TY>
@@ -1335,8 +1339,7 @@ cudaError_t launch_fa_rb(const FieldP& p, cudaStream_t s) {
         configured = true;
     }
     dim3 grid((p.g.nz + TZ - 1) / TZ, (p.g.nx + TX - 1) / TX, NDIM == 3 ? (p.g.ny + TY - 1) / TY : 1);
-    k<<<grid, 256, T::smem_bytes, s>>>(p);
-    return cudaGetLastError();
+    return launch_chained_if(few_cells(p.g), k, grid, 256, T::smem_bytes, s, p);
 }
 
 // Rows (2D) or planes (3D) per marching chunk: the chunk count that minimises the number of waves
@@ -1377,8 +1380,7 @@ cudaError_t launch_fa_march(const FieldP& p, cudaStream_t s) {
     per_sm = per_sm < 1 ? 1 : (per_sm > 2048 / NT ? 2048 / NT : per_sm);
     const int yc = march_chunk(p.g.ny, cols, nsm * per_sm, 8);
     dim3 grid((p.g.nz + TZ - 1) / TZ, (p.g.nx + TX - 1) / TX, (p.g.ny + yc - 1) / yc);
-    k<<<grid, NT, T::smem_bytes, s>>>(p, yc);
-    return cudaGetLastError();
+    return launch_chained_if(few_cells(p.g), k, grid, NT, T::smem_bytes, s, p, yc);
 }
 
 // CTAs of k that one SM holds (k already has its shared-memory limit), once per kernel
@@ -1410,8 +1412,7 @@ cudaError_t launch_fa_rows_v(const FieldP& p, cudaStream_t s) {
     const int nseg = (p.g.nz + T::OUT - 1) / T::OUT, tz = row_segment(p.g.nz, nseg);
     const int cols = (p.g.nz + tz - 1) / tz;
     const int xc = march_chunk(p.g.nx, cols, sm_count() * per_sm, 8);
-    k<<<dim3(cols, (p.g.nx + xc - 1) / xc, 1), NT, T::smem_bytes, s>>>(p, tz, xc);
-    return cudaGetLastError();
+    return launch_chained_if(few_cells(p.g), k, dim3(cols, (p.g.nx + xc - 1) / xc, 1), NT, T::smem_bytes, s, p, tz, xc);
 }
 
 template <int MAXM, int NT>
@@ -1438,8 +1439,7 @@ cudaError_t launch_fa_march_ring(const FieldP& p, cudaStream_t s) {
     per_sm = per_sm < 1 ? 1 : (per_sm > 2048 / NT ? 2048 / NT : per_sm);
     const int yc = march_chunk(p.g.ny, cols, nsm * per_sm, 8);
     dim3 grid((p.g.nz + TZ - 1) / TZ, (p.g.nx + TX - 1) / TX, (p.g.ny + yc - 1) / yc);
-    k<<<grid, NT, T::smem_bytes, s>>>(p, yc);
-    return cudaGetLastError();
+    return launch_chained_if(few_cells(p.g), k, grid, NT, T::smem_bytes, s, p, yc);
 }
 
 template <int NDIM, int MAXM, int TZ, int TX, int TY>
@@ -1586,6 +1586,53 @@ cudaError_t launch_field_advance_batch(const FieldP* inst, const int4* work, int
     if (maxm <= 4) return launch_fa_batch<3, 4, 64, 4, 4>(inst, work, total_tiles, parity, s);
     if (maxm <= 8) return launch_fa_batch<3, 8, 64, 4, 4>(inst, work, total_tiles, parity, s);
     return launch_fa_batch<3, 16, 64, 4, 4>(inst, work, total_tiles, parity, s);
+}
+
+namespace {
+__global__ void __launch_bounds__(256) zero_kernel(float* f, long long n) {
+    chain_enter();
+    const long long n4 = ((uintptr_t)f & 15) ? 0 : n / 4, step = (long long)gridDim.x * 256;
+    const long long t = (long long)blockIdx.x * 256 + threadIdx.x;
+    for (long long i = t; i < n4; i += step) reinterpret_cast<float4*>(f)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (long long i = 4 * n4 + t; i < n; i += step) f[i] = 0.f;
+}
+__global__ void __launch_bounds__(256) copy2_kernel(float* d0, const float* s0, float* d1, const float* s1, long long n) {
+    chain_enter();
+    const bool vec = (((uintptr_t)d0 | (uintptr_t)s0 | (uintptr_t)d1 | (uintptr_t)s1) & 15) == 0;
+    const long long n4 = vec ? n / 4 : 0, step = (long long)gridDim.x * 256;
+    const long long t = (long long)blockIdx.x * 256 + threadIdx.x;
+    for (long long i = t; i < n4; i += step) {
+        const float4 a = reinterpret_cast<const float4*>(s0)[i], b = reinterpret_cast<const float4*>(s1)[i];
+        reinterpret_cast<float4*>(d0)[i] = a;
+        reinterpret_cast<float4*>(d1)[i] = b;
+    }
+    for (long long i = 4 * n4 + t; i < n; i += step) {
+        d0[i] = s0[i];
+        d1[i] = s1[i];
+    }
+}
+
+// Arrays up to this many floats are cleared and copied by the kernels above, chained to the step's other
+// kernels; longer ones by the driver's memset and copies, where the gap does not matter.
+constexpr long long CHAIN_FLOATS = 3 << 20;
+
+unsigned chain_blocks(long long n) {
+    const long long b = (n / 4 + 255) / 256;
+    return (unsigned)(b < 1 ? 1 : b > 152 * 8 ? 152 * 8 : b);
+}
+}  // namespace
+
+cudaError_t launch_zero(float* f, long long n, cudaStream_t s) {
+    if (n > CHAIN_FLOATS) return cudaMemsetAsync(f, 0, sizeof(float) * n, s);
+    return launch_chained(zero_kernel, chain_blocks(n), 256, 0, s, f, n);
+}
+
+cudaError_t launch_copy2(float* d0, const float* s0, float* d1, const float* s1, long long n, cudaStream_t s) {
+    if (n > CHAIN_FLOATS) {
+        cudaError_t e = cudaMemcpyAsync(d0, s0, sizeof(float) * n, cudaMemcpyDeviceToDevice, s);
+        return e != cudaSuccess ? e : cudaMemcpyAsync(d1, s1, sizeof(float) * n, cudaMemcpyDeviceToDevice, s);
+    }
+    return launch_chained(copy2_kernel, chain_blocks(n), 256, 0, s, d0, s0, d1, s1, n);
 }
 
 // Tile variants the autotuner chooses from.  2D: (TZ, TX); 3D: (TZ, TX, TY); rb = register-

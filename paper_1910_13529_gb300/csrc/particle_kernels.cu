@@ -474,6 +474,7 @@ __device__ __forceinline__ bool advance_one(const GridP& g, const SpeciesP& sp, 
 template <int NDIM, int SHAPE>
 __global__ void __launch_bounds__(256) push_kernel(GridP g, SpeciesP sp, const float* __restrict__ E,
                                                    const float* __restrict__ B, int shift) {
+    chain_enter();
     const long long n = *sp.count;
     const long long cap = sp.cap;
     for (long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x; p < n;
@@ -1572,6 +1573,7 @@ __global__ void __launch_bounds__(FUSED_T, 3) push_deposit_3d_kernel(GridP g, Sp
                                                                      int* __restrict__ defer2,
                                                                      const __grid_constant__ CUtensorMap mapE,
                                                                      const __grid_constant__ CUtensorMap mapB, int* status) {
+    chain_enter();
     extern __shared__ __align__(128) float4 smem4[];
     float* smem = reinterpret_cast<float*>(smem4);
     __shared__ int box[BW_SHARED];
@@ -1926,6 +1928,7 @@ __global__ void __launch_bounds__(FUSED_T, 2) push_deposit_3d_leftover_kernel(Gr
                                                                               const float* __restrict__ E,
                                                                               const float* __restrict__ B,
                                                                               float* __restrict__ J, int shift) {
+    chain_enter();
     extern __shared__ float4 smem4[];
     float* smem = reinterpret_cast<float*>(smem4);
     __shared__ int box[14];
@@ -1986,6 +1989,7 @@ template <int SHAPE>
 __global__ void __launch_bounds__(FUSED_T, 4) push_deposit_2d_kernel(GridP g, SpeciesP sp, const float* __restrict__ E,
                                                                      const float* __restrict__ B, float* __restrict__ J,
                                                                      int shift) {
+    chain_enter();
     extern __shared__ float4 smem4[];      // 16-byte aligned: the boxes are read and written as float4
     float* smem = reinterpret_cast<float*>(smem4);
     __shared__ int box[BW2_SHARED];
@@ -2052,6 +2056,7 @@ __device__ __forceinline__ void deposit_one(const GridP& g, const SpeciesP& sp, 
 // Unfused deposition from the positions saved by push_kernel<MODE_PUSH_ONLY>.
 template <int NDIM, int SHAPE>
 __global__ void __launch_bounds__(256) deposit_kernel(GridP g, SpeciesP sp, float* __restrict__ J) {
+    chain_enter();
     const long long n = *sp.count;
     for (long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x; p < n;
          p += (long long)gridDim.x * blockDim.x)
@@ -2067,6 +2072,7 @@ __global__ void __launch_bounds__(256) deposit_kernel(GridP g, SpeciesP sp, floa
 // the new column, as after a sort, instead of a long row of cells.
 __global__ void inject_kernel(GridP g, SpeciesP sp, int pz, int px, int py, int pxc, int pyc, int align,
                               long long nnew, long long next_id, int* status) {
+    chain_enter();
     const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= nnew + align - 1) return;
     const long long base0 = *sp.count;
@@ -2110,6 +2116,7 @@ __global__ void inject_kernel(GridP g, SpeciesP sp, int pz, int px, int py, int 
 }
 
 __global__ void add_count_kernel(int32_t* count, long long nnew, int align, long long cap) {
+    chain_enter();
     const long long base = ((long long)*count + align - 1) / align * align;
     if (base + nnew <= cap) *count = (int32_t)(base + nnew);
 }
@@ -2513,7 +2520,7 @@ cudaError_t launch_push(const GridP& g0, const SpeciesP& sp, const float* E, con
                 if (e != cudaSuccess) return e;
                 configured = true;
             }
-            k<<<pblocks(extent), FUSED_T, smem, s>>>(g, sp, E, B, J, shift);
+            return launch_chained(k, pblocks(extent), FUSED_T, smem, s, g, sp, E, B, J, shift);
         } else if (mode == MODE_FUSED) {
             const size_t smem = SMEM_3D * sizeof(float);
             CUtensorMap mapE{}, mapB{};
@@ -2525,12 +2532,11 @@ cudaError_t launch_push(const GridP& g0, const SpeciesP& sp, const float* E, con
                 if (e != cudaSuccess) return e;
                 configured[tma] = true;
             }
-            k<<<pblocks(extent), FUSED_T, smem, s>>>(g, sp, E, B, J, shift, defer, defer + defer_len(sp.cap), mapE, mapB,
-                                                     status);
+            return launch_chained(k, pblocks(extent), FUSED_T, smem, s, g, sp, E, B, J, shift, defer,
+                                  defer + defer_len(sp.cap), mapE, mapB, status);
         } else {
-            push_kernel<ND, SH><<<pblocks(extent), 256, 0, s>>>(g, sp, E, B, shift);
+            return launch_chained(push_kernel<ND, SH>, pblocks(extent), 256, 0, s, g, sp, E, B, shift);
         }
-        return cudaGetLastError();
     });
 }
 
@@ -2561,8 +2567,7 @@ cudaError_t launch_push_leftover(const GridP& g0, const SpeciesP* sp, int* const
         }
         // the lists' lengths are on the device: a full grid, or one CTA per warp of a small extent
         const long long want = nchunk * (FUSED_T / 32);
-        k<<<(unsigned)(want < 152 * 2 ? want : 152 * 2), FUSED_T, smem, s>>>(g, lp, E, B, J, shift);
-        return cudaGetLastError();
+        return launch_chained(k, (unsigned)(want < 152 * 2 ? want : 152 * 2), FUSED_T, smem, s, g, lp, E, B, J, shift);
     });
 }
 
@@ -2612,8 +2617,7 @@ cudaError_t launch_deposit_unfused(const GridP& g0, const SpeciesP& sp, float* J
     if (extent <= 0) return cudaSuccess;
     return dispatch(g.ndim, g.shape, [&](auto nd, auto sh) {
         constexpr int ND = decltype(nd)::value, SH = decltype(sh)::value;
-        deposit_kernel<ND, SH><<<pblocks(extent), 256, 0, s>>>(g, sp, J);
-        return cudaGetLastError();
+        return launch_chained(deposit_kernel<ND, SH>, pblocks(extent), 256, 0, s, g, sp, J);
     });
 }
 
@@ -2636,12 +2640,12 @@ cudaError_t launch_inject(const GridP& g, const SpeciesP& sp, const int ppc[3], 
             else pyc *= 2;
         }
     }
-    inject_kernel<<<nblocks(nnew + align - 1, 256), 256, 0, s>>>(g, sp, pz, px, py, pxc, pyc, align, nnew, next_id,
-                                                                 status);
-    add_count_kernel<<<1, 1, 0, s>>>(sp.count, nnew, align, sp.cap);
+    cudaError_t e = launch_chained(inject_kernel, nblocks(nnew + align - 1, 256), 256, 0, s, g, sp, pz, px, py, pxc, pyc,
+                                   align, nnew, next_id, status);
+    if (e == cudaSuccess) e = launch_chained(add_count_kernel, 1, 1, 0, s, sp.count, nnew, align, sp.cap);
     const long long ext = (*extent + align - 1) / align * align + nnew;
     *extent = ext < sp.cap ? ext : sp.cap;
-    return cudaGetLastError();
+    return e;
 }
 
 long long sort_bins(const GridP& g) {

@@ -320,7 +320,7 @@ pic_status one_step(pic_t* h, const float* Ein, const float* Bin, float* Eout, f
         if ((st = do_sort(h, s))) return st;
     {
         Scope sc(h, PIC_T_DEPOSIT, 1, s);
-        CK(h, cudaMemsetAsync(h->J, 0, sizeof(float) * 3 * h->g.ncell, s), "zero J");
+        CK(h, launch_zero(h->J, 3 * h->g.ncell, s), "zero J");
     }
     SpeciesP sps[PIC_MAX_SPECIES];
     int* defers[PIC_MAX_SPECIES];
@@ -639,7 +639,7 @@ pic_status pic_deposit(pic_t* h, void* stream) {
     const long long N = h->g.ncell;
     {
         Scope sc(h, PIC_T_DEPOSIT, 1, s);
-        CK(h, cudaMemsetAsync(h->J, 0, sizeof(float) * 3 * N, s), "zero J");
+        CK(h, launch_zero(h->J, 3 * N, s), "zero J");
     }
     for (int i = 0; i < PIC_MAX_SPECIES; ++i) {
         if (!h->sp[i].bound) continue;
@@ -660,8 +660,7 @@ pic_status pic_field_advance(pic_t* h, void* stream) {
     const long long N = h->g.ncell;
     if ((st = advance_fields(h, h->E, h->B, h->E2, h->B2, true, true, s))) return st;
     Scope sc(h, PIC_T_FIELDS, 2, s);
-    CK(h, cudaMemcpyAsync(h->E, h->E2, sizeof(float) * 3 * N, cudaMemcpyDeviceToDevice, s), "copy E");
-    CK(h, cudaMemcpyAsync(h->B, h->B2, sizeof(float) * 3 * N, cudaMemcpyDeviceToDevice, s), "copy B");
+    CK(h, launch_copy2(h->E, h->E2, h->B, h->B2, 3 * N, s), "copy E, B");
     h->state = 0;
     return PIC_OK;
 }
@@ -686,8 +685,7 @@ pic_status pic_step(pic_t* h, int nsteps, void* stream) {
     }
     if (Ec != h->E) {
         Scope sc(h, PIC_T_FIELDS, 2, s);
-        CK(h, cudaMemcpyAsync(h->E, Ec, sizeof(float) * 3 * N, cudaMemcpyDeviceToDevice, s), "copy E");
-        CK(h, cudaMemcpyAsync(h->B, Bc, sizeof(float) * 3 * N, cudaMemcpyDeviceToDevice, s), "copy B");
+        CK(h, launch_copy2(h->E, Ec, h->B, Bc, 3 * N, s), "copy E, B");
     }
     h->state = 0;
     return PIC_OK;
