@@ -34,6 +34,7 @@ struct KSpaceState {
     int solver = 0;
     long long nk = 0;          // modes: (nz/2 + 1) nx ny
     int nzk = 0;
+    bool keep = false;         // buf has the second six
     float2* buf = nullptr;     // in k space: E, B and J, then the scaled E and B that the inverse
                                // transforms consume: 15 nk complex values
     float4* tab = nullptr;     // per axis and index, z then x then y: spectral/KT (d+ re, d+ im,
@@ -70,8 +71,8 @@ __device__ __forceinline__ void ccurl(float2 dz, float2 dx, float2 dy, const flo
 }
 
 // W: the six scaled fields for the inverse transforms; keep: E and B are also wanted in k space
-__global__ void __launch_bounds__(256) kspace_update_kernel(float2* __restrict__ Ek, float2* __restrict__ Bk,
-                                                            const float2* __restrict__ Jk, float2* __restrict__ W, int keep,
+__global__ void __launch_bounds__(256) kspace_update_kernel(float2* Ek, float2* Bk,
+                                                            const float2* __restrict__ Jk, float2* W, int keep,
                                                             const float4* __restrict__ tab, int nzk, int nx,
                                                             long long nk, float dt, float scale) {
     const float4* tz = tab;
@@ -126,8 +127,8 @@ __device__ __forceinline__ float2 ci(float2 a) { return make_float2(-a.y, a.x); 
 __device__ __forceinline__ float2 cscale(float s, float2 a) { return make_float2(s * a.x, s * a.y); }
 __device__ __forceinline__ float2 cadd(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
 
-__global__ void __launch_bounds__(256) psatd_update_kernel(float2* __restrict__ Ek, float2* __restrict__ Bk,
-                                                           const float2* __restrict__ Jk, float2* __restrict__ W, int keep,
+__global__ void __launch_bounds__(256) psatd_update_kernel(float2* Ek, float2* Bk,
+                                                           const float2* __restrict__ Jk, float2* W, int keep,
                                                            const float4* __restrict__ tab, int nzk, int nx,
                                                            long long nk, float dt, float scale) {
     const float4* tz = tab;
@@ -247,8 +248,9 @@ void fill_axis(std::vector<float4>& out, int solver, int axis, int n, double h, 
 
 }  // namespace
 
-int kspace_create(const GridP& g, int solver, double dz, double dx, double dy, double dt, KSpaceState** out,
-                  char* err, size_t nerr) {
+// keep: room for the scaled copies as well (15 nk complex values, 9 without)
+static int kspace_create_with(const GridP& g, int solver, double dz, double dx, double dy, double dt, bool keep,
+                              KSpaceState** out, char* err, size_t nerr) {
     *out = nullptr;
 #ifndef PIC_HAVE_CUFFT
     (void)g; (void)solver; (void)dz; (void)dx; (void)dy; (void)dt;
@@ -258,13 +260,14 @@ int kspace_create(const GridP& g, int solver, double dz, double dx, double dy, d
     KSpaceState* k = new KSpaceState();
     k->g = g;
     k->solver = solver;
+    k->keep = keep;
     k->nzk = g.nz / 2 + 1;
     k->nk = (long long)k->nzk * g.nx * g.ny;
     std::vector<float4> tab;
     fill_axis(tab, solver, 0, g.nz, dz, dt, true, false);
     fill_axis(tab, solver, 1, g.nx, dx, dt, false, false);
     fill_axis(tab, solver, 2, g.ny, dy, dt, false, g.ndim == 2);
-    cudaError_t e = cudaMalloc(&k->buf, sizeof(float2) * 15 * k->nk);
+    cudaError_t e = cudaMalloc(&k->buf, sizeof(float2) * (keep ? 15 : 9) * k->nk);
     if (e == cudaSuccess) e = cudaMalloc(&k->tab, sizeof(float4) * tab.size());
     if (e == cudaSuccess) e = cudaMemcpy(k->tab, tab.data(), sizeof(float4) * tab.size(), cudaMemcpyHostToDevice);
     if (e != cudaSuccess) {
@@ -289,6 +292,15 @@ int kspace_create(const GridP& g, int solver, double dz, double dx, double dy, d
     *out = k;
     return 0;
 #endif
+}
+
+// Where the memory does not reach for the copies, every step transforms the fields anew.
+int kspace_create(const GridP& g, int solver, double dz, double dx, double dy, double dt, KSpaceState** out,
+                  char* err, size_t nerr) {
+    const int r = kspace_create_with(g, solver, dz, dx, dy, dt, true, out, err, nerr);
+    if (r != 2) return r;
+    cudaGetLastError();   // the failed allocation is dealt with here
+    return kspace_create_with(g, solver, dz, dx, dy, dt, false, out, err, nerr);
 }
 
 void kspace_destroy(KSpaceState* k) {
@@ -317,7 +329,10 @@ int kspace_advance(KSpaceState* k, const float* Ein, const float* Bin, const flo
     float2* Ek = k->buf;
     float2* Bk = Ek + 3 * k->nk;
     float2* Jk = Bk + 3 * k->nk;
-    float2* W = Jk + 3 * k->nk;
+    // without room for copies the scaled fields take the place of Ek and Bk, mode by mode
+    float2* W = k->keep ? Jk + 3 * k->nk : Ek;
+    cont = cont && k->keep;
+    keep = keep && k->keep;
     cufftResult r = cufftSetStream(k->r2c, s);
     if (r == CUFFT_SUCCESS) r = cufftSetStream(k->c2r, s);
     if (r == CUFFT_SUCCESS && !cont)
