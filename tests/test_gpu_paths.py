@@ -217,3 +217,29 @@ def test_correction_of_paired_rows(nz):
     assert np.abs(J - osim.J).max() < TOL * np.abs(osim.J).max()
     assert field_error(sim, osim) < TOL
     sim.close()
+
+
+@pytest.mark.parametrize("ndim,nz,nx,ny,filt", [(2, 130, 24, 1, False), (2, 131, 25, 1, True), (2, 4100, 260, 1, False),
+                                                (3, 50, 20, 18, False), (3, 48, 20, 18, True)])
+def test_captured_steps(ndim, nz, nx, ny, filt):
+    """Three steps captured into a CUDA graph by the caller and replayed once (launches chained from
+    kernel to kernel, from the memset of a large J, and into the copies back), against the oracle."""
+    d = (0.5, 0.4, 0.45)[:ndim]
+    C = fit.fit_coefficients(2.5, M=4)
+    grid = dict(ndim=ndim, nz=nz, nx=nx, ny=ny, dz=d[0], dx=d[1], dy=d[2] if ndim == 3 else 1.0,
+                dt=0.8 * fit.cfl_dt(d[0], d[1:], C), solver="custom", shape=2, current_filter=filt)
+    sp = wl.random_particles(ndim, nz, nx, ny, 900, seed=nz, u_scale=0.5, u_drift=(2.0, 0, 0), margin=8)
+    sim, osim = gpu_sim(grid, [sp], coef=C), oracle_sim(grid, [sp], coef=C)
+    sim.step(1)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        sim.step(3)
+    graph.replay()
+    torch.cuda.synchronize()
+    for _ in range(4):
+        osim.step()
+    assert field_error(sim, osim) < TOL
+    dx, du = particle_errors(sim, osim, 0, ndim)
+    assert dx < TOL and du < TOL
+    sim.close()
