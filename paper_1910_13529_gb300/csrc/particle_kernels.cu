@@ -15,6 +15,7 @@
 #include <climits>
 #include <type_traits>
 
+#include "box_fit.h"
 #include "pair_math.h"
 #include "pic_internal.h"
 
@@ -102,6 +103,9 @@ __device__ __forceinline__ int encode(const GridP& g, int iz, int ix, int iy) {
     return (iz + 1) + g.nzg * (ix + g.nx * iy);
 }
 
+// first element of component c: three components of close to 2^31 cells pass 32 bits
+__device__ __forceinline__ size_t comp(uint32_t ncell, int c) { return (size_t)ncell * (uint32_t)c; }
+
 // ---------------------------------------------------------------- gather ----
 // sum_a,b(,c) Wz[a] Wx[b] (Wy[c]) F[row(b, c) + bz + a]; rows are precomputed z-row offsets
 template <int NDIM, int SHAPE>
@@ -155,22 +159,22 @@ __device__ __forceinline__ void gather(const GridP& g, const float* __restrict__
         byn = p.iy + Shape<SHAPE>::w(p.oy, Wyn);
         byh = half_weights<SHAPE>(p.iy, p.oy, Wyh);
     }
-    const int N = (int)g.ncell;
+    const uint32_t N = (uint32_t)g.ncell;
     int rnn[R], rhn[R];            // x node / x half rows, y node
     row_offsets<NDIM, K>(g, bxn, byn, rnn);
     row_offsets<NDIM, K>(g, bxh, byn, rhn);
     eb[0] = interp<NDIM, SHAPE>(g, E, bzh, Wzh, rnn, Wxn, Wyn);
     eb[1] = interp<NDIM, SHAPE>(g, E + N, bzn, Wzn, rhn, Wxh, Wyn);
-    eb[5] = interp<NDIM, SHAPE>(g, B + 2 * N, bzh, Wzh, rhn, Wxh, Wyn);
+    eb[5] = interp<NDIM, SHAPE>(g, B + comp(N, 2), bzh, Wzh, rhn, Wxh, Wyn);
     if (NDIM == 3) {
         int rnh[R], rhh[R];        // y half rows
         row_offsets<NDIM, K>(g, bxn, byh, rnh);
         row_offsets<NDIM, K>(g, bxh, byh, rhh);
-        eb[2] = interp<NDIM, SHAPE>(g, E + 2 * N, bzn, Wzn, rnh, Wxn, Wyh);
+        eb[2] = interp<NDIM, SHAPE>(g, E + comp(N, 2), bzn, Wzn, rnh, Wxn, Wyh);
         eb[3] = interp<NDIM, SHAPE>(g, B, bzn, Wzn, rhh, Wxh, Wyh);
         eb[4] = interp<NDIM, SHAPE>(g, B + N, bzh, Wzh, rnh, Wxn, Wyh);
     } else {
-        eb[2] = interp<NDIM, SHAPE>(g, E + 2 * N, bzn, Wzn, rnn, Wxn, Wyn);
+        eb[2] = interp<NDIM, SHAPE>(g, E + comp(N, 2), bzn, Wzn, rnn, Wxn, Wyn);
         eb[3] = interp<NDIM, SHAPE>(g, B, bzn, Wzn, rhn, Wxh, Wyn);
         eb[4] = interp<NDIM, SHAPE>(g, B + N, bzh, Wzh, rnn, Wxn, Wyn);
     }
@@ -272,7 +276,7 @@ struct GlobalAcc {
     __device__ __forceinline__ void add(int c, int gz, int gx, int gy, float v) const {
         if (gz < 0 || gz >= g->nz) return;
         int o = (wrapi(gy, g->ny) * g->nx + wrapi(gx, g->nx)) * g->nz + gz;
-        atomicAdd(J + c * (int)g->ncell + o, v);
+        atomicAdd(J + comp((uint32_t)g->ncell, c) + o, v);
     }
 };
 // Old-position weights w0 (first node b0) and the new position (i1, o1) -> the deposition
@@ -634,7 +638,7 @@ __device__ __forceinline__ void push_deposit_2d_chunks(const GridP& g, const Spe
     constexpr int KW = K + 1;
     const long long n = *sp.count;
     const long long cap = sp.cap;
-    const int N = (int)g.ncell;
+    const uint32_t N = (uint32_t)g.ncell;
     const bool fvec = (g.nz & 3) == 0 && aligned16(E) && aligned16(B);
     const bool jvec = (g.nz & 3) == 0 && aligned16(J);
     int* const iJ = reinterpret_cast<int*>(sJ);
@@ -701,7 +705,7 @@ __device__ __forceinline__ void push_deposit_2d_chunks(const GridP& g, const Spe
         e.any = bw[0] != INT_MAX;
         e.fz0 = e.any ? (bw[0] & ~3) : 0, e.fx0 = bw[1];
         e.fzl = e.any ? ((1 - bw[2] - e.fz0 + 3) & ~3) : 0, e.fxl = e.any ? 1 - bw[3] - bw[1] : 0;
-        e.ftile = e.any && 6 * e.fzl * e.fxl <= F_CAP && e.fxl <= g.nx + 2 * K;
+        e.ftile = e.any && box_fits<6, F_CAP>(e.fzl, e.fxl) && e.fxl <= g.nx + 2 * K;
         return e;
     };
     // the fields of the next chunk: component c at sF + c fzl fxl, [x][z], zero outside the z range
@@ -714,7 +718,7 @@ __device__ __forceinline__ void push_deposit_2d_chunks(const GridP& g, const Spe
         for (int i = threadIdx.x; i < 3 * rows * ng; i += FUSED_T) {     // the groups of E_c and B_c
             const int r = box_div(i, rg), zg = i - r * ng;
             const int c = box_div(r, rx), x = r - c * rows;
-            const long long row = (long long)c * N + (long long)wrapi(e.fx0 + x, g.nx) * g.nz;
+            const size_t row = comp(N, c) + wrapi(e.fx0 + x, g.nx) * g.nz;
             const float *fe = E + row, *fb = B + row;
             float* d = sF + 4 * i;                   // (c rows + x) fzl + 4 zg
             const int gz = e.fz0 + 4 * zg;
@@ -752,13 +756,13 @@ __device__ __forceinline__ void push_deposit_2d_chunks(const GridP& g, const Spe
         if (more) agree(base + stride * FUSED_T, buf ^ 1, box + nxt * BW2_N);
         const Ext e = extents(bc);
         const bool any = e.any;
-        const int fz0 = e.fz0, fx0 = e.fx0, fzl = e.fzl, fvol = e.fzl * e.fxl;
+        const int fz0 = e.fz0, fx0 = e.fx0, fzl = e.fzl, fvol = e.ftile ? e.fzl * e.fxl : 0;
         // current box: every deposition window starts at most one node below the gather stencils and
         // its K + 1 nodes end at most one node above them (the move is under one cell per axis)
         const int jz0 = any ? ((bc[0] - 1) & ~3) : 0, jx0 = fx0 - 1;
         const int jzl = any ? ((2 - bc[2] - jz0 + 3) & ~3) : 0, jxl = any ? e.fxl + 2 : 0;
-        const int jvol = jzl * jxl;
-        const bool jtile = any && 3 * jvol <= J_CAP && jxl <= g.nx + 2 * KW;
+        const bool jtile = any && box_fits<3, J_CAP>(jzl, jxl) && jxl <= g.nx + 2 * KW;
+        const int jvol = jtile ? jzl * jxl : 0;
         // the flush clears what a chunk used: only the first chunk and a larger box clear anything here
         if (jtile && 3 * (jvol >> 2) > clear) {
             for (int i = clear + threadIdx.x; i < 3 * (jvol >> 2); i += FUSED_T)
@@ -961,7 +965,7 @@ __device__ __forceinline__ void push_deposit_2d_chunks(const GridP& g, const Spe
                     float v;
                     if (a < KW - 1 && (v = f1 * cz[a] * tx) != 0.f) atomicAdd(d, v);
                     if (b < KW - 1 && (v = (S0z[a] + 0.5f * DSz[a]) * f2 * cx[b]) != 0.f) atomicAdd(d + N, v);
-                    if ((v = fmaf(S0z[a], ax, DSz[a] * bxv)) != 0.f) atomicAdd(d + 2 * N, v);
+                    if ((v = fmaf(S0z[a], ax, DSz[a] * bxv)) != 0.f) atomicAdd(d + comp(N, 2), v);
                 }
             }
         }
@@ -981,7 +985,7 @@ __device__ __forceinline__ void push_deposit_2d_chunks(const GridP& g, const Spe
                 const int r = box_div(i, rg), zg = i - r * ng;
                 const int c = box_div(r, rx), x = r - c * jxl;
                 const int gz = jz0 + 4 * zg;
-                float* dst = J + c * N + wrapi(jx0 + x, g.nx) * g.nz + gz;
+                float* dst = J + comp(N, c) + wrapi(jx0 + x, g.nx) * g.nz + gz;
                 if (jvec && gz >= 0 && gz + 3 < g.nz) {
                     atomicAdd(reinterpret_cast<float4*>(dst), v);
                 } else {
@@ -1150,7 +1154,7 @@ __device__ __forceinline__ void push_deposit_3d_chunks(const GridP& g, const Spe
     constexpr int KW = K + 1;
     const long long n = *sp.count;
     const long long cap = sp.cap;
-    const int N = (int)g.ncell;
+    const uint32_t N = (uint32_t)g.ncell;
     const bool fvec = (g.nz & 3) == 0 && aligned16(E) && aligned16(B);
     const bool jvec = (g.nz & 3) == 0 && aligned16(J);
     int* const iJ = reinterpret_cast<int*>(sJ);
@@ -1241,7 +1245,7 @@ __device__ __forceinline__ void push_deposit_3d_chunks(const GridP& g, const Spe
     auto stage = [&](const Ext& e) {
         staged(e, [&](int c, int x, int y, int zg) {
             const long long row = ((long long)wrapi(e.fy0 + y, g.ny) * g.nx + wrapi(e.fx0 + x, g.nx)) * g.nz;
-            const float* f = (c < 3 ? E + c * N : B + (c - 3) * N) + row;
+            const float* f = (c < 3 ? E + comp(N, c) : B + comp(N, c - 3)) + row;
             float* d = sF + c * FV3 + (y * FX3 + x) * FZP3 + 4 * zg;
             const int gz = e.fz0 + 4 * zg;
             if (fvec) {
@@ -1309,8 +1313,9 @@ __device__ __forceinline__ void push_deposit_3d_chunks(const GridP& g, const Spe
             // boxes the general path holds in shared memory (its own rounding of the z extents) go to
             // its list, the rest to the per-particle one
             const int gfz = (e.fzl + 3) & ~3, gjz = (jzl + 3) & ~3;
-            const bool general = 6 * gfz * e.fxl * e.fyl <= F_CAP3 && e.fxl <= g.nx + 2 * K && e.fyl <= g.ny + 2 * K &&
-                                 3 * gjz * jxl * jyl <= J_CAP3 && jxl <= g.nx + 2 * KW && jyl <= g.ny + 2 * KW;
+            const bool general = box_fits<6, F_CAP3>(gfz, e.fxl, e.fyl) && e.fxl <= g.nx + 2 * K &&
+                                 e.fyl <= g.ny + 2 * K && box_fits<3, J_CAP3>(gjz, jxl, jyl) && jxl <= g.nx + 2 * KW &&
+                                 jyl <= g.ny + 2 * KW;
             int* list = general ? defer : defer2;
             list[2 + atomicAdd(list, 1)] = (int)(base / FUSED_T);
         }
@@ -1550,7 +1555,7 @@ __device__ __forceinline__ void push_deposit_3d_chunks(const GridP& g, const Spe
                 const float4 v = make_float4((float)q.x * inv_s, (float)q.y * inv_s, (float)q.z * inv_s,
                                              (float)q.w * inv_s);
                 const int gz = jz0 + 4 * zg;
-                float* dst = J + c * N + (wrapi(jy0 + y, g.ny) * g.nx + wrapi(jx0 + x, g.nx)) * g.nz + gz;
+                float* dst = J + comp(N, c) + (wrapi(jy0 + y, g.ny) * g.nx + wrapi(jx0 + x, g.nx)) * g.nz + gz;
                 if (jvec && gz >= 0 && gz + 3 < g.nz) {
                     atomicAdd(reinterpret_cast<float4*>(dst), v);
                 } else {
@@ -1622,7 +1627,7 @@ __device__ __forceinline__ void push_deposit_3d_general(const GridP& g, const Sp
     constexpr int KW = K + 1;
     const long long n = *sp.count;
     const long long cap = sp.cap;
-    const int N = (int)g.ncell;
+    const uint32_t N = (uint32_t)g.ncell;
     const bool fvec = (g.nz & 3) == 0 && aligned16(E) && aligned16(B);
     const bool jvec = (g.nz & 3) == 0 && aligned16(J);
     float* const pfb = sJ + J_CAP3;                   // [2][PF3][FUSED_T]
@@ -1708,13 +1713,13 @@ __device__ __forceinline__ void push_deposit_3d_general(const GridP& g, const Sp
         const int fz0 = any ? (bc[0] & ~3) : 0, fx0 = bc[2], fy0 = bc[4];
         const int fzl = any ? ((bc[1] + 1 - fz0 + 3) & ~3) : 0;
         const int fxl = any ? bc[3] - bc[2] + 1 : 0, fyl = any ? bc[5] - bc[4] + 1 : 0;
-        const int fvol = fzl * fxl * fyl;
-        const bool ftile = any && 6 * fvol <= F_CAP3 && fxl <= g.nx + 2 * K && fyl <= g.ny + 2 * K;
+        const bool ftile = any && box_fits<6, F_CAP3>(fzl, fxl, fyl) && fxl <= g.nx + 2 * K && fyl <= g.ny + 2 * K;
+        const int fvol = ftile ? fzl * fxl * fyl : 0;
         const int jz0 = any ? ((bc[0] - 1) & ~3) : 0, jx0 = bc[2] - 1, jy0 = bc[4] - 1;
         const int jzl = any ? ((bc[1] + 2 - jz0 + 3) & ~3) : 0;
         const int jxl = any ? bc[3] - bc[2] + 3 : 0, jyl = any ? bc[5] - bc[4] + 3 : 0;
-        const int jvol = jzl * jxl * jyl;
-        const bool jtile = any && 3 * jvol <= J_CAP3 && jxl <= g.nx + 2 * KW && jyl <= g.ny + 2 * KW;
+        const bool jtile = any && box_fits<3, J_CAP3>(jzl, jxl, jyl) && jxl <= g.nx + 2 * KW && jyl <= g.ny + 2 * KW;
+        const int jvol = jtile ? jzl * jxl * jyl : 0;
         // groups (c, y, x, z4) of the [c][y][x][z] box, copied asynchronously (all of a thread's
         // groups in flight at once); z groups start at multiples of 4, so with nz % 4 == 0 a group
         // lies wholly inside or wholly outside 0 <= z < nz
@@ -1731,7 +1736,7 @@ __device__ __forceinline__ void push_deposit_3d_general(const GridP& g, const Sp
             staged([&](int c, int q, int zg) {
                 const int y = box_div(q, rx), x = q - y * fxl;
                 const long long row = ((long long)wrapi(fy0 + y, g.ny) * g.nx + wrapi(fx0 + x, g.nx)) * g.nz;
-                const float* f = (c < 3 ? E + c * N : B + (c - 3) * N) + row;
+                const float* f = (c < 3 ? E + comp(N, c) : B + comp(N, c - 3)) + row;
                 float* d = sF + c * fvol + q * fzl + 4 * zg;
                 const int gz = fz0 + 4 * zg;
                 if (fvec) {
@@ -1900,7 +1905,7 @@ __device__ __forceinline__ void push_deposit_3d_general(const GridP& g, const Sp
                 const int c = box_div(r, rr), qq = r - c * rows;
                 const int y = box_div(qq, rx), x = qq - y * jxl;
                 const int gz = jz0 + 4 * zg;
-                float* dst = J + c * N + (wrapi(jy0 + y, g.ny) * g.nx + wrapi(jx0 + x, g.nx)) * g.nz + gz;
+                float* dst = J + comp(N, c) + (wrapi(jy0 + y, g.ny) * g.nx + wrapi(jx0 + x, g.nx)) * g.nz + gz;
                 if (jvec && gz >= 0 && gz + 3 < g.nz) {
                     atomicAdd(reinterpret_cast<float4*>(dst), v);
                 } else {
