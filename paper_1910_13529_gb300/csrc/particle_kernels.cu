@@ -1920,14 +1920,15 @@ __device__ __forceinline__ void push_deposit_3d_general(const GridP& g, const Sp
     cp_async_wait_all_p();                         // the last (empty) prefetch group
 }
 
-// Everything push_deposit_3d_kernel left, of all species, in one launch: defer[s][2 ..] holds the
-// chunks for the general path (count in defer[s][0]), defer2[s][2 ..] those whose boxes are beyond it
-// (a chunk of particles that crossed the periodic seam since the last sort).  The latter go per
-// particle (gather from global memory, global atomics, exact zeros not added) in units of one warp,
-// dealt to the CTAs in turn: a warp's scattered atomics pass through its SM one lane at a time, so a
-// chunk's eight warps on eight SMs finish in an eighth of the time of one CTA.  One launch for all
-// species: the few chunks of one species run beside those of the others.
-// The last CTA to finish clears the lists (defer[0][1] counts finished CTAs).
+// What push_deposit_3d_kernel left on the lists of all species: defer[s][2 ..] holds the chunks for the
+// general path (count in defer[s][0]), defer2[s][2 ..] those whose boxes are beyond it (particles that
+// crossed the periodic seam or have not been sorted for a while).  One launch per kind for all species:
+// the few chunks of one species run beside those of the others.  Two launches, because the first kind
+// wants shared memory and the second the L1 cache that it leaves.  With 28 KB of L1, as the tail of the
+// general kernel or behind it under its split, the per-particle path took more than twice as long: 1e6 unsorted
+// particles on 128 x 64 x 64 726 us a step (linear) and 2270 (quadratic), 312 and 870 now; 8.4e6 on
+// 256 x 128 x 128 11.8 and 32.2 ms, 4.0 and 9.6 now.
+// The last CTA of each to finish clears its lists (word 1 of the first species' list counts).
 template <int SHAPE>
 __global__ void __launch_bounds__(FUSED_T, 2) push_deposit_3d_leftover_kernel(GridP g, LeftoverP lp,
                                                                               const float* __restrict__ E,
@@ -1949,16 +1950,39 @@ __global__ void __launch_bounds__(FUSED_T, 2) push_deposit_3d_leftover_kernel(Gr
         first = (first + nd) % grid;
         __syncthreads();
     }
-    const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    int item = wid * grid + ((int)blockIdx.x >= first ? (int)blockIdx.x - first : (int)blockIdx.x - first + grid);
+    if (threadIdx.x == 0) {
+        __threadfence();
+        if (atomicAdd(lp.defer[0] + 1, 1) == grid - 1) {
+            for (int s = 0; s < lp.n; ++s) lp.defer[s][0] = 0;
+            lp.defer[0][1] = 0;
+            __threadfence();
+        }
+    }
+}
+
+// Per particle: gather from global memory, global atomics, exact zeros not added.  Few chunks go in units of
+// one warp, dealt to the CTAs in turn: a warp's scattered atomics pass through its SM one lane at a time, so a
+// chunk's eight warps on eight SMs finish in an eighth of the time of one CTA.  Many go one to a CTA,
+// whose warps find one another's fields in L1.
+template <int SHAPE>
+__global__ void __launch_bounds__(FUSED_T, 2) push_deposit_3d_particles_kernel(GridP g, LeftoverP lp,
+                                                                               const float* __restrict__ E,
+                                                                               const float* __restrict__ B,
+                                                                               float* __restrict__ J, int shift) {
+    chain_enter();
+    constexpr int WARPS = FUSED_T / 32;
+    const int grid = (int)gridDim.x, wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    int chunks = 0;
+#pragma unroll 1
+    for (int s = 0; s < lp.n; ++s) chunks += *(volatile int*)lp.defer2[s];
+    int item = chunks >= grid ? (int)blockIdx.x * WARPS + wid : wid * grid + (int)blockIdx.x;
 #pragma unroll 1
     for (int s = 0; s < lp.n; ++s) {
         const SpeciesP& sp = lp.sp[s];
-        const int nw = *(volatile int*)lp.defer2[s] * (FUSED_T / 32);
+        const int nw = *(volatile int*)lp.defer2[s] * WARPS;
         const long long n = *sp.count;
-        for (; item < nw; item += grid * (FUSED_T / 32)) {
-            const long long p =
-                (long long)lp.defer2[s][2 + item / (FUSED_T / 32)] * FUSED_T + (item % (FUSED_T / 32)) * 32 + lane;
+        for (; item < nw; item += grid * WARPS) {
+            const long long p = (long long)lp.defer2[s][2 + item / WARPS] * FUSED_T + (item % WARPS) * 32 + lane;
             Pos p0, p1;
             float v3;
             if (p < n && advance_one<3, SHAPE, MODE_FUSED>(g, sp, E, B, shift, p, sp.cap, p0, p1, v3)) {
@@ -1971,9 +1995,9 @@ __global__ void __launch_bounds__(FUSED_T, 2) push_deposit_3d_leftover_kernel(Gr
     __syncthreads();
     if (threadIdx.x == 0) {
         __threadfence();
-        if (atomicAdd(lp.defer[0] + 1, 1) == grid - 1) {
-            for (int s = 0; s < lp.n; ++s) lp.defer[s][0] = lp.defer2[s][0] = 0;
-            lp.defer[0][1] = 0;
+        if (atomicAdd(lp.defer2[0] + 1, 1) == grid - 1) {
+            for (int s = 0; s < lp.n; ++s) lp.defer2[s][0] = 0;
+            lp.defer2[0][1] = 0;
             __threadfence();
         }
     }
@@ -2570,9 +2594,12 @@ cudaError_t launch_push_leftover(const GridP& g0, const SpeciesP* sp, int* const
             if (e != cudaSuccess) return e;
             configured = true;
         }
-        // the lists' lengths are on the device: a full grid, or one CTA per warp of a small extent
+        // the lists' lengths are on the device: full grids, or one CTA per chunk and per warp of a small extent
         const long long want = nchunk * (FUSED_T / 32);
-        return launch_chained(k, (unsigned)(want < 152 * 2 ? want : 152 * 2), FUSED_T, smem, s, g, lp, E, B, J, shift);
+        cudaError_t e = launch_chained(k, (unsigned)(nchunk < 152 * 2 ? nchunk : 152 * 2), FUSED_T, smem, s, g, lp, E, B, J, shift);
+        if (e != cudaSuccess) return e;
+        return launch_split(true, 0, push_deposit_3d_particles_kernel<decltype(sh)::value>,
+                            (unsigned)(want < 152 * 4 ? want : 152 * 4), FUSED_T, 0, s, g, lp, E, B, J, shift);
     });
 }
 

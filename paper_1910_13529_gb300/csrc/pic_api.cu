@@ -344,9 +344,9 @@ pic_status one_step(pic_t* h, const float* Ein, const float* Bin, float* Eout, f
            "fused push/deposit kernel");
     }
     if (h->cfg.ndim == 3 && nsp > 0) {
-        Scope sc(h, PIC_T_PARTICLES, 1, s);
+        Scope sc(h, PIC_T_PARTICLES, 2, s);
         CK(h, launch_push_leftover(h->g, sps, defers, extents, nsp, Ein, Bin, h->J, h->pending_shift, s),
-           "deferred chunks kernel");
+           "deferred chunks kernels");
     }
     h->pending_shift = 0;
     if ((st = smooth_current(h, s))) return st;

@@ -129,19 +129,31 @@ __device__ __forceinline__ void chain_enter() {
     asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
     asm volatile("griddepcontrol.wait;\n" ::: "memory");
 }
+// A chained kernel starts with the split between shared memory and L1 that the one before it left, unless it asks
+// for another: carveout, percent of the shared memory that an SM can give; -1 asks for nothing.
 template <typename... P, typename... A>
-cudaError_t launch_chained_if(bool chain, void (*k)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A&&... args) {
+cudaError_t launch_split(bool chain, int carveout, void (*k)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                         A&&... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = block;
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
-    cudaLaunchAttribute attr;
-    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr.val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = &attr;
-    cfg.numAttrs = chain ? 1 : 0;
+    cudaLaunchAttribute attr[2];
+    if (chain) {
+        attr[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[cfg.numAttrs++].val.programmaticStreamSerializationAllowed = 1;
+    }
+    if (carveout >= 0) {
+        attr[cfg.numAttrs].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+        attr[cfg.numAttrs++].val.sharedMemCarveout = (unsigned)carveout;
+    }
+    cfg.attrs = attr;
     return cudaLaunchKernelEx(&cfg, k, static_cast<A&&>(args)...);
+}
+template <typename... P, typename... A>
+cudaError_t launch_chained_if(bool chain, void (*k)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A&&... args) {
+    return launch_split(chain, -1, k, grid, block, smem, s, static_cast<A&&>(args)...);
 }
 template <typename... P, typename... A>
 cudaError_t launch_chained(void (*k)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A&&... args) {

@@ -1,0 +1,48 @@
+"""Cost of one input relative to another through the same call, where a route once cost several times what its work
+does.  Ratios of medians on one device with wide margins: no absolute times."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():
+    pytest.skip("no CUDA device", allow_module_level=True)
+
+from paper_1910_13529_gb300 import workloads as wl  # noqa: E402
+from paper_1910_13529_gb300.runtime import Simulation  # noqa: E402
+
+
+def median_ms(f, reps=9):
+    for _ in range(3):
+        f()
+    ts = []
+    for _ in range(reps):
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        a.record()
+        f()
+        b.record()
+        torch.cuda.synchronize()
+        ts.append(a.elapsed_time(b))
+    return float(np.median(ts))
+
+
+def slow_particles(ndim, nz, nx, ny, n, seed=1):
+    """In no order, slow enough to keep the order that a sort gives them."""
+    return wl.random_particles(ndim, nz, nx, ny, n, seed=seed, u_scale=1e-3, margin=4)
+
+
+def add(sim, sp):
+    sim.add_species(0, sp["iz"], sp["ix"], sp["iy"], sp["off"], sp["u"], sp["q"], sp["m"], sp["w"])
+
+
+@pytest.mark.parametrize("shape", [1, 2])
+def test_unsorted_particles_3d(shape):
+    """A step that gathers and deposits per particle (nothing sorted) against one whose chunks fit their boxes: 2.2 to
+    4.7 times as long, 5.9 to 11 when the per-particle path had hardly any L1."""
+    sim = Simulation(ndim=3, nz=128, nx=64, ny=64, dz=0.05, dx=0.05, dy=0.05, dt=0.025, shape=shape)
+    add(sim, slow_particles(3, 128, 64, 64, 1 << 20))
+    unsorted = median_ms(lambda: sim.step(1))
+    sim.sort()
+    assert unsorted < (4.2 if shape == 1 else 7.5) * median_ms(lambda: sim.step(1))
+    sim.close()
