@@ -514,8 +514,11 @@ struct Never {
 // Bound by instruction issue (77% of the slots at 47% of the warps, 64 registers).  Six barriers per
 // chunk and exposed loads before, three barriers now: 2048 x 512, 5.2e6 particles, quadratic, wake state,
 // 268 us per step before, 242 us now; 1001 x 237 linear 49.4 and 48.4 us.
-// Boxes larger than the shared-memory caps fall back to global loads / global atomics.
-constexpr int F_CAP = 6 * 1024;    // field box floats (6 components)
+// Boxes larger than the shared-memory caps fall back to global loads / global atomics.  That path (runs without
+// sorts, sparse species, every batch) lives on L1: with 48 KB per CTA the four of an SM left it 28 KB, and a batch of
+// 16 x 256 x 128 cells, 4 per cell, unsorted, took 692 us a step (linear) and 1651 (quadratic); at 41 KB, 270 and
+// 690.  2048 x 512, 4.2e6 unsorted: 776 and 473 us (linear), 1658 and 1060 (quadratic).  Sorted: 157 and 162, 208 and 208.
+constexpr int F_CAP = 4032;        // field box floats (6 components): four CTAs leave 92 KB of L1 to an SM
 constexpr int J_CAP = 3 * 1024;    // current box floats (3 components)
 constexpr int PF2 = 6;             // prefetched words per particle (cell, 2 offsets, 3 momenta)
 constexpr int SMEM_2D = F_CAP + J_CAP + 2 * PF2 * FUSED_T;
@@ -628,6 +631,13 @@ __device__ __forceinline__ float4 load_group(const float* __restrict__ row, int 
 }
 
 __device__ __forceinline__ bool aligned16(const void* q) { return ((uintptr_t)q & 15) == 0; }
+
+// Out of line: inlined, its registers made the whole kernel spill.
+template <int SHAPE>
+__device__ __noinline__ void gather2_global(const GridP g, const float* __restrict__ E, const float* __restrict__ B,
+                                            const Pos p0, float* eb) {
+    gather<2, SHAPE>(g, E, B, p0, eb);
+}
 
 template <int SHAPE>
 __device__ __forceinline__ void push_deposit_2d_chunks(const GridP& g, const SpeciesP& sp,
@@ -806,7 +816,7 @@ __device__ __forceinline__ void push_deposit_2d_chunks(const GridP& g, const Spe
                 eb[2] = q3.x;
                 eb[5] = q3.y;
             } else {
-                gather<2, SHAPE>(g, E, B, p0, eb);
+                gather2_global<SHAPE>(g, E, B, p0, eb);
             }
         }
         // ---- push and move ----
@@ -2542,14 +2552,15 @@ cudaError_t launch_push(const GridP& g0, const SpeciesP& sp, const float* E, con
         constexpr int ND = decltype(nd)::value, SH = decltype(sh)::value;
         if (mode == MODE_FUSED && ND == 2) {
             auto k = push_deposit_2d_kernel<SH>;
-            const size_t smem = SMEM_2D * sizeof(float);
-            static bool configured = false;
-            if (!configured) {
+            const unsigned ctas = pblocks(extent);
+            const size_t smem = spread_shared(ctas, SMEM_2D * sizeof(float));
+            static size_t granted = 0;
+            if (smem > granted) {
                 cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
                 if (e != cudaSuccess) return e;
-                configured = true;
+                granted = smem;
             }
-            return launch_chained(k, pblocks(extent), FUSED_T, smem, s, g, sp, E, B, J, shift);
+            return launch_split(true, STEP_CARVEOUT, k, ctas, FUSED_T, smem, s, g, sp, E, B, J, shift);
         } else if (mode == MODE_FUSED) {
             const size_t smem = SMEM_3D * sizeof(float);
             CUtensorMap mapE{}, mapB{};

@@ -130,7 +130,25 @@ __device__ __forceinline__ void chain_enter() {
     asm volatile("griddepcontrol.wait;\n" ::: "memory");
 }
 // A chained kernel starts with the split between shared memory and L1 that the one before it left, unless it asks
-// for another: carveout, percent of the shared memory that an SM can give; -1 asks for nothing.
+// for another, and where the split changes the device runs empty first.  So the kernels of a 2D step
+// ask for one split, 164 KB of shared memory and 92 KB of L1: what the particle kernel's four CTAs need, with
+// the L1 of its path for unsorted particles.  Left to the driver (field kernels 228 KB): 2048 x 512 with
+// 1000 scattered particles 45 us a step, 34 now; 511 x 255 with 524288 sorted ones 37 and 32.  Only a kernel
+// whose grid fits the device at once under that split asks (in_step): it loses nothing.
+constexpr int STEP_CARVEOUT = 71;                    // percent of 228 KB, rounded down to the next split
+constexpr size_t STEP_SHARED = 164 * 1024, CTA_RESERVED = 2 * 1024;
+inline int in_step(dim3 grid, size_t smem) {
+    const unsigned long long ctas = (unsigned long long)grid.x * grid.y * grid.z;
+    return smem > 0 && ctas <= 152ull * (STEP_SHARED / (smem + CTA_RESERVED)) ? STEP_CARVEOUT : -1;
+}
+// Dynamic shared memory that spreads a grid of less than a wave evenly over the SMs: the CTAs of a chained kernel
+// settle on the SMs that the kernel before it leaves first, as many as fit there (2048 x 512, 20000 scattered
+// particles, quadratic: 61 us a step, 33 with one CTA per SM).
+inline size_t spread_shared(unsigned ctas, size_t smem) {
+    const size_t share = STEP_SHARED / ((ctas + 151) / 152) - CTA_RESERVED;
+    return share > smem ? share : smem;
+}
+// carveout: percent of the shared memory that an SM can give; -1 asks for nothing
 template <typename... P, typename... A>
 cudaError_t launch_split(bool chain, int carveout, void (*k)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
                          A&&... args) {
@@ -153,7 +171,7 @@ cudaError_t launch_split(bool chain, int carveout, void (*k)(P...), dim3 grid, d
 }
 template <typename... P, typename... A>
 cudaError_t launch_chained_if(bool chain, void (*k)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A&&... args) {
-    return launch_split(chain, -1, k, grid, block, smem, s, static_cast<A&&>(args)...);
+    return launch_split(chain, chain ? in_step(grid, smem) : -1, k, grid, block, smem, s, static_cast<A&&>(args)...);
 }
 template <typename... P, typename... A>
 cudaError_t launch_chained(void (*k)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A&&... args) {
