@@ -1312,6 +1312,11 @@ __global__ void __launch_bounds__(256, 2) field_advance_rb_batch_kernel(const Fi
     advance_tile_rb<NDIM, MAXM, TZ, TX, TY>(sp, it.y, it.z, it.w, reinterpret_cast<float*>(smem4));
 }
 
+// 3D field kernels are launched plainly: behind the particle kernels the early blocks pile up on the SMs that
+// end first (a step of 1e6 particles on 127 x 63 x 65 cells: 170 us chained, 145 us not; 1.3e5 on 65 x 33 x
+// 31: 90 and 75 us; one particle on 128 x 64 x 64: 38.9 and 39.1 us).
+inline bool chain_fields(const GridP& g) { return g.ndim == 2 && few_cells(g); }
+
 template <int NDIM, int MAXM, int TZ, int TX, int TY>
 cudaError_t launch_fa(const FieldP& p, cudaStream_t s) {
     using T = Tile<NDIM, MAXM, TZ, TX, TY>;
@@ -1324,7 +1329,7 @@ cudaError_t launch_fa(const FieldP& p, cudaStream_t s) {
         configured = true;
     }
     dim3 grid((p.g.nz + TZ - 1) / TZ, (p.g.nx + TX - 1) / TX, NDIM == 3 ? (p.g.ny + TY - 1) / TY : 1);
-    return launch_chained_if(few_cells(p.g), k, grid, 256, T::smem_bytes, s, p);
+    return launch_chained_if(chain_fields(p.g), k, grid, 256, T::smem_bytes, s, p);
 }
 
 template <int NDIM, int MAXM, int TZ, int TX, int TY>
@@ -1339,7 +1344,7 @@ cudaError_t launch_fa_rb(const FieldP& p, cudaStream_t s) {
         configured = true;
     }
     dim3 grid((p.g.nz + TZ - 1) / TZ, (p.g.nx + TX - 1) / TX, NDIM == 3 ? (p.g.ny + TY - 1) / TY : 1);
-    return launch_chained_if(few_cells(p.g), k, grid, 256, T::smem_bytes, s, p);
+    return launch_chained_if(chain_fields(p.g), k, grid, 256, T::smem_bytes, s, p);
 }
 
 // Rows (2D) or planes (3D) per marching chunk: the chunk count that minimises the number of waves
@@ -1380,7 +1385,7 @@ cudaError_t launch_fa_march(const FieldP& p, cudaStream_t s) {
     per_sm = per_sm < 1 ? 1 : (per_sm > 2048 / NT ? 2048 / NT : per_sm);
     const int yc = march_chunk(p.g.ny, cols, nsm * per_sm, 8);
     dim3 grid((p.g.nz + TZ - 1) / TZ, (p.g.nx + TX - 1) / TX, (p.g.ny + yc - 1) / yc);
-    return launch_chained_if(few_cells(p.g), k, grid, NT, T::smem_bytes, s, p, yc);
+    return launch_chained_if(chain_fields(p.g), k, grid, NT, T::smem_bytes, s, p, yc);
 }
 
 // CTAs of k that one SM holds (k already has its shared-memory limit), once per kernel
@@ -1412,7 +1417,7 @@ cudaError_t launch_fa_rows_v(const FieldP& p, cudaStream_t s) {
     const int nseg = (p.g.nz + T::OUT - 1) / T::OUT, tz = row_segment(p.g.nz, nseg);
     const int cols = (p.g.nz + tz - 1) / tz;
     const int xc = march_chunk(p.g.nx, cols, sm_count() * per_sm, 8);
-    return launch_chained_if(few_cells(p.g), k, dim3(cols, (p.g.nx + xc - 1) / xc, 1), NT, T::smem_bytes, s, p, tz, xc);
+    return launch_chained_if(chain_fields(p.g), k, dim3(cols, (p.g.nx + xc - 1) / xc, 1), NT, T::smem_bytes, s, p, tz, xc);
 }
 
 template <int MAXM, int NT>
@@ -1439,7 +1444,7 @@ cudaError_t launch_fa_march_ring(const FieldP& p, cudaStream_t s) {
     per_sm = per_sm < 1 ? 1 : (per_sm > 2048 / NT ? 2048 / NT : per_sm);
     const int yc = march_chunk(p.g.ny, cols, nsm * per_sm, 8);
     dim3 grid((p.g.nz + TZ - 1) / TZ, (p.g.nx + TX - 1) / TX, (p.g.ny + yc - 1) / yc);
-    return launch_chained_if(few_cells(p.g), k, grid, NT, T::smem_bytes, s, p, yc);
+    return launch_chained_if(chain_fields(p.g), k, grid, NT, T::smem_bytes, s, p, yc);
 }
 
 template <int NDIM, int MAXM, int TZ, int TX, int TY>

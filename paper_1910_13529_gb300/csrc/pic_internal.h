@@ -121,9 +121,10 @@ enum : int { STATUS_CAPACITY = 1, STATUS_TIMEOUT = 2 };
 // that is launched so) until that one has completed and its writes are visible: 1 to 2 us less between
 // two kernels, which is what steps of small grids consist of (256 x 128 cells, one particle: a step 24.2
 // -> 11.8 us; the separate phases at 1024 x 256: 106 -> 96 us; the gradient of 500 steps there: 42.8 ->
-// 36.8 ms).  Field and current kernels over more than CHAIN_CELLS cells are launched plainly: there the
-// blocks of the early kernel settle where the other ends first instead of evenly (8192 x 2048, M = 16,
-// four steps: 1166 us chained, 1148 us not; 2048 x 512 still gains, 2860 -> 2790 us for eight steps).
+// 36.8 ms).  Field and current kernels over more than CHAIN_CELLS cells, and 3D field kernels, are launched
+// plainly: there the blocks of the early kernel settle where the other ends first instead of evenly (8192 x
+// 2048, M = 16, four steps: 1166 us chained, 1148 us not; 2048 x 512 still gains, 2860 -> 2790 us for eight
+// steps).
 constexpr long long CHAIN_CELLS = 1 << 20;
 __device__ __forceinline__ void chain_enter() {
     asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
