@@ -1349,10 +1349,11 @@ cudaError_t launch_fa_rb(const FieldP& p, cudaStream_t s) {
 
 // Rows (2D) or planes (3D) per marching chunk: the chunk count that minimises the number of waves
 // times the rows a CTA walks (its chunk plus the two its prologue recomputes), chunks of at least
-// `minc` rows.  `cols` CTAs march side by side; `slots` CTAs run at once.
+// `minc` rows.  `cols` CTAs march side by side; `slots` CTAs run at once.  Tried: 1 to 64 chunks and those
+// that fill 1 to 8 waves (few columns of many rows: 128 x 16384 cells are one column).
 inline int march_chunk(int n, int cols, int slots, int minc) {
     int best = n, best_cost = INT_MAX;
-    for (int chunks = 1; chunks <= 64; ++chunks) {
+    auto look = [&](int chunks) {
         int c = (n + chunks - 1) / chunks;
         if (c < minc) c = minc;
         const long long ctas = (long long)cols * ((n + c - 1) / c);
@@ -1362,7 +1363,10 @@ inline int march_chunk(int n, int cols, int slots, int minc) {
             best_cost = (int)cost;
             best = c;
         }
-    }
+    };
+    for (int chunks = 1; chunks <= 64; ++chunks) look(chunks);
+    for (int waves = 1; waves <= 8; ++waves)
+        if (waves * slots / cols > 64) look(waves * slots / cols);
     return best;
 }
 
@@ -1657,7 +1661,9 @@ int field_variants(int ndim) { return ndim == 2 ? 12 : 12; }
 //   3D: the y-march, up to M = 8 128 x 4 (Yee 512 x 256 x 256: a 1527, b 597; 251 x 120 x 117: a 182, b 119;
 //   M = 8: a 718, b 670), for M = 16 the prefetch ring 128 x 8 (862, next best 1066).
 //   2D from 2e6 cells: the x-march with 64 threads (4096 x 1024 Yee: a 76, b 48; M = 16: a 86, b 64; 4099 x
-//   1030 M = 16: a 145, b 91), but not Yee on rows that are not 16-byte aligned (74 against 72).
+//   1030 M = 16: a 145, b 91), but not Yee on rows that are not 16-byte aligned (74 against 72), and not on short
+//   rows, which leave most of a segment's 464 or 416 cells idle (128 x 16384 Yee and M = 16: x-march 53 and 87,
+//   128 x 8 35 and 47; 256 x 8192: 35 and 52, 35 and 48; 320 x 6400: 32 and 44, 36 and 53).
 //   2D below: rows not 16-byte aligned want the one-cell tiles up to M = 4 (1501 x 700 Yee: 64 x 16 16.8,
 //   128 x 8 18.8, register-blocked 30; M = 4: 22.9 and 31) and the register-blocked ones above; aligned
 //   rows the register-blocked 128 x 8, on fewer than 1.3e5 cells 128 x 4 (256 x 128 Yee: a 8.7, b 5), and
@@ -1665,7 +1671,7 @@ int field_variants(int ndim) { return ndim == 2 ? 12 : 12; }
 int default_field_variant(const GridP& g, int M) {
     if (g.ndim == 3) return M <= 8 ? 6 : 10;
     const bool aligned = g.nz % 4 == 0, yee = M <= 1;
-    if (g.ncell >= 2000000 && (aligned || !yee)) return 11;
+    if (g.ncell >= 2000000 && g.nz >= 256 && (aligned || !yee)) return 11;
     if (!aligned) return yee ? 2 : M <= 4 ? 0 : 4;
     if (g.ncell < 130000) return 6;
     return yee && g.ncell >= 500000 ? 2 : 4;

@@ -9,6 +9,7 @@ torch = pytest.importorskip("torch")
 if not torch.cuda.is_available():
     pytest.skip("no CUDA device", allow_module_level=True)
 
+from oracle import fit  # noqa: E402
 from paper_1910_13529_gb300 import workloads as wl  # noqa: E402
 from paper_1910_13529_gb300.runtime import Batch, Simulation  # noqa: E402
 
@@ -66,3 +67,16 @@ def test_unsorted_particles_of_a_batch(shape):
         times.append(median_ms(lambda: batch.step(8)))
         batch.close()
     assert times[0] < (4.0 if shape == 1 else 6.0) * times[1]
+
+
+@pytest.mark.parametrize("M", [1, 4, 16])
+def test_field_advance_of_short_rows(M):
+    """128 x 16384 cells against 16384 x 128: 0.7 to 1.2 times as long, 6 to 8 when the short rows' one column of segments was
+    cut into 64 chunks."""
+    times = []
+    for nz, nx in ((128, 16384), (16384, 128)):
+        kw = dict(solver="custom", coef=fit.fit_coefficients(4.0, M=M)) if M > 1 else {}
+        sim = Simulation(ndim=2, nz=nz, nx=nx, dz=0.05, dx=0.05, dt=0.0125, **kw)
+        times.append(median_ms(lambda: [sim.field_advance() for _ in range(4)]))
+        sim.close()
+    assert times[0] < 2.5 * times[1]
