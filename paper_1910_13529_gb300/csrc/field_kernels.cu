@@ -1659,7 +1659,10 @@ int field_variants(int ndim) { return ndim == 2 ? 12 : 12; }
 // Variant used before (or without) pic_autotune.  The lines lie where the measured times of the variants
 // cross (us per advance on 16 to 33.6e6 cells; a before the rule, b with it):
 //   3D: the y-march, up to M = 8 128 x 4 (Yee 512 x 256 x 256: a 1527, b 597; 251 x 120 x 117: a 182, b 119;
-//   M = 8: a 718, b 670), for M = 16 the prefetch ring 128 x 8 (862, next best 1066).
+//   M = 8: a 718, b 670), for M = 16 the prefetch ring 128 x 8 (862, next best 1066).  Few cells want the
+//   register-blocked 64 x 4 x 4, whose CTAs wait for one staging instead of one per plane (kernel alone, M = 1
+//   and 16: 64 x 32 x 32 10 and 14, y-march 27, ring 41; 65 x 33 x 31 13 and 17, 33 and 56; 64 x 64 x 64 12 and 22,
+//   27 and 41; 128 x 64 x 64 20 and 38, 28 and 42; 127 x 63 x 65 M = 4 33 and 35; 256 x 64 x 64 M = 4 35 and 33).
 //   2D from 2e6 cells: the x-march with 64 threads (4096 x 1024 Yee: a 76, b 48; M = 16: a 86, b 64; 4099 x
 //   1030 M = 16: a 145, b 91), but not Yee on rows that are not 16-byte aligned (74 against 72), and not on short
 //   rows, which leave most of a segment's 464 or 416 cells idle (128 x 16384 Yee and M = 16: x-march 53 and 87,
@@ -1669,8 +1672,11 @@ int field_variants(int ndim) { return ndim == 2 ? 12 : 12; }
 //   rows the register-blocked 128 x 8, on fewer than 1.3e5 cells 128 x 4 (256 x 128 Yee: a 8.7, b 5), and
 //   Yee from 5e5 cells 64 x 16 (2048 x 512: a 18.8, b 16.8; register-blocked 18.8).
 int default_field_variant(const GridP& g, int M) {
-    if (g.ndim == 3) return M <= 8 ? 6 : 10;
     const bool aligned = g.nz % 4 == 0, yee = M <= 1;
+    if (g.ndim == 3) {
+        if (g.ncell <= 300000 || (aligned && M <= 4 && g.ncell <= 600000)) return 3;
+        return M <= 8 ? 6 : 10;
+    }
     if (g.ncell >= 2000000 && g.nz >= 256 && (aligned || !yee)) return 11;
     if (!aligned) return yee ? 2 : M <= 4 ? 0 : 4;
     if (g.ncell < 130000) return 6;
