@@ -283,16 +283,15 @@ __device__ __forceinline__ void load_taps(float2* h2, const float* __restrict__ 
     for (int k = threadIdx.x; k <= 2 * kHL; k += blockDim.x) h2[k] = make_float2(h[k], h[k]);
 }
 
-// CP_NT / tpr pairs of rows per CTA, tpr threads each (a multiple of 32)
-__global__ void __launch_bounds__(CP_NT) correct_j1_pairs_kernel(const __grid_constant__ CorrP p, long long rows, int tpr,
-                                                                 int vec4) {
+// CP_NT / tpr pairs of rows per CTA, tpr threads each (a multiple of 32); 16-byte aligned rows
+__global__ void __launch_bounds__(CP_NT) correct_j1_pairs_kernel(const __grid_constant__ CorrP p, long long rows, int tpr) {
     chain_enter();
     extern __shared__ float4 s4[];
     __shared__ float2 h2[2 * kHL + 1];
     load_taps(h2, p.h);
     const int grp = threadIdx.x / tpr, nz = p.g.nz;
     const long long r = 2 * ((long long)blockIdx.x * (CP_NT / tpr) + grp);
-    correct_pair(p.J1 + (r < rows ? r : 0) * nz, nz, r < rows, r + 1 < rows, vec4 != 0, h2,
+    correct_pair(p.J1 + (r < rows ? r : 0) * nz, nz, r < rows, r + 1 < rows, true, h2,
                  reinterpret_cast<float*>(s4) + grp * pair_floats(nz), threadIdx.x - grp * tpr, tpr);
 }
 
@@ -446,10 +445,12 @@ cudaError_t launch_correct_j1(const GridP& g, const float* taps, int hlen, float
     CorrP p = corr_params(g, taps, hlen, J1);
     const long long rows = (long long)g.nx * g.ny;
     const int vec4 = (g.nz % 4 == 0 && ((uintptr_t)J1 & 15) == 0) ? 1 : 0;
-    // Pairs of rows where they are short and many: a pair's buffer is 2.5 times a row's and there are half
-    // as many CTAs.  One row at a time and pairs: 512 cells x 65536 rows 128 and 86 us; 8192 x 2048 41 and 46,
-    // 2048 x 512 5.7 and 6.1 (256 CTAs on 152 SMs).
-    if (g.nz <= 1024 && rows >= 4096) {
+    // Pairs of rows where they are of middle length, aligned and many: a pair's buffer is 2.5 times a row's, there
+    // are half as many CTAs, and a lane's eight cells leave most of a warp idle on short rows.  One row at a time and
+    // pairs, us: 512 cells x 65536 rows 128 and 86; 1024 x 4096 19.4 and 17.6, x 16384 65 and 53; 512 x 4096 12.5
+    // and 11.9; the other side of the line: 260 x 4096 10.6 and 12.0, 64 x 16384 12.8 and 16.6; rows that
+    // are not 16-byte aligned 1021 x 4096 23 and 29, x 16384 90 and 99; 8192 x 2048 41 and 46, 2048 x 512 5.7 and 6.1.
+    if (vec4 && g.nz >= 512 && g.nz <= 1024 && rows >= 4096) {
         // threads per pair: a lane each, in whole warps; short rows share a CTA
         int tpr = ((g.nz + 7) / 8 + 31) / 32 * 32;
         tpr = tpr > CP_NT / 2 ? CP_NT : tpr;
@@ -457,7 +458,7 @@ cudaError_t launch_correct_j1(const GridP& g, const float* taps, int hlen, float
         const size_t smem = sizeof(float) * pair_floats(g.nz) * per;
         static_assert(sizeof(float) * pair_floats(1024) < 48 * 1024, "default shared memory");
         return launch_chained_if(few_cells(p.g), correct_j1_pairs_kernel, (unsigned)((rows + 2 * per - 1) / (2 * per)), per * tpr, smem, s, p,
-                              rows, tpr, vec4);
+                                 rows, tpr);
     }
     // threads per row: enough for one pass of four outputs each, in whole warps, at most 256
     int tpr = (((g.nz + 3) / 4) + 31) / 32 * 32;

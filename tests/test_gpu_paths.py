@@ -243,3 +243,21 @@ def test_captured_steps(ndim, nz, nx, ny, filt):
     dx, du = particle_errors(sim, osim, 0, ndim)
     assert dx < TOL and du < TOL
     sim.close()
+
+
+@pytest.mark.parametrize("nz,nx,ny", [(512, 65, 65), (512, 64, 64), (516, 64, 65), (1020, 65, 65), (1024, 63, 67)])
+def test_correction_in_pairs_of_rows(nz, nx, ny):
+    """The Sec. 3 correction where it takes two rows at a time (at least 4096 aligned rows of 512 to 1024 cells): two pairs
+    and one pair per CTA, an odd number of rows, a last CTA with an idle group, rows that end inside a lane's eight
+    cells; against the oracle as above."""
+    assert nz % 4 == 0 and nx * ny >= 4096
+    C = fit.fit_coefficients(2.5, M=8)
+    grid = dict(ndim=3, nz=nz, nx=nx, ny=ny, dz=0.5, dx=0.6, dy=0.7, dt=0.2, solver="custom", shape=1)
+    sp = wl.random_particles(3, nz, nx, ny, 4000, seed=nz + nx, u_scale=1.0, margin=1)
+    sim, osim = gpu_sim(grid, [sp], coef=C), oracle_sim(grid, [sp], coef=C)
+    sim.step(1)
+    osim.step()
+    J = sim.J.double().cpu().numpy()
+    assert np.abs(J - osim.J).max() < TOL * np.abs(osim.J).max()
+    assert field_error(sim, osim) < TOL
+    sim.close()
