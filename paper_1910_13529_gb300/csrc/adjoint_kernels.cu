@@ -17,18 +17,20 @@
 // memory.  A CTA owns ADJ_SEG cells of one z row, four per thread; rows that are differentiated along z
 // are staged with their halo, everything else is read at the cell.
 //
-// The gradient sums of FP32 fields are kept to about 48 bits in pairs of FP32 numbers (pair_math.h: exact
-// differences, products and sums) and added up in FP64 from the warp
-// totals on.  FP64 arithmetic per cell was what the step waited for: this chip does 64 FP32 operations
-// for one in FP64, so that 1024 x 256 cells with M = 4 took 34 us per gradient kernel, 127 us of the
-// 163 us of an adjoint step (now 26 us).  The pairs cost 17 FP32 operations per tap and component and the step is
-// bound by its launches and their latency.
+// The gradient sums of FP32 fields are wide sums (wide_math.h: exact differences and products, sums kept to
+// about 2^-72), which become FP64 at the warp totals.  FP64 arithmetic per cell was what the step waited for: this
+// chip does 64 FP32 operations for one in FP64.  1024 x 256, M = 4: pic_adjoint_step 200 us with FP64 sums, 58 with
+// these; the gradient of 500 steps 128 and 45 ms.  (Sums in pairs, 48 bits, took 42 us and 37 ms: too few bits.)
+// A term costs 40 FP32 operations; half of the rest is launches and their latency.  Each warp scales its
+// cells and its windows by powers of two to about 1, so that fields may be as small or large as FP32 holds; where
+// the largest product of a warp is still below 1e-18 of what its largest cells could give, and for values that
+// are not finite, the warp adds in FP64.
 #include <cuda_runtime.h>
 
 #include <type_traits>
 
-#include "pair_math.h"
 #include "pic_internal.h"
+#include "wide_math.h"
 
 namespace pic {
 
@@ -39,23 +41,75 @@ constexpr int HL = PIC_MAX_HLEN;
 
 __device__ __forceinline__ int wrapm(int a, int n) { return a < 0 ? a + n : (a >= n ? a - n : a); }
 
-// grad[l] += scale * the block's sum of acc[l], l < M
-template <int MAXM>
-__device__ __forceinline__ void flush_grad(PairSum (&acc)[MAXM], int M, double scale, double* grad) {
-    __shared__ double part[MAXM][ADJ_NT / 32];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-#pragma unroll
-    for (int l = 0; l < MAXM; ++l) {
-        if (l >= M) break;
-        acc[l].warp_sum();
-        if (lane == 0) part[l][w] = acc[l].value();
-    }
+constexpr int ADJ_W = ADJ_NT / 32;
+
+// grad[l] += scale * the sum of part[l] over the warps, l < M (ends what the warps wrote to part)
+template <int MP>
+__device__ __forceinline__ void flush_grad(const double (&part)[MP][ADJ_W], int M, double scale, double* grad) {
     __syncthreads();
     if (threadIdx.x < M) {
         double v = 0.0;
-        for (int q = 0; q < ADJ_NT / 32; ++q) v += part[threadIdx.x][q];
+        for (int q = 0; q < ADJ_W; ++q) v += part[threadIdx.x][q];
         if (v != 0.0) atomicAdd(grad + threadIdx.x, scale * v);
     }
+}
+
+__device__ __forceinline__ double warp_sum(double v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+
+// The largest |a| of a warp: its bits, and the power of two that brings it to about 1.
+struct WarpScale {
+    unsigned bits = 0u;
+    template <int N>
+    __device__ __forceinline__ void look(const float (&a)[N]) {
+#pragma unroll
+        for (int k = 0; k < N; ++k) bits = max(bits, __float_as_uint(fabsf(a[k])));
+    }
+    __device__ __forceinline__ void agree() { bits = __reduce_max_sync(0xffffffffu, bits); }
+    __device__ __forceinline__ bool finite() const { return bits < 0x7f800000u; }
+    __device__ __forceinline__ float factor() const {
+        return __uint_as_float((unsigned)min(max(254 - (int)(bits >> 23), 1), 253) << 23);
+    }
+};
+template <int N>
+__device__ __forceinline__ void scale_by(float (&a)[N], float f) {
+#pragma unroll
+    for (int k = 0; k < N; ++k) a[k] *= f;
+}
+// The sums of a warp's scaled terms stand when the largest product (top) leaves its residuals in range.
+__device__ __forceinline__ bool wide_enough(float top) {
+    return __reduce_max_sync(0xffffffffu, __float_as_uint(top)) >= __float_as_uint(1e-18f);
+}
+// Sums of acc[0 .. N) over the lanes at distances O, O / 2, .., 1: a lane hands over half of its sums at each step until
+// it has one left, in the end that of acc[lane MP / 32].  MP + 4 - log2(MP) additions where summing each over the warp takes 5 MP (M = 16: 16
+// and 80).
+template <int N, int O, int MP>
+__device__ __forceinline__ void fold_sums(WideSum (&acc)[MP]) {
+    if constexpr (O > 0) {
+        if constexpr (N == 1) {
+            acc[0].add_lane(acc[0], O);
+        } else {
+            const bool up = threadIdx.x & O;
+#pragma unroll
+            for (int k = 0; k < N / 2; ++k) {
+                const WideSum give = up ? acc[k] : acc[k + N / 2];
+                if (up) acc[k] = acc[k + N / 2];
+                acc[k].add_lane(give, O);
+            }
+        }
+        fold_sums<(N > 1 ? N / 2 : 1), O / 2>(acc);
+    }
+}
+// part[l] = the warp's sum of acc[l], unscaled; zero: nothing was added
+template <int MP>
+__device__ __forceinline__ void keep_sums(WideSum (&acc)[MP], bool zero, int M, float fa, float fb,
+                                          double (&part)[MP][ADJ_W]) {
+    if (!zero) fold_sums<MP, 16>(acc);
+    const int l = (threadIdx.x & 31) * MP / 32;
+    if ((threadIdx.x & (32 / MP - 1)) == 0 && l < M) part[l][threadIdx.x >> 5] = acc[0].value() / ((double)fa * (double)fb);
 }
 
 // Cells [zlo, zlo + n) of a row into s, zero outside 0 <= z < nz, asynchronously: a stage's rows are
@@ -97,27 +151,123 @@ template <int MP, bool PLUS>
 __device__ __forceinline__ float axial(const StencilP& st, const float (&w)[2 * MP + 4], int j) {
     float s = 0.f;
 #pragma unroll
-    for (int l = 1; l <= MP; ++l)
+    for (int l = 1; l <= MP; ++l) {
+        if (l > st.M) break;
         s = fmaf(st.C[l - 1], PLUS ? w[MP + j + l] - w[MP + j - l + 1] : w[MP + j + l - 1] - w[MP + j - l], s);
+    }
     return s;
 }
 
-// acc[l - 1] += sum_j l3[j] D_l f2 - l2[j] D_l f3 over the thread's four cells, D_l tap l of d+ (PLUS)
-// or d- without its 1/dz
+// part[l - 1] = the warp's sum of l3 D_l f2 - l2 D_l f3 over its cells, D_l tap l of d+ (PLUS) or d-
+// without its 1/dz.  L2, L3: the thread's four cells; F2, F3: its windows (cell 0 at F + MP); all staged,
+// zero outside the grid.
 template <int MP, bool PLUS>
-__device__ __forceinline__ void grad_terms(PairSum (&acc)[MP], const float (&l2)[4], const float (&l3)[4],
-                                           const float (&f2)[2 * MP + 4], const float (&f3)[2 * MP + 4]) {
+__device__ __forceinline__ void grad_terms(double (&part)[MP][ADJ_W], int M, const float* L2, const float* L3,
+                                           const float* F2, const float* F3) {
+    float l2[4], l3[4], f2[2 * MP + 4], f3[2 * MP + 4];
+    load_window(l2, L2);
+    load_window(l3, L3);
+    load_window(f2, F2);
+    load_window(f3, F3);
+    WarpScale ml, mf;
+    ml.look(l2);
+    ml.look(l3);
+    mf.look(f2);
+    mf.look(f3);
+    ml.agree();
+    mf.agree();
+    bool wide = ml.finite() && mf.finite();
+    if (wide) {
+        const float a = ml.factor(), b = mf.factor();
+        scale_by(l2, a);
+        scale_by(l3, a);
+        scale_by(f2, b);
+        scale_by(f3, b);
+        WideSum acc[MP];
+        const bool zero = ml.bits == 0u || mf.bits == 0u;
+        float top = 0.f;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        if (l2[j] == 0.f && l3[j] == 0.f) continue;
+        for (int j = 0; j < 4; ++j) {
+            if (zero || (l2[j] == 0.f && l3[j] == 0.f)) continue;
 #pragma unroll
-        for (int l = 1; l <= MP; ++l) {
-            const int a = PLUS ? MP + j + l : MP + j + l - 1, b = PLUS ? MP + j - l + 1 : MP + j - l;
-            float d, e;
-            add2(f3[a], -f3[b], d, e);
-            acc[l - 1].fma(-l2[j], d, e);
-            add2(f2[a], -f2[b], d, e);
-            acc[l - 1].fma(l3[j], d, e);
+            for (int l = 1; l <= MP; ++l) {
+                if (l > M) break;
+                const int hi = PLUS ? MP + j + l : MP + j + l - 1, lo = PLUS ? MP + j - l + 1 : MP + j - l;
+                float d, e;
+                two_sum(f3[hi], -f3[lo], d, e);
+                top = fmaxf(top, fabsf(acc[l - 1].fma(-l2[j], d, e)));
+                two_sum(f2[hi], -f2[lo], d, e);
+                top = fmaxf(top, fabsf(acc[l - 1].fma(l3[j], d, e)));
+            }
+        }
+        wide = zero || wide_enough(top);
+        if (wide) keep_sums(acc, zero, M, a, b, part);
+    }
+    if (!wide) {
+#pragma unroll 1
+        for (int l = 1; l <= M; ++l) {
+            const int hi = PLUS ? MP + l : MP + l - 1, lo = PLUS ? MP - l + 1 : MP - l;
+            double v = 0.0;
+            for (int j = 0; j < 4; ++j) {
+                const double a2 = L2[j], a3 = L3[j];
+                if (a2 == 0.0 && a3 == 0.0) continue;
+                v += -a2 * ((double)F3[j + hi] - (double)F3[j + lo]) + a3 * ((double)F2[j + hi] - (double)F2[j + lo]);
+            }
+            v = warp_sum(v);
+            if ((threadIdx.x & 31) == 0) part[l - 1][threadIdx.x >> 5] = v;
+        }
+    }
+}
+
+// part[l - 1] = the warp's sum of v (sum of J1 over |m| < l), J: the thread's window (cell 0 at J + MP).
+template <int MP>
+__device__ __forceinline__ void correction_terms(double (&part)[MP][ADJ_W], int M, const float (&v)[4], const float* J) {
+    float w[4], jw[2 * MP + 4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) w[j] = v[j];
+    load_window(jw, J);
+    WarpScale mv, mj;
+    mv.look(w);
+    mj.look(jw);
+    mv.agree();
+    mj.agree();
+    bool wide = mv.finite() && mj.finite();
+    if (wide) {
+        const float a = mv.factor(), b = mj.factor();
+        scale_by(w, a);
+        scale_by(jw, b);
+        WideSum acc[MP];
+        const bool zero = mv.bits == 0u || mj.bits == 0u;
+        float top = 0.f;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            if (zero || w[j] == 0.f) continue;
+            WideSum box;                                       // of J1 over |m| < l
+            box.h = jw[MP + j];
+            top = fmaxf(top, fabsf(acc[0].fma(w[j], box.h, 0.f)));
+#pragma unroll
+            for (int l = 2; l <= MP; ++l) {
+                if (l > M) break;
+                box.add(jw[MP + j - (l - 1)]);
+                box.add(jw[MP + j + (l - 1)]);
+                top = fmaxf(top, fabsf(acc[l - 1].fma(w[j], box.h, box.m, box.l)));
+            }
+        }
+        wide = zero || wide_enough(top);
+        if (wide) keep_sums(acc, zero, M, a, b, part);
+    }
+    if (!wide) {
+#pragma unroll 1
+        for (int l = 1; l <= M; ++l) {
+            double s = 0.0;
+            for (int j = 0; j < 4; ++j) {
+                if (v[j] == 0.f) continue;
+                double box = J[MP + j];
+                for (int m = 1; m < l; ++m) box += (double)J[MP + j - m] + (double)J[MP + j + m];
+                s += (double)v[j] * box;
+            }
+            s = warp_sum(s);
+            if ((threadIdx.x & 31) == 0) part[l - 1][threadIdx.x >> 5] = s;
         }
     }
 }
@@ -144,6 +294,7 @@ __global__ void __launch_bounds__(ADJ_NT) adjoint_ampere_kernel(GridP g, Stencil
     chain_enter();
     constexpr int W = ADJ_SEG + 2 * MP;
     __shared__ __align__(16) float sB[2][W], sF[2][W];
+    __shared__ double part[MP][ADJ_W];
     const long long N = g.ncell;
     const RowAt q = row_at(g, blockIdx.x);
     const int z0 = blockIdx.y * ADJ_SEG, nz = g.nz;
@@ -167,7 +318,6 @@ __global__ void __launch_bounds__(ADJ_NT) adjoint_ampere_kernel(GridP g, Stencil
     }
     stage_wait();
     __syncthreads();
-    PairSum acc[MP];
     float b2[2 * MP + 4], b3[2 * MP + 4];
     load_window(b2, sB[0] + t4);
     load_window(b3, sB[1] + t4);
@@ -184,15 +334,8 @@ __global__ void __launch_bounds__(ADJ_NT) adjoint_ampere_kernel(GridP g, Stencil
         o[N] = e2[j] + s2;
         o[2 * N] = e3[j] + (hz * axial<MP, false>(st, b2, j) - hx * (b1[j] - x1[j]));
     }
-    {
-        const float l2[4] = {b2[MP], b2[MP + 1], b2[MP + 2], b2[MP + 3]};
-        const float l3[4] = {b3[MP], b3[MP + 1], b3[MP + 2], b3[MP + 3]};
-        float f2[2 * MP + 4], f3[2 * MP + 4];
-        load_window(f2, sF[0] + t4);
-        load_window(f3, sF[1] + t4);
-        grad_terms<MP, true>(acc, l2, l3, f2, f3);
-    }
-    flush_grad<MP>(acc, st.M, -(double)h / (double)g.dz, grad);
+    grad_terms<MP, true>(part, st.M, sB[0] + t4 + MP, sB[1] + t4 + MP, sF[0] + t4, sF[1] + t4);
+    flush_grad<MP>(part, st.M, -(double)h / (double)g.dz, grad);
 }
 
 // rows of B' (components 2, 3) over [z0 - MP, z0 + ADJ_SEG + MP) into sH, by way of E2, E3 staged in sE
@@ -239,6 +382,7 @@ __global__ void __launch_bounds__(ADJ_NT) adjoint_faraday_kernel(GridP g, Stenci
     chain_enter();
     constexpr int W = ADJ_SEG + 2 * MP, W1 = ADJ_SEG + 2 * HL;
     __shared__ __align__(16) float sE[2][ADJ_SEG + 4 * MP], sH[2][W], sA[2][W], sA1[W1], sJ[W];
+    __shared__ double part[MP][ADJ_W];
     const long long N = g.ncell;
     const RowAt q = row_at(g, blockIdx.x);
     const int z0 = blockIdx.y * ADJ_SEG, nz = g.nz;
@@ -262,7 +406,6 @@ __global__ void __launch_bounds__(ADJ_NT) adjoint_faraday_kernel(GridP g, Stenci
         cells4(y2, aE + N + q.yp, zi, nz);
     }
     stage_b_half<MP>(g, st, E, B, q, z0, sE, sH);
-    PairSum acc[MP];
     {
         float a2[2 * MP + 4], a3[2 * MP + 4];
         load_window(a2, sA[0] + t4);
@@ -280,40 +423,23 @@ __global__ void __launch_bounds__(ADJ_NT) adjoint_faraday_kernel(GridP g, Stenci
             o[N] = b2[j] + s2;
             o[2 * N] = b3[j] + (fz * axial<MP, true>(st, a2, j) - fx * (x1[j] - a1[j]));
         }
-        const float l2[4] = {a2[MP], a2[MP + 1], a2[MP + 2], a2[MP + 3]};
-        const float l3[4] = {a3[MP], a3[MP + 1], a3[MP + 2], a3[MP + 3]};
-        float f2[2 * MP + 4], f3[2 * MP + 4];
-        load_window(f2, sH[0] + t4);
-        load_window(f3, sH[1] + t4);
-        grad_terms<MP, false>(acc, l2, l3, f2, f3);
     }
+    grad_terms<MP, false>(part, st.M, sA[0] + t4 + MP, sA[1] + t4 + MP, sH[0] + t4, sH[1] + t4);
     // the correction's sum has another factor: flushed on its own
-    flush_grad<MP>(acc, st.M, (double)dt / (double)g.dz, grad);
+    flush_grad<MP>(part, st.M, (double)dt / (double)g.dz, grad);
     if (!correct) return;
     __syncthreads();
-    PairSum cor[MP];
-    float w[2 * HL + 4], jw[2 * MP + 4];
+    float w[2 * HL + 4], v[4];
     load_window(w, sA1 + t4);
-    load_window(jw, sJ + t4);
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-        float v = 0.f;                                         // P^{-1} l_E1
+        v[j] = 0.f;                                            // P^{-1} l_E1
 #pragma unroll
-        for (int k = 0; k <= 2 * HL; ++k) v = fmaf(taps.h[k], w[j + 2 * HL - k], v);
-        if (v == 0.f || zi + j >= nz) continue;
-        float bh = jw[MP + j], bl = 0.f;                       // sum of J1 over |m| < l
-        cor[0].fma(v, bh, 0.f);
-#pragma unroll
-        for (int l = 2; l <= MP; ++l) {
-            float s, e;
-            add2(bh, jw[MP + j - (l - 1)], s, e);
-            bl += e;
-            add2(s, jw[MP + j + (l - 1)], bh, e);
-            bl += e;
-            cor[l - 1].fma(v, bh, bl);
-        }
+        for (int k = 0; k <= 2 * HL; ++k) v[j] = fmaf(taps.h[k], w[j + 2 * HL - k], v[j]);
+        if (zi + j >= nz) v[j] = 0.f;
     }
-    flush_grad<MP>(cor, st.M, (double)dt, grad);
+    correction_terms<MP>(part, st.M, v, sJ + t4);
+    flush_grad<MP>(part, st.M, (double)dt, grad);
 }
 
 // E' = E + dt (S B' - J), components 2 and 3, into out (component stride N, component 1 not written).

@@ -1,0 +1,131 @@
+"""What the library forms in FP64, or wider out of FP32 parts, against exact rational arithmetic.  Tolerances
+count the FP64 roundings of the result (u = 2^-53 each); the parts before them lose less than 2^-60."""
+from fractions import Fraction as Fr
+
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():
+    pytest.skip("no CUDA device", allow_module_level=True)
+
+import paper_1910_13529_gb300 as P  # noqa: E402
+from oracle import fit  # noqa: E402
+from paper_1910_13529_gb300.runtime import Simulation  # noqa: E402
+
+U = 2.0 ** -53
+
+
+def _sim(nz, M=1, nx=4, **kw):
+    C = dict(solver="custom", coef=fit.fit_coefficients(4.0, M=M)) if M > 1 else dict(solver="yee")
+    return Simulation(device="cuda:0", ndim=2, nz=nz, nx=nx, dz=0.5, dx=0.5, dt=0.125, **C, **kw)
+
+
+def _dev(a):
+    return torch.from_numpy(np.ascontiguousarray(a, dtype=np.float32)).cuda()
+
+
+def _gradient(sim, M, E1, aE, aB, J):
+    """The gradient of one recorded step whose first fields are zero: only the third stage (E1, aB) and the
+    correction (J, aE) contribute."""
+    E = torch.stack([torch.zeros_like(_dev(E1)), _dev(E1)])
+    B, Jd, aEd, aBd = torch.zeros_like(E), _dev(J), _dev(aE), _dev(aB)
+    grad = torch.zeros(M, dtype=torch.float64, device="cuda")
+    P.pic_adjoint_run(sim.h, 1, E.data_ptr(), B.data_ptr(), Jd.data_ptr(), aEd.data_ptr(), aBd.data_ptr(),
+                      grad.data_ptr(), sim.stream)
+    torch.cuda.synchronize()
+    return grad.cpu().numpy()
+
+
+def _at(row, z):
+    return Fr(float(row[z])) if 0 <= z < len(row) else Fr(0)
+
+
+def _third_stage(E1, aB, M, scale):
+    """scale sum l3 D+_l F2 - l2 D+_l F3 over the cells with (l2, l3) != 0, and the sum of the terms' sizes."""
+    out, size = [Fr(0)] * M, [Fr(0)] * M
+    _, _, nx, nz = E1.shape
+    for x in range(nx):
+        for z in range(nz):
+            l2, l3 = Fr(float(aB[1, 0, x, z])), Fr(float(aB[2, 0, x, z]))
+            if not l2 and not l3:
+                continue
+            for l in range(1, M + 1):
+                for v, f in ((l3, E1[1, 0, x]), (-l2, E1[2, 0, x])):
+                    t = v * (_at(f, z + l) - _at(f, z - l + 1))
+                    out[l - 1] += scale * t
+                    size[l - 1] += abs(scale * t)
+    return out, size
+
+
+@pytest.mark.parametrize("M", [3, 8, 16])
+@pytest.mark.parametrize("la,lf", [(0, 0), (-60, -60), (-120, 30), (60, 63), (-20, -128)])
+def test_gradient_sums(M, la, lf):
+    """The third stage's terms over the range of FP32 (aB times 2^la, E' times 2^lf).  Roundings: two where a
+    warp's sum becomes FP64 and three of the four rows' additions; the factor -h/dz is a power of two."""
+    nz = 4
+    sim = _sim(nz, M)
+    worst = 0.0
+    for seed in range(12):
+        rng = np.random.default_rng(1000 * M + seed)
+        E1, aB = np.zeros((3, 1, 4, nz), np.float32), np.zeros((3, 1, 4, nz), np.float32)
+        E1[1:] = np.ldexp(rng.normal(size=(2, 1, 4, nz)).astype(np.float32), lf)
+        aB[1:] = np.ldexp(rng.normal(size=(2, 1, 4, nz)).astype(np.float32), la)
+        got = _gradient(sim, M, E1, np.zeros_like(E1), aB, np.zeros_like(E1))
+        ref, size = _third_stage(E1, aB, M, Fr(-1, 8))
+        for l in range(M):
+            if size[l]:
+                worst = max(worst, float(abs(Fr(float(got[l])) - ref[l]) / size[l]))
+            else:
+                assert got[l] == 0.0
+    assert worst <= 5 * U + 2.0 ** -60, worst
+    sim.close()
+
+
+@pytest.mark.parametrize("far", [1.0, np.inf])
+def test_gradient_sums_where_large_cells_take_no_part(far):
+    """Products 2^-100 of what the largest cells of the row could give: a warp that spans both, and one that
+    spans an infinity that no term reads."""
+    M, nz = 4, 120
+    sim = _sim(nz, M)
+    rng = np.random.default_rng(7)
+    E1, aB = np.zeros((3, 1, 4, nz), np.float32), np.zeros((3, 1, 4, nz), np.float32)
+    E1[1:, :, :, :12] = np.ldexp(rng.normal(size=(2, 1, 4, 12)).astype(np.float32), -100)
+    aB[1:, :, :, :8] = rng.normal(size=(2, 1, 4, 8)).astype(np.float32)
+    E1[1:, :, :, 100] = far
+    got = _gradient(sim, M, E1, np.zeros_like(E1), aB, np.zeros_like(E1))
+    E1[1:, :, :, 100] = 0.0                                  # (no cell with aB != 0 reaches it)
+    ref, size = _third_stage(E1, aB, M, Fr(-1, 8))
+    for l in range(M):
+        # in FP64 from the first difference on: 16 terms, five shuffles, four warps, four rows
+        assert abs(Fr(float(got[l])) - ref[l]) <= 32 * U * size[l]
+    sim.close()
+
+
+@pytest.mark.parametrize("M", [2, 5, 16])
+@pytest.mark.parametrize("la,lj", [(0, 0), (-70, -60), (50, 70)])
+def test_gradient_of_the_correction(M, la, lj):
+    """dt <P^-1 aE1, P_l J1> for an aE1 of one cell per row, so that P^-1 aE1 is the taps themselves: 2 + 1 + 3
+    FP64 roundings (rows of three warps; the factor dt is a power of two)."""
+    nz = 96
+    sim = _sim(nz, M)
+    taps = sim.coefficients()[1].astype(np.float32)
+    rng = np.random.default_rng(M)
+    aE, J = np.zeros((3, 1, 4, nz), np.float32), np.zeros((3, 1, 4, nz), np.float32)
+    aE[0, 0, :, 41] = np.ldexp(1.0, la)
+    J[0] = np.ldexp(rng.normal(size=(1, 4, nz)).astype(np.float32), lj)
+    got = _gradient(sim, M, np.zeros_like(aE), aE, np.zeros_like(aE), J)
+    c = len(taps) // 2
+    for l in range(1, M + 1):
+        ref, size = Fr(0), Fr(0)
+        for x in range(4):
+            for m in range(-c, c + 1):
+                v = Fr(float(np.ldexp(taps[c + m], la)))
+                for k in range(-(l - 1), l):
+                    t = Fr(1, 8) * v * _at(J[0, 0, x], 41 + m + k)
+                    ref += t
+                    size += abs(t)
+        assert abs(Fr(float(got[l - 1])) - ref) <= 6 * U * size + size * Fr(1, 2 ** 60)
+    sim.close()
