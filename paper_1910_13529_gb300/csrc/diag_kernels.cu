@@ -11,6 +11,7 @@
 
 #include "pair_math.h"
 #include "pic_internal.h"
+#include "wide_math.h"
 
 namespace pic {
 
@@ -186,42 +187,25 @@ __global__ void __launch_bounds__(DG_NT) diag_kernel(GridP g, StencilP st, InvP 
 }
 
 __global__ void __launch_bounds__(256) kinetic_kernel(SpeciesP sp, double* acc) {
-    PairSum e;
+    WideSum e;
     double big = 0.0;                                 // momenta beyond the range of FP32 squares
     int alive = 0;
     const long long n = *sp.count;
     for (long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x; p < n;
          p += (long long)gridDim.x * blockDim.x) {
         if (sp.cell[p] < 0) continue;
-        // gamma - 1 = u^2 / (gamma + 1): no cancellation for slow particles
-        PairSum u2;
-#pragma unroll
-        for (int d = 0; d < 3; ++d) {
-            const float u = sp.u[d * sp.cap + p];
-            u2.fma(u, u, 0.f);
-        }
-        float s, t;
-        if (!(u2.h < 1e30f)) {
-            const double a = sp.u[p], b = sp.u[sp.cap + p], c = sp.u[2 * sp.cap + p];
+        const float u0 = sp.u[p], u1 = sp.u[sp.cap + p], u2 = sp.u[2 * sp.cap + p];
+        if (u0 * u0 + u1 * u1 + u2 * u2 < 1e30f) {
+            const WideSum k = gamma_minus_one(u0, u1, u2);
+            e.add(k.h, k.m, k.l);
+        } else {
+            const double a = u0, b = u1, c = u2;
             big += sqrt(1.0 + a * a + b * b + c * c) - 1.0;
-            ++alive;
-            continue;
         }
-        add2(u2.h, u2.l, s, t);                       // renormalised
-        u2.h = s;
-        u2.l = t;
-        PairSum g2 = u2;
-        g2.add(1.f, 0.f);
-        // gamma = gh + gl (one Newton step on the pair), then the quotient likewise
-        const float gh = sqrtf(g2.h), gl = (fmaf(-gh, gh, g2.h) + g2.l) * __fdividef(0.5f, gh);
-        float dh, dl;
-        add2(gh, 1.f, dh, dl);
-        dl += gl;
-        const float qh = u2.h / dh, ql = (fmaf(-qh, dh, u2.h) + (u2.l - qh * dl)) / dh;
-        e.add(qh, ql);
         ++alive;
     }
-    e.warp_sum();
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) e.add_lane(e, o);
     big = warp_sum(big);
     alive = __reduce_add_sync(0xffffffffu, alive);
     __shared__ double sh[2][8];

@@ -62,6 +62,13 @@ struct WideSum {
         add(p, r, fmaf(x, dl, e + t));
         return p;
     }
+    PIC_HD void normalise() {                              // h the nearest FP32 of the sum, m of the rest
+        float e;
+        two_sum(h, m, h, m);
+        two_sum(m, l, m, l);
+        two_sum(h, m, h, e);
+        m = e;
+    }
 #ifdef __CUDACC__
     __device__ __forceinline__ void add_lane(const WideSum& s, int o) {       // += the s of the lane at distance o
         add(__shfl_xor_sync(0xffffffffu, s.h, o), __shfl_xor_sync(0xffffffffu, s.m, o), __shfl_xor_sync(0xffffffffu, s.l, o));
@@ -69,5 +76,44 @@ struct WideSum {
 #endif
     PIC_HD double value() const { return (double)h + ((double)m + (double)l); }
 };
+
+// gamma - 1 of a momentum u as a WideSum, for |u|^2 below 1e30: u^2 / (gamma + 1), which cancels nothing for
+// slow particles.  The root and the quotient start from FP32 and take two corrections from exact
+// residuals each (2^-22, 2^-46, 2^-70).
+PIC_HD WideSum gamma_minus_one(float u0, float u1, float u2) {
+    WideSum s;                                     // |u|^2
+    float p, e, r, f, q, t, v, w;
+    two_prod(u0, u0, s.h, s.m);
+    two_prod(u1, u1, p, e);
+    s.add(p, e, 0.f);
+    two_prod(u2, u2, p, e);
+    s.add(p, e, 0.f);
+    s.normalise();
+    WideSum g2 = s;                                // gamma^2
+    g2.add(1.f);
+    g2.normalise();
+    // gamma = a + b + c: g2 - a^2 and then g2 - (a + b)^2, each sum ordered so that its large parts cancel
+    const float a = sqrtf(g2.h), ra = 0.5f / a;
+    two_prod(a, a, p, e);
+    two_sum(g2.h - p, -e, r, f);                   // (the difference is exact)
+    two_sum(r, g2.m, r, v);
+    const float b = r * ra;
+    two_prod(2.f * a, b, q, t);
+    const float c = ((r - q) + ((f + v) + g2.l) - (t + b * b)) * ra;
+    // d = gamma + 1 and s / d
+    WideSum d{a, b, c};
+    d.add(1.f);
+    d.normalise();
+    const float q0 = s.h / d.h;
+    two_prod(q0, d.h, p, e);
+    two_prod(q0, d.m, q, t);
+    two_sum(s.h - p, s.m, r, f);                   // (s.h - q0 d.h is exact with e)
+    two_sum(r, -e, r, v);
+    two_sum(r, -q, r, w);
+    const float rest = ((f + v) + w) + (s.l - t - q0 * d.l);
+    const float q1 = r / d.h;
+    const float q2 = (fmaf(-q1, d.h, r) + (rest - q1 * d.m)) / d.h;
+    return WideSum{q0, q1, q2};
+}
 
 }  // namespace pic

@@ -1,5 +1,6 @@
 """What the library forms in FP64, or wider out of FP32 parts, against exact rational arithmetic.  Tolerances
 count the FP64 roundings of the result (u = 2^-53 each); the parts before them lose less than 2^-60."""
+from decimal import Decimal, getcontext
 from fractions import Fraction as Fr
 
 import numpy as np
@@ -128,4 +129,22 @@ def test_gradient_of_the_correction(M, la, lj):
                     ref += t
                     size += abs(t)
         assert abs(Fr(float(got[l - 1])) - ref) <= 6 * U * size + size * Fr(1, 2 ** 60)
+    sim.close()
+
+
+def test_kinetic_energy():
+    """gamma - 1 of one particle, from slow to fast and beyond the range of FP32 squares."""
+    getcontext().prec = 60
+    sim = _sim(16)
+    rng = np.random.default_rng(2)
+    for k in range(48):
+        u = (rng.normal(size=3) * 2.0 ** rng.uniform(-14, 40 if k % 8 else 80)).astype(np.float32)
+        if k % 5 == 0:
+            u[1:] = 0.0
+        one = np.ones(1, np.int64)
+        sim.add_species(0, 8 * one, 2 * one, 0 * one, np.full((2, 1), 0.25, np.float32), u[:, None], -1.0, 1.0, 1.0)
+        x = sum(Decimal(float(v)) ** 2 for v in u)
+        ref = x / (1 + (1 + x).sqrt())
+        got = Decimal(sim.diag()["kinetic"])
+        assert abs(got - ref) <= 3 * Decimal(U) * ref, (u, got, ref)
     sim.close()
