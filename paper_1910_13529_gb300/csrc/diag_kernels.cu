@@ -1,15 +1,12 @@
-// FP64 diagnostics: Gauss residual d-.E - rho - rho_bg (Eq. Gauss of Sec. 2.1, with the same
-// axial d- as Ampere's law), field and kinetic energy.  The divergence and each particle's gamma - 1 are
-// formed as pairs of FP32 numbers (pair_math.h, 48 bits) and become FP64 where they meet rho or the sum
-// of a warp; the field energy and the residual's reductions are FP64 throughout.  With FP64 from the first
-// difference on, the FP64 pipe and its conversions were busy all the time: the 32-point divergence of
-// 2048 x 512 nodes took 215 us (now 15), with the reductions 274 us (61, the energies' FP64), the kinetic
-// energy of 5.2e6 particles 187 us (60).
+// Diagnostics: Gauss residual d-.E - rho - rho_bg (Eq. Gauss of Sec. 2.1, with the same axial d- as Ampere's
+// law), field and kinetic energy.  The divergence and each particle's gamma - 1 are wide sums of FP32 parts
+// (wide_math.h, about 2^-70), which become FP64 where they meet rho and the sums; the rest is FP64 throughout.  With FP64 from the
+// first difference on, the FP64 pipe and its conversions were busy all the time: pic_gauss on 1024 x 256 nodes 39 us
+// (M = 1) and 77 (M = 16), now 29 and 36; on 128 x 64 x 64 with 1e6 particles 126 and 60.
 #include <cuda_runtime.h>
 
 #include <type_traits>
 
-#include "pair_math.h"
 #include "pic_internal.h"
 #include "wide_math.h"
 
@@ -19,17 +16,21 @@ namespace {
 
 constexpr int DG_NT = 128, DG_SEG = 4 * DG_NT;
 
-// 1/h of the axes as pairs
+// Cell sizes of the axes, their reciprocals in three parts, -rho_bg as well; plain: reciprocals of a size
+// that FP32 products can take.
 struct InvP {
-    float z[2], x[2], y[2];
-    float bg[2];                   // -rho_bg
+    double h[3], bg;
+    float z[3], x[3], y[3], back[3];
+    bool plain;
 };
 
-// Nodes of one row segment [z0, z0 + DG_SEG): d-.E - rho_bg at the thread's four nodes.  sE: the E1 cells
-// the windows need (staged here).
+// Nodes of one row segment [z0, z0 + DG_SEG): d-.E - rho_bg at the thread's four nodes.  sE: the E1 cells the
+// windows need (staged here).  Differences are exact, and the sum of all axes is wide as long as its largest
+// term lies where FP32 products leave exact residuals; outside (fields below about 1e-18 or above 1e30) and
+// for values that are not finite the node takes FP64 from the first difference on.
 template <int MP>
 __device__ __forceinline__ void div_row(const GridP& g, const StencilP& st, const InvP& inv, const float* __restrict__ E,
-                                        int row_index, int z0, float* sE, PairSum (&out)[4]) {
+                                        int row_index, int z0, float* sE, double (&out)[4]) {
     constexpr int W = DG_SEG + 2 * MP;
     const long long N = g.ncell;
     const int j = row_index % g.nx, k = row_index / g.nx;
@@ -66,42 +67,64 @@ __device__ __forceinline__ void div_row(const GridP& g, const StencilP& st, cons
     }
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-        PairSum s;
+        out[q] = 0.0;
+        if (zi + q >= g.nz) continue;
+        WideSum s, t;
+        float top = 0.f, range = 0.f;                 // largest term, largest difference
 #pragma unroll
         for (int l = 1; l <= MP; ++l) {
+            if (l > st.M) break;
             float d, e;
-            add2(w[MP + q + l - 1], -w[MP + q - l], d, e);
-            s.fma(st.Cm[l - 1], d, e);                // the B-side d- of Ampere's law
+            two_sum(w[MP + q + l - 1], -w[MP + q - l], d, e);
+            range = fmaxf(range, fabsf(d));
+            top = fmaxf(top, fabsf(s.fma(st.Cm[l - 1], d, e)));      // the B-side d- of Ampere's law
         }
-        s.scale(inv.z[0], inv.z[1]);
-        PairSum t;
-        add2(x1[q], -x0[q], t.h, t.l);
-        t.scale(inv.x[0], inv.x[1]);
-        s.add(t.h, t.l);
+        s.scale(inv.z[0], inv.z[1], inv.z[2]);
+        two_sum(x1[q], -x0[q], t.h, t.m);
+        top = fmaxf(top, fabsf(t.h));
+        range = fmaxf(range, fabsf(t.h));
+        t.l = 0.f;
+        t.scale(inv.x[0], inv.x[1], inv.x[2]);
+        s.add(t.h, t.m, t.l);
         if (g.ndim == 3) {
-            add2(y1[q], -y0[q], t.h, t.l);
-            t.scale(inv.y[0], inv.y[1]);
-            s.add(t.h, t.l);
+            two_sum(y1[q], -y0[q], t.h, t.m);
+            top = fmaxf(top, fabsf(t.h));
+            range = fmaxf(range, fabsf(t.h));
+            t.l = 0.f;
+            t.scale(inv.y[0], inv.y[1], inv.y[2]);
+            s.add(t.h, t.m, t.l);
         }
-        s.add(inv.bg[0], inv.bg[1]);
-        out[q] = s;
+        s.add(inv.back[0], inv.back[1], inv.back[2]);
+        if (inv.plain && fabsf(s.h) < 1e30f && (top > 1e-18f || range == 0.f)) {
+            out[q] = s.value();
+        } else {
+            double dz = 0.0;
+#pragma unroll 1
+            for (int l = 1; l <= st.M; ++l) {
+                const float* c = sE + 4 * threadIdx.x + MP + q;
+                dz += (double)st.Cm[l - 1] * ((double)c[l - 1] - (double)c[-l]);
+            }
+            out[q] = dz / inv.h[0] + ((double)x1[q] - (double)x0[q]) / inv.h[1];
+            if (g.ndim == 3) out[q] += ((double)y1[q] - (double)y0[q]) / inv.h[2];
+            out[q] += inv.bg;
+        }
     }
     __syncthreads();                                  // sE may be filled again
 }
 
 template <int MP>
-__global__ void __launch_bounds__(DG_NT) gauss_kernel(GridP g, StencilP st, InvP inv, const float* E, const double* rho,
+__global__ void __launch_bounds__(DG_NT, 5) gauss_kernel(GridP g, StencilP st, InvP inv, const float* E, const double* rho,
                                                       double* G) {
     __shared__ __align__(16) float sE[DG_SEG + 2 * MP];
     const int z0 = blockIdx.y * DG_SEG;
-    PairSum d[4];
+    double d[4];
     div_row<MP>(g, st, inv, E, blockIdx.x, z0, sE, d);
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
         const int z = z0 + 4 * threadIdx.x + q;
         if (z >= g.nz) break;
         const long long c = (long long)blockIdx.x * g.nz + z;
-        G[c] = (double)d[q].h + ((double)d[q].l - rho[c]);
+        G[c] = d[q] - rho[c];
     }
 }
 
@@ -133,7 +156,7 @@ __global__ void __launch_bounds__(DG_NT) diag_kernel(GridP g, StencilP st, InvP 
     int cnt = 0;
     for (long long it = blockIdx.x; it < items; it += gridDim.x) {
         const int r = (int)(it / segs), z0 = (int)(it - (long long)r * segs) * DG_SEG;
-        PairSum d[4];
+        double d[4];
         div_row<MP>(g, st, inv, E, r, z0, sE, d);
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
@@ -148,7 +171,7 @@ __global__ void __launch_bounds__(DG_NT) diag_kernel(GridP g, StencilP st, InvP 
             const double rv = rho[c];
             rmax = fmax(rmax, fabs(rv));
             if (z >= margin && z < g.nz - margin) {
-                const double G = (double)d[q].h + ((double)d[q].l - rv);
+                const double G = d[q] - rv;
                 gmax = fmax(gmax, fabs(G));
                 g2 += G * G;
                 ++cnt;
@@ -226,15 +249,25 @@ __global__ void __launch_bounds__(256) kinetic_kernel(SpeciesP sp, double* acc) 
 }
 
 InvP inverses(const GridP& g, double rho_bg) {
-    auto split = [](double v, float* p) {
+    InvP q;
+    q.plain = true;
+    // v + rest in three parts
+    auto parts = [](double v, double rest, float* p) {
         p[0] = (float)v;
         p[1] = (float)(v - (double)p[0]);
+        p[2] = (float)(v - (double)p[0] - (double)p[1] + rest);
     };
-    InvP q;
-    split(1.0 / (double)g.dz, q.z);
-    split(1.0 / (double)g.dx, q.x);
-    split(g.ndim == 3 ? 1.0 / (double)g.dy : 0.0, q.y);
-    split(-rho_bg, q.bg);
+    float* const inv[3] = {q.z, q.x, q.y};
+    const float h[3] = {g.dz, g.dx, g.dy};
+    for (int a = 0; a < 3; ++a) {
+        q.h[a] = h[a];
+        const double r = 1.0 / q.h[a];
+        parts(r, std::fma(-r, q.h[a], 1.0) * r, inv[a]);
+        if (a < g.ndim) q.plain = q.plain && r > 1e-10 && r < 1e10;
+    }
+    q.bg = -rho_bg;
+    parts(q.bg, 0.0, q.back);
+    q.plain = q.plain && (rho_bg == 0.0 || (std::fabs(rho_bg) > 1e-18 && std::fabs(rho_bg) < 1e30));
     return q;
 }
 

@@ -62,6 +62,18 @@ struct WideSum {
         add(p, r, fmaf(x, dl, e + t));
         return p;
     }
+    // *= ch + cm + cl
+    PIC_HD void scale(float ch, float cm, float cl) {
+        float p, e, q, t, r, u, f, g;
+        two_prod(h, ch, p, e);
+        two_prod(h, cm, q, t);
+        two_prod(m, ch, r, u);
+        two_sum(q, r, q, f);
+        two_sum(e, q, e, g);
+        l = ((f + g) + (t + u)) + fmaf(h, cl, fmaf(m, cm, l * ch));
+        h = p;
+        m = e;
+    }
     PIC_HD void normalise() {                              // h the nearest FP32 of the sum, m of the rest
         float e;
         two_sum(h, m, h, m);

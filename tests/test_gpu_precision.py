@@ -148,3 +148,51 @@ def test_kinetic_energy():
         got = Decimal(sim.diag()["kinetic"])
         assert abs(got - ref) <= 3 * Decimal(U) * ref, (u, got, ref)
     sim.close()
+
+
+def _exact_gauss(E, C, h):
+    _, _, nx, nz = E.shape
+    G, size = np.empty((nx, nz), object), np.empty((nx, nz), object)
+    for x in range(nx):
+        for z in range(nz):
+            a = [Fr(float(C[l])) * s * _at(E[0, 0, x], z + o) / h for l in range(len(C))
+                 for s, o in ((1, l), (-1, -l - 1))]
+            a += [_at(E[1, 0, x], z) / h, -_at(E[1, 0, (x - 1) % nx], z) / h]
+            G[x, z], size[x, z] = sum(a), sum(abs(v) for v in a)
+    return G, size
+
+
+@pytest.mark.parametrize("M", [1, 3, 8, 16])
+@pytest.mark.parametrize("lf", [0, -115, 100])
+def test_gauss_residual(M, lf):
+    """d-.E of random fields times 2^lf, without particles: two roundings where the axial sum becomes FP64, one of the
+    x difference and three sums (the divisions by 1/2 are exact); out of the range of FP32 products FP64
+    from the first difference on, M + 6."""
+    nz = 21
+    sim = _sim(nz, M)
+    rng = np.random.default_rng(M)
+    E = np.ldexp(rng.normal(size=(3, 1, 4, nz)).astype(np.float32), lf)
+    sim.E.copy_(_dev(E))
+    C = np.ones(1, np.float32) if M == 1 else sim.coefficients()[0].astype(np.float32)
+    ref, size = _exact_gauss(E, C, Fr(1, 2))
+    got = sim.gauss().cpu().numpy()[0]
+    worst = max(float(abs(Fr(float(got[x, z])) - ref[x, z]) / size[x, z]) for x in range(4) for z in range(nz))
+    assert worst <= (6 if lf == 0 else M + 6) * U, worst
+    sim.close()
+
+
+@pytest.mark.parametrize("M", [1, 3, 16])
+def test_gauss_residual_of_infinite_fields(M):
+    """A field that has overflowed shows: the nodes whose difference reads it are infinite or not a number as FP64
+    has them, the others stay finite, and gauss_max is infinite."""
+    nz, z0 = 160, 80
+    sim = _sim(nz, M)
+    E = np.ones((3, 1, 4, nz), np.float32)
+    E[0, 0, 1, z0] = np.inf
+    sim.E.copy_(_dev(E))
+    got = sim.gauss().cpu().numpy()[0]
+    hit = np.zeros((4, nz), bool)
+    hit[1, z0 - M + 1:z0 + M + 1] = True
+    assert np.array_equal(np.isinf(got), hit) and np.isfinite(got[~hit]).all()
+    assert np.isinf(sim.diag()["gauss_max"])
+    sim.close()
