@@ -16,8 +16,8 @@
 #include <type_traits>
 
 #include "box_fit.h"
-#include "pair_math.h"
 #include "pic_internal.h"
+#include "wide_math.h"
 
 namespace pic {
 
@@ -200,17 +200,6 @@ __device__ __forceinline__ void boris(float eps, const float* eb, float* u) {
     u[0] = ul0 + eps * eb[0];
     u[1] = ul1 + eps * eb[1];
     u[2] = ul2 + eps * eb[2];
-}
-
-// Error-free transforms (Knuth TwoSum, FMA TwoProd) for float-float arithmetic.
-__device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
-    s = a + b;
-    float bb = s - a;
-    e = (a - (s - bb)) + (b - bb);
-}
-__device__ __forceinline__ void two_prod(float a, float b, float& p, float& e) {
-    p = a * b;
-    e = fmaf(a, b, -p);
 }
 
 // gamma = sqrt(1 + |u|^2) as an unevaluated float-float sum gh + gl; rg ~ 1/gh (approximate:
@@ -2361,42 +2350,35 @@ __device__ __forceinline__ void rho_one(const GridP& g, const SpeciesP& sp, int 
 }
 
 
-// weights of a position as pairs of FP32 numbers (pair_math.h); the first node is that of Shape::w
+// weights of a position in units of 2^-63 (o in [0, 1]; the first node is that of Shape::w)
 template <int SHAPE>
-__device__ __forceinline__ void pair_weights(float o, PairSum* W) {
+__device__ __forceinline__ void fixed_weights(float o, unsigned long long* W) {
+    const unsigned long long one = 1ull << 63, x = __float2ull_rz(o * 9223372036854775808.f);
     if (SHAPE == 1) {
-        add2(1.f, -o, W[0].h, W[0].l);
-        W[1].h = o;
-        W[1].l = 0.f;
+        W[0] = one - x;
+        W[1] = x;
         return;
     }
-    const float d = o >= 0.5f ? o - 1.f : o;              // exact
-    float ah, al, bh, bl;
-    add2(0.5f, -d, ah, al);
-    add2(0.5f, d, bh, bl);
-    W[0].h = 0.5f * ah;
-    W[0].l = 0.5f * al;
-    W[0].scale(ah, al);
-    W[2].h = 0.5f * bh;
-    W[2].l = 0.5f * bl;
-    W[2].scale(bh, bl);
-    W[1].h = 0.75f;
-    W[1].l = 0.f;
-    W[1].fma(-d, d, 0.f);
+    // o - node + 1/2 and node + 1/2 - o, both in [0, 1]
+    const unsigned long long b = o >= 0.5f ? x - (one >> 1) : x + (one >> 1), a = one - b;
+    W[0] = __umul64hi(a, a);                              // a^2 / 2
+    W[2] = __umul64hi(b, b);
+    W[1] = one - W[0] - W[2];
 }
 
 // Charge density of chunks of FUSED_T particles: the chunk's nodes are summed in shared memory and
-// added to rho once per node.  A contribution (a product of weights, at most 1) is formed as a pair of
-// FP32 numbers and added as two fixed-point words, units 2^-22 and 2^-44: integer shared atomics, no FP64
-// until the flush (two operations per node).  FP64 weights and one FP64 global atomic per node and
-// particle took 237 us for 2.6e6 particles (quadratic, 2D; the FP64 pipe), this takes 48 us.  A chunk whose nodes
-// do not fit (particles not sorted) takes that path still.
+// added to rho once per node.  Weights and their products are whole numbers in units of 2^-63 to 2^-61
+// (an offset's bits below 2^-63 and the products' below those units are cut), and a contribution is added as three
+// 21-bit words: integer shared atomics, no FP64 until the flush.  FP64 weights and one FP64 global atomic
+// per node and particle took 237 us for 2.6e6 particles (quadratic, 2D; the FP64 pipe), this takes 75 us.
+// A chunk whose nodes do not fit (particles not sorted) takes that path still, and so does a particle whose
+// offset is not a number in [0, 1].
 constexpr int RHO_CAP = 2048;      // nodes of the box
 
 template <int NDIM, int SHAPE>
 __global__ void __launch_bounds__(FUSED_T) rho_kernel(GridP g, SpeciesP sp, int shift, double* rho) {
     constexpr int K = Shape<SHAPE>::K;
-    __shared__ __align__(16) int hi[RHO_CAP], lo[RHO_CAP];
+    __shared__ unsigned sum[3][RHO_CAP];                    // words of 21 bits, the lowest first
     __shared__ int box[2][6];
     const long long n = *sp.count;
     const int n3[3] = {g.nz, g.nx, g.ny};
@@ -2413,10 +2395,16 @@ __global__ void __launch_bounds__(FUSED_T) rho_kernel(GridP g, SpeciesP sp, int 
             decode(g, sp.cell[p], izg, ix, iy);
             const int c[3] = {izg - 1 - shift, ix, iy};
             ok = c[0] >= 0 && c[0] < g.nz;
+            bool plain = true;
 #pragma unroll
             for (int a = 0; a < NDIM; ++a) {
                 o[a] = sp.off[a * sp.cap + p];
+                plain = plain && o[a] >= 0.f && o[a] <= 1.f;
                 b[a] = SHAPE == 1 ? c[a] : o[a] >= 0.5f ? c[a] : c[a] - 1;
+            }
+            if (ok && !plain) {
+                rho_one<NDIM, SHAPE>(g, sp, shift, rho, p);
+                ok = false;
             }
         }
         int* const bw = box[cur];
@@ -2445,7 +2433,7 @@ __global__ void __launch_bounds__(FUSED_T) rho_kernel(GridP g, SpeciesP sp, int 
         fits = fits && vol <= RHO_CAP;
         const int b0[3] = {bw[0], bw[1], NDIM == 3 ? bw[2] : 0};
         if (fits)
-            for (int i = threadIdx.x; i < (int)vol; i += FUSED_T) hi[i] = lo[i] = 0;
+            for (int i = threadIdx.x; i < (int)vol; i += FUSED_T) sum[0][i] = sum[1][i] = sum[2][i] = 0u;
         __syncthreads();
         if (threadIdx.x < 6) bw[threadIdx.x] = INT_MAX;     // read by all; used again two chunks on
         if (!fits) {
@@ -2453,41 +2441,38 @@ __global__ void __launch_bounds__(FUSED_T) rho_kernel(GridP g, SpeciesP sp, int 
             continue;
         }
         if (ok) {
-            PairSum wz[K], wx[K], wy[K];
-            pair_weights<SHAPE>(o[0], wz);
-            pair_weights<SHAPE>(o[1], wx);
-            if (NDIM == 3) pair_weights<SHAPE>(o[2], wy);
+            unsigned long long wz[K], wx[K], wy[K];
+            fixed_weights<SHAPE>(o[0], wz);
+            fixed_weights<SHAPE>(o[1], wx);
+            if (NDIM == 3) fixed_weights<SHAPE>(o[2], wy);
             const int at = ((NDIM == 3 ? b[2] - b0[2] : 0) * ext[1] + b[1] - b0[1]) * ext[0] + b[0] - b0[0];
 #pragma unroll
             for (int q = 0; q < (NDIM == 3 ? K : 1); ++q)
 #pragma unroll
                 for (int r = 0; r < K; ++r) {
-                    PairSum w = wx[r];
-                    if (NDIM == 3) w.scale(wy[q].h, wy[q].l);
+                    const unsigned long long w = NDIM == 3 ? __umul64hi(wx[r], wy[q]) : wx[r];
 #pragma unroll
                     for (int t = 0; t < K; ++t) {
-                        PairSum v = w;
-                        v.scale(wz[t].h, wz[t].l);
-                        const float MAGIC = 12582912.f;    // 1.5 2^23
-                        const float f1 = fmaf(v.h, 4194304.f, MAGIC);
-                        const float rest = fmaf(f1 - MAGIC, -1.f / 4194304.f, v.h) + v.l;   // |rest| < 2^-22
-                        const float f2 = fmaf(rest, 17592186044416.f, MAGIC);               // 2^44
+                        const unsigned long long v = __umul64hi(w, wz[t]);
                         const int k = at + (q * ext[1] + r) * ext[0] + t;
-                        atomicAdd(hi + k, __float_as_int(f1) - 0x4B400000);
-                        atomicAdd(lo + k, __float_as_int(f2) - 0x4B400000);
+                        atomicAdd(&sum[0][k], (unsigned)v & 0x1fffffu);
+                        atomicAdd(&sum[1][k], (unsigned)(v >> 21) & 0x1fffffu);
+                        atomicAdd(&sum[2][k], (unsigned)(v >> 42));
                     }
                 }
         }
         __syncthreads();
         const float rz = 1.f / (float)ext[0], rx = 1.f / (float)ext[1];
-        const double unit = sp.qv64 / 17592186044416.0;
+        const double unit = sp.qv64 / (NDIM == 3 ? 2305843009213693952.0 : 4611686018427387904.0);   // 2^61, 2^62
         for (int i = threadIdx.x; i < (int)vol; i += FUSED_T) {
-            if ((hi[i] | lo[i]) == 0) continue;
-            const long long v = (long long)hi[i] * 4194304 + lo[i];
+            if ((sum[0][i] | sum[1][i] | sum[2][i]) == 0u) continue;
+            // the lower two words have at most 50 bits together: exact in FP64
+            const double v = fma((double)sum[2][i], 4398046511104.0,
+                                 (double)((unsigned long long)sum[1][i] * 2097152u + sum[0][i]));
             const int r = box_div(i, rz), z = b0[0] + i - r * ext[0];
             const int q = box_div(r, rx), x = wrapi(b0[1] + r - q * ext[1], g.nx);
             const int y = NDIM == 3 ? wrapi(b0[2] + q, g.ny) : 0;
-            if ((unsigned)z < (unsigned)g.nz) atomicAdd(rho + ((long long)y * g.nx + x) * g.nz + z, unit * (double)v);
+            if ((unsigned)z < (unsigned)g.nz) atomicAdd(rho + ((long long)y * g.nx + x) * g.nz + z, unit * v);
         }
         __syncthreads();
     }

@@ -196,3 +196,49 @@ def test_gauss_residual_of_infinite_fields(M):
     assert np.array_equal(np.isinf(got), hit) and np.isfinite(got[~hit]).all()
     assert np.isinf(sim.diag()["gauss_max"])
     sim.close()
+
+
+@pytest.mark.parametrize("ndim,shape", [(2, 1), (2, 2), (3, 1), (3, 2)])
+def test_charge_density(ndim, shape):
+    """rho of five particles in one cell.  Weights in units of 2^-63 and products in units of 2^-62 and 2^-61 put a
+    contribution within 2^-59 of a particle's density; then three roundings of the node's sum."""
+    nz, nx, ny = 12, 6, 6 if ndim == 3 else 1
+    sim = Simulation(device="cuda:0", ndim=ndim, nz=nz, nx=nx, ny=ny, dz=0.5, dx=0.5, dy=0.5, dt=0.125, shape=shape)
+    qv = Fr(-1) / Fr(1, 2) ** ndim
+    rng = np.random.default_rng(10 * ndim + shape)
+    for _ in range(6):
+        off = rng.random((ndim, 5)).astype(np.float32)
+        one = np.ones(5, np.int64)
+        sim.add_species(0, 5 * one, 2 * one, 2 * one if ndim == 3 else 0 * one, off, np.zeros((3, 5), np.float32), -1.0, 1.0, 1.0)
+
+        def weights(o):
+            o = Fr(float(o))
+            if shape == 1:
+                return {0: 1 - o, 1: o}
+            b = 1 if o >= Fr(1, 2) else 0
+            d = o - b
+            return {b - 1: (Fr(1, 2) - d) ** 2 / 2, b: Fr(3, 4) - d * d, b + 1: (Fr(1, 2) + d) ** 2 / 2}
+
+        ref = {}
+        for p in range(5):
+            w = [weights(off[a, p]) for a in range(ndim)] + ([{0: Fr(1)}] if ndim == 2 else [])
+            for a, wa in w[0].items():
+                for b, wb in w[1].items():
+                    for c, wc in w[2].items():
+                        n = (c + 2 if ndim == 3 else 0, b + 2, a + 5)
+                        ref[n] = ref.get(n, Fr(0)) + qv * wa * wb * wc
+        got = sim.rho().cpu().numpy()
+        for n, v in ref.items():
+            assert abs(Fr(float(got[n])) - v) <= 3 * U * abs(v) + 5 * abs(qv) * Fr(1, 2 ** 59)
+    sim.close()
+
+
+def test_charge_density_of_an_offset_that_is_not_a_number():
+    sim = _sim(16, nx=8, shape=2)
+    one = np.ones(3, np.int64)
+    off = np.full((2, 3), 0.25, np.float32)
+    off[0, 1] = np.nan
+    sim.add_species(0, 8 * one, 4 * one, 0 * one, off, np.zeros((3, 3), np.float32), -1.0, 1.0, 1.0)
+    bad = np.isnan(sim.rho().cpu().numpy()[0])
+    assert bad[3:6, 7:10].all() and bad.sum() == 9
+    sim.close()
