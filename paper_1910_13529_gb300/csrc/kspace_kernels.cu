@@ -13,10 +13,13 @@
 //   (curl F)_1 = d_x F3 - d_y F2,  (curl F)_2 = d_y F1 - d_z F3,  (curl F)_3 = d_z F2 - d_x F1,
 // E and B scaled by 1/(nz nx ny) for the unnormalised inverse transform.  Memory per mode: 9 complex
 // values read, 6 written.
-// Between two steps of one call nothing but this update changes the fields, so their transforms stay
-// in k space (written beside the scaled copies, 12 values a mode) and the next step transforms only
-// the current: 9 transforms a step instead of 15 and fewer roundings.  Four steps of 2048 x 512
-// (spectral): 371 us before, 297 now; two of 256 x 128 x 128 (PSATD): 742 and 639.
+// Between two steps of one call nothing but this update changes the fields, so their transforms stay in k
+// space and the next step transforms only the current: 9 transforms a step instead of 15 and fewer
+// roundings.  The inverse transforms consume their input: the scaled E takes the place of J in the update
+// itself, the scaled B after E's inverse transform, by a pass of its own, so that a handle needs no more memory
+// than one that transforms everything (room for both copies, 15 arrays, saves that pass: 512 x 256, eight steps
+// 310 us for 335; everything transformed: 440).  us per call, everything transformed and now: four steps of 2048 x 512
+// (spectral) 488 and 380, two of 256 x 128 x 128 (PSATD) 826 and 720.
 #include "pic_internal.h"
 
 #include <cmath>
@@ -34,9 +37,7 @@ struct KSpaceState {
     int solver = 0;
     long long nk = 0;          // modes: (nz/2 + 1) nx ny
     int nzk = 0;
-    bool keep = false;         // buf has the second six
-    float2* buf = nullptr;     // in k space: E, B and J, then the scaled E and B that the inverse
-                               // transforms consume: 15 nk complex values
+    float2* buf = nullptr;     // E, B, J in k space: 9 nk complex values
     float4* tab = nullptr;     // per axis and index, z then x then y: spectral/KT (d+ re, d+ im,
                                // [k]_Yee / [k], 0); PSATD (cos(k h/2), sin(k h/2), k, ratio or -1)
 #ifdef PIC_HAVE_CUFFT
@@ -70,9 +71,22 @@ __device__ __forceinline__ void ccurl(float2 dz, float2 dx, float2 dy, const flo
     out[2] = csub(cmul(dz, F[1]), cmul(dx, F[0]));
 }
 
-// W: the six scaled fields for the inverse transforms; keep: E and B are also wanted in k space
-__global__ void __launch_bounds__(256) kspace_update_kernel(float2* Ek, float2* Bk,
-                                                            const float2* __restrict__ Jk, float2* W, int keep,
+// The fields for the inverse transforms are scaled: in place, or, where E and B are wanted in k space
+// as well (keep), E in the place of J.
+__device__ __forceinline__ void put_mode(float2* Ek, float2* Bk, float2* Jk, int keep, long long c, float2 e, float2 b,
+                                         float scale) {
+    (keep ? Jk : Ek)[c] = make_float2(e.x * scale, e.y * scale);
+    if (keep) Ek[c] = e;
+    Bk[c] = keep ? b : make_float2(b.x * scale, b.y * scale);
+}
+
+__global__ void __launch_bounds__(256) scaled_copy_kernel(float2* __restrict__ dst, const float2* __restrict__ src,
+                                                          long long n, float scale) {
+    for (long long i = (long long)blockIdx.x * 256 + threadIdx.x; i < n; i += (long long)gridDim.x * 256)
+        dst[i] = make_float2(src[i].x * scale, src[i].y * scale);
+}
+
+__global__ void __launch_bounds__(256) kspace_update_kernel(float2* Ek, float2* Bk, float2* Jk, int keep,
                                                             const float4* __restrict__ tab, int nzk, int nx,
                                                             long long nk, float dt, float scale) {
     const float4* tz = tab;
@@ -104,12 +118,7 @@ __global__ void __launch_bounds__(256) kspace_update_kernel(float2* Ek, float2* 
 #pragma unroll
         for (int q = 0; q < 3; ++q) {
             B[q] = cfma(-0.5f * dt, t[q], B[q]);
-            W[q * nk + m] = make_float2(E[q].x * scale, E[q].y * scale);
-            W[(3 + q) * nk + m] = make_float2(B[q].x * scale, B[q].y * scale);
-            if (keep) {
-                Ek[q * nk + m] = E[q];
-                Bk[q * nk + m] = B[q];
-            }
+            put_mode(Ek, Bk, Jk, keep, q * nk + m, E[q], B[q], scale);
         }
     }
 }
@@ -127,8 +136,7 @@ __device__ __forceinline__ float2 ci(float2 a) { return make_float2(-a.y, a.x); 
 __device__ __forceinline__ float2 cscale(float s, float2 a) { return make_float2(s * a.x, s * a.y); }
 __device__ __forceinline__ float2 cadd(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
 
-__global__ void __launch_bounds__(256) psatd_update_kernel(float2* Ek, float2* Bk,
-                                                           const float2* __restrict__ Jk, float2* W, int keep,
+__global__ void __launch_bounds__(256) psatd_update_kernel(float2* Ek, float2* Bk, float2* Jk, int keep,
                                                            const float4* __restrict__ tab, int nzk, int nx,
                                                            long long nk, float dt, float scale) {
     const float4* tz = tab;
@@ -142,11 +150,8 @@ __global__ void __launch_bounds__(256) psatd_update_kernel(float2* Ek, float2* B
         const float4 a = __ldg(tz + iz), b = __ldg(tx + ix), c = __ldg(ty + iy);
         if (a.w < 0.f || b.w < 0.f || c.w < 0.f) {          // Nyquist plane: removed
 #pragma unroll
-            for (int q = 0; q < 6; ++q) W[q * nk + m] = make_float2(0.f, 0.f);
-            if (keep) {
-#pragma unroll
-                for (int q = 0; q < 3; ++q) Ek[q * nk + m] = Bk[q * nk + m] = make_float2(0.f, 0.f);
-            }
+            for (int q = 0; q < 3; ++q)
+                put_mode(Ek, Bk, Jk, keep, q * nk + m, make_float2(0.f, 0.f), make_float2(0.f, 0.f), 0.f);
             continue;
         }
         // e^{-i k h/2} per axis (z, x, y)
@@ -205,12 +210,7 @@ __global__ void __launch_bounds__(256) psatd_update_kernel(float2* Ek, float2* B
 #pragma unroll
         for (int q = 0; q < 3; ++q) {
             const float2 e = cmul(En[q], cconj(pE[q])), b = cmul(Bn[q], cconj(pB[q]));
-            W[q * nk + m] = cscale(scale, e);
-            W[(3 + q) * nk + m] = cscale(scale, b);
-            if (keep) {
-                Ek[q * nk + m] = e;
-                Bk[q * nk + m] = b;
-            }
+            put_mode(Ek, Bk, Jk, keep, q * nk + m, e, b, scale);
         }
     }
 }
@@ -248,9 +248,8 @@ void fill_axis(std::vector<float4>& out, int solver, int axis, int n, double h, 
 
 }  // namespace
 
-// keep: room for the scaled copies as well (15 nk complex values, 9 without)
-static int kspace_create_with(const GridP& g, int solver, double dz, double dx, double dy, double dt, bool keep,
-                              KSpaceState** out, char* err, size_t nerr) {
+int kspace_create(const GridP& g, int solver, double dz, double dx, double dy, double dt, KSpaceState** out,
+                  char* err, size_t nerr) {
     *out = nullptr;
 #ifndef PIC_HAVE_CUFFT
     (void)g; (void)solver; (void)dz; (void)dx; (void)dy; (void)dt;
@@ -260,14 +259,13 @@ static int kspace_create_with(const GridP& g, int solver, double dz, double dx, 
     KSpaceState* k = new KSpaceState();
     k->g = g;
     k->solver = solver;
-    k->keep = keep;
     k->nzk = g.nz / 2 + 1;
     k->nk = (long long)k->nzk * g.nx * g.ny;
     std::vector<float4> tab;
     fill_axis(tab, solver, 0, g.nz, dz, dt, true, false);
     fill_axis(tab, solver, 1, g.nx, dx, dt, false, false);
     fill_axis(tab, solver, 2, g.ny, dy, dt, false, g.ndim == 2);
-    cudaError_t e = cudaMalloc(&k->buf, sizeof(float2) * (keep ? 15 : 9) * k->nk);
+    cudaError_t e = cudaMalloc(&k->buf, sizeof(float2) * 9 * k->nk);
     if (e == cudaSuccess) e = cudaMalloc(&k->tab, sizeof(float4) * tab.size());
     if (e == cudaSuccess) e = cudaMemcpy(k->tab, tab.data(), sizeof(float4) * tab.size(), cudaMemcpyHostToDevice);
     if (e != cudaSuccess) {
@@ -292,15 +290,6 @@ static int kspace_create_with(const GridP& g, int solver, double dz, double dx, 
     *out = k;
     return 0;
 #endif
-}
-
-// Where the memory does not reach for the copies, every step transforms the fields anew.
-int kspace_create(const GridP& g, int solver, double dz, double dx, double dy, double dt, KSpaceState** out,
-                  char* err, size_t nerr) {
-    const int r = kspace_create_with(g, solver, dz, dx, dy, dt, true, out, err, nerr);
-    if (r != 2) return r;
-    cudaGetLastError();   // the failed allocation is dealt with here
-    return kspace_create_with(g, solver, dz, dx, dy, dt, false, out, err, nerr);
 }
 
 void kspace_destroy(KSpaceState* k) {
@@ -329,10 +318,6 @@ int kspace_advance(KSpaceState* k, const float* Ein, const float* Bin, const flo
     float2* Ek = k->buf;
     float2* Bk = Ek + 3 * k->nk;
     float2* Jk = Bk + 3 * k->nk;
-    // without room for copies the scaled fields take the place of Ek and Bk, mode by mode
-    float2* W = k->keep ? Jk + 3 * k->nk : Ek;
-    cont = cont && k->keep;
-    keep = keep && k->keep;
     cufftResult r = cufftSetStream(k->r2c, s);
     if (r == CUFFT_SUCCESS) r = cufftSetStream(k->c2r, s);
     if (r == CUFFT_SUCCESS && !cont)
@@ -350,17 +335,26 @@ int kspace_advance(KSpaceState* k, const float* Ein, const float* Bin, const flo
     const unsigned nb = (unsigned)(blocks < 152 * 8 ? (blocks < 1 ? 1 : blocks) : 152 * 8);
     const float scale = (float)(1.0 / ((double)g.nz * g.nx * g.ny));
     if (k->solver == PIC_SOLVER_PSATD)
-        psatd_update_kernel<<<nb, 256, 0, s>>>(Ek, Bk, Jk, W, keep ? 1 : 0, k->tab, k->nzk, g.nx, k->nk, g.dt, scale);
+        psatd_update_kernel<<<nb, 256, 0, s>>>(Ek, Bk, Jk, keep ? 1 : 0, k->tab, k->nzk, g.nx, k->nk, g.dt, scale);
     else
-        kspace_update_kernel<<<nb, 256, 0, s>>>(Ek, Bk, Jk, W, keep ? 1 : 0, k->tab, k->nzk, g.nx, k->nk, g.dt, scale);
+        kspace_update_kernel<<<nb, 256, 0, s>>>(Ek, Bk, Jk, keep ? 1 : 0, k->tab, k->nzk, g.nx, k->nk, g.dt, scale);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) {
         snprintf(err, nerr, "k-space update kernel: %s", cudaGetErrorString(e));
         return 1;
     }
-    r = cufftExecC2R(k->c2r, reinterpret_cast<cufftComplex*>(W), reinterpret_cast<cufftReal*>(Eout));
+    float2 *We = keep ? Jk : Ek, *Wb = keep ? Jk : Bk;
+    r = cufftExecC2R(k->c2r, reinterpret_cast<cufftComplex*>(We), reinterpret_cast<cufftReal*>(Eout));
+    if (keep && r == CUFFT_SUCCESS) {
+        scaled_copy_kernel<<<nb, 256, 0, s>>>(Jk, Bk, 3 * k->nk, scale);
+        e = cudaGetLastError();
+        if (e != cudaSuccess) {
+            snprintf(err, nerr, "k-space copy kernel: %s", cudaGetErrorString(e));
+            return 1;
+        }
+    }
     if (r == CUFFT_SUCCESS)
-        r = cufftExecC2R(k->c2r, reinterpret_cast<cufftComplex*>(W + 3 * k->nk), reinterpret_cast<cufftReal*>(Bout));
+        r = cufftExecC2R(k->c2r, reinterpret_cast<cufftComplex*>(Wb), reinterpret_cast<cufftReal*>(Bout));
     if (r != CUFFT_SUCCESS) {
         snprintf(err, nerr, "cuFFT inverse transform failed (%d)", (int)r);
         return 1;

@@ -179,3 +179,40 @@ def test_psatd_drifting_charge_fields_of_appendix_b(beta):
     assert np.abs(sim.E.double().cpu().numpy() - E1).max() < TOL * scale
     assert np.abs(sim.B.double().cpu().numpy() - B1).max() < TOL * scale
     sim.close()
+
+
+@pytest.mark.parametrize("solver", ["spectral", "kt", "psatd"])
+@pytest.mark.parametrize("nd,nz,nx,ny", [(2, 95, 20, 1), (2, 96, 21, 1), (3, 32, 10, 9)])
+def test_several_steps_in_one_call(nd, nz, nx, ny, solver):
+    """Five steps in one call (E and B stay in k space between them) against five calls and the oracle, fields and
+    particles; then one more step, which starts from the fields again."""
+    grid = kgrid(nd, nz, nx, ny, solver)
+    sp = wl.random_particles(nd, nz, nx, ny, 300, seed=nz, u_scale=0.4, margin=8)
+    together, apart, osim = gpu_sim(grid, [sp]), gpu_sim(grid, [sp]), oracle_sim(grid, [sp])
+    together.step(5)
+    together.step(1)
+    for _ in range(6):
+        apart.step(1)
+        osim.step()
+    for sim in (together, apart):
+        assert field_error(sim, osim) < TOL
+        dx, du = particle_errors(sim, osim, 0, nd)
+        assert dx < TOL and du < TOL
+        sim.close()
+
+
+def test_memory_of_a_handle():
+    """A k-space handle's own memory, in floats per cell: 8 as any handle's and 9 complex values per mode; 23 when
+    it kept room for copies of the transforms."""
+    import paper_1910_13529_gb300 as P
+    from paper_1910_13529_gb300.runtime import make_config
+    nz, nx = 4096, 2048
+    taken = []
+    for _ in range(2):                                     # the first creation loads cuFFT's kernels as well
+        c, keep = make_config(ndim=2, nz=nz, nx=nx, dz=0.5, dx=0.5, dt=0.1, solver="spectral")
+        torch.cuda.synchronize()
+        before = torch.cuda.mem_get_info()[0]
+        h = P.pic_create(c)
+        taken.append((before - torch.cuda.mem_get_info()[0]) / (4 * nz * nx))
+        P.pic_destroy(h)
+    assert taken[1] < 19
