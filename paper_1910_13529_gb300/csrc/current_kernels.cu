@@ -403,9 +403,8 @@ cudaError_t launch_fc(const CorrP& p, int vec4, cudaStream_t s) {
     const size_t smem = sizeof(float) * corr_floats(p.g.nz);
     // the default limit is 48 KB for static and dynamic shared memory together
     if (smem + sizeof(float) * (8 * NT + 16) > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(filter_correct_kernel<NT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)smem);
-        if (e != cudaSuccess) return e;
+        static PerDevice granted;
+        if (cudaError_t e = allow_shared(granted, filter_correct_kernel<NT>, smem)) return e;
     }
     return launch_chained_if(few_cells(p.g), filter_correct_kernel<NT>, (unsigned)(3LL * p.g.nx * p.g.ny), NT, smem, s, p, vec4);
 }
@@ -465,12 +464,9 @@ cudaError_t launch_correct_j1(const GridP& g, const float* taps, int hlen, float
     tpr = tpr > 256 ? 256 : tpr;
     const int rpc = 256 / tpr;
     const size_t smem = sizeof(float) * corr_floats(g.nz) * rpc;
-    static size_t opted = 48 * 1024;
-    if (smem > opted) {
-        cudaError_t e = cudaFuncSetAttribute(correct_j1_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)smem);
-        if (e != cudaSuccess) return e;
-        opted = smem;
+    if (smem > 48 * 1024) {
+        static PerDevice granted;
+        if (cudaError_t e = allow_shared(granted, correct_j1_rows_kernel, smem)) return e;
     }
     return launch_chained_if(few_cells(p.g), correct_j1_rows_kernel, (unsigned)((rows + rpc - 1) / rpc), rpc * tpr, smem, s, p, rows, tpr, vec4);
 }
@@ -492,9 +488,8 @@ cudaError_t launch_correct_j1_batch(const CorrInst* inst, int ninst, int max_row
     size_t smem = sizeof(float) * pair_floats(paired);
     if (max_nz > CP_MAX_NZ && sizeof(float) * corr_floats(max_nz) > smem) smem = sizeof(float) * corr_floats(max_nz);
     if (smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(correct_j1_batch_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)smem);
-        if (e != cudaSuccess) return e;
+        static PerDevice granted;
+        if (cudaError_t e = allow_shared(granted, correct_j1_batch_kernel, smem)) return e;
     }
     correct_j1_batch_kernel<<<dim3((unsigned)((max_rows + 1) / 2), (unsigned)ninst), CP_NT, smem, s>>>(inst);
     return cudaGetLastError();

@@ -1321,13 +1321,8 @@ template <int NDIM, int MAXM, int TZ, int TX, int TY>
 cudaError_t launch_fa(const FieldP& p, cudaStream_t s) {
     using T = Tile<NDIM, MAXM, TZ, TX, TY>;
     auto k = field_advance_kernel<NDIM, MAXM, TZ, TX, TY>;
-    static bool configured = false;   // attribute is per function; setting it twice is harmless
-    if (!configured) {
-        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)T::smem_bytes);
-        if (e != cudaSuccess) return e;
-        configured = true;
-    }
+    static PerDevice granted;
+    if (cudaError_t e = allow_shared(granted, k, T::smem_bytes)) return e;
     dim3 grid((p.g.nz + TZ - 1) / TZ, (p.g.nx + TX - 1) / TX, NDIM == 3 ? (p.g.ny + TY - 1) / TY : 1);
     return launch_chained_if(chain_fields(p.g), k, grid, 256, T::smem_bytes, s, p);
 }
@@ -1336,13 +1331,8 @@ template <int NDIM, int MAXM, int TZ, int TX, int TY>
 cudaError_t launch_fa_rb(const FieldP& p, cudaStream_t s) {
     using T = TileRB<NDIM, MAXM, TZ, TX, TY>;
     auto k = field_advance_rb_kernel<NDIM, MAXM, TZ, TX, TY>;
-    static bool configured = false;
-    if (!configured) {
-        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)T::smem_bytes);
-        if (e != cudaSuccess) return e;
-        configured = true;
-    }
+    static PerDevice granted;
+    if (cudaError_t e = allow_shared(granted, k, T::smem_bytes)) return e;
     dim3 grid((p.g.nz + TZ - 1) / TZ, (p.g.nx + TX - 1) / TX, NDIM == 3 ? (p.g.ny + TY - 1) / TY : 1);
     return launch_chained_if(chain_fields(p.g), k, grid, 256, T::smem_bytes, s, p);
 }
@@ -1374,12 +1364,8 @@ template <int MAXM, int TZ, int TX, int NT>
 cudaError_t launch_fa_march(const FieldP& p, cudaStream_t s) {
     using T = MarchT<MAXM, TZ, TX>;
     auto k = field_advance_march_kernel<MAXM, TZ, TX, NT>;
-    static bool configured = false;
-    if (!configured) {
-        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)T::smem_bytes);
-        if (e != cudaSuccess) return e;
-        configured = true;
-    }
+    static PerDevice granted;
+    if (cudaError_t e = allow_shared(granted, k, T::smem_bytes)) return e;
     // y chunks: about four waves of CTAs over the SMs, each chunk at least 8 planes
     int dev = 0, nsm = 152;
     cudaGetDevice(&dev);
@@ -1392,7 +1378,7 @@ cudaError_t launch_fa_march(const FieldP& p, cudaStream_t s) {
     return launch_chained_if(chain_fields(p.g), k, grid, NT, T::smem_bytes, s, p, yc);
 }
 
-// CTAs of k that one SM holds (k already has its shared-memory limit), once per kernel
+// CTAs of k that one SM holds (k already has its shared-memory limit)
 template <typename K>
 int resident_ctas(K k, int nt, size_t smem) {
     int n = 0;
@@ -1410,12 +1396,9 @@ template <int MAXM, int NT, bool VEC>
 cudaError_t launch_fa_rows_v(const FieldP& p, cudaStream_t s) {
     using T = RowT<MAXM, NT, VEC>;
     auto k = field_advance_rows_kernel<MAXM, NT, VEC>;
-    static int per_sm = 0;
-    if (!per_sm) {
-        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)T::smem_bytes);
-        if (e != cudaSuccess) return e;
-        per_sm = resident_ctas(k, NT, T::smem_bytes);
-    }
+    static PerDevice granted, resident;
+    if (cudaError_t e = allow_shared(granted, k, T::smem_bytes)) return e;
+    const int per_sm = resident.number(current_device(), [&] { return resident_ctas(k, NT, T::smem_bytes); });
     // equal segments along z; x chunks for one wave of CTAs, each of at least 8 rows (a chunk's first
     // two rows of B^{n+1/2} and one of E^{n+1} are computed by its neighbours as well)
     const int nseg = (p.g.nz + T::OUT - 1) / T::OUT, tz = row_segment(p.g.nz, nseg);
@@ -1433,12 +1416,8 @@ template <int MAXM, int TZ, int TX, int NT>
 cudaError_t launch_fa_march_ring(const FieldP& p, cudaStream_t s) {
     using T = MarchRingT<MAXM, TZ, TX>;
     auto k = field_advance_march_ring_kernel<MAXM, TZ, TX, NT>;
-    static bool configured = false;
-    if (!configured) {
-        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)T::smem_bytes);
-        if (e != cudaSuccess) return e;
-        configured = true;
-    }
+    static PerDevice granted;
+    if (cudaError_t e = allow_shared(granted, k, T::smem_bytes)) return e;
     // y chunks: one wave of CTAs, each chunk at least 8 planes
     int dev = 0, nsm = 152;
     cudaGetDevice(&dev);
@@ -1456,12 +1435,8 @@ cudaError_t launch_fa_batch(const FieldP* inst, const int4* work, int total, int
                             cudaStream_t s) {
     using T = Tile<NDIM, MAXM, TZ, TX, TY>;
     auto k = field_advance_batch_kernel<NDIM, MAXM, TZ, TX, TY>;
-    static bool configured = false;
-    if (!configured) {
-        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)T::smem_bytes);
-        if (e != cudaSuccess) return e;
-        configured = true;
-    }
+    static PerDevice granted;
+    if (cudaError_t e = allow_shared(granted, k, T::smem_bytes)) return e;
     k<<<(unsigned)total, 256, T::smem_bytes, s>>>(inst, work, parity);
     return cudaGetLastError();
 }
@@ -1473,12 +1448,8 @@ cudaError_t launch_fa_rb_batch(const FieldP* inst, const int4* work, int total, 
                                cudaStream_t s) {
     using T = TileRB<NDIM, MAXM, TZ, TX, TY>;
     auto k = field_advance_rb_batch_kernel<NDIM, MAXM, TZ, TX, TY>;
-    static bool configured = false;
-    if (!configured) {
-        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)T::smem_bytes);
-        if (e != cudaSuccess) return e;
-        configured = true;
-    }
+    static PerDevice granted;
+    if (cudaError_t e = allow_shared(granted, k, T::smem_bytes)) return e;
     k<<<(unsigned)total, 256, T::smem_bytes, s>>>(inst, work, parity);
     return cudaGetLastError();
 }
@@ -1487,13 +1458,10 @@ cudaError_t launch_fa_rb_batch(const FieldP* inst, const int4* work, int total, 
 template <int MAXM>
 int rows_batch_slots_m() {
     using T = RowT<MAXM, ROWS_BATCH_NT, false>;
-    static int per_sm = 0;
-    if (!per_sm) {
-        auto k = field_advance_rows_batch_kernel<MAXM, ROWS_BATCH_NT>;
-        if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)T::smem_bytes) != cudaSuccess)
-            return 1;
-        per_sm = resident_ctas(k, ROWS_BATCH_NT, T::smem_bytes);
-    }
+    auto k = field_advance_rows_batch_kernel<MAXM, ROWS_BATCH_NT>;
+    static PerDevice granted, resident;
+    if (allow_shared(granted, k, T::smem_bytes) != cudaSuccess) return 1;
+    const int per_sm = resident.number(current_device(), [&] { return resident_ctas(k, ROWS_BATCH_NT, T::smem_bytes); });
     return sm_count() * per_sm;
 }
 

@@ -2539,24 +2539,16 @@ cudaError_t launch_push(const GridP& g0, const SpeciesP& sp, const float* E, con
             auto k = push_deposit_2d_kernel<SH>;
             const unsigned ctas = pblocks(extent);
             const size_t smem = spread_shared(ctas, SMEM_2D * sizeof(float));
-            static size_t granted = 0;
-            if (smem > granted) {
-                cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-                if (e != cudaSuccess) return e;
-                granted = smem;
-            }
+            static PerDevice granted;
+            if (cudaError_t e = allow_shared(granted, k, smem)) return e;
             return launch_split(true, STEP_CARVEOUT, k, ctas, FUSED_T, smem, s, g, sp, E, B, J, shift);
         } else if (mode == MODE_FUSED) {
             const size_t smem = SMEM_3D * sizeof(float);
             CUtensorMap mapE{}, mapB{};
             const bool tma = field_box_map(&mapE, E, g) && field_box_map(&mapB, B, g);
             auto k = tma ? push_deposit_3d_kernel<SH, true> : push_deposit_3d_kernel<SH, false>;
-            static bool configured[2] = {false, false};
-            if (!configured[tma]) {
-                cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-                if (e != cudaSuccess) return e;
-                configured[tma] = true;
-            }
+            static PerDevice granted[2];
+            if (cudaError_t e = allow_shared(granted[tma], k, smem)) return e;
             return launch_chained(k, pblocks(extent), FUSED_T, smem, s, g, sp, E, B, J, shift, defer,
                                   defer + defer_len(sp.cap), mapE, mapB, status);
         } else {
@@ -2584,12 +2576,8 @@ cudaError_t launch_push_leftover(const GridP& g0, const SpeciesP* sp, int* const
         (void)nd;
         auto k = push_deposit_3d_leftover_kernel<decltype(sh)::value>;
         const size_t smem = SMEM_3D_GEN * sizeof(float);
-        static bool configured = false;
-        if (!configured) {
-            cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            if (e != cudaSuccess) return e;
-            configured = true;
-        }
+        static PerDevice granted;
+        if (cudaError_t e = allow_shared(granted, k, smem)) return e;
         // the lists' lengths are on the device: full grids, or one CTA per chunk and per warp of a small extent
         const long long want = nchunk * (FUSED_T / 32);
         cudaError_t e = launch_chained(k, (unsigned)(nchunk < 152 * 2 ? nchunk : 152 * 2), FUSED_T, smem, s, g, lp, E, B, J, shift);
@@ -2609,23 +2597,15 @@ cudaError_t launch_push_batch(const PartInst* inst, int ninst, int ndim, int sha
         if (ND == 2) {
             auto k = push_deposit_2d_batch_kernel<SH>;
             const size_t smem = SMEM_2D * sizeof(float);
-            static bool configured = false;
-            if (!configured) {
-                cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-                if (e != cudaSuccess) return e;
-                configured = true;
-            }
+            static PerDevice granted;
+            if (cudaError_t e = allow_shared(granted, k, smem)) return e;
             k<<<grid, FUSED_T, smem, s>>>(inst, parity);
             return cudaGetLastError();
         }
         auto k = push_deposit_3d_batch_kernel<SH>;
         const size_t smem = SMEM_3D * sizeof(float);
-        static bool configured = false;
-        if (!configured) {
-            cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            if (e != cudaSuccess) return e;
-            configured = true;
-        }
+        static PerDevice granted;
+        if (cudaError_t e = allow_shared(granted, k, smem)) return e;
         k<<<grid, FUSED_T, smem, s>>>(inst, parity);
         return cudaGetLastError();
     });

@@ -6,6 +6,7 @@
 #include <cuda_runtime.h>
 
 #include "../../include/pic.h"
+#include "per_device.h"
 
 namespace pic {
 
@@ -177,6 +178,17 @@ cudaError_t launch_chained_if(bool chain, void (*k)(P...), dim3 grid, dim3 block
 template <typename... P, typename... A>
 cudaError_t launch_chained(void (*k)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A&&... args) {
     return launch_chained_if(true, k, grid, block, smem, s, static_cast<A&&>(args)...);
+}
+inline int current_device() {
+    int dev = -1;
+    return cudaGetDevice(&dev) == cudaSuccess ? dev : -1;
+}
+// Allows k `bytes` of dynamic shared memory on the current device; granted: the launch's own static.
+template <typename K>
+cudaError_t allow_shared(PerDevice& granted, K k, size_t bytes) {
+    return (cudaError_t)granted.grant(current_device(), (int)bytes, [&] {
+        return (int)cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    });
 }
 inline bool few_cells(const GridP& g) { return g.ncell <= CHAIN_CELLS; }
 #endif

@@ -44,3 +44,50 @@ def test_cell_counts_are_not_narrowed(name):
     text = open(os.path.join(CSRC, name)).read()
     assert not re.search(r"\(int\)\s*\w+(\.|->)ncell", text)
     assert not re.search(r"\bint\s+\w+\s*=\s*\w+(\.|->)ncell", text)
+
+
+def test_launch_setup_is_kept_per_device(tmp_path):
+    """PerDevice: a device that has not been set up is, one that has been is not, a larger amount is granted again, a failure
+    is not remembered, and threads that ask together are granted once and for the largest amount."""
+    source = r"""#include "per_device.h"
+    #include <cstdio>
+    #include <thread>
+    #include <vector>
+    int main() {
+      static pic::PerDevice p;
+      int calls = 0;
+      auto ask = [&](int dev, int amount, int err) { return p.grant(dev, amount, [&] { ++calls; return err; }); };
+      ask(0, 100, 0); ask(0, 100, 0); ask(0, 50, 0);
+      std::printf("%d ", calls);
+      ask(1, 100, 0);
+      std::printf("%d ", calls);
+      ask(0, 200, 0); ask(0, 150, 0);
+      std::printf("%d ", calls);
+      const int failed = ask(2, 10, 7), again = ask(2, 10, 0);
+      std::printf("%d %d %d ", failed, again, calls);
+      ask(-1, 10, 0); ask(-1, 10, 0); ask(1000, 10, 0);
+      std::printf("%d\n", calls);
+      static pic::PerDevice q, r;
+      int sets = 0, last = 0;
+      std::vector<std::thread> t;
+      for (int k = 0; k < 8; ++k)
+        t.emplace_back([&, k] { for (int i = 0; i < 2000; ++i)
+          q.grant(3, 1 + (i + 250 * k) % 2000, [&] { ++sets; last = 1 + (i + 250 * k) % 2000; return 0; }); });
+      for (auto& x : t) x.join();
+      int asked = 0;
+      auto make = [&] { return ++asked == 1 ? 0 : 5; };
+      const int none = r.number(0, make), five = r.number(0, make), kept = r.number(0, make), other = r.number(1, make);
+      std::printf("%d %d %d %d %d %d\n", last, none, five, kept, other, asked);
+    }"""
+    lines = run_cpp(tmp_path, source).splitlines()
+    assert lines[0].split() == ["1", "2", "3", "7", "0", "5", "8"]
+    # the last amount set is the largest asked for: none was lowered after it
+    assert lines[1].split() == ["2000", "0", "5", "5", "5", "3"]
+
+
+def test_launches_keep_no_state_of_one_device():
+    """No launch remembers in a plain static what belongs to the device that was current."""
+    for name in os.listdir(CSRC):
+        if name.endswith((".cu", ".h")):
+            text = open(os.path.join(CSRC, name)).read()
+            assert not re.search(r"^\s*static (bool|int|size_t|unsigned|long long) \w+\s*(\[\d+\]\s*)?=", text, flags=re.M), name
