@@ -326,7 +326,8 @@ pic_status pic_adjoint_run(pic_t* h, int nsteps, const float* E, const float* B,
 /* ---- tile autotuner ----------------------------------------------------------------------
  * pic_autotune times each field-advance tile variant on the handle's bound fields (results go
  * to library scratch; the state is unchanged; synchronises stream) and keeps the fastest for
- * later steps.  The choice is cached per (ndim, stencil class, grid) for the process.
+ * later steps.  The choice is cached per device, (ndim, stencil class, grid) and whether the bound
+ * arrays can be moved in 16-byte groups, for the process.
  * pic_get_tuning: chosen variant, per-variant time in ms (0: not timed; ms needs
  * PIC_MAX_TILE_VARIANTS entries) and the number of variants.  2D (z x x): 0 = 128x8,
  * 1 = 256x4, 2 = 64x16, 3 = 256x8 with one cell per thread and stage, 4 = 128x8, 5 = 256x4,

@@ -1689,10 +1689,14 @@ cudaError_t launch_fa_variant(const FieldP& p, int v, cudaStream_t s) {
 bool aligned16(const void* q) { return ((uintptr_t)q & 15) == 0; }
 }  // namespace
 
+int field_vec4(const FieldP& p) {
+    return (p.g.nz % 4 == 0) && aligned16(p.Ein) && aligned16(p.Bin) && aligned16(p.J1) && aligned16(p.J2) &&
+           aligned16(p.J3) && aligned16(p.Eout) && aligned16(p.Bout);
+}
+
 cudaError_t launch_field_advance(const FieldP& p_in, cudaStream_t s, int variant) {
     FieldP p = p_in;
-    p.vec4 = (p.g.nz % 4 == 0) && aligned16(p.Ein) && aligned16(p.Bin) && aligned16(p.J1) && aligned16(p.J2) &&
-             aligned16(p.J3) && aligned16(p.Eout) && aligned16(p.Bout);
+    p.vec4 = field_vec4(p);
     const int M = p.st.M;
     if (p.g.ndim == 2) {
         if (M <= 1) return launch_fa_variant<2, 1>(p, variant, s);

@@ -8,6 +8,7 @@
 #include <cstring>
 #include <new>
 #include <algorithm>
+#include <mutex>
 #include <vector>
 
 #include "pic_internal.h"
@@ -904,20 +905,16 @@ pic_status pic_adjoint_run(pic_t* h, int nsteps, const float* E, const float* B,
 
 // Tile autotuner: time every field-advance tile variant on this handle's bound fields (the
 // output goes to the library's second buffer, so the state is unchanged) and keep the fastest.
-// The choice is cached per (ndim, stencil class, nz, nx, ny) for the process.
+// The choice is cached per device, (ndim, stencil class, nz, nx, ny) and whether rows can be moved in 16-byte
+// groups (other kernels than where they cannot) for the process.
 pic_status pic_autotune(pic_t* h, void* stream) {
     if (!h) return PIC_ERR_ARG;
     pic_status st = need_fields(h);
     if (st) return st;
     if (h->ks) return PIC_OK;           // one k-space advance: nothing to choose
+    static std::mutex lock;
     static std::vector<std::pair<std::vector<long long>, int>> cache;
     const int mclass = h->st.M <= 1 ? 1 : h->st.M <= 4 ? 4 : h->st.M <= 8 ? 8 : 16;
-    std::vector<long long> key = {h->g.ndim, mclass, h->g.nz, h->g.nx, h->g.ny};
-    for (auto& e : cache)
-        if (e.first == key) {
-            h->fa_variant = e.second;
-            return PIC_OK;
-        }
     cudaStream_t s = (cudaStream_t)stream;
     const long long N = h->g.ncell;
     FieldP p;
@@ -931,6 +928,15 @@ pic_status pic_autotune(pic_t* h, void* stream) {
     p.Eout = h->E2;
     p.Bout = h->B2;
     p.shift = 0;
+    std::vector<long long> key = {h->device, field_vec4(p), h->g.ndim, mclass, h->g.nz, h->g.nx, h->g.ny};
+    {
+        std::lock_guard<std::mutex> hold(lock);
+        for (auto& e : cache)
+            if (e.first == key) {
+                h->fa_variant = e.second;
+                return PIC_OK;
+            }
+    }
     cudaEvent_t a, b;
     CK(h, cudaEventCreate(&a), "event");
     CK(h, cudaEventCreate(&b), "event");
@@ -960,6 +966,7 @@ pic_status pic_autotune(pic_t* h, void* stream) {
     cudaEventDestroy(a);
     cudaEventDestroy(b);
     h->fa_variant = best;
+    std::lock_guard<std::mutex> hold(lock);
     cache.push_back({key, best});
     return PIC_OK;
 }

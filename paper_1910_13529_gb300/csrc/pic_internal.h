@@ -199,6 +199,7 @@ cudaError_t launch_field_advance(const FieldP& p, cudaStream_t s, int variant = 
 cudaError_t launch_zero(float* f, long long n, cudaStream_t s);
 cudaError_t launch_copy2(float* d0, const float* s0, float* d1, const float* s1, long long n, cudaStream_t s);
 int field_variants(int ndim);
+int field_vec4(const FieldP& p);     // 1: its arrays can be moved in 16-byte groups
 int default_field_variant(const GridP& g, int M);
 
 // batched: instance tables live in device memory

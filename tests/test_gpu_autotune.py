@@ -139,3 +139,20 @@ def test_marching_variants_across_chunks(nd, nz, nx, ny, solver, C, variants):
             assert sim.state()[1] == osim.shifts
             assert field_error(sim, osim) < 1e-5, (v, moving)
             sim.close()
+
+
+def test_choice_is_not_shared_between_aligned_and_unaligned_arrays():
+    """A handle whose bound arrays do not start on 16 bytes runs other kernels than one of the same grid whose arrays do:
+    it is timed itself; a third, aligned again, takes the first one's choice."""
+    from paper_1910_13529_gb300 import pic_bind_fields
+    timed = []
+    for shifted in (False, True, False):
+        grid = dict(ndim=2, nz=516, nx=36, ny=1, dz=0.5, dx=0.4, dy=1.0, dt=0.08, solver="custom", shape=1)
+        sim = gpu_sim(grid, [], coef=TABLE1)
+        n = sim.E.numel()
+        keep = [torch.zeros(n + 4, dtype=torch.float32, device="cuda")[1 if shifted else 0:] for _ in range(3)]
+        pic_bind_fields(sim.h, *(t.data_ptr() for t in keep))
+        _, ms = sim.autotune()
+        timed.append(bool(np.all(ms > 0)))
+        sim.close()
+    assert timed == [True, True, False]
