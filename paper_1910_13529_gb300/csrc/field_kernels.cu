@@ -1604,6 +1604,8 @@ cudaError_t launch_zero(float* f, long long n, cudaStream_t s) {
     return launch_chained(zero_kernel, chain_blocks(n), 256, 0, s, f, n);
 }
 
+int copy2_launches(long long n) { return n > CHAIN_FLOATS ? 2 : 1; }
+
 cudaError_t launch_copy2(float* d0, const float* s0, float* d1, const float* s1, long long n, cudaStream_t s) {
     if (n > CHAIN_FLOATS) {
         cudaError_t e = cudaMemcpyAsync(d0, s0, sizeof(float) * n, cudaMemcpyDeviceToDevice, s);

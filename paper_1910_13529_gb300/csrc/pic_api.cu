@@ -205,7 +205,7 @@ pic_status advance_fields(pic_t* h, const float* Ein, const float* Bin, float* E
     p.Bout = Bout;
     p.shift = shift;
     if (h->ks) {
-        Scope sc(h, PIC_T_FIELDS, 1, s);
+        Scope sc(h, PIC_T_FIELDS, last ? 1 : 2, s);      // the update, and the copy of the B that is kept
         char kerr[256] = {0};
         if (kspace_advance(h->ks, Ein, Bin, h->J, Eout, Bout, !first, !last, s, kerr, sizeof kerr))
             return fail(h, PIC_ERR_CUDA, "%s", kerr);
@@ -660,7 +660,7 @@ pic_status pic_field_advance(pic_t* h, void* stream) {
     cudaStream_t s = (cudaStream_t)stream;
     const long long N = h->g.ncell;
     if ((st = advance_fields(h, h->E, h->B, h->E2, h->B2, true, true, s))) return st;
-    Scope sc(h, PIC_T_FIELDS, 2, s);
+    Scope sc(h, PIC_T_FIELDS, copy2_launches(3 * N), s);
     CK(h, launch_copy2(h->E, h->E2, h->B, h->B2, 3 * N, s), "copy E, B");
     h->state = 0;
     return PIC_OK;
@@ -685,7 +685,7 @@ pic_status pic_step(pic_t* h, int nsteps, void* stream) {
         Bn = t;
     }
     if (Ec != h->E) {
-        Scope sc(h, PIC_T_FIELDS, 2, s);
+        Scope sc(h, PIC_T_FIELDS, copy2_launches(3 * N), s);
         CK(h, launch_copy2(h->E, Ec, h->B, Bc, 3 * N, s), "copy E, B");
     }
     h->state = 0;

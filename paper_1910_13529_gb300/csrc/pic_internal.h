@@ -198,6 +198,7 @@ cudaError_t launch_field_advance(const FieldP& p, cudaStream_t s, int variant = 
 // f = 0 (n floats); d0 = s0 and d1 = s1 (n floats each)
 cudaError_t launch_zero(float* f, long long n, cudaStream_t s);
 cudaError_t launch_copy2(float* d0, const float* s0, float* d1, const float* s1, long long n, cudaStream_t s);
+int copy2_launches(long long n);     // 1 kernel, or 2 copies
 int field_variants(int ndim);
 int field_vec4(const FieldP& p);     // 1: its arrays can be moved in 16-byte groups
 int default_field_variant(const GridP& g, int M);

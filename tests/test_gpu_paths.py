@@ -261,3 +261,25 @@ def test_correction_in_pairs_of_rows(nz, nx, ny):
     assert np.abs(J - osim.J).max() < TOL * np.abs(osim.J).max()
     assert field_error(sim, osim) < TOL
     sim.close()
+
+
+@pytest.mark.parametrize("nz,nx,copies", [(64, 32, 1), (1500, 800, 2)])
+def test_counted_launches(nz, nx, copies):
+    """pic_timing_read counts what is launched: a call that ends in the second field buffers copies E and B back by one
+    kernel, on large grids by two copies."""
+    import paper_1910_13529_gb300 as P
+    grid = dict(ndim=2, nz=nz, nx=nx, ny=1, dz=0.5, dx=0.5, dy=1.0, dt=0.1, solver="yee", shape=1)
+    sim = gpu_sim(grid, [wl.random_particles(2, nz, nx, 1, 50, seed=1)])
+    for nsteps in (1, 2, 3):
+        P.pic_timing(sim.h, 1)
+        sim.step(nsteps)
+        _, n = P.pic_timing_read(sim.h, sim.stream)
+        P.pic_timing(sim.h, 0)
+        assert n["fields"] == nsteps + (copies if nsteps % 2 else 0)
+        assert n["deposit"] == n["particles"] == nsteps
+    P.pic_timing(sim.h, 1)
+    sim.gather_push()
+    sim.deposit()
+    sim.field_advance()
+    assert P.pic_timing_read(sim.h, sim.stream)[1]["fields"] == 1 + copies
+    sim.close()
