@@ -279,6 +279,11 @@ pic_status pic_set_state(pic_t* h, int64_t step, int64_t shifts, int pending_shi
 
 /* Synchronise stream and report any CUDA or device-side error. */
 pic_status pic_sync(pic_t* h, void* stream);
+/* Limit of the particle kernel's wait for a copy of its fields, in looks of up to a microsecond (2^20 when the
+ * handle is created).  Where it runs out the kernel reports PIC_ERR_TIMEOUT through pic_sync and pic_diag,
+ * waits once more, by the limit at creation, for what it has in flight, and stops; the step is not valid.  0 gives
+ * up before the first look, which shows that path without anything going wrong.                   */
+pic_status pic_set_wait_limit(pic_t* h, int polls);
 
 /* ---- kernel timing (CUDA events on the caller's stream) --------------------------------
  * pic_timing(h, 1) starts collecting: every later kernel launch of h is bracketed by a pair

@@ -30,7 +30,7 @@ EXPORTS = ["pic_create", "pic_destroy", "pic_last_error", "pic_fit_coefficients"
            "pic_deposit", "pic_field_advance", "pic_step", "pic_filter_current", "pic_sort", "pic_diag", "pic_rho", "pic_gauss",
            "pic_get_count", "pic_get_state", "pic_sync", "pic_timing", "pic_timing_read", "pic_gauss_static",
            "pic_batch_create", "pic_batch_instance", "pic_batch_step", "pic_batch_destroy", "pic_batch_get_tuning",
-           "pic_autotune", "pic_get_tuning", "pic_set_tuning", "pic_adjoint_step",
+           "pic_autotune", "pic_get_tuning", "pic_set_tuning", "pic_set_wait_limit", "pic_adjoint_step",
            "pic_step_record", "pic_adjoint_run", "pic_set_state", "pic_get_next_id"]
 TIMING_KEYS = ["particles", "deposit", "correction", "fields", "sort", "window", "diag", "filter"]
 
@@ -100,6 +100,7 @@ def _load():
         "pic_autotune": ([vp, vp], ctypes.c_int),
         "pic_get_tuning": ([vp, ip, dp, ip], ctypes.c_int),
         "pic_set_tuning": ([vp, ctypes.c_int], ctypes.c_int),
+        "pic_set_wait_limit": ([vp, ctypes.c_int], ctypes.c_int),
         "pic_adjoint_step": ([vp, vp, vp, vp, vp, vp, vp, vp], ctypes.c_int),
         "pic_step_record": ([vp, ctypes.c_int, vp, vp, vp, vp], ctypes.c_int),
         "pic_adjoint_run": ([vp, ctypes.c_int, vp, vp, vp, vp, vp, vp, vp], ctypes.c_int),
@@ -304,6 +305,10 @@ def pic_get_tuning(h):
 
 def pic_set_tuning(h, variant):
     _check(lib.pic_set_tuning(h, int(variant)), h)
+
+
+def pic_set_wait_limit(h, polls):
+    _check(lib.pic_set_wait_limit(h, int(polls)), h)
 
 
 def pic_adjoint_step(h, E_ptr, B_ptr, J_ptr, aE_ptr, aB_ptr, grad_ptr, stream):

@@ -1099,10 +1099,10 @@ __device__ __noinline__ void deposit3_global(const GridP g, float qv, const Pos 
     deposit<3, SHAPE>(g, qv, 0.f, p0, p1, acc);
 }
 
-// Waits for phase `parity` of an mbarrier that a TMA copy completes; gives up after about a second
-// (false).
-__device__ __forceinline__ bool mbar_wait(unsigned bar, unsigned parity) {
-    for (int k = 0; k < (1 << 20); ++k) {
+// Waits for phase `parity` of an mbarrier that a TMA copy completes; gives up after `polls` looks of up to
+// a microsecond each (false).
+__device__ __forceinline__ bool mbar_wait(unsigned bar, unsigned parity, int polls) {
+    for (int k = 0; k < polls; ++k) {
         unsigned done;
         asm volatile("{\n.reg .pred q;\nmbarrier.try_wait.parity.shared::cta.b64 q, [%1], %2, 0x3e8;\n"
                      "selp.u32 %0, 1, 0, q;\n}\n"
@@ -1148,7 +1148,7 @@ __device__ __forceinline__ void push_deposit_3d_chunks(const GridP& g, const Spe
                                                        long long stride, float* sF, float* sJ, int* box,
                                                        int* __restrict__ defer, int* __restrict__ defer2,
                                                        const CUtensorMap* mapE, const CUtensorMap* mapB,
-                                                       unsigned long long* mbar, int* status) {
+                                                       unsigned long long* mbar, int* status, int polls) {
     constexpr int K = Shape<SHAPE>::K;
     constexpr int KW = K + 1;
     const long long n = *sp.count;
@@ -1319,9 +1319,9 @@ __device__ __forceinline__ void push_deposit_3d_chunks(const GridP& g, const Spe
             list[2 + atomicAdd(list, 1)] = (int)(base / FUSED_T);
         }
         if (e.tma) {
-            if (!mbar_wait(bar, parity)) {         // the copy did not arrive: report, give it more time, stop
+            if (!mbar_wait(bar, parity, polls)) {  // the copy did not arrive: report, give it more time, stop
                 atomicOr(status, STATUS_TIMEOUT);
-                mbar_wait(bar, parity);
+                mbar_wait(bar, parity, WAIT_POLLS);
                 box[BW_ABORT] = 1;
             }
             parity ^= 1;
@@ -1576,14 +1576,14 @@ __global__ void __launch_bounds__(FUSED_T, 3) push_deposit_3d_kernel(GridP g, Sp
                                                                      int shift, int* __restrict__ defer,
                                                                      int* __restrict__ defer2,
                                                                      const __grid_constant__ CUtensorMap mapE,
-                                                                     const __grid_constant__ CUtensorMap mapB, int* status) {
+                                                                     const __grid_constant__ CUtensorMap mapB, int* status, int polls) {
     chain_enter();
     extern __shared__ __align__(128) float4 smem4[];
     float* smem = reinterpret_cast<float*>(smem4);
     __shared__ int box[BW_SHARED];
     __shared__ __align__(8) unsigned long long mbar;
     push_deposit_3d_chunks<SHAPE, true, TMA>(g, sp, E, B, J, shift, blockIdx.x, gridDim.x, smem, smem + 6 * FV3, box,
-                                             defer, defer2, &mapE, &mapB, &mbar, status);
+                                             defer, defer2, &mapE, &mapB, &mbar, status, polls);
 }
 
 constexpr int SMEM_3D_GEN = F_CAP3 + J_CAP3 + 2 * PF3 * FUSED_T;
@@ -2010,7 +2010,7 @@ __global__ void __launch_bounds__(FUSED_T, 2) push_deposit_3d_batch_kernel(const
     const PartInst& q = inst[blockIdx.y];
     const GridP g = prep_device(q.g);
     push_deposit_3d_chunks<SHAPE, false, false>(g, q.sp, q.E[parity], q.B[parity], q.J, 0, blockIdx.x, gridDim.x, smem,
-                                                smem + 6 * FV3, box, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr);
+                                                smem + 6 * FV3, box, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, 0);
 }
 
 template <int SHAPE>
@@ -2530,7 +2530,7 @@ bool field_box_map(CUtensorMap* map, const float* F, const GridP& g) {
 }  // namespace
 
 cudaError_t launch_push(const GridP& g0, const SpeciesP& sp, const float* E, const float* B, float* J,
-                        int shift, int mode, long long extent, int* defer, int* status, cudaStream_t s) {
+                        int shift, int mode, long long extent, int* defer, int* status, int polls, cudaStream_t s) {
     const GridP g = prep(g0);
     if (extent <= 0) return cudaSuccess;
     return dispatch(g.ndim, g.shape, [&](auto nd, auto sh) {
@@ -2550,7 +2550,7 @@ cudaError_t launch_push(const GridP& g0, const SpeciesP& sp, const float* E, con
             static PerDevice granted[2];
             if (cudaError_t e = allow_shared(granted[tma], k, smem)) return e;
             return launch_chained(k, pblocks(extent), FUSED_T, smem, s, g, sp, E, B, J, shift, defer,
-                                  defer + defer_len(sp.cap), mapE, mapB, status);
+                                  defer + defer_len(sp.cap), mapE, mapB, status, polls);
         } else {
             return launch_chained(push_kernel<ND, SH>, pblocks(extent), 256, 0, s, g, sp, E, B, shift);
         }

@@ -71,6 +71,7 @@ struct pic_t {
     float* adj_scratch = nullptr; // adjoint: E' of the step (3 N floats)
     double* static_rho = nullptr; // device address of g_static_rho on this handle's device
     int fa_variant = 0;           // field-advance tile variant (pic_autotune)
+    int wait_polls = WAIT_POLLS;  // limit of the particle kernel's waits for its field copies
     KSpaceState* ks = nullptr;    // k-space solvers: transforms, buffers and symbol tables
     double fa_ms[PIC_MAX_TILE_VARIANTS] = {0};   // measured time per variant (ms), 0 = not measured
 };
@@ -341,7 +342,7 @@ pic_status one_step(pic_t* h, const float* Ein, const float* Bin, float* Eout, f
         defers[nsp] = q.defer;
         extents[nsp++] = q.extent;
         Scope sc(h, PIC_T_PARTICLES, 1, s);
-        CK(h, launch_push(h->g, sp, Ein, Bin, h->J, h->pending_shift, 0, q.extent, q.defer, h->status, s),
+        CK(h, launch_push(h->g, sp, Ein, Bin, h->J, h->pending_shift, 0, q.extent, q.defer, h->status, h->wait_polls, s),
            "fused push/deposit kernel");
     }
     if (h->cfg.ndim == 3 && nsp > 0) {
@@ -623,7 +624,7 @@ pic_status pic_gather_push(pic_t* h, void* stream) {
         }
         SpeciesP sp = species_params(h, i);
         Scope sc(h, PIC_T_PARTICLES, 1, s);
-        CK(h, launch_push(h->g, sp, h->E, h->B, nullptr, h->pending_shift, 1, q.extent, nullptr, h->status, s),
+        CK(h, launch_push(h->g, sp, h->E, h->B, nullptr, h->pending_shift, 1, q.extent, nullptr, h->status, h->wait_polls, s),
            "push kernel");
     }
     h->pending_shift = 0;
@@ -975,6 +976,13 @@ pic_status pic_set_tuning(pic_t* h, int variant) {
     if (!h) return PIC_ERR_ARG;
     if (variant < 0 || variant >= field_variants(h->g.ndim)) return fail(h, PIC_ERR_ARG, "tile variant %d", variant);
     h->fa_variant = variant;
+    return PIC_OK;
+}
+
+pic_status pic_set_wait_limit(pic_t* h, int polls) {
+    if (!h) return PIC_ERR_ARG;
+    if (polls < 0) return fail(h, PIC_ERR_ARG, "pic_set_wait_limit: polls < 0");
+    h->wait_polls = polls;
     return PIC_OK;
 }
 

@@ -114,6 +114,7 @@ struct FiltInst {
 
 // Device status word bits.
 enum : int { STATUS_CAPACITY = 1, STATUS_TIMEOUT = 2 };
+constexpr int WAIT_POLLS = 1 << 20;      // looks of a bounded device-side wait, of up to a microsecond each
 
 #ifdef __CUDACC__
 // ---- chained launches ----
@@ -225,7 +226,7 @@ cudaError_t launch_zero_j_batch(const PartInst* inst, int ninst, long long max_n
 // after launch_push of every species, processes the lists of all of them and clears them.
 constexpr long long defer_len(long long cap) { return 2 + (cap + 255) / 256; }
 cudaError_t launch_push(const GridP& g, const SpeciesP& sp, const float* E, const float* B,
-                        float* J, int shift, int mode, long long extent, int* defer, int* status, cudaStream_t s);
+                        float* J, int shift, int mode, long long extent, int* defer, int* status, int polls, cudaStream_t s);
 cudaError_t launch_push_leftover(const GridP& g, const SpeciesP* sp, int* const* defer, const long long* extent, int n,
                                  const float* E, const float* B, float* J, int shift, cudaStream_t s);
 cudaError_t launch_deposit_unfused(const GridP& g, const SpeciesP& sp, float* J, long long extent,

@@ -283,3 +283,29 @@ def test_counted_launches(nz, nx, copies):
     sim.field_advance()
     assert P.pic_timing_read(sim.h, sim.stream)[1]["fields"] == 1 + copies
     sim.close()
+
+
+def test_wait_for_field_copies_runs_out():
+    """With no look at all the 3D kernel gives up its copies (which do arrive), reports it and returns; the context stays
+    usable, and a handle that has not been limited steps as ever."""
+    import paper_1910_13529_gb300 as P
+    grid = _grid3(48, 16, 16, 2)
+    sp = _patch(600, 48, 16, 16, (9, 5, 5), 1)
+    sim = gpu_sim(grid, [sp])
+    sim.step(1)
+    sim.sync()
+    with pytest.raises(P.PicError):
+        P.pic_set_wait_limit(sim.h, -1)
+    P.pic_set_wait_limit(sim.h, 0)
+    sim.step(1)
+    with pytest.raises(P.PicError) as e:
+        sim.sync()
+    assert "did not arrive" in str(e.value)
+    sim.close()
+    other, osim = gpu_sim(grid, [sp]), oracle_sim(grid, [sp])
+    other.step(2)
+    other.sync()
+    for _ in range(2):
+        osim.step()
+    assert field_error(other, osim) < TOL
+    other.close()
