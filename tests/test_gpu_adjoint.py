@@ -163,3 +163,60 @@ def test_stencil_tuning_lowers_the_wake_energy():
     L_or1 = _oracle_loss(hist["C_final"], grid, sps, nsteps)
     assert L_or1 < L_or0
     assert hist["loss_final"] == pytest.approx(L_or1, rel=1e-4)
+
+
+@pytest.mark.parametrize("ndim,nz,nx,ny,M", [(2, 85, 9, 1, 5), (2, 530, 6, 1, 16), (2, 517, 7, 1, 8), (2, 515, 5, 1, 2),
+                                             (3, 69, 6, 5, 3), (3, 94, 5, 4, 16), (3, 78, 6, 5, 8)])
+def test_adjoint_of_recorded_steps_with_currents(ndim, nz, nx, ny, M):
+    """Three recorded steps of rigid particles in random fields: the correction's gradient and the current in the rebuilt E'
+    take part.  The currents keep the reach of the taps and of the widest box filter away from the z ends, outside of
+    which the adjoint takes the corrected current as zero.  Gradient against FP64 central differences of the oracle (whose correction follows the
+    coefficients), to 1e-4 of its largest entry, the framework's bound; pic_adjoint_run and pic_adjoint_step called
+    step by step give the same gradient and adjoint fields to rounding of FP32."""
+    from parity_util import gpu_sim, oracle_sim
+    C = fit.fit_coefficients(2.5, M=M)
+    d = (0.5, 0.45, 0.4)[:ndim]
+    grid = dict(ndim=ndim, nz=nz, nx=nx, ny=ny, dz=d[0], dx=d[1], dy=d[2] if ndim == 3 else 1.0,
+                dt=0.8 * fit.cfl_dt(d[0], d[1:], C), solver="custom", shape=2)
+    sp = wl.random_particles(ndim, nz, nx, ny, 80, seed=nz + M, u_scale=1.0, u_drift=(3.0, 0, 0), margin=24 + M + 2, m=1e30,
+                             w=0.4)
+    rng = np.random.default_rng(100 * M + nz)
+    shp, n = (3, ny, nx, nz), 3
+    E0, B0, lE, lB = (rng.normal(size=shp).astype(np.float32) for _ in range(4))
+
+    def loss(Cx):
+        osim = oracle_sim(grid, [sp], coef=Cx)
+        osim.E[:], osim.B[:] = E0, B0
+        for _ in range(n):
+            osim.step()
+        return np.sum(lE * osim.E) + np.sum(lB * osim.B), np.abs(osim.J).max()
+
+    ref = np.zeros(M)
+    for l in range(M):
+        h = np.zeros(M)
+        h[l] = 1e-5
+        ref[l] = (loss(C + h)[0] - loss(C - h)[0]) / 2e-5
+    assert loss(C)[1] > 0.05                                  # currents of the size of the fields
+    sim = gpu_sim(grid, [sp], coef=C)
+    dev = lambda a: torch.from_numpy(a).cuda()                                       # noqa: E731
+    E = torch.empty((n + 1, *shp), device="cuda")
+    B, J = torch.empty_like(E), torch.empty((n, *shp), device="cuda")
+    E[0], B[0] = dev(E0), dev(B0)
+    P.pic_step_record(sim.h, n, E.data_ptr(), B.data_ptr(), J.data_ptr(), sim.stream)
+    out = []
+    for one_by_one in (False, True):
+        aE, aB = dev(lE), dev(lB)
+        grad = torch.zeros(M, dtype=torch.float64, device="cuda")
+        if one_by_one:
+            for k in reversed(range(n)):
+                P.pic_adjoint_step(sim.h, E[k].data_ptr(), B[k].data_ptr(), J[k].data_ptr(), aE.data_ptr(), aB.data_ptr(),
+                                   grad.data_ptr(), sim.stream)
+        else:
+            P.pic_adjoint_run(sim.h, n, E.data_ptr(), B.data_ptr(), J.data_ptr(), aE.data_ptr(), aB.data_ptr(),
+                              grad.data_ptr(), sim.stream)
+        torch.cuda.synchronize()
+        out.append((grad.cpu().numpy(), aE.double().cpu().numpy(), aB.double().cpu().numpy()))
+        assert np.abs(out[-1][0] - ref).max() < 1e-4 * np.abs(ref).max()
+    for a, b in zip(out[0], out[1]):
+        assert np.abs(a - b).max() < 1e-5 * np.abs(b).max()
+    sim.close()

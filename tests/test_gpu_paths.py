@@ -292,8 +292,6 @@ def test_wait_for_field_copies_runs_out():
     grid = _grid3(48, 16, 16, 2)
     sp = _patch(600, 48, 16, 16, (9, 5, 5), 1)
     sim = gpu_sim(grid, [sp])
-    sim.step(1)
-    sim.sync()
     with pytest.raises(P.PicError):
         P.pic_set_wait_limit(sim.h, -1)
     P.pic_set_wait_limit(sim.h, 0)
