@@ -206,7 +206,7 @@ pic_status advance_fields(pic_t* h, const float* Ein, const float* Bin, float* E
     p.Bout = Bout;
     p.shift = shift;
     if (h->ks) {
-        Scope sc(h, PIC_T_FIELDS, last ? 1 : 2, s);      // the update, and the copy of the B that is kept
+        Scope sc(h, PIC_T_FIELDS, 1, s);                 // counted once per advance, whatever cuFFT launches
         char kerr[256] = {0};
         if (kspace_advance(h->ks, Ein, Bin, h->J, Eout, Bout, !first, !last, s, kerr, sizeof kerr))
             return fail(h, PIC_ERR_CUDA, "%s", kerr);

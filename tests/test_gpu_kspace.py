@@ -216,3 +216,17 @@ def test_memory_of_a_handle():
         taken.append((before - torch.cuda.mem_get_info()[0]) / (4 * nz * nx))
         P.pic_destroy(h)
     assert taken[1] < 19
+
+
+def test_advances_are_counted_once():
+    """pic_timing_read's count of a k-space run is its advances (and the copies back of an odd number of steps), by which
+    the time per advance is formed."""
+    import paper_1910_13529_gb300 as P
+    sim = gpu_sim(kgrid(2, 48, 20, 1, "spectral"), [])
+    for nsteps in (1, 4, 5):
+        P.pic_timing(sim.h, 1)
+        sim.step(nsteps)
+        _, n = P.pic_timing_read(sim.h, sim.stream)
+        P.pic_timing(sim.h, 0)
+        assert n["fields"] == nsteps + nsteps % 2
+    sim.close()
