@@ -142,7 +142,8 @@ typedef struct pic_config {
                                with [k]_E1 [k]_B1 = [k1]_t^2.  Not supported by pic_adjoint_step. */
     int precision;          /* arithmetic of fields, currents, offsets and momenta: 0 or 32 = FP32
                                (the only one built); any other value is refused with PIC_ERR_ARG.
-                               Diagnostics always reduce in FP64. */
+                               Diagnostics and the adjoint's gradient are summed in FP64 or
+                               wider (parts in FP32 or 64-bit whole numbers). */
 } pic_config;
 
 /* ---- handle ------------------------------------------------------------------------
@@ -230,7 +231,7 @@ pic_status pic_filter_current(pic_t* h, void* stream);
  * columns: consecutive tiles are neighbours); cells z-fastest then x then y inside a tile. */
 pic_status pic_sort(pic_t* h, void* stream);
 
-/* ---- diagnostics (FP64 on the GPU) ----------------------------------------------------
+/* ---- diagnostics (FP64 or wider on the GPU) ---------------------------------------------
  * pic_diag fills out[PIC_DIAG_N] (indices above) and synchronises stream.  The Gauss
  * residual d-.E - rho - rho_bg uses the same d- as Ampere's law (customised stencil
  * included) and skips nodes within (M + hlen + 2) cells of the z ends (2 for Yee), plus 5

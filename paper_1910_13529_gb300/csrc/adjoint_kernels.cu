@@ -83,9 +83,9 @@ __device__ __forceinline__ void scale_by(float (&a)[N], float f) {
 __device__ __forceinline__ bool wide_enough(float top) {
     return __reduce_max_sync(0xffffffffu, __float_as_uint(top)) >= __float_as_uint(1e-18f);
 }
-// Sums of acc[0 .. N) over the lanes at distances O, O / 2, .., 1: a lane hands over half of its sums at each step until
-// it has one left, in the end that of acc[lane MP / 32].  MP + 4 - log2(MP) additions where summing each over the warp takes 5 MP (M = 16: 16
-// and 80).
+// Sums of acc[0 .. N) over the lanes at distances O, O / 2, .., 1: a lane hands over half of its sums at each step
+// until it has one left, in the end that of acc[lane MP / 32].  MP + 4 - log2(MP) additions where summing
+// each over the warp takes 5 MP (M = 16: 16 and 80).
 template <int N, int O, int MP>
 __device__ __forceinline__ void fold_sums(WideSum (&acc)[MP]) {
     if constexpr (O > 0) {

@@ -1,8 +1,9 @@
 // Diagnostics: Gauss residual d-.E - rho - rho_bg (Eq. Gauss of Sec. 2.1, with the same axial d- as Ampere's
 // law), field and kinetic energy.  The divergence and each particle's gamma - 1 are wide sums of FP32 parts
-// (wide_math.h, about 2^-70), which become FP64 where they meet rho and the sums; the rest is FP64 throughout.  With FP64 from the
-// first difference on, the FP64 pipe and its conversions were busy all the time: pic_gauss on 1024 x 256 nodes 39 us
-// (M = 1) and 77 (M = 16), now 29 and 36; on 128 x 64 x 64 with 1e6 particles 126 and 60.
+// (wide_math.h, about 2^-70), which become FP64 where they meet rho and the sums; the rest is FP64
+// throughout.  With FP64 from the first difference on, the FP64 pipe and its conversions were busy all the
+// time: pic_gauss on 1024 x 256 nodes 39 us (M = 1) and 77 (M = 16), now 29 and 36; on 128 x 64 x 64 with 1e6
+// particles 126 and 66.
 #include <cuda_runtime.h>
 
 #include <type_traits>

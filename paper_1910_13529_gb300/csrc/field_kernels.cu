@@ -803,9 +803,10 @@ __device__ __forceinline__ void march_bnew_store(const FieldP& p, const float* e
 // its halo and read two windows of 2 M + 4 floats for four cells (69% of the shared-memory rate, issue
 // 71%).  Before and now, us per advance, best segment length: 8192 x 2048 Yee 188 and 163 (91% of the
 // copy bandwidth), M = 16 240 and 213 (69%); 4099 x 1030 M = 16 145 and 91 (rows not 16-byte aligned);
-// 4096 x 1024 M = 16 84 and 64.  64 threads win everywhere: fewer barrier partners outweigh the
-// 6 D lanes of a segment that produce nothing.  Below about 1e6 cells the blocked tiles are faster
-// (one row at a time is a serial chain).
+// 4096 x 1024 M = 16 84 and 64.  64 threads are the default (fewer barrier partners outweigh the 6 D lanes
+// of a segment that produce nothing); 96 are up to 10% faster on rows of 512 and 700 cells, 128 and 256 on none
+// measured, but pic_set_tuning takes their numbers.  Below about 2e6 cells the blocked tiles are faster (one
+// row at a time is a serial chain).
 constexpr int ROW_Z = 8;                                       // cells of a lane
 constexpr int ROW_G = 5;                                       // 16-byte groups of a lane's pairs
 

@@ -506,7 +506,8 @@ struct Never {
 // Boxes larger than the shared-memory caps fall back to global loads / global atomics.  That path (runs without
 // sorts, sparse species, every batch) lives on L1: with 48 KB per CTA the four of an SM left it 28 KB, and a batch of
 // 16 x 256 x 128 cells, 4 per cell, unsorted, took 692 us a step (linear) and 1651 (quadratic); at 41 KB, 270 and
-// 690.  2048 x 512, 4.2e6 unsorted: 776 and 473 us (linear), 1658 and 1060 (quadratic).  Sorted: 157 and 162, 208 and 208.
+// 690.  2048 x 512, 4.2e6 unsorted: 776 and 473 us (linear), 1658 and 1060 (quadratic); sorted 157 and 162, 208
+// and 208.
 constexpr int F_CAP = 4032;        // field box floats (6 components): four CTAs leave 92 KB of L1 to an SM
 constexpr int J_CAP = 3 * 1024;    // current box floats (3 components)
 constexpr int PF2 = 6;             // prefetched words per particle (cell, 2 offsets, 3 momenta)
