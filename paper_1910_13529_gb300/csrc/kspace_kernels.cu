@@ -19,7 +19,8 @@
 // itself, the scaled B after E's inverse transform, by a pass of its own, so that a handle needs no more memory
 // than one that transforms everything (room for both copies, 15 arrays, saves that pass: 512 x 256, eight steps
 // 310 us for 335; everything transformed: 440).  us per call, everything transformed and now: four steps of 2048 x 512
-// (spectral) 488 and 380, two of 256 x 128 x 128 (PSATD) 826 and 720.
+// (spectral) 488 and 380, two of 256 x 128 x 128 (PSATD) 826 and 720; an advance of many, 8192 x 2048 1.24 ms and
+// 0.92 (0.88 with 15 arrays), 512 x 256 x 256 2.9 and 2.11 (2.04).
 #include "pic_internal.h"
 
 #include <cmath>
